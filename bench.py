@@ -190,6 +190,8 @@ def kernel_specs(wl, peaks, sustained, D=None, n_keep=None, cache_rows=None):
         "decode_logits": ("hbm", cache_rows * (d * s + wl.G * 4.0) / 1e9 if cache_rows else None, hbm, "GB/s"),
         "decode_accumulate": ("hbm", cache_rows * (wl.G * 4.0 + 12.0) / 1e9 if cache_rows else None, hbm, "GB/s"),
         "decode_commit": ("hbm", None, None, None),
+        # the same in one launch, the logits in shared memory
+        "decode_step": ("hbm", cache_rows * (d * s + 12.0) / 1e9 if cache_rows else None, hbm, "GB/s"),
         "prepare_vote": ("alu", None, None, None),
         "prepare_finish": ("alu", None, None, None),
         "wide_gram": ("tensor", None, None, None),

@@ -128,13 +128,22 @@ def _check(code: int, where: str) -> None:
         raise UncompError(code, where)
 
 
+# A call's host time is mostly argument marshalling (a decode step takes a dozen tensors and a few microseconds on the
+# device), so pointers and streams go to ctypes as plain integers, and the current stream's handle is asked for without
+# building a torch.cuda.Stream around it.
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream: Optional[torch.cuda.Stream]):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def make_shape(B, L, H, Hq, N, d, w, dtype) -> uncomp_shape:
@@ -144,9 +153,10 @@ def make_shape(B, L, H, Hq, N, d, w, dtype) -> uncomp_shape:
 
 def strides_of(t: torch.Tensor) -> uncomp_strides:
     """Element strides of a [B, L, H, N, d] tensor (d contiguous)."""
-    if t.dim() != 5 or t.stride(4) != 1:
+    st = t.stride()
+    if len(st) != 5 or st[4] != 1:
         raise ValueError("expected a [B, L, H, N, d] tensor with a contiguous last dimension")
-    return uncomp_strides(t.stride(0), t.stride(1), t.stride(2), t.stride(3))
+    return uncomp_strides(st[0], st[1], st[2], st[3])
 
 
 def uncomp_workspace_bytes(shape: uncomp_shape) -> int:

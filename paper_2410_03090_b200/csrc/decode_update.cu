@@ -11,13 +11,16 @@
 //               scores: the lower position; no such entry: every cached entry is a candidate) and the new
 //               token takes its row, so the slab is not kept in position order: `pos` names each row.
 //
-// The step is bound by reading the cached keys once.  Three launches:
+// The step is bound by reading the cached keys once.  One launch while the logits of a unit fit into the shared memory
+// of a cluster (decode_step_kernel below); otherwise three:
 //   1. logits      grid (chunks of 1024 entries, units): the G logits of every entry (log2 domain) to scratch,
 //                  per chunk the softmax statistics (max, sum of 2^(x - max)) per query head;
 //   2. accumulate  same grid: merges the chunk statistics, forms p, updates cum, and leaves per chunk the
 //                  lexicographic minimum of (cum, pos) over the candidates and over all entries;
 //   3. commit      one small CTA per unit: picks the row, copies the new key / value rows, updates pos, cum, len.
 // Positions are unique inside a unit, so every minimum is unique and no result depends on thread order.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 
 namespace uncomp {
@@ -346,6 +349,340 @@ __global__ void __launch_bounds__(64) decode_commit_kernel(DecArgs a, int H_per_
     if (tid < 32) { if (tid < vecs) dstK[tid] = srcK[tid]; }
     else if (tid - 32 < vecs) dstV[tid - 32] = srcV[tid - 32];
 }
+// ---- the whole step in one launch: a cluster of CTAs per unit ---------------------------------------------------
+// Bound by reading the cached keys once.  A unit is one CTA, or a cluster of 2, 4 or 8 when its cache is large or the
+// units are few.  The logits stay in shared memory between the statistics and the probabilities; softmax statistics and
+// eviction minima of a cluster meet in distributed shared memory, and CTA 0 writes the new token.  Three CTAs per SM are
+// in different phases, so the latency of the barriers hides behind other units' loads; scores, positions and the new
+// token's row are prefetched past the barriers.  Against three launches over a logits array in global memory (device
+// time, back to back): 1024 caches of 3080 rows 194 -> 145 us = 5.9 TB/s of keys, scores and positions, 256 caches of
+// 410 rows 16.0 -> 8.2 us.
+constexpr int kStepMaxCluster = 8;
+constexpr int kPre = 3;                                  // entries per thread whose score and position are prefetched
+constexpr size_t kStepSmem = 200 * 1024;                 // logits of one CTA's share at most
+
+struct StepSmem {
+    unsigned long long wkey[kDecWarps][2];
+    float red_m[kDecWarps][16], red_l[kDecWarps][16];
+    float stat_m[16], stat_l[16];                        // this CTA's softmax statistics per head
+    float mprime[16];
+    unsigned long long key[kStepMaxCluster][2];          // CTA 0: smallest (cum, pos) of every CTA, old enough / any
+    int32_t slot[kStepMaxCluster][2];
+    float new_cum;                                       // CTA 0
+    int row;
+};
+
+// order-preserving image of (cum, pos): the lexicographic minimum is the smallest key
+__device__ __forceinline__ unsigned long long min_key(float c, int32_t pos) {
+    const uint32_t b = __float_as_uint(c + 0.f);         // -0 and +0 are equal scores
+    const uint32_t o = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+    return ((unsigned long long)o << 32) | (uint32_t)pos;
+}
+__device__ __forceinline__ unsigned long long warp_min(unsigned long long v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
+// logits of the entries t0 .. t1 - 1 to lg[head * pitch + t - t0]; running (max, sum) of this thread's heads
+template <int G>
+__device__ __forceinline__ void step_logits(const DecArgs &a, int u, int64_t off, int len, int t0, int t1, float *lg, int pitch,
+                                            StepSmem &S, __nv_bfloat16) {
+    constexpr int NB = (G + 7) / 8;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, gid = lane >> 2, tig = lane & 3;
+    const __nv_bfloat16 *qb = (const __nv_bfloat16 *)a.q + (size_t)u * G * kD;
+    const __nv_bfloat16 *Kb = (const __nv_bfloat16 *)a.Kc + off * kD;
+    const __nv_bfloat16 *kn = (const __nv_bfloat16 *)a.knew + (size_t)u * kD;
+    uint32_t bq[NB][16];
+#pragma unroll
+    for (int nb = 0; nb < NB; ++nb) {
+        const int h = nb * 8 + gid;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            uint4 x = make_uint4(0u, 0u, 0u, 0u);
+            if (h < G) x = reinterpret_cast<const uint4 *>(qb + (size_t)h * kD)[4 * j + tig];
+            bq[nb][4 * j] = x.x; bq[nb][4 * j + 1] = x.y; bq[nb][4 * j + 2] = x.z; bq[nb][4 * j + 3] = x.w;
+        }
+    }
+    float m_run[NB][2], l_run[NB][2];
+#pragma unroll
+    for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) { m_run[nb][i] = -1e30f; l_run[nb][i] = 0.f; }
+    for (int base = t0 + wid * 32; base < t1; base += kDecWarps * 32) {
+        uint4 ka[2][2][4];
+#pragma unroll
+        for (int tile = 0; tile < 2; ++tile)
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                const int row = base + tile * 16 + half * 8 + gid;
+                const uint4 *src = reinterpret_cast<const uint4 *>(row < len ? Kb + (int64_t)row * kD : kn);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) ka[tile][half][j] = row < t1 ? src[4 * j + tig] : make_uint4(0u, 0u, 0u, 0u);
+            }
+#pragma unroll
+        for (int tile = 0; tile < 2; ++tile)
+#pragma unroll
+            for (int nb = 0; nb < NB; ++nb) {
+                float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint4 lo = ka[tile][0][j], hi = ka[tile][1][j];
+                    mma_bf16_16816(acc, lo.x, hi.x, lo.y, hi.y, bq[nb][4 * j], bq[nb][4 * j + 1]);
+                    mma_bf16_16816(acc, lo.z, hi.z, lo.w, hi.w, bq[nb][4 * j + 2], bq[nb][4 * j + 3]);
+                }
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int h = nb * 8 + 2 * tig + i;
+                    if (h < G) {
+#pragma unroll
+                        for (int half = 0; half < 2; ++half) {
+                            const int t = base + tile * 16 + half * 8 + gid;
+                            if (t < t1) {
+                                const float v = acc[2 * half + i] * a.c_log2;
+                                lg[h * pitch + t - t0] = v;
+                                const float m_new = fmaxf(m_run[nb][i], v);
+                                l_run[nb][i] = fmaf(l_run[nb][i], ex2f(m_run[nb][i] - m_new), ex2f(v - m_new));
+                                m_run[nb][i] = m_new;
+                            }
+                        }
+                    }
+                }
+            }
+    }
+    // over the 8 row lanes, then one value per warp and head
+#pragma unroll
+    for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            float m = m_run[nb][i], l = l_run[nb][i];
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1) {
+                const float mo = __shfl_xor_sync(0xffffffffu, m, o), lo = __shfl_xor_sync(0xffffffffu, l, o);
+                const float mn = fmaxf(m, mo);
+                l = l * ex2f(m - mn) + lo * ex2f(mo - mn);
+                m = mn;
+            }
+            const int h = nb * 8 + 2 * tig + i;
+            if (gid == 0 && h < G) { S.red_m[wid][h] = m; S.red_l[wid][h] = l; }
+        }
+}
+
+template <int G>
+__device__ __forceinline__ void step_logits(const DecArgs &a, int u, int64_t off, int len, int t0, int t1, float *lg, int pitch,
+                                            StepSmem &S, float) {
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const float4 *q4 = reinterpret_cast<const float4 *>((const float *)a.q + (size_t)u * G * kD) + lane;
+    float4 q[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) q[g] = q4[g * (kD / 4)];
+    const float *Kb = (const float *)a.Kc + off * kD;
+    const float *kn = (const float *)a.knew + (size_t)u * kD;
+    float m_run = -1e30f, l_run = 0.f;                   // lane g < G keeps the statistics of head g
+    for (int t = t0 + wid; t < t1; t += kDecWarps) {
+        const float4 k4 = *reinterpret_cast<const float4 *>((t < len ? Kb + (int64_t)t * kD : kn) + lane * 4);
+        float mine = 0.f;
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            float v = fmaf(k4.x, q[g].x, fmaf(k4.y, q[g].y, fmaf(k4.z, q[g].z, k4.w * q[g].w)));
+            v = warp_sum(v) * a.c_log2;
+            if (lane == g) mine = v;
+        }
+        if (lane < G) {
+            lg[lane * pitch + t - t0] = mine;
+            const float m_new = fmaxf(m_run, mine);
+            l_run = fmaf(l_run, ex2f(m_run - m_new), ex2f(mine - m_new));
+            m_run = m_new;
+        }
+    }
+    if (lane < G) { S.red_m[wid][lane] = m_run; S.red_l[wid][lane] = l_run; }
+}
+
+struct StepArgs {
+    const int32_t *new_pos;
+    const void *vnew;
+    void *Kc, *Vc;
+    int32_t *pos, *lens, *evicted;
+    float *cum, *p_out;
+    uint32_t *status;
+    int H_per_seq, protect, pitch;
+};
+
+template <int G, typename T>
+__global__ void __launch_bounds__(kDecThreads, 3) decode_step_kernel(DecArgs a, StepArgs b) {
+    namespace cg = cooperative_groups;
+    __shared__ StepSmem S;
+    extern __shared__ float lg[];                        // [G][pitch]
+    cg::cluster_group cluster = cg::this_cluster();
+    const int ctas = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int u = blockIdx.x / ctas, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    // the new token's row and position are not needed before the end: on their way from the start
+    constexpr int kVecs = kD * (int)sizeof(T) / 16;      // 16-byte vectors per row
+    int4 fresh = make_int4(0, 0, 0, 0);
+    if (rank == 0 && tid < 2 * kVecs)
+        fresh = (reinterpret_cast<const int4 *>(tid < kVecs ? a.knew : b.vnew) + (size_t)u * kVecs)[tid % kVecs];
+    const int32_t newest = b.new_pos[u / b.H_per_seq], limit = newest - b.protect;     // candidates have pos <= limit
+    int64_t off;
+    int len;
+    if (!unit_ok(a, u, off, len)) {                      // uniform over the cluster
+        if (tid == 0 && rank == 0) {
+            atomicOr(b.status, (uint32_t)UNCOMP_STATUS_BOUNDS);
+            if (b.evicted) b.evicted[u] = -1;
+        }
+        return;
+    }
+    const int64_t cap = a.offsets[u + 1] - off;
+    const bool full = len >= cap;
+    const int n = len + 1, share = (n + ctas - 1) / ctas;
+    const int t0 = min(n, rank * share), t1 = min(n, t0 + share);
+    StepSmem *S0 = cluster.map_shared_rank(&S, 0);
+
+    // ---- logits, softmax statistics over the cluster -------------------------------------------------
+    step_logits<G>(a, u, off, len, t0, t1, lg, b.pitch, S, T());
+    // cumulative scores and positions of this thread's first entries are on their way during the barriers
+    float c_pre[kPre];
+    int32_t p_pre[kPre];
+#pragma unroll
+    for (int i = 0; i < kPre; ++i) {
+        const int j = t0 + tid + i * kDecThreads;
+        c_pre[i] = j < t1 && j < len ? b.cum[off + j] : 0.f;
+        p_pre[i] = j < t1 && j < len ? b.pos[off + j] : 0;
+    }
+    __syncthreads();
+    if (tid < G) {
+        float m = -1e30f, l = 0.f;
+#pragma unroll
+        for (int x = 0; x < kDecWarps; ++x) m = fmaxf(m, S.red_m[x][tid]);
+#pragma unroll
+        for (int x = 0; x < kDecWarps; ++x) l += S.red_l[x][tid] * ex2f(S.red_m[x][tid] - m);
+        S.stat_m[tid] = m;
+        S.stat_l[tid] = l;
+        if (ctas == 1) S.mprime[tid] = m + log2f(l);
+    }
+    if (ctas > 1) {
+        cluster.sync();
+        if (tid < G) {
+            float m[kStepMaxCluster], l[kStepMaxCluster], top = -1e30f, sum = 0.f;
+#pragma unroll
+            for (int c = 0; c < kStepMaxCluster; ++c) {
+                const StepSmem *Sc = cluster.map_shared_rank(&S, c < ctas ? c : 0);
+                m[c] = c < ctas ? Sc->stat_m[tid] : -1e30f;
+                l[c] = c < ctas ? Sc->stat_l[tid] : 0.f;
+            }
+#pragma unroll
+            for (int c = 0; c < kStepMaxCluster; ++c) top = fmaxf(top, m[c]);
+#pragma unroll
+            for (int c = 0; c < kStepMaxCluster; ++c) sum += l[c] * exp2f(m[c] - top);
+            S.mprime[tid] = top + log2f(sum);
+        }
+    }
+    __syncthreads();
+
+    // ---- probabilities, cumulative scores, the lowest of this CTA -------------------------------------
+    float mp[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) mp[g] = S.mprime[g];
+    unsigned long long best_el = ~0ull, best_any = ~0ull;
+    int j_el = -1, j_any = -1;
+    auto entry = [&](int j, float c_old, int32_t ps) {
+        float p = 0.f;                                   // heads in ascending order
+#pragma unroll
+        for (int g = 0; g < G; ++g) p += ex2f(lg[g * b.pitch + j - t0] - mp[g]);
+        if (b.p_out) b.p_out[off + u + j] = p;
+        if (j < len) {
+            const float cn = c_old + p;
+            b.cum[off + j] = cn;
+            if (full) {
+                const unsigned long long k = min_key(cn, ps);
+                if (k < best_any) { best_any = k; j_any = j; }
+                if (ps <= limit && k < best_el) { best_el = k; j_el = j; }
+            }
+        } else {
+            S0->new_cum = p;
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < kPre; ++i) {
+        const int j = t0 + tid + i * kDecThreads;
+        if (j < t1) entry(j, c_pre[i], p_pre[i]);
+    }
+#pragma unroll 4
+    for (int j = t0 + tid + kPre * kDecThreads; j < t1; j += kDecThreads)
+        entry(j, j < len ? b.cum[off + j] : 0.f, j < len ? b.pos[off + j] : 0);
+    if (full) {
+        const unsigned long long we = warp_min(best_el), wa = warp_min(best_any);
+        if (lane == 0) { S.wkey[wid][0] = we; S.wkey[wid][1] = wa; }
+        __syncthreads();
+        unsigned long long be = ~0ull, ba = ~0ull;
+#pragma unroll
+        for (int x = 0; x < kDecWarps; ++x) { be = min(be, S.wkey[x][0]); ba = min(ba, S.wkey[x][1]); }
+        // keys are unique inside a unit: the one thread that holds the minimum names its row
+        if (be != ~0ull ? best_el == be : tid == 0) { S0->key[rank][0] = be; S0->slot[rank][0] = j_el; }
+        if (ba != ~0ull ? best_any == ba : tid == 0) { S0->key[rank][1] = ba; S0->slot[rank][1] = j_any; }
+    }
+    if (ctas > 1) cluster.sync();
+    else __syncthreads();
+    if (rank != 0) return;
+
+    // ---- the new token takes its row -----------------------------------------------------------------
+    if (tid == 0) {
+        int slot = len, gone = -1;
+        if (full) {
+            unsigned long long k[2] = {~0ull, ~0ull};
+            int s[2] = {-1, -1};
+            for (int c = 0; c < ctas; ++c)
+                for (int w = 0; w < 2; ++w)
+                    if (S.key[c][w] < k[w]) { k[w] = S.key[c][w]; s[w] = S.slot[c][w]; }
+            const int w = s[0] >= 0 ? 0 : 1;
+            slot = s[w];
+            gone = (int32_t)(uint32_t)k[w];
+        } else {
+            b.lens[u] = len + 1;
+        }
+        if (!UNCOMP_INDEX_OK(slot, cap, b.status)) slot = -1;     // debug library: the row must lie in the unit's slab
+        if (slot >= 0) {
+            b.pos[off + slot] = newest;
+            b.cum[off + slot] = S.new_cum;
+        }
+        if (b.evicted) b.evicted[u] = gone;
+        S.row = slot;
+    }
+    __syncthreads();
+    if (S.row < 0) return;                               // only the debug library can get here
+    if (tid < 2 * kVecs)
+        (reinterpret_cast<int4 *>(tid < kVecs ? b.Kc : b.Vc) + (off + S.row) * kVecs)[tid % kVecs] = fresh;
+}
+
+template <int G, typename T>
+cudaError_t launch_step(const DecArgs &a, const StepArgs &b, int units, int ctas, size_t smem, cudaStream_t st) {
+    static bool done[64] = {};
+    cudaError_t e = allow_dynamic_smem((const void *)decode_step_kernel<G, T>, kStepSmem, done);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = ctas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(units * ctas);
+    cfg.blockDim = dim3(kDecThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = ctas > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, decode_step_kernel<G, T>, a, b);
+}
+template <typename T>
+cudaError_t launch_step_g(const DecArgs &a, const StepArgs &b, int units, int ctas, size_t smem, cudaStream_t st) {
+    switch (a.G) {
+        case 1: return launch_step<1, T>(a, b, units, ctas, smem, st);
+        case 2: return launch_step<2, T>(a, b, units, ctas, smem, st);
+        case 4: return launch_step<4, T>(a, b, units, ctas, smem, st);
+        case 8: return launch_step<8, T>(a, b, units, ctas, smem, st);
+        case 16: return launch_step<16, T>(a, b, units, ctas, smem, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
 // Cumulative scores right after prefill: a kept prefix position takes its prefill score, a window position the
 // largest score among the kept prefix positions of its head (0 if there is none).  One CTA per unit.
 __global__ void __launch_bounds__(256) decode_seed_kernel(const float *__restrict__ scores, int P,
@@ -396,6 +733,28 @@ cudaError_t launch_decode_update(const Plan &p, const void *d_q, const void *d_k
     a.units = p.units; a.G = p.G; a.max_cap = max_cap; a.chunks_max = decode_chunks(max_cap);
     a.c_log2 = scale * 1.4426950408889634f;
     a.logits = d_logits; a.stats = d_stats;
+    {
+        // One launch with the logits in shared memory.  A cluster barrier costs a microsecond of a CTA's time, so a unit
+        // stays on one CTA up to 4096 entries (64 KB of logits at 4 heads, three CTAs per SM); beyond, the cluster grows
+        // to 8 CTAs, then the share.  Only where the units leave half the SMs idle smaller shares pay.
+        int ctas = 1;
+        while (ctas < kStepMaxCluster && (max_cap + 1 > 4096 * ctas ||
+                                          ((int64_t)p.units * ctas * 2 <= kTargetSms && max_cap + 1 > 512 * ctas)))
+            ctas *= 2;
+        const int share = (max_cap + 1 + ctas - 1) / ctas;
+        StepArgs b;
+        b.pitch = (share + 31) / 32 * 32 + 8;            // heads 8 banks apart
+        const size_t smem = (size_t)b.pitch * p.G * sizeof(float);
+        if (smem <= kStepSmem) {
+            b.new_pos = d_new_pos; b.vnew = d_vnew; b.Kc = d_Kc; b.Vc = d_Vc; b.pos = d_pos; b.lens = d_lens;
+            b.evicted = d_evicted; b.cum = d_cum; b.p_out = d_p; b.status = d_status;
+            b.H_per_seq = s.L * s.H; b.protect = protect;
+            ProfScope ps(prof, kSlotDecodeStep, st);
+            return s.dtype == UNCOMP_FP32 ? launch_step_g<float>(a, b, p.units, ctas, smem, st)
+                                          : launch_step_g<__nv_bfloat16>(a, b, p.units, ctas, smem, st);
+        }
+    }
+    // caches whose logits do not fit into the shared memory of a cluster: three launches over a global logits array
     const dim3 grid(a.chunks_max, p.units);
     const int row_bytes = kD * (s.dtype == UNCOMP_FP32 ? 4 : 2);
     {
