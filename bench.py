@@ -198,6 +198,7 @@ def kernel_specs(wl, peaks, sustained, D=None, n_keep=None, cache_rows=None):
         "wide_assemble": ("hbm", None, None, None),
         "wide_tridiag": ("alu", None, None, None),
         "wide_eigen_entropy": ("alu", None, None, None),
+        "wide_krylov": ("alu", None, None, None),
     }
 
 
@@ -770,7 +771,7 @@ def run_wide(args):
             ach = flops_gram / 1e12 / (avg / 1e3)
             ent_k.update({"bound": "tensor", "achieved": round(ach, 1), "peak": peaks["bf16_sustained"], "unit": "TFLOP/s",
                           "frac": round(ach / peaks["bf16_sustained"], 4)})
-        elif name == "wide_tridiag":
+        elif name == "wide_tridiag" and avg > 0.1:      # it leaves at once when block Lanczos has converged
             # the trailing matrix is read and written once per column: (2/3) D^3 floats each way
             gb = 2.0 * (Dt ** 3) / 3.0 * 4 / 1e9
             ent_k.update({"bound": "l2", "achieved": round(gb / (avg / 1e3), 1), "peak": round(l2_peak, 1),

@@ -239,7 +239,7 @@ const char *uncomp_profile_slot_name(int slot) {
                                             "decode_logits", "decode_accumulate", "decode_commit",
                                             "prepare_vote", "prepare_finish",
                                             "wide_gram", "wide_assemble", "wide_tridiag", "wide_eigen_entropy",
-                                            "gram_score_colsum", "decode_step"};
+                                            "gram_score_colsum", "decode_step", "wide_krylov"};
     return slot >= 0 && slot < kSlotCount ? names[slot] : "";
 }
 

@@ -122,7 +122,7 @@ inline cudaError_t allow_dynamic_smem(const void *fn, size_t bytes, bool (&done)
 enum Slot { kSlotGram = 0, kSlotEigen, kSlotBudgets, kSlotScoreStats, kSlotStatsMerge, kSlotScoreColsum,
             kSlotPoolSelect, kSlotCompact, kSlotGramStats, kSlotEvictLogits, kSlotEvictScores, kSlotEvictGather,
             kSlotDecodeLogits, kSlotDecodeAccumulate, kSlotDecodeCommit, kSlotPrepareVote,
-            kSlotPrepareFinish, kSlotWideGram, kSlotWideAssemble, kSlotWideTridiag, kSlotWideSturm, kSlotGramColsum, kSlotDecodeStep, kSlotCount };
+            kSlotPrepareFinish, kSlotWideGram, kSlotWideAssemble, kSlotWideTridiag, kSlotWideSturm, kSlotGramColsum, kSlotDecodeStep, kSlotWideKrylov, kSlotCount };
 enum { kScorePhaseStats = 1, kScorePhaseColsum = 2 };
 struct Profiler;
 void prof_begin(Profiler *p, int slot, cudaStream_t st);

@@ -22,7 +22,9 @@
 // poll limit after which the kernel raises UNCOMP_STATUS_TIMEOUT and all CTAs leave.
 #include <math.h>
 
+#include "grid_barrier.cuh"
 #include "tc_common.cuh"
+#include "wide_krylov.cuh"
 
 namespace uncomp {
 
@@ -303,7 +305,6 @@ __global__ void __launch_bounds__(256) wide_rowdot_kernel(const __nv_bfloat16 *_
 // ------------------------------------------------------------------------------------- 4. tridiagonalisation
 constexpr int kTriThreads = 1024;
 constexpr int kTriWarps = kTriThreads / 32;
-constexpr unsigned kBarrierSpin = 1u << 22;
 
 // Three block-wide sums at once; every thread gets the totals.  Warp 0 adds the per-warp sums (a butterfly: a fixed
 // order) and publishes them.  `red` must not be the array of the previous call: the calls alternate between two
@@ -325,27 +326,6 @@ __device__ __forceinline__ void tri_block_sum3(float &x, float &y, float &z, flo
     z = red[2][kTriWarps];
 }
 
-// All CTAs of a cooperative launch meet here.  `bar` counts arrivals monotonically.
-__device__ __forceinline__ bool tri_grid_barrier(unsigned *bar, unsigned &phase, uint32_t *status, int *flag) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(bar, 1u);
-        const unsigned target = (phase + 1u) * gridDim.x;
-        bool ok = false;
-        for (unsigned it = 0; it < kBarrierSpin; ++it) {
-            unsigned cur;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(cur) : "l"(bar) : "memory");
-            if (cur >= target) { ok = true; break; }
-        }
-        if (!ok) atomicOr(status, (uint32_t)UNCOMP_STATUS_TIMEOUT);
-        *flag = ok ? 1 : 0;
-    }
-    __syncthreads();
-    ++phase;
-    return *flag != 0;
-}
-
 // A: full symmetric fp32 matrix [D, D], destroyed.  Output: diagonal a[D] and off-diagonal e[D - 1].
 // State at the top of iteration k: rows >= k of A hold the matrix after the reflections of columns 0 .. k - 2;
 // the rank-2 update of column k - 1, A -= 2 (v w^T + w v^T) on rows and columns >= k, is still pending: its
@@ -356,8 +336,13 @@ constexpr int kTriQ = 4;   // columns per thread: D <= kTriQ * kTriThreads
 
 __global__ void __launch_bounds__(kTriThreads, 1) tridiag_wide_kernel(float *__restrict__ A, int D, double *__restrict__ a_out,
                                                                      double *__restrict__ e_out, float *__restrict__ pbuf,
-                                                                     unsigned *bar, uint32_t *__restrict__ status) {
+                                                                     unsigned *bar, int *kry, const double *lam, int k_wanted,
+                                                                     uint32_t *__restrict__ status) {
     extern __shared__ float sm[];
+    if (kry && krylov_done(kry, lam, k_wanted)) {          // the same answer in every CTA
+        if (blockIdx.x == 0 && threadIdx.x == 0) kry[2] = 1;
+        return;
+    }
     float *v = sm, *w = sm + D, *vn = sm + 2 * D;
     __shared__ float redA[3][kTriWarps + 1], redB[3][kTriWarps + 1];
     __shared__ int flag;
@@ -451,7 +436,7 @@ __global__ void __launch_bounds__(kTriThreads, 1) tridiag_wide_kernel(float *__r
             acc = warp_sum(acc);
             if (lane == 0) __stcg(pw + i, acc);
         }
-        if (!tri_grid_barrier(bar, phase, status, &flag)) return;
+        if (!grid_barrier(bar, phase, status, &flag)) return;
     }
     // the last 2 x 2 block: its pending update comes from column D - 3
     if (blockIdx.x == 0 && tid == 0) {
@@ -516,8 +501,9 @@ __device__ int sturm_count_wide(const double *__restrict__ a, const double *__re
 // grid (k): CTA t finds the t-th largest eigenvalue by 256-section (every CTA repeats the cheap set-up);
 // lam_out[t] and, from CTA 0, the trace in lam_out[k]
 __global__ void __launch_bounds__(kSturmThreads) sturm_wide_kernel(const double *__restrict__ a, const double *__restrict__ e,
-                                                                  int D, int k, int max_iters, double *__restrict__ lam_out,
+                                                                  int D, int k, int max_iters, const int *kry, double *__restrict__ lam_out,
                                                                   uint32_t *__restrict__ status) {
+    if (kry && kry[2]) return;                             // set by the launch before this one
     __shared__ double redlo[kSturmThreads / 32], redhi[kSturmThreads / 32], redtr[kSturmThreads / 32];
     __shared__ int redc[kSturmThreads / 32];
     __shared__ double bounds[3];
@@ -582,25 +568,30 @@ __global__ void __launch_bounds__(kSturmThreads) sturm_wide_kernel(const double 
 }
 
 // H_k and erank_k from the kf largest eigenvalues (descending; eigenvalues kf .. k - 1 are zero) and the trace at
-// lam[kf]
-__global__ void wide_entropy_kernel(const double *__restrict__ lam, int k, int kf, int norm, float *__restrict__ H_out,
-                                    float *__restrict__ erank_out, double *__restrict__ spectrum) {
-    if (threadIdx.x != 0) return;
+// lam[kf]; one warp, lane i takes eigenvalues i, i + 32, ...
+__global__ void __launch_bounds__(32) wide_entropy_kernel(const double *__restrict__ lam, int k, int kf, int norm,
+                                                         float *__restrict__ H_out, float *__restrict__ erank_out,
+                                                         double *__restrict__ spectrum) {
+    const int lane = threadIdx.x;
     double denom = 0.0;
     if (norm == 0) {
-        for (int i = 0; i < kf; ++i) denom += fmax(lam[i], 0.0);
+        for (int i = lane; i < kf; i += 32) denom += fmax(lam[i], 0.0);
+        denom = warp_sum(denom);
     } else {
         denom = lam[kf];
     }
     double h = 0.0;
-    for (int i = 0; i < kf; ++i) {
+    for (int i = lane; i < kf; i += 32) {
         const double pi = denom > 0.0 ? fmax(lam[i], 0.0) / denom : 0.0;
         if (pi > 0.0) h -= pi * log(pi);
     }
-    *H_out = (float)h;
-    if (erank_out) *erank_out = (float)exp(h);
+    h = warp_sum(h);
+    if (lane == 0) {
+        *H_out = (float)h;
+        if (erank_out) *erank_out = (float)exp(h);
+    }
     if (spectrum)
-        for (int i = 0; i < k; ++i) spectrum[i] = i < kf ? lam[i] : 0.0;
+        for (int i = lane; i < k; i += 32) spectrum[i] = i < kf ? lam[i] : 0.0;
 }
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -609,7 +600,9 @@ struct WideLayout {
     bool dual;          // token-space path (N < D)
     int Dt;             // size of the symmetric matrix that is tridiagonalised
     int nblk, pairs, chunk, chunks;
-    size_t off_bar, off_s, off_colpart, off_a, off_e, off_lam, off_g, off_p, off_C, off_part, bytes;
+    size_t off_bar, off_s, off_colpart, off_a, off_e, off_lam, off_g, off_p, off_C, off_part;
+    size_t off_state, off_Q, off_kpart, off_H, off_G, off_T;      // block Lanczos
+    size_t zero_bytes, bytes;
 };
 
 WideLayout wide_layout(int N, int D) {
@@ -627,16 +620,25 @@ WideLayout wide_layout(int N, int D) {
     w.chunk = (((contract + chunks - 1) / chunks) + kWTok - 1) / kWTok * kWTok;
     w.chunks = (contract + w.chunk - 1) / w.chunk;
     size_t o = 0;
+    // cleared before every matrix: barrier counters, block Lanczos state, eigenvalues
     w.off_bar = o;      o = align256(o + 256);
+    w.off_state = o;    o = align256(o + kKryStateInts * sizeof(int));
+    w.off_lam = o;      o = align256(o + (size_t)(kSturmMaxK + 1) * sizeof(double));
+    w.zero_bytes = o;
     w.off_s = o;        o = align256(o + (size_t)D * sizeof(double));
     w.off_colpart = o;  o = align256(o + (size_t)kColChunks * D * sizeof(double));
     w.off_a = o;        o = align256(o + (size_t)w.Dt * sizeof(double));
     w.off_e = o;        o = align256(o + (size_t)w.Dt * sizeof(double));
-    w.off_lam = o;      o = align256(o + (size_t)(kSturmMaxK + 1) * sizeof(double));
     w.off_g = o;        o = align256(o + (size_t)(w.Dt + 1) * sizeof(double));
     w.off_p = o;        o = align256(o + (size_t)2 * w.Dt * sizeof(float));
     w.off_C = o;        o = align256(o + (size_t)w.Dt * w.Dt * sizeof(float));
     w.off_part = o;     o = align256(o + (size_t)w.chunks * w.pairs * 2 * 128 * kWBlock * sizeof(float));
+    const size_t steps = krylov_steps(w.Dt);
+    w.off_Q = o;        o = align256(o + (steps ? (steps + 1) * kKryBlock * w.Dt * sizeof(float) : 0));
+    w.off_kpart = o;    o = align256(o + (steps ? (steps + 3) * (w.Dt / kKryBlock) * kKryBlock * kKryBlock * sizeof(float) : 0));
+    w.off_H = o;        o = align256(o + (steps + 1) * kKryBlock * kKryBlock * sizeof(float));
+    w.off_G = o;        o = align256(o + kKryBlock * kKryBlock * sizeof(double));
+    w.off_T = o;        o = align256(o + (steps + 1) * kKryBlock * kKryBand * sizeof(double));
     w.bytes = o;
     return w;
 }
@@ -664,7 +666,7 @@ cudaError_t launch_entropy_wide(const void *d_X, int64_t sN, int N, int D, const
     float *pbuf = (float *)(scratch + w.off_p), *C = (float *)(scratch + w.off_C), *part = (float *)(scratch + w.off_part);
     double *g = (double *)(scratch + w.off_g);
     unsigned *bar = (unsigned *)(scratch + w.off_bar);
-    cudaError_t err = cudaMemsetAsync(bar, 0, 256, st);
+    cudaError_t err = cudaMemsetAsync(bar, 0, w.zero_bytes, st);        // off_bar is 0
     if (err != cudaSuccess) return err;
     {
         ProfScope ps(prof, kSlotWideGram, st);
@@ -696,6 +698,25 @@ cudaError_t launch_entropy_wide(const void *d_X, int64_t sN, int N, int D, const
     }
     err = cudaGetLastError();
     if (err != cudaSuccess) return err;
+    const int k = ep.k_trunc < D ? ep.k_trunc : D;                // entries of the outputs
+    const int kf = k < w.Dt ? k : w.Dt;                           // eigenvalues the matrix can have; the rest are zero
+    double *lam = (double *)(scratch + w.off_lam);
+    int *kry = nullptr;
+    // A few of the eigenvalues of a large matrix: block Lanczos.  What follows leaves at once when it has converged.
+    if (krylov_applies(w.Dt, kf)) {
+        ProfScope ps(prof, kSlotWideKrylov, st);
+        KrylovBuffers b;
+        b.Q = (float *)(scratch + w.off_Q);
+        b.part = (float *)(scratch + w.off_kpart);
+        b.H = (float *)(scratch + w.off_H);
+        b.G = (double *)(scratch + w.off_G);
+        b.T = (double *)(scratch + w.off_T);
+        b.lam = lam;
+        b.state = kry = (int *)(scratch + w.off_state);
+        b.bar = bar + 8;
+        err = launch_krylov(C, w.Dt, kf, ep.max_iters, b, d_status, st);
+        if (err != cudaSuccess) return err;
+    }
     {
         ProfScope ps(prof, kSlotWideTridiag, st);
         int dev = 0, sms = 0, per_sm = 0;
@@ -710,19 +731,16 @@ cudaError_t launch_entropy_wide(const void *d_X, int64_t sN, int N, int D, const
         if (per_sm < 1) return cudaErrorLaunchOutOfResources;
         int grid = sms;                                          // one CTA per SM: all of them are resident
         if (grid > Dt / 8) grid = Dt / 8;                         // small matrices: fewer CTAs, cheaper barrier
-        int Di = Dt;
-        void *args[] = {(void *)&C, (void *)&Di, (void *)&a, (void *)&e, (void *)&pbuf, (void *)&bar, (void *)&d_status};
+        int Di = Dt, kw = kf;
+        const double *lam_in = lam;
+        void *args[] = {(void *)&C, (void *)&Di, (void *)&a, (void *)&e, (void *)&pbuf, (void *)&bar, (void *)&kry, (void *)&lam_in,
+                        (void *)&kw, (void *)&d_status};
         err = cudaLaunchCooperativeKernel((const void *)tridiag_wide_kernel, dim3(grid), dim3(kTriThreads), args, smem, st);
         if (err != cudaSuccess) return err;
     }
     {
         ProfScope ps(prof, kSlotWideSturm, st);
-        const int k = ep.k_trunc < D ? ep.k_trunc : D;            // entries of the outputs
-        const int kf = k < w.Dt ? k : w.Dt;                       // eigenvalues the matrix can have; the rest are zero
-        double *lam = (double *)(scratch + w.off_lam);
-        err = cudaMemsetAsync(lam, 0, (size_t)(kSturmMaxK + 1) * sizeof(double), st);
-        if (err != cudaSuccess) return err;
-        sturm_wide_kernel<<<kf, kSturmThreads, 0, st>>>(a, e, w.Dt, kf, ep.max_iters, lam, d_status);
+        sturm_wide_kernel<<<kf, kSturmThreads, 0, st>>>(a, e, w.Dt, kf, ep.max_iters, kry, lam, d_status);
         wide_entropy_kernel<<<1, 32, 0, st>>>(lam, k, kf, ep.norm, d_entropy, d_erank, d_spectrum);
     }
     return cudaGetLastError();

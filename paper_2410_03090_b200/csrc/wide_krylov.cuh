@@ -1,0 +1,43 @@
+// The k largest eigenvalues of a large symmetric matrix by block Lanczos (see wide_krylov.cu).
+#pragma once
+
+#include "common.cuh"
+
+namespace uncomp {
+
+constexpr int kKryBlock = 32;        // vectors per block
+constexpr int kKryMaxK = 64;         // eigenvalues wanted at most
+constexpr int kKryMaxSteps = 40;     // block steps at most
+constexpr int kKryMinN = 384;        // smaller matrices: the column-by-column reduction is as fast
+
+// Scratch of one matrix (device pointers), and what the kernels leave there.
+struct KrylovBuffers {
+    float *Q;            // [steps + 1][32][n] orthonormal blocks, a vector contiguous
+    float *part;         // [n / 32][steps + 1][1024] partial products of the CTAs
+    float *H;            // [steps][1024] their sums
+    double *G;           // [1024] Gram matrix of the new block
+    double *T;           // [32 steps + 32][kKryBand] projected matrix, column c: entry (c - o, c) at [c][o], o <= 32
+    double *lam;         // [k + 1] eigenvalues descending, then the trace
+    int *state;          // [0] steps in Q, [1] broken, [2] first unconverged count; [8 ..] converged, one per eigenvalue
+    unsigned *bar;       // grid barrier counters, one per launch, zero at the start
+};
+constexpr int kKryBand = 34;
+constexpr int kKryStateInts = 8 + kKryMaxK;
+constexpr int kKryMaxLaunches = 4;
+
+// true when all k eigenvalues have converged (every kernel behind the first asks this before it does anything)
+__device__ __forceinline__ bool krylov_done(const int *state, const double *lam, int k) {
+    if (state[1]) return false;
+    for (int i = 0; i < k; ++i)
+        if (!state[8 + i]) return false;
+    // a block of 32 start vectors shows an eigenvalue at most 32 times: a cluster of that size may be larger
+    for (int i = 0; i + kKryBlock <= k - 1; ++i)
+        if (lam[i] - lam[i + kKryBlock - 1] <= 1e-6 * lam[0]) return false;
+    return true;
+}
+
+bool krylov_applies(int n, int k);
+int krylov_steps(int n);             // blocks the buffers hold besides the first
+cudaError_t launch_krylov(const float *C, int n, int k, int max_iters, const KrylovBuffers &b, uint32_t *d_status, cudaStream_t st);
+
+}  // namespace uncomp

@@ -1,0 +1,49 @@
+"""Wide entropy where a few eigenvalues of a large matrix come from block Lanczos: the edges of its range, slow
+convergence (a second and third launch), and the inputs that must end in the full reduction, against the oracle."""
+import pytest
+import torch
+
+import test_gpu_wide as tw
+
+pytestmark = pytest.mark.gpu
+
+
+def _gauss(N, D, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.randn(1, N, D, generator=g, device="cuda").to(torch.bfloat16)
+
+
+@pytest.mark.parametrize("N,D,rank,k", [
+    (900, 320, 30, 32),      # one size below its range
+    (900, 384, 30, 32),      # the smallest matrix
+    (420, 1024, 200, 32),    # token space, padded from 420 to 448, nearly all directions wanted or close
+    (1300, 448, 60, 33),     # ten blocks from the start
+    (1300, 512, 60, 64),     # the largest k
+    (1300, 512, 60, 65),     # one more: the full reduction
+    (2100, 1088, 300, 48),   # 34 CTAs
+])
+def test_edges(N, D, rank, k):
+    from paper_2410_03090_b200 import binding as ub
+    X = tw._matrix(1, N, D, rank, 0.1, seed=N + D)
+    tw._check(ub, X, k, 1, 0)
+    tw._check(ub, X, k, 0, 1)
+
+
+@pytest.mark.parametrize("N,D,k", [(1500, 640, 32), (3000, 1536, 64)])
+def test_isotropic_needs_more_steps(N, D, k):
+    from paper_2410_03090_b200 import binding as ub
+    tw._check(ub, _gauss(N, D, 3), k, 1, 0)
+
+
+def test_multiple_eigenvalues_rank_loss_and_zero():
+    from paper_2410_03090_b200 import binding as ub
+    eye = torch.eye(512, device="cuda").repeat(4, 1)[None].to(torch.bfloat16)     # 511 equal eigenvalues
+    tw._check(ub, eye, 32, 1, 0)
+    tw._check(ub, eye, 64, 1, 0)                                                  # more than a block can show
+    low = torch.zeros(1, 1024, 512, dtype=torch.bfloat16, device="cuda")
+    low[:, :, :8] = _gauss(1024, 8, 5)                                            # rank 8
+    tw._check(ub, low, 32, 1, 0)
+    ctx = ub.Context(ub.make_shape(1, 1, 1, 1, 256, 128, 8, "bf16"))
+    ent, er = ub.uncomp_entropy_wide(ctx, torch.ones(1, 1024, 512, dtype=torch.bfloat16, device="cuda"), 32)
+    torch.cuda.synchronize()
+    assert ub.uncomp_status(ctx) == 0 and float(ent[0]) == 0.0 and float(er[0]) == 1.0
