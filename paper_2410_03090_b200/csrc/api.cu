@@ -41,9 +41,11 @@ Plan make_plan(const uncomp_shape &s) {
         p.gram_splits = (s.N + chunk - 1) / chunk;
     }
     {
-        // scorer: chunks of 8192 tokens (a multiple of the 128-token tile), halved while the grid is small
+        // scorer: chunks of 8192 tokens (a multiple of the 128-token tile), halved while the grid is small; the
+        // CUDA-core kernels of fp32 keys need no long pipeline and go down to one of their blocks of 64 tokens
         int chunk = 8192;
-        while (chunk > 512 && (int64_t)p.units * ((s.N + chunk - 1) / chunk) < target_ctas) chunk >>= 1;
+        const int least = s.dtype == UNCOMP_FP32 ? 64 : 512;
+        while (chunk > least && (int64_t)p.units * ((s.N + chunk - 1) / chunk) < target_ctas) chunk >>= 1;
         p.score_chunk = chunk;
         p.score_splits = (s.N + chunk - 1) / chunk;
     }
