@@ -11,18 +11,27 @@
 // K tiles (128 tokens x 128 features, two 128B-swizzled boxes of 64 features) stream through a TMA ring;
 // the unit's window queries stay in shared memory for the whole CTA.  Both operands are K-major.
 //
-// CTA on one SM: warps 0-15 softmax in two groups of eight that take alternate token tiles (so the four
+// One CTA per SM works through its share of the (unit, token chunk) items.  The TMA producer runs ahead into the next item,
+// so a CTA's pipeline fills once and not once per item (a CTA per item spent 8,000 of 38,000 cycles on a 3712-token unit
+// before its first tile arrived and 6,000 after its last).
+// Warps 0-15 softmax in two groups of eight that take alternate token tiles (so the four
 // warps of an SM sub-partition are in different phases: while one group waits for its accumulator, the
 // other keeps the exponential unit busy); inside a group warp % 4 selects the TMEM lane quarter and bit 2
 // of the warp index the 64-column half of an accumulator.  Warp 16 is the TMA producer, warp 17 allocates
-// TMEM and issues the MMAs.  The 128-column accumulators form one ring that both groups draw from in item
-// order (item = one 128-row block of one tile): four buffers in modes 0 and 1, three in mode 2.
+// TMEM and issues the MMAs: one ELECTED lane (elect.sync lets the compiler keep descriptors in uniform registers; with
+// `lane == 0` an MMA took 130 cycles to issue, twice what the tensor pipe needs for it, and paced the kernel).  The
+// 128-column accumulators form one ring that both groups draw from in order
+// (block = one 128-row block of one tile): four buffers in modes 0 and 1, three in modes 2 and 3.
 // Mode 2 of the kernel is pass A with the Gram stage folded in: the K tile that is in shared memory for
 // Qw K^T is also the MN-major operand of G += K_tile^T K_tile, so the entropy stage costs no second sweep
 // over K.  The Gram block takes the last 128 TMEM columns; the column sums s = K^T 1 are added up by two
-// extra warps (18, 19) with plain global loads of the same tokens (L2 hits), in a fixed order.
+// extra warps (18, 19) that read the tile from shared memory as well (from global memory, 3,000 cycles of latency per
+// tile paced the kernel).
 // Mode 3 is pass B with the Gram stage folded in the same way, for callers who bring the row normalisers (their
 // prefill attention kernel's log-sum-exp): entropy stage and scores from ONE sweep over K.
+// What bounds it: power.  With keys streaming and the tensor pipe busy the SM clock falls from 1.9 to 1.2 - 1.6 GHz; a
+// micro-benchmark of the same MMAs, TMA loads and exponentials without any hand-over takes 1,180 cycles = 0.95 us per tile
+// of one row block, modes 2 and 3 take about 1.1 us.  Two row blocks are bound by the exponential unit (2,048 cycles).
 // Every wait is bounded; a timeout raises UNCOMP_STATUS_TIMEOUT and the CTA drains and exits.
 #include "tc_common.cuh"
 
@@ -39,15 +48,16 @@ constexpr int kGramThreads = kScoreThreads + 64;  // mode 2: two more warps for 
 constexpr int kMaxStages = 4;
 
 struct ScoreTail {
-    uint64_t full[kMaxStages], empty[kMaxStages], qfull, tfull[2 * kNB], tempty[kNB], gfull;
+    uint64_t full[kMaxStages], empty[kMaxStages], qfull[2], qempty[2], tfull[2 * kNB], tempty[kNB], gfull, gdrained;
     uint32_t tmem_base;
-    float sum_xch[kD];     // hand-over of the second column-sum warp (mode 2 and 3)
+    float sum_xch[2][kD];  // hand-over of the second column-sum warp (modes 2 and 3)
 };
 
 __host__ __device__ constexpr int score_stages(int MB) { return MB <= 2 ? 4 : (MB == 3 ? 3 : 2); }
+__host__ __device__ constexpr int query_buffers(int MB) { return MB == 1 ? 2 : 1; }
 __host__ __device__ constexpr int score_smem(int MB) {
-    return 1024 + MB * kBlockBytes + score_stages(MB) * kBlockBytes + MB * 128 * 4 + 2 * 4 * 128 * 4 +
-           (int)sizeof(ScoreTail);
+    return 1024 + query_buffers(MB) * MB * kBlockBytes + score_stages(MB) * kBlockBytes + 2 * MB * 128 * 4 + 2 * 4 * 128 * 4 +
+           4 * MB * 128 * 8 + (int)sizeof(ScoreTail);
 }
 
 __device__ __forceinline__ float ex2(float x) {
@@ -60,17 +70,15 @@ __device__ __forceinline__ void group_barrier(int g) { asm volatile("bar.sync %0
 __device__ __forceinline__ void sum_warps_barrier() { asm volatile("bar.sync 4, 64;" ::: "memory"); }
 __device__ __forceinline__ float bf16_lo(uint32_t x) { return __uint_as_float(x << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t x) { return __uint_as_float(x & 0xffff0000u); }
-__device__ __forceinline__ void add_bf16x8(float (&acc)[8], const uint4 &x) {
-    acc[0] += bf16_lo(x.x); acc[1] += bf16_hi(x.x);
-    acc[2] += bf16_lo(x.y); acc[3] += bf16_hi(x.y);
-    acc[4] += bf16_lo(x.z); acc[5] += bf16_hi(x.z);
-    acc[6] += bf16_lo(x.w); acc[7] += bf16_hi(x.w);
+__device__ __forceinline__ void add_bf16x8(f32x2 (&acc)[4], const uint4 &x) {
+    acc[0] = add2(acc[0], pack2(bf16_lo(x.x), bf16_hi(x.x)));
+    acc[1] = add2(acc[1], pack2(bf16_lo(x.y), bf16_hi(x.y)));
+    acc[2] = add2(acc[2], pack2(bf16_lo(x.z), bf16_hi(x.z)));
+    acc[3] = add2(acc[3], pack2(bf16_lo(x.w), bf16_hi(x.w)));
 }
-// 16-byte read-only global load that does not allocate in L1
-__device__ __forceinline__ uint4 ld_stream16(const void *p) {
+__device__ __forceinline__ uint4 ld_shared16(uint32_t addr) {
     uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
     return v;
 }
 __device__ __forceinline__ float max3(float a, float b, float c) {
@@ -79,19 +87,20 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     return d;
 }
 
-// Pass A: fold 64 logits of one row into its running (m, l), log2 domain.  m only has to stay at or above
-// every logit seen so far (it is the exact running maximum here, raised lazily), l = sum 2^(x c - m).
-template <bool MASKED>
-__device__ __forceinline__ void stats_update(uint32_t (&v)[64], float c_log2, int pos0, int last, float &m_run,
+// Pass A: fold NC logits of one row into its running (m, l), log2 domain.  m only has to stay at or above
+// every logit seen so far (it is the exact running maximum here, raised lazily), l = sum 2^(x c - m).  Multiply-adds and
+// sums work on pairs.
+template <bool MASKED, int NC>
+__device__ __forceinline__ void stats_update(uint32_t (&v)[NC], float c_log2, int pos0, int last, float &m_run,
                                              float &l_run) {
     if (MASKED) {
 #pragma unroll
-        for (int j = 0; j < 64; ++j)
+        for (int j = 0; j < NC; ++j)
             if (pos0 + j > last) v[j] = 0xff800000u;            // -inf: not visible to this row
     }
     float pm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-    for (int j = 0; j < 64; j += 8) {
+    for (int j = 0; j < NC; j += 8) {
         pm[0] = max3(pm[0], __uint_as_float(v[j]), __uint_as_float(v[j + 1]));
         pm[1] = max3(pm[1], __uint_as_float(v[j + 2]), __uint_as_float(v[j + 3]));
         pm[2] = max3(pm[2], __uint_as_float(v[j + 4]), __uint_as_float(v[j + 5]));
@@ -103,80 +112,123 @@ __device__ __forceinline__ void stats_update(uint32_t (&v)[64], float c_log2, in
         m_run = mx;
     }
     if (m_run > -INFINITY) {
-        float sum[4] = {0.f, 0.f, 0.f, 0.f};
+        const f32x2 c2 = pack2(c_log2, c_log2), m2 = pack2(-m_run, -m_run);
+        f32x2 sum[2] = {0ull, 0ull};
 #pragma unroll
-        for (int j = 0; j < 64; ++j) sum[j & 3] += ex2(fmaf(__uint_as_float(v[j]), c_log2, -m_run));
-        l_run += (sum[0] + sum[1]) + (sum[2] + sum[3]);
+        for (int j = 0; j < NC; j += 2) {
+            float a, b;
+            unpack2(fma2(pack2(__uint_as_float(v[j]), __uint_as_float(v[j + 1])), c2, m2), a, b);
+            sum[(j >> 1) & 1] = add2(sum[(j >> 1) & 1], pack2(ex2(a), ex2(b)));
+        }
+        l_run += sum2(sum[0]) + sum2(sum[1]);
     }
 }
 
-// Pass B: sum over 64 window rows of 2^(s c - m'_r) for one token.
-__device__ __forceinline__ float colsum_partial(const uint32_t (&v)[64], float c_log2, const float *mrow) {
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+// Pass B: sum over NC window rows of 2^(s c - m'_r) for one token; `mneg` holds -m'_r.
+template <int NC>
+__device__ __forceinline__ float colsum_partial(const uint32_t (&v)[NC], float c_log2, const float *mneg) {
+    const f32x2 c2 = pack2(c_log2, c_log2);
+    f32x2 acc[2] = {0ull, 0ull};
 #pragma unroll
-    for (int j = 0; j < 64; j += 4) {
-        const float4 m4 = *reinterpret_cast<const float4 *>(mrow + j);
-        acc[0] += ex2(fmaf(__uint_as_float(v[j]), c_log2, -m4.x));
-        acc[1] += ex2(fmaf(__uint_as_float(v[j + 1]), c_log2, -m4.y));
-        acc[2] += ex2(fmaf(__uint_as_float(v[j + 2]), c_log2, -m4.z));
-        acc[3] += ex2(fmaf(__uint_as_float(v[j + 3]), c_log2, -m4.w));
+    for (int j = 0; j < NC; j += 4) {
+        const ulonglong2 m4 = *reinterpret_cast<const ulonglong2 *>(mneg + j);
+        float a, b;
+        unpack2(fma2(pack2(__uint_as_float(v[j]), __uint_as_float(v[j + 1])), c2, m4.x), a, b);
+        acc[0] = add2(acc[0], pack2(ex2(a), ex2(b)));
+        unpack2(fma2(pack2(__uint_as_float(v[j + 2]), __uint_as_float(v[j + 3])), c2, m4.y), a, b);
+        acc[1] = add2(acc[1], pack2(ex2(a), ex2(b)));
     }
-    return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    return sum2(acc[0]) + sum2(acc[1]);
+}
+
+// NC columns of this warp's 32 TMEM lanes
+template <int NC>
+__device__ __forceinline__ void load_columns(uint32_t taddr, uint32_t (&v)[NC]) {
+    if constexpr (NC == 16) {
+        tc::tmem_ld16(taddr, v);
+        tc::tmem_ld_wait();
+    } else if constexpr (NC == 32) {
+        tc::tmem_ld32(taddr, v);
+        tc::tmem_ld_wait();
+    } else {
+        uint32_t va[32], vb[32];
+        tc::tmem_ld32(taddr, va);
+        tc::tmem_ld32(taddr + 32, vb);
+        tc::tmem_ld_wait();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) { v[j] = va[j]; v[32 + j] = vb[j]; }
+    }
 }
 }  // namespace
 
-template <int MB, int MODE>   // MODE 0: pass A, 1: pass B, 2: pass A fused with the Gram stage, 3: pass B fused with it
+// MODE 0: pass A, 1: pass B, 2: pass A fused with the Gram stage, 3: pass B fused with it.
+// SPLIT 2 and 4 (MB = 1 only): at most 64 or 32 window rows.  A block of 128 rows would be mostly padding, and every
+// padded row costs as many exponentials as a real one.  Pass A keeps M = 128 but fills it with SPLIT copies of the rows;
+// the lanes of a copy take their own part of the tile's tokens.  Pass B takes N = 128 / SPLIT instead of 128.  (Copies of
+// 16 rows were no faster: the keys' bandwidth and the Gram MMAs bound it then.)
+template <int MB, int MODE, int SPLIT>
 __global__ void __launch_bounds__(kGramThreads, 1)
 score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant__ CUtensorMap tmapK, int L, int H,
-                int N, int w, int rows, int chunk, int splits, float c_log2, float *__restrict__ stats_part,
+                int N, int w, int rows, int units, int chunk, int splits, float c_log2, float *__restrict__ stats_part,
                 const float *__restrict__ mprime, float *__restrict__ raw, float *__restrict__ gram_part,
-                const void *__restrict__ Kraw, const UnitAddr kaddr, uint32_t *__restrict__ status) {
+                uint32_t *__restrict__ status) {
     constexpr bool PASS_B = MODE == 1 || MODE == 3, GRAM = MODE >= 2;
-    // Accumulator buffers (128 TMEM columns each).  An item is one 128-row block of one tile; tile i belongs to
-    // softmax group i & 1.  Modes 0 and 1: four buffers, two owned by each group, which it fills alternately
-    // with its own items (so each group runs up to two items ahead, independent of the other).  Mode 2: the
-    // Gram block leaves room for three, which form one ring over all items in issue order.
+    // Accumulator buffers (128 TMEM columns each).  An accumulator holds one 128-row block of one tile; tile n (counted
+    // over everything the CTA does) belongs to softmax group n & 1.  Modes 0 and 1: four buffers, two owned by each group,
+    // which it fills alternately (so each group runs up to two blocks ahead, independent of the other).  Modes 2 and 3:
+    // the Gram block leaves room for three, which form one ring in issue order.
     constexpr int NB = GRAM ? 3 : kNB;
-    // Mode 2: "item n is ready" is signalled on barrier n % (2 NB).  A softmax group that waits for the first item
-    // of its next tile may get there before the other group's item n - NB has completed, and with one barrier per
+    // Modes 2 and 3: "block q is ready" is signalled on barrier q % (2 NB).  A softmax group that waits for the first block
+    // of its next tile may get there before the other group's block q - NB has completed, and with one barrier per
     // buffer the parity of that unfinished phase could not be told from the one waited for.  The user of barrier
-    // n % (2 NB) before item n is item n - 2 NB, which lies in a tile this group has already consumed (2 NB > MB).
+    // q % (2 NB) before block q is block q - 2 NB, which lies in a tile this group has already consumed (2 NB > MB).
     // Modes 0 and 1 need no such care: a group only ever waits on its own buffers.
     constexpr int NF = 2 * NB;
-    // item (tile i, block mb) -> buffer, ready barrier and its parity, and the drain phase the MMA thread waits for
+    // block (tile n, mb) -> buffer, ready barrier and its parity, and the drain phase the MMA thread waits for
     // (-1: the buffer has not been used yet)
-    auto item_buf = [](int i, int mb) { return GRAM ? (i * MB + mb) % NB : 2 * (i & 1) + (((i >> 1) * MB + mb) & 1); };
-    auto item_ready_bar = [](int i, int mb) { return GRAM ? (i * MB + mb) % NF : 2 * (i & 1) + (((i >> 1) * MB + mb) & 1); };
-    auto item_ready_parity = [](int i, int mb) { return GRAM ? ((i * MB + mb) / NF) & 1 : ((((i >> 1) * MB + mb) >> 1) & 1); };
-    auto item_drain_phase = [](int i, int mb) { return GRAM ? (i * MB + mb) / NB - 1 : ((((i >> 1) * MB + mb) >> 1) - 1); };
-    constexpr uint32_t kGramCol = 384;               // TMEM columns of the Gram block (mode 2)
-    constexpr int S = score_stages(MB);
+    auto item_buf = [](int n, int mb) { return GRAM ? (n * MB + mb) % NB : 2 * (n & 1) + (((n >> 1) * MB + mb) & 1); };
+    auto item_ready_bar = [](int n, int mb) { return GRAM ? (n * MB + mb) % NF : 2 * (n & 1) + (((n >> 1) * MB + mb) & 1); };
+    auto item_ready_parity = [](int n, int mb) { return GRAM ? ((n * MB + mb) / NF) & 1 : ((((n >> 1) * MB + mb) >> 1) & 1); };
+    auto item_drain_phase = [](int n, int mb) { return GRAM ? (n * MB + mb) / NB - 1 : ((((n >> 1) * MB + mb) >> 1) - 1); };
+    constexpr uint32_t kGramCol = 384;               // TMEM columns of the Gram block (modes 2 and 3)
+    constexpr int kRows = 128 / SPLIT;               // rows of a copy (pass A), columns of an accumulator (pass B)
+    constexpr int NC = 64 / SPLIT;                   // logits a thread takes from an accumulator
+    static_assert(kRows >= 32, "a TMEM load has one address per warp: a warp belongs to one copy");
+    static_assert(SPLIT == 1 || MB == 1, "more than 128 rows are never split");
+    constexpr int S = score_stages(MB), QB = query_buffers(MB);
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw_addr = tc::smem_u32(smem_raw);
     const uint32_t pad = (1024u - (raw_addr & 1023u)) & 1023u;
     unsigned char *smem = smem_raw + pad;
     const uint32_t q_addr = raw_addr + pad;
-    const uint32_t k_addr = q_addr + MB * kBlockBytes;
-    float *mp = reinterpret_cast<float *>(smem + (MB + S) * kBlockBytes);      // [MB * 128]
-    float *colsum = mp + MB * 128;                                             // [2][4][128]
-    ScoreTail &T = *reinterpret_cast<ScoreTail *>(colsum + 2 * 4 * 128);
+    const uint32_t k_addr = q_addr + QB * MB * kBlockBytes;
+    float *mp = reinterpret_cast<float *>(smem + (QB * MB + S) * kBlockBytes);     // [2][MB * 128], by unit
+    float *colsum = mp + 2 * MB * 128;                                             // [2][4][128]
+    float2 *merge = reinterpret_cast<float2 *>(colsum + 2 * 4 * 128);              // [4][MB * 128]
+    ScoreTail &T = *reinterpret_cast<ScoreTail *>(merge + 4 * MB * 128);
 
-    const int c = blockIdx.x, u = blockIdx.y;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int h = u % H, l = (u / H) % L, b = u / (H * L);
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int P = N - w;
     const int limit = (PASS_B && !GRAM) ? P : N;   // pass B only scores the prefix; the Gram stage needs every token
-    const int t0 = c * chunk;
-    const int t1 = min(limit, t0 + chunk);
-    const int ntiles = t1 > t0 ? (t1 - t0 + kTile - 1) / kTile : 0;
+    // this CTA's share of the work items; item j is chunk j % splits of unit j / splits
+    const int64_t total = (int64_t)units * splits;
+    const int first = (int)(total * blockIdx.x / gridDim.x), last_item = (int)(total * (blockIdx.x + 1) / gridDim.x);
+    auto tiles_of = [&](int j) {
+        const int t0 = (j % splits) * chunk;
+        return (min(limit, t0 + chunk) - t0 + kTile - 1) / kTile;
+    };
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             tc::mbar_init(tc::smem_u32(&T.full[s]), 1);
-            tc::mbar_init(tc::smem_u32(&T.empty[s]), 1);
+            tc::mbar_init(tc::smem_u32(&T.empty[s]), GRAM ? 3 : 1);     // the MMAs and the two column-sum warps
         }
-        tc::mbar_init(tc::smem_u32(&T.qfull), 1);
+        for (int q = 0; q < QB; ++q) {
+            tc::mbar_init(tc::smem_u32(&T.qfull[q]), 1);
+            tc::mbar_init(tc::smem_u32(&T.qempty[q]), 1);
+        }
         tc::mbar_init(tc::smem_u32(&T.gfull), 1);
+        tc::mbar_init(tc::smem_u32(&T.gdrained), kSoftThreads / 32);
         for (int i = 0; i < 2 * kNB; ++i) tc::mbar_init(tc::smem_u32(&T.tfull[i]), 1);
         for (int i = 0; i < kNB; ++i) tc::mbar_init(tc::smem_u32(&T.tempty[i]), kSoftThreads / 64);   // the 8 warps of one group
         tc::fence_mbar_init();
@@ -195,259 +247,335 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
     const uint32_t tmem = T.tmem_base;
 
     if (warp == 16) {
-        // ---------------- TMA producer ----------------
-        if (lane == 0 && ntiles > 0) {
-            const uint32_t qbar = tc::smem_u32(&T.qfull);
-            tc::mbar_expect_tx(qbar, MB * kBlockBytes);
-            for (int mb = 0; mb < MB; ++mb) {
-                tc::tma_load_3d(q_addr + mb * kBlockBytes, &tmapQ, qbar, 0, mb * 128, u);
-                tc::tma_load_3d(q_addr + mb * kBlockBytes + kHalfBytes, &tmapQ, qbar, 64, mb * 128, u);
+        // ---------------- TMA producer: runs ahead into the next items ----------------
+        if (lane == 0) {
+            int n = 0, useq = -1, cur_u = -1, q_sent = 0;      // tiles sent, units seen, query blocks sent
+            bool ok = true, q_pending = false;
+            auto q_free = [&]() {
+                return useq < QB || tc::mbar_test_wait(tc::smem_u32(&T.qempty[useq % QB]), ((useq / QB) - 1) & 1);
+            };
+            auto send_q = [&]() {
+                constexpr int kCopies = PASS_B ? 1 : SPLIT;
+                const uint32_t bar = tc::smem_u32(&T.qfull[useq % QB]);
+                tc::mbar_expect_tx(bar, MB * kCopies * (kBlockBytes / SPLIT));
+                for (int mb = 0; mb < MB; ++mb)
+                    for (int cp = 0; cp < kCopies; ++cp) {
+                        const uint32_t dst = q_addr + ((useq % QB) * MB + mb) * kBlockBytes + cp * (kHalfBytes / SPLIT);
+                        tc::tma_load_3d(dst, &tmapQ, bar, 0, mb * 128, cur_u);
+                        tc::tma_load_3d(dst + kHalfBytes, &tmapQ, bar, 64, mb * 128, cur_u);
+                    }
+                q_pending = false;
+                ++q_sent;
+            };
+            // the queries' buffer may still be in use by the unit before: key tiles go ahead, the queries as soon as it is free
+            auto wait_q = [&]() {
+                if (useq >= QB) ok = tc::mbar_wait(tc::smem_u32(&T.qempty[useq % QB]), ((useq / QB) - 1) & 1, status);
+                if (ok) send_q();
+            };
+            for (int j = first; j < last_item && ok; ++j) {
+                const int u = j / splits, t0 = (j % splits) * chunk, ntiles = tiles_of(j);
+                const int h = u % H, l = (u / H) % L, b = u / (H * L);
+                if (u != cur_u) {
+                    if (q_pending) wait_q();
+                    if (!ok) break;
+                    cur_u = u;
+                    ++useq;
+                    q_pending = true;
+                    if (q_free()) send_q();
+                }
+                for (int i = 0; i < ntiles; ++i, ++n) {
+                    const int s = n % S;
+                    if (n >= S) {
+                        const uint32_t bar = tc::smem_u32(&T.empty[s]), parity = ((n / S) - 1) & 1;
+                        uint32_t spins = 0;
+                        while (q_pending && !tc::mbar_test_wait(bar, parity) && ++spins < tc::kSpinLimit)
+                            if (q_free()) send_q();
+                        ok = tc::mbar_wait(bar, parity, status);
+                        if (!ok) break;
+                    }
+                    const uint32_t bar = tc::smem_u32(&T.full[s]);
+                    const uint32_t dst = k_addr + s * kBlockBytes;
+                    tc::mbar_expect_tx(bar, kBlockBytes);
+                    tc::tma_load_5d(dst, &tmapK, bar, 0, t0 + i * kTile, h, l, b);
+                    tc::tma_load_5d(dst + kHalfBytes, &tmapK, bar, 64, t0 + i * kTile, h, l, b);
+                    if (q_pending && q_free()) send_q();
+                }
             }
-            int issued = 0;
-            bool ok = true;
-            for (int i = 0; i < ntiles; ++i, ++issued) {
-                const int s = i % S;
-                if (i >= S) ok = tc::mbar_wait(tc::smem_u32(&T.empty[s]), ((i / S) - 1) & 1, status);
-                if (!ok) break;
-                const uint32_t bar = tc::smem_u32(&T.full[s]);
-                const uint32_t dst = k_addr + s * kBlockBytes;
-                tc::mbar_expect_tx(bar, kBlockBytes);
-                tc::tma_load_5d(dst, &tmapK, bar, 0, t0 + i * kTile, h, l, b);
-                tc::tma_load_5d(dst + kHalfBytes, &tmapK, bar, 64, t0 + i * kTile, h, l, b);
-            }
+            if (ok && q_pending) wait_q();
             if (!ok) {   // let the copies in flight land before the CTA may exit (bounded)
-                tc::mbar_wait(qbar, 0, status);
-                for (int i = max(0, issued - S); i < issued; ++i)
+                for (int q = max(0, q_sent - QB); q < q_sent; ++q)
+                    tc::mbar_wait(tc::smem_u32(&T.qfull[q % QB]), (q / QB) & 1, status);
+                for (int i = max(0, n - S); i < n; ++i)
                     tc::mbar_wait(tc::smem_u32(&T.full[i % S]), (i / S) & 1, status);
             }
         }
     } else if (warp == 17) {
         // ---------------- MMA issue ----------------
-        if (lane == 0 && ntiles > 0) {
-            constexpr uint32_t idesc = tc::idesc_bf16_f32(128, 128, 0, 0);
+        if (tc::elect_one()) {
+            constexpr uint32_t idesc = tc::idesc_bf16_f32(128, PASS_B ? kRows : 128, 0, 0);
             // descriptors: K-major, 128-byte swizzle, 8-row groups 1024 B apart.  Only the address field
             // (16-byte units) of the lower half changes: +2 per 16 features inside a 128-byte row, +1024 for
             // the second 64-feature half.
             const uint64_t d0 = tc::smem_desc_sw128(q_addr, 16, 1024);
-            const uint32_t dhi = tc::desc_hi(d0);
-            uint32_t q_lo[MB];
-#pragma unroll
-            for (int mb = 0; mb < MB; ++mb) q_lo[mb] = tc::desc_lo(d0) + (uint32_t)(mb * kBlockBytes >> 4);
+            const uint32_t dhi = tc::desc_hi(d0), q_lo0 = tc::desc_lo(d0);
             const uint32_t k_lo0 = tc::desc_lo(tc::smem_desc_sw128(k_addr, 16, 1024));
             const uint64_t gd = tc::smem_desc_sw128(k_addr, kHalfBytes, 1024);
             const uint32_t g_lo0 = tc::desc_lo(gd), g_hi = tc::desc_hi(gd);
-            // Mode 2: the Gram MMAs of a tile only have to be issued before its stage is handed back, so they
-            // are deferred by up to one tile and issued while this thread would otherwise wait for an
-            // accumulator: the latency-critical QK^T MMAs never queue behind them.
+            int n = 0, useq = -1, cur_u = -1, iseq = 0, item_start = 0;
+            bool ok = true;
+            bool have_tile = false, have_buf = false;   // known of the next tile before this one's Gram MMAs are issued
+            // Modes 2 and 3: the Gram MMAs of a tile only have to be issued before its stage is handed back, so they
+            // are deferred by up to one tile: the latency-critical QK^T MMAs never queue behind them, and while the
+            // tensor pipe works on them this thread finds out about the next tile and accumulator.
+            // One 128-row block per tile: three accumulators are three tiles ahead, nothing waits behind the Gram MMAs, and
+            // issuing them at once frees the stage earlier (c4: 2204 -> 2126 us); with more blocks the lag pays (c3: 866 -> 838).
+            constexpr int kLag = MB == 1 ? 0 : 1;
             int g_done = 0;                    // tiles whose Gram MMAs are issued (and whose stage is released)
-            auto issue_gram = [&](int t) {
+            auto issue_gram = [&]() {
                 constexpr uint32_t idesc_g = tc::idesc_bf16_f32(128, 128, 1, 1);
-                const int sg = t % S;
+                const int t = g_done, sg = t % S;
+                if (t == item_start && iseq > 0) {      // the softmax warps have read the item before
+                    ok = tc::mbar_wait(tc::smem_u32(&T.gdrained), (iseq - 1) & 1, status);
+                    tc::tc_fence_after();
+                    if (!ok) return;
+                }
                 const uint32_t g_lo = g_lo0 + (uint32_t)(sg * (kBlockBytes >> 4));
 #pragma unroll
                 for (int k = 0; k < kTile / 16; ++k) {
                     // the same stage read MN-major (feature halves kHalfBytes apart, 8-token groups 1024 B
                     // apart); 16 tokens further = +128 address units
-                    const uint32_t acc = (t > 0 || k > 0) ? 1u : 0u;
+                    const uint32_t acc = (t > item_start || k > 0) ? 1u : 0u;
                     tc::mma_f16_ss_lohi(tmem + kGramCol, g_lo + k * 128, g_lo + k * 128, g_hi, idesc_g, acc);
                 }
                 tc::mma_commit(tc::smem_u32(&T.empty[sg]));
+                ++g_done;
             };
-            bool ok = tc::mbar_wait(tc::smem_u32(&T.qfull), 0, status);
-            for (int i = 0; i < ntiles && ok; ++i) {
-                const int s = i % S;
-                ok = tc::mbar_wait(tc::smem_u32(&T.full[s]), (i / S) & 1, status);
-                if (!ok) break;
-                const uint32_t k_lo = k_lo0 + (uint32_t)(s * (kBlockBytes >> 4));
+            for (int j = first; j < last_item && ok; ++j) {
+                const int u = j / splits, ntiles = tiles_of(j);
+                const bool more = j + 1 < last_item;
+                if (u != cur_u) {
+                    cur_u = u;
+                    ++useq;
+                    ok = tc::mbar_wait(tc::smem_u32(&T.qfull[useq % QB]), (useq / QB) & 1, status);
+                }
+                const bool leaves_q = !more || (j + 1) / splits != u;      // the unit's last item of this CTA
+                const uint32_t q_lo = q_lo0 + (uint32_t)((useq % QB) * MB * (kBlockBytes >> 4));
+                item_start = n;
+                for (int i = 0; i < ntiles && ok; ++i, ++n) {
+                    const int s = n % S;
+                    if (!have_tile) ok = tc::mbar_wait(tc::smem_u32(&T.full[s]), (n / S) & 1, status);
+                    if (!ok) break;
+                    const uint32_t k_lo = k_lo0 + (uint32_t)(s * (kBlockBytes >> 4));
 #pragma unroll
-                for (int mb = 0; mb < MB; ++mb) {
-                    // the item's buffer must have been drained of its previous item
-                    const int buf = item_buf(i, mb), drain = item_drain_phase(i, mb);
-                    if (ok && drain >= 0) {
-                        const uint32_t bar = tc::smem_u32(&T.tempty[buf]);
-                        const uint32_t parity = drain & 1;
-                        if (GRAM) {
-                            uint32_t spins = 0;
-                            while (!tc::mbar_try_wait(bar, parity)) {
-                                if (g_done < i) issue_gram(g_done++);
-                                else if (++spins >= tc::kSpinLimit) {
-                                    atomicOr(status, (uint32_t)UNCOMP_STATUS_TIMEOUT);
-                                    ok = false;
-                                    break;
-                                }
+                    for (int mb = 0; mb < MB; ++mb) {
+                        // the block's buffer must have been drained of its previous block
+                        const int buf = item_buf(n, mb), drain = item_drain_phase(n, mb);
+                        if (ok && drain >= 0 && !(mb == 0 && have_buf)) {
+                            const uint32_t bar = tc::smem_u32(&T.tempty[buf]);
+                            const uint32_t parity = drain & 1;
+                            if (GRAM) {
+                                while (ok && g_done < n && !tc::mbar_test_wait(bar, parity)) issue_gram();
                             }
-                        } else {
-                            ok = tc::mbar_wait(bar, parity, status);
+                            if (ok) ok = tc::mbar_wait(bar, parity, status);
                         }
+                        if (!ok) break;
+                        tc::tc_fence_after();
+                        const uint32_t d_tmem = tmem + buf * 128;
+                        const uint32_t qb_lo = q_lo + (uint32_t)(mb * (kBlockBytes >> 4));
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            const uint32_t off = (uint32_t)(k >> 2) * (kHalfBytes >> 4) + (uint32_t)(k & 3) * 2;
+                            if (PASS_B) tc::mma_f16_ss_lohi(d_tmem, k_lo + off, qb_lo + off, dhi, idesc, k > 0);
+                            else tc::mma_f16_ss_lohi(d_tmem, qb_lo + off, k_lo + off, dhi, idesc, k > 0);
+                        }
+                        tc::mma_commit(tc::smem_u32(&T.tfull[item_ready_bar(n, mb)]));
                     }
                     if (!ok) break;
-                    tc::tc_fence_after();
-                    const uint32_t d_tmem = tmem + buf * 128;
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const uint32_t off = (uint32_t)(k >> 2) * (kHalfBytes >> 4) + (uint32_t)(k & 3) * 2;
-                        if (PASS_B) tc::mma_f16_ss_lohi(d_tmem, k_lo + off, q_lo[mb] + off, dhi, idesc, k > 0);
-                        else tc::mma_f16_ss_lohi(d_tmem, q_lo[mb] + off, k_lo + off, dhi, idesc, k > 0);
+                    if (leaves_q && i == ntiles - 1) tc::mma_commit(tc::smem_u32(&T.qempty[useq % QB]));
+                    if (!GRAM) tc::mma_commit(tc::smem_u32(&T.empty[s]));
+                    const int m = n + 1, nd = item_drain_phase(m, 0);
+                    const bool next = i + 1 < ntiles || more;
+                    have_tile = next && tc::mbar_test_wait(tc::smem_u32(&T.full[m % S]), (m / S) & 1);
+                    have_buf = next && nd >= 0 && tc::mbar_test_wait(tc::smem_u32(&T.tempty[item_buf(m, 0)]), nd & 1);
+                    if (GRAM) {
+                        while (ok && g_done < n + 1 - kLag) issue_gram();  // at most kLag tiles may stay pending
                     }
-                    tc::mma_commit(tc::smem_u32(&T.tfull[item_ready_bar(i, mb)]));
                 }
-                if (!ok) break;
-                if (GRAM) {
-                    while (g_done < i) issue_gram(g_done++);      // at most one tile may stay pending
-                } else {
-                    tc::mma_commit(tc::smem_u32(&T.empty[s]));
+                if (GRAM && ok) {
+                    while (ok && g_done < n) issue_gram();
+                    if (ok) tc::mma_commit(tc::smem_u32(&T.gfull));
+                    ++iseq;
                 }
-            }
-            if (GRAM) {
-                if (ok) while (g_done < ntiles) issue_gram(g_done++);
-                tc::mma_commit(tc::smem_u32(&T.gfull));
             }
         }
     } else if (warp >= 18) {
-        // ---------------- column sums s = K^T 1 (mode 2 only) ----------------
-        // Two warps add up the CTA's token chunk with plain 16-byte global loads (the lines are in L2: the TMA
-        // stream fetches the same tokens), so the shared-memory banks stay with the MMA operands and the sums
-        // need no place in the tile pipeline.  A lane owns one 16-byte chunk (8 features) of the 256-byte row and
-        // one of four row phases; its rows are added in increasing order, the phases in a fixed order below.
+        // ---------------- column sums s = K^T 1 (modes 2 and 3) ----------------
+        // Two warps read every tile from its stage, beside the MMAs, and hand the stage back like the MMA thread does.  A
+        // lane owns one 16-byte chunk (8 features) of the row and one of four row phases; its rows are added in
+        // increasing order, the phases in a fixed order below.
         if (GRAM) {
             const int sw = warp - 18, ch = lane & 15, phase = 2 * sw + (lane >> 4);
-            float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            const unsigned char *rowp = reinterpret_cast<const unsigned char *>(Kraw) +
-                                        2 * (kaddr.base(u) + (int64_t)(t0 + phase) * kaddr.sN) + 16 * ch;
-            const int64_t step = 2 * 4 * kaddr.sN;                 // four rows further, in bytes
-            const int nrows = t1 > t0 + phase ? (t1 - t0 - phase + 3) / 4 : 0;
-            int r = 0;
-            for (; r + 16 <= nrows; r += 16) {          // 16 loads in flight per lane cover the L2 latency
-                uint4 x[16];
+            // row phase + 4 q of the swizzled half: chunk c sits at c ^ (row & 7)
+            const uint32_t at0 = k_addr + (uint32_t)(ch >> 3) * kHalfBytes + phase * 128, c8 = ch & 7;
+            const uint32_t even = at0 + ((c8 ^ phase) << 4), odd = at0 + 512 + ((c8 ^ (phase + 4)) << 4);
+            bool ok = true;                            // after a timeout the warp only keeps its barrier
+            int n = 0;
+            for (int j = first; j < last_item; ++j) {
+                const int ntiles = tiles_of(j);
+                f32x2 acc2[4] = {0ull, 0ull, 0ull, 0ull};
+                for (int i = 0; i < ntiles && ok; ++i, ++n) {
+                    const int s = n % S;
+                    ok = tc::mbar_wait(tc::smem_u32(&T.full[s]), (n / S) & 1, status);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+#pragma unroll 1
+                    for (int q = 0; q < 4; ++q) {
+                        uint4 x[8];
 #pragma unroll
-                for (int q = 0; q < 16; ++q) x[q] = ld_stream16(rowp + (int64_t)(r + q) * step);
+                        for (int e = 0; e < 8; ++e) x[e] = ld_shared16((e & 1 ? odd : even) + s * kBlockBytes + (q * 4 + (e >> 1)) * 1024);
 #pragma unroll
-                for (int q = 0; q < 16; ++q) add_bf16x8(acc, x[q]);
-            }
-            for (; r < nrows; ++r) add_bf16x8(acc, ld_stream16(rowp + (int64_t)r * step));
+                        for (int e = 0; e < 8; ++e) add_bf16x8(acc2, x[e]);
+                    }
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(tc::smem_u32(&T.empty[s]));
+                }
+                float acc[8];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], 16);   // phases 2 sw, 2 sw + 1
-            float *xch = T.sum_xch;
-            if (sw == 1 && lane < 16) {
+                for (int e = 0; e < 4; ++e) unpack2(acc2[e], acc[2 * e], acc[2 * e + 1]);
 #pragma unroll
-                for (int e = 0; e < 8; ++e) xch[ch * 8 + e] = acc[e];
-            }
-            sum_warps_barrier();
-            if (sw == 0 && lane < 16 && ntiles > 0) {
-                float *out = gram_part + ((size_t)u * splits + c) * (kD * kD + kD) + kD * kD;
+                for (int e = 0; e < 8; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], 16);   // phases 2 sw, 2 sw + 1
+                float *xch = T.sum_xch[j & 1];         // the array of item j - 2 has been read: the barrier of j - 1 is past
+                if (sw == 1 && lane < 16) {
 #pragma unroll
-                for (int e = 0; e < 8; ++e) out[ch * 8 + e] = acc[e] + xch[ch * 8 + e];
+                    for (int e = 0; e < 8; ++e) xch[ch * 8 + e] = acc[e];
+                }
+                sum_warps_barrier();
+                if (sw == 0 && lane < 16 && ok) {
+                    float *out = gram_part + (size_t)j * (kD * kD + kD) + kD * kD;
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) out[ch * 8 + e] = acc[e] + xch[ch * 8 + e];
+                }
             }
         }
     } else {
         // ---------------- softmax warps ----------------
         const int quarter = warp & 3, half = (warp >> 2) & 1, group = warp >> 3;
         const int lane_row = quarter * 32 + lane;          // TMEM lane: a window row (A) or a token (B)
-        const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)half * 64;
+        const int copy = PASS_B ? 0 : lane_row / kRows;    // pass A: the copy of the rows this lane belongs to
+        const int col0 = PASS_B ? half * NC : half * 64 + copy * NC;
+        const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)col0;
         bool dead = false;
-        if (PASS_B) {
-            for (int r = threadIdx.x; r < MB * 128; r += kSoftThreads)
-                mp[r] = r < rows ? mprime[(size_t)u * kMaxRows + r] : INFINITY;
-            all_soft_barrier();
-        }
-        float m_run[MB], l_run[MB];
+        int n0 = 0, useq = -1, cur_u = -1;                 // tiles before this item, units seen
+        for (int j = first; j < last_item; ++j) {
+            const int u = j / splits, t0 = (j % splits) * chunk, t1 = min(limit, t0 + chunk), ntiles = tiles_of(j);
+            if (PASS_B && u != cur_u) {
+                // two arrays in turn: the one written here belonged to the unit before the last, which everyone has left
+                // since the barrier of the last
+                cur_u = u;
+                ++useq;
+                for (int r = threadIdx.x; r < MB * 128; r += kSoftThreads)
+                    mp[(useq & 1) * (MB * 128) + r] = r < rows ? -mprime[(size_t)u * kMaxRows + r] : -INFINITY;
+                all_soft_barrier();
+            }
+            const float *mpu = mp + (useq & 1) * (MB * 128);
+            float m_run[MB], l_run[MB];
 #pragma unroll
-        for (int mb = 0; mb < MB; ++mb) { m_run[mb] = -INFINITY; l_run[mb] = 0.f; }
+            for (int mb = 0; mb < MB; ++mb) { m_run[mb] = -INFINITY; l_run[mb] = 0.f; }
 
-        for (int i = group; i < ntiles; i += 2) {           // this group's tiles
-            const int tile_t0 = t0 + i * kTile;
-            const bool masked = tile_t0 + kTile > P;            // uniform over the CTA
-            float acc = 0.f;
+            for (int i = group ^ (n0 & 1); i < ntiles; i += 2) {    // this group's tiles
+                const int n = n0 + i, tile_t0 = t0 + i * kTile;
+                const bool masked = tile_t0 + kTile > P;            // uniform over the CTA
+                float acc = 0.f;
 #pragma unroll
-            for (int mb = 0; mb < MB; ++mb) {
-                const int buf = item_buf(i, mb);
-                uint32_t v[64];
+                for (int mb = 0; mb < MB; ++mb) {
+                    const int buf = item_buf(n, mb);
+                    uint32_t v[NC];
+                    if (!dead) {
+                        const bool ok = tc::mbar_wait(tc::smem_u32(&T.tfull[item_ready_bar(n, mb)]), item_ready_parity(n, mb),
+                                                      status);
+                        dead = !__all_sync(0xffffffffu, ok);
+                    }
+                    if (!dead) {
+                        tc::tc_fence_after();
+                        load_columns<NC>(tbase + buf * 128, v);
+                        tc::tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) tc::mbar_arrive(tc::smem_u32(&T.tempty[buf]));
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < NC; ++e) v[e] = 0u;
+                    }
+                    if (PASS_B) {
+                        acc += colsum_partial<NC>(v, c_log2, mpu + mb * 128 + half * NC);
+                    } else {
+                        const int r = mb * 128 + lane_row % kRows;
+                        const int last = P + (r % w);                       // last visible position of this row
+                        const int pos0 = tile_t0 + col0;
+                        if (masked) stats_update<true, NC>(v, c_log2, pos0, last, m_run[mb], l_run[mb]);
+                        else stats_update<false, NC>(v, c_log2, pos0, last, m_run[mb], l_run[mb]);
+                    }
+                }
+                if (PASS_B) {
+                    // the two column halves of this group meet in shared memory (slot = tile parity within the group)
+                    float *cs = colsum + ((n >> 1) & 1) * 512 + group * 256;
+                    cs[half * 128 + lane_row] = acc;
+                    group_barrier(group);
+                    const int pos = tile_t0 + lane_row;
+                    if (half == 0 && pos < min(t1, P) && !dead) raw[(size_t)u * P + pos] = cs[lane_row] + cs[128 + lane_row];
+                }
+            }
+            n0 += ntiles;
+            if (GRAM) {
+                // drain the Gram block: warp (quarter, cb) stores rows 32 quarter .. +31, columns 32 cb .. +31
                 if (!dead) {
-                    const bool ok = tc::mbar_wait(tc::smem_u32(&T.tfull[item_ready_bar(i, mb)]), item_ready_parity(i, mb),
-                                                  status);
+                    const bool ok = tc::mbar_wait(tc::smem_u32(&T.gfull), (j - first) & 1, status);
                     dead = !__all_sync(0xffffffffu, ok);
                 }
                 if (!dead) {
                     tc::tc_fence_after();
-                    uint32_t va[32], vb[32];
-                    tc::tmem_ld32(tbase + buf * 128, va);
-                    tc::tmem_ld32(tbase + buf * 128 + 32, vb);
+                    const int cb = warp >> 2;
+                    float *out = gram_part + (size_t)j * (kD * kD + kD);
+                    uint32_t r[32];
+                    tc::tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + kGramCol + cb * 32, r);
                     tc::tmem_ld_wait();
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) { v[j] = va[j]; v[32 + j] = vb[j]; }
                     tc::tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) tc::mbar_arrive(tc::smem_u32(&T.tempty[buf]));
-                } else {
+                    if (lane == 0) tc::mbar_arrive(tc::smem_u32(&T.gdrained));
+                    float4 *dst = reinterpret_cast<float4 *>(out + (size_t)lane_row * kD + cb * 32);
 #pragma unroll
-                    for (int j = 0; j < 64; ++j) v[j] = 0u;
-                }
-                if (PASS_B) {
-                    acc += colsum_partial(v, c_log2, mp + mb * 128 + half * 64);
-                } else {
-                    const int r = mb * 128 + lane_row;
-                    const int last = P + (r % w);                       // last visible position of this row
-                    const int pos0 = tile_t0 + half * 64;
-                    if (masked) stats_update<true>(v, c_log2, pos0, last, m_run[mb], l_run[mb]);
-                    else stats_update<false>(v, c_log2, pos0, last, m_run[mb], l_run[mb]);
+                    for (int q4 = 0; q4 < 8; ++q4)
+                        dst[q4] = make_float4(__uint_as_float(r[4 * q4]), __uint_as_float(r[4 * q4 + 1]),
+                                              __uint_as_float(r[4 * q4 + 2]), __uint_as_float(r[4 * q4 + 3]));
                 }
             }
-            if (PASS_B) {
-                // the two column halves of this group meet in shared memory (slot = tile parity within the group)
-                float *cs = colsum + ((i >> 1) & 1) * 512 + group * 256;
-                cs[half * 128 + lane_row] = acc;
-                group_barrier(group);
-                const int pos = tile_t0 + lane_row;
-                if (half == 0 && pos < min(t1, P) && !dead) raw[(size_t)u * P + pos] = cs[lane_row] + cs[128 + lane_row];
-            }
-        }
-        if (!PASS_B) {
-            // merge the four (group, half) partials of every row in a fixed order.  Scratch: the query blocks,
-            // which no MMA reads any more once both groups have consumed every accumulator (the K stages may still
-            // feed deferred Gram MMAs).
-            float2 *merge = reinterpret_cast<float2 *>(smem);                         // [4][MB * 128]
-            all_soft_barrier();            // both groups have consumed their last accumulator
-            const int slot = group * 2 + half;
+            if (!PASS_B) {
+                // merge the four (group, half) partials of every row, and of its copies, in a fixed order
+                all_soft_barrier();            // the item before has been read
+                const int slot = group * 2 + half;
 #pragma unroll
-            for (int mb = 0; mb < MB; ++mb) merge[slot * (MB * 128) + mb * 128 + lane_row] = make_float2(m_run[mb], l_run[mb]);
-            all_soft_barrier();
-            if (slot == 0 && !dead) {
+                for (int mb = 0; mb < MB; ++mb) merge[slot * (MB * 128) + mb * 128 + lane_row] = make_float2(m_run[mb], l_run[mb]);
+                all_soft_barrier();
+                if (slot == 0 && !dead) {
 #pragma unroll
-                for (int mb = 0; mb < MB; ++mb) {
-                    const int r = mb * 128 + lane_row;
-                    if (r < rows) {
-                        float m = -INFINITY;
+                    for (int mb = 0; mb < MB; ++mb) {
+                        const int r = mb * 128 + lane_row;
+                        if (r < rows) {                                 // SPLIT > 1: rows <= kRows, the lanes of copy 0
+                            float m = -INFINITY;
 #pragma unroll
-                        for (int sl = 0; sl < 4; ++sl) m = fmaxf(m, merge[sl * (MB * 128) + r].x);
-                        float lsum = 0.f;
+                            for (int sl = 0; sl < 4 * SPLIT; ++sl)
+                                m = fmaxf(m, merge[(sl / SPLIT) * (MB * 128) + r + (sl % SPLIT) * kRows].x);
+                            float lsum = 0.f;
 #pragma unroll
-                        for (int sl = 0; sl < 4; ++sl) {
-                            const float2 ml = merge[sl * (MB * 128) + r];
-                            if (ml.x > -INFINITY) lsum += ml.y * ex2(ml.x - m);
+                            for (int sl = 0; sl < 4 * SPLIT; ++sl) {
+                                const float2 ml = merge[(sl / SPLIT) * (MB * 128) + r + (sl % SPLIT) * kRows];
+                                if (ml.x > -INFINITY) lsum += ml.y * ex2(ml.x - m);
+                            }
+                            float *o = stats_part + ((size_t)j * kMaxRows + r) * 2;
+                            o[0] = m;
+                            o[1] = lsum;
                         }
-                        float *o = stats_part + (((size_t)u * splits + c) * kMaxRows + r) * 2;
-                        o[0] = m;
-                        o[1] = lsum;
                     }
                 }
-            }
-        }
-        if (GRAM) {
-            // drain the Gram block: warp (quarter, cb) stores rows 32 quarter .. +31, columns 32 cb .. +31
-            bool ok = ntiles > 0 && tc::mbar_wait(tc::smem_u32(&T.gfull), 0, status);
-            ok = __all_sync(0xffffffffu, ok) && !dead;
-            if (ok) {
-                tc::tc_fence_after();
-                const int cb = warp >> 2;
-                float *out = gram_part + ((size_t)u * splits + c) * (kD * kD + kD);
-                uint32_t r[32];
-                tc::tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + kGramCol + cb * 32, r);
-                tc::tmem_ld_wait();
-                float4 *dst = reinterpret_cast<float4 *>(out + (size_t)lane_row * kD + cb * 32);
-#pragma unroll
-                for (int q4 = 0; q4 < 8; ++q4)
-                    dst[q4] = make_float4(__uint_as_float(r[4 * q4]), __uint_as_float(r[4 * q4 + 1]),
-                                          __uint_as_float(r[4 * q4 + 2]), __uint_as_float(r[4 * q4 + 3]));
             }
         }
     }
@@ -472,55 +600,37 @@ __global__ void score_tc_merge_kernel(const float *__restrict__ stats_part, int 
     mprime[(size_t)u * kMaxRows + r] = m + log2f(l);
 }
 
-// cudaFuncSetAttribute is sticky per function and device: done once per device and instantiation
-template <int MB>
-static cudaError_t raise_smem_limit_once() {
+template <int MB, int MODE, int SPLIT>
+static cudaError_t raise_smem_limit() {
     static bool done[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
-    const int smem = score_smem(MB);
-    e = cudaFuncSetAttribute(score_tc_kernel<MB, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(score_tc_kernel<MB, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(score_tc_kernel<MB, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
-    return e;
+    return allow_dynamic_smem((const void *)score_tc_kernel<MB, MODE, SPLIT>, score_smem(MB), done);
 }
 
-template <int MB>
-static cudaError_t raise_smem_limit_mode3() {
-    static bool done[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
-    e = cudaFuncSetAttribute(score_tc_kernel<MB, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, score_smem(MB));
-    if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
-    return e;
-}
-
-template <int MB>
-static cudaError_t launch_scores_tc_mb(const Plan &p, const CUtensorMap &tq, const CUtensorMap &tk, const void *dK,
-                                       const UnitAddr &addr, float c_log2,
+template <int MB, int SPLIT>
+static cudaError_t launch_scores_tc_mb(const Plan &p, const CUtensorMap &tq, const CUtensorMap &tk, float c_log2,
                                        const float *d_lse, float *d_stats_part, float *d_mprime, float *d_raw,
                                        float *d_gram_part, int phases, uint32_t *d_status, Profiler *prof,
                                        cudaStream_t st) {
     const uncomp_shape &s = p.shape;
     const int smem = score_smem(MB);
-    cudaError_t e = raise_smem_limit_once<MB>();
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    int dev = 0, sms = kTargetSms;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // one CTA per SM, each with an equal share of the (unit, chunk) items
+    auto ctas = [&](int splits) { return (unsigned)min((int64_t)sms, (int64_t)p.units * splits); };
     if (phases & kScorePhaseStats) {
+        e = d_gram_part ? raise_smem_limit<MB, 2, SPLIT>() : raise_smem_limit<MB, 0, SPLIT>();
+        if (e != cudaSuccess) return e;
         ProfScope ps(prof, d_gram_part ? kSlotGramStats : kSlotScoreStats, st);
-        dim3 grid(p.score_splits, p.units);
         if (d_gram_part)
-            score_tc_kernel<MB, 2><<<grid, kGramThreads, smem, st>>>(tq, tk, s.L, s.H, s.N, s.w, p.rows, p.score_chunk,
-                                                                      p.score_splits, c_log2, d_stats_part, nullptr,
-                                                                      nullptr, d_gram_part, dK, addr, d_status);
+            score_tc_kernel<MB, 2, SPLIT><<<ctas(p.score_splits), kGramThreads, smem, st>>>(
+                tq, tk, s.L, s.H, s.N, s.w, p.rows, p.units, p.score_chunk, p.score_splits, c_log2, d_stats_part, nullptr, nullptr,
+                d_gram_part, d_status);
         else
-            score_tc_kernel<MB, 0><<<grid, kScoreThreads, smem, st>>>(tq, tk, s.L, s.H, s.N, s.w, p.rows, p.score_chunk,
-                                                                      p.score_splits, c_log2, d_stats_part, nullptr,
-                                                                      nullptr, nullptr, nullptr, addr, d_status);
+            score_tc_kernel<MB, 0, SPLIT><<<ctas(p.score_splits), kScoreThreads, smem, st>>>(
+                tq, tk, s.L, s.H, s.N, s.w, p.rows, p.units, p.score_chunk, p.score_splits, c_log2, d_stats_part, nullptr, nullptr,
+                nullptr, d_status);
     }
     if (phases & kScorePhaseColsum) {
         const bool with_gram = (phases & kScorePhaseStats) == 0 && d_gram_part != nullptr;   // mode 3
@@ -538,18 +648,18 @@ static cudaError_t launch_scores_tc_mb(const Plan &p, const CUtensorMap &tq, con
         ProfScope ps(prof, with_gram ? kSlotGramColsum : kSlotScoreColsum, st);
         const int splitsB = (p.prefix + p.score_chunk - 1) / p.score_chunk;
         if (with_gram) {
-            e = raise_smem_limit_mode3<MB>();
+            e = raise_smem_limit<MB, 3, SPLIT>();
             if (e != cudaSuccess) return e;
-            dim3 grid3(p.score_splits, p.units);
-            score_tc_kernel<MB, 3><<<grid3, kGramThreads, smem, st>>>(tq, tk, s.L, s.H, s.N, s.w, p.rows, p.score_chunk,
-                                                                     p.score_splits, c_log2, nullptr, d_mprime, d_raw,
-                                                                     d_gram_part, dK, addr, d_status);
+            score_tc_kernel<MB, 3, SPLIT><<<ctas(p.score_splits), kGramThreads, smem, st>>>(
+                tq, tk, s.L, s.H, s.N, s.w, p.rows, p.units, p.score_chunk, p.score_splits, c_log2, nullptr, d_mprime, d_raw,
+                d_gram_part, d_status);
             return cudaGetLastError();
         }
-        dim3 grid(splitsB, p.units);
-        score_tc_kernel<MB, 1><<<grid, kScoreThreads, smem, st>>>(tq, tk, s.L, s.H, s.N, s.w, p.rows, p.score_chunk,
-                                                                  splitsB, c_log2, nullptr, d_mprime, d_raw, nullptr,
-                                                                  nullptr, addr, d_status);
+        e = raise_smem_limit<MB, 1, SPLIT>();
+        if (e != cudaSuccess) return e;
+        score_tc_kernel<MB, 1, SPLIT><<<ctas(splitsB), kScoreThreads, smem, st>>>(tq, tk, s.L, s.H, s.N, s.w, p.rows, p.units,
+                                                                                 p.score_chunk, splitsB, c_log2, nullptr, d_mprime,
+                                                                                 d_raw, nullptr, d_status);
     }
     return cudaGetLastError();
 }
@@ -562,11 +672,13 @@ cudaError_t launch_scores_tc(const Plan &p, const void *dQw, const void *dK, con
     if (e != cudaSuccess) return e;
     const float c_log2 = scale * 1.4426950408889634f;
     const int MB = (p.rows + 127) / 128;
+    if (p.rows <= 32) return launch_scores_tc_mb<1, 4>(p, tq, tk, c_log2, d_lse, d_stats_part, d_stats, d_raw, d_gram_part, phases, d_status, prof, st);
+    if (p.rows <= 64) return launch_scores_tc_mb<1, 2>(p, tq, tk, c_log2, d_lse, d_stats_part, d_stats, d_raw, d_gram_part, phases, d_status, prof, st);
     switch (MB) {
-        case 1: return launch_scores_tc_mb<1>(p, tq, tk, dK, addr, c_log2, d_lse, d_stats_part, d_stats, d_raw, d_gram_part, phases, d_status, prof, st);
-        case 2: return launch_scores_tc_mb<2>(p, tq, tk, dK, addr, c_log2, d_lse, d_stats_part, d_stats, d_raw, d_gram_part, phases, d_status, prof, st);
-        case 3: return launch_scores_tc_mb<3>(p, tq, tk, dK, addr, c_log2, d_lse, d_stats_part, d_stats, d_raw, d_gram_part, phases, d_status, prof, st);
-        default: return launch_scores_tc_mb<4>(p, tq, tk, dK, addr, c_log2, d_lse, d_stats_part, d_stats, d_raw, d_gram_part, phases, d_status, prof, st);
+        case 1: return launch_scores_tc_mb<1, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_stats, d_raw, d_gram_part, phases, d_status, prof, st);
+        case 2: return launch_scores_tc_mb<2, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_stats, d_raw, d_gram_part, phases, d_status, prof, st);
+        case 3: return launch_scores_tc_mb<3, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_stats, d_raw, d_gram_part, phases, d_status, prof, st);
+        default: return launch_scores_tc_mb<4, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_stats, d_raw, d_gram_part, phases, d_status, prof, st);
     }
 }
 

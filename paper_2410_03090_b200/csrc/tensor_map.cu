@@ -44,12 +44,13 @@ cudaError_t make_key_tensor_map(CUtensorMap *map, const uncomp_shape &s, const U
     return encode_tensor_map(map, dK, 5, dims, str, box, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
-// Tensor map over the window queries [units, rows, d] (contiguous bf16): box = 64 features x 128 rows.
+// Tensor map over the window queries [units, rows, d] (contiguous bf16): box = 64 features x 128 rows, or 64 or 32 rows
+// when there are no more.
 // Rows beyond `rows` read as zero.
 cudaError_t make_query_tensor_map(CUtensorMap *map, const void *dQw, int units, int rows) {
     uint64_t dims[3] = {(uint64_t)kD, (uint64_t)rows, (uint64_t)units};
     uint64_t str[2] = {(uint64_t)kD * 2, (uint64_t)rows * kD * 2};
-    uint32_t box[3] = {64, 128, 1};
+    uint32_t box[3] = {64, rows <= 32 ? 32u : (rows <= 64 ? 64u : 128u), 1};
     return encode_tensor_map(map, dQw, 3, dims, str, box, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 

@@ -1,0 +1,50 @@
+"""The persistent scorer where its variants and its work split change: numbers of window rows around 32, 64, 128 and 512,
+several (unit, chunk) items per CTA with units changing inside a CTA, ragged last tiles; scores, entropies and the
+log-sum-exp form against the oracle."""
+from dataclasses import replace
+
+import pytest
+import torch
+
+import parity
+from paper_2410_03090_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _lse(wl, K, Qw):
+    q = Qw.float().view(wl.B, wl.L, wl.H, wl.G * wl.w, wl.d)
+    s = torch.einsum("blhrd,blhnd->blhrn", q, K.float()) / wl.d ** 0.5
+    last = (wl.N - wl.w + torch.arange(wl.w, device="cuda")).repeat(wl.G)
+    s.masked_fill_(torch.arange(wl.N, device="cuda")[None, :] > last[:, None], float("-inf"))
+    return torch.logsumexp(s, dim=-1).view(wl.B, wl.L, wl.Hq, wl.w)
+
+
+@pytest.mark.parametrize("L,H,G,w,N", [
+    (1, 1, 1, 1, 129),        # one row, one item
+    (20, 8, 4, 8, 700),       # 32 rows; 320 items, two chunks per unit
+    (1, 3, 3, 11, 1300),      # 33 rows
+    (19, 8, 1, 64, 640),      # 64 rows; 152 units of two chunks, the second is one full tile
+    (1, 2, 5, 13, 641),       # 65 rows, one token in the last tile
+    (40, 8, 4, 32, 512),      # 128 rows; 320 units of one chunk: the queries change with every item
+    (20, 8, 3, 43, 520),      # 129 rows, one query buffer
+    (20, 8, 8, 48, 600),      # 384 rows
+    (20, 8, 8, 64, 1100),     # 512 rows
+])
+def test_items(L, H, G, w, N):
+    from paper_2410_03090_b200.compress import CompressionPass
+    avg = w + 20
+    wl = replace(synth.WORKLOADS["c2"], L=L, H=H, Hq=H * G, N=N, w=w, avg_budget=avg, M=1, n_max=avg, seed=31)
+    K, V, Qw = synth.generate(wl, "cuda")
+    cp = CompressionPass(wl, "cuda")
+    units = sorted({0, 1 % wl.units, wl.units // 2, wl.units - 1})
+    for out in (lambda: cp.run(K, V, Qw), lambda: cp.run_one_call(K, V, Qw), lambda: cp.run_one_call(K, V, Qw, lse=_lse(wl, K, Qw)),
+                lambda: cp.run(K, V, Qw, lse=_lse(wl, K, Qw))):
+        cp.out.scores.fill_(-1)
+        cp.out.entropy.fill_(-1)
+        o = out()
+        torch.cuda.synchronize()
+        assert cp.status() == 0
+        assert bool((o.scores >= 0).all()) and bool((o.entropy >= 0).all())
+        parity.check_scores(wl, K, Qw, o.scores, units)
+        parity.check_entropy(wl, K, o.entropy, o.erank, units)
