@@ -7,103 +7,110 @@
 // t_g = n_max - g * n (n_max - avg) / S, S = sum_g n_g g, is kept as the exact fraction num_g / S, heads
 // get floor(t_g) and the tokens still missing go to the largest remainders (ties: better rank).  Every
 // step is integer arithmetic, so the budgets are reproducible bit for bit.
+//
+// What bounds it is latency.  A remainder belongs to a group, so who gets a missing token follows from a table of the M
+// groups (remainder, heads ahead of the group) and a head's rank inside its group; S and the number of missing tokens
+// come from the host; ranks are counted in shared memory; the prefix sum is one of warps.  With 64-bit divisions in every
+// thread, remainders compared head by head in global memory and a scan with 20 barriers 256 units took 15 us
+// (of which 9 are the launch and its event records), now 11.
 #include "common.cuh"
 
 namespace uncomp {
 
 constexpr int kBudThreads = 1024;
+constexpr int kBudShared = 4096;      // effective ranks and groups held in shared memory
 
-__host__ __device__ __forceinline__ int group_lo(int g, int n, int M) { return (int)(((int64_t)g * n) / M); }
+// first rank of group g: floor(g n / M)
+__host__ __device__ __forceinline__ int group_lo(int g, int n, int M) {
+    const uint64_t p = (uint64_t)g * (uint64_t)n;
+    return p >> 32 ? (int)(p / (uint64_t)M) : (int)((uint32_t)p / (uint32_t)M);
+}
 
+struct BudSched {
+    int64_t S;            // sum_g n_g g
+    int missing;          // tokens of a ranking set that the floors leave undistributed
+};
+
+// grid (1).  table_ahead [M] and table_rem [M]: scratch for the group table when M > kBudShared.
 __global__ void __launch_bounds__(kBudThreads) budgets_kernel(const float *__restrict__ erank, int B, int L, int H,
-                                                             int N, int w, uncomp_budget_params bp,
+                                                             int N, int w, uncomp_budget_params bp, BudSched sched,
                                                              int32_t *__restrict__ budgets,
                                                              int64_t *__restrict__ offsets,
                                                              int32_t *__restrict__ layer_group,
                                                              int32_t *__restrict__ layer_ctx,
-                                                             int32_t *__restrict__ rank_ws,
-                                                             int64_t *__restrict__ rem_ws) {
-    const int tid = threadIdx.x;
+                                                             int32_t *__restrict__ table_ahead,
+                                                             int64_t *__restrict__ table_rem) {
+    extern __shared__ int64_t bud_smem[];
+    __shared__ int64_t warp_total[kBudThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int units = B * L * H;
     const int n = bp.scope ? L * H : H;          // ranking-set size
     const int M = bp.M;
-    const int64_t avg = bp.avg_budget, n_max = bp.n_max;
-
-    // S = sum_g n_g * g and the tokens the floors leave undistributed (same for every ranking set)
-    int64_t S = 0, floor_total = 0;
-    for (int g = 0; g < M; ++g) S += (int64_t)(group_lo(g + 1, n, M) - group_lo(g, n, M)) * g;
-    for (int g = 0; g < M; ++g) {
-        const int64_t ng = group_lo(g + 1, n, M) - group_lo(g, n, M);
-        const int64_t fl = M == 1 ? avg : (n_max * S - (int64_t)g * n * (n_max - avg)) / S;
-        floor_total += ng * fl;
-    }
-    const int missing = (int)((int64_t)n * avg - floor_total);
-
-    // phase 1: rank within the set, group, floor and remainder
-    for (int u = tid; u < units; u += kBudThreads) {
-        const int set_base = (u / n) * n;
-        const float e = erank[u];
-        int r = 0;
-        for (int j = 0; j < n; ++j) {
-            const float ej = erank[set_base + j];
-            r += (ej > e) || (ej == e && set_base + j < u);
-        }
-        int g = (int)(((int64_t)r * M) / n);
-        while (g + 1 < M && group_lo(g + 1, n, M) <= r) ++g;
-        while (g > 0 && group_lo(g, n, M) > r) --g;
-        int64_t fl, rem;
-        if (M == 1) { fl = avg; rem = 0; }
-        else {
-            const int64_t num = n_max * S - (int64_t)g * n * (n_max - avg);
-            fl = num / S;
-            rem = num % S;
-        }
-        rank_ws[u] = r;
-        rem_ws[u] = rem;
-        budgets[u] = (int32_t)fl;
-    }
+    const int64_t avg = bp.avg_budget, n_max = bp.n_max, S = sched.S;
+    const bool shared_tab = M <= kBudShared, shared_er = units <= kBudShared;
+    int64_t *rem_t = shared_tab ? bud_smem : table_rem;                              // [M]
+    int32_t *ahead_t = shared_tab ? reinterpret_cast<int32_t *>(bud_smem + M) : table_ahead;   // [M]
+    float *er_s = reinterpret_cast<float *>(shared_tab ? reinterpret_cast<int32_t *>(bud_smem + M) + M
+                                                       : reinterpret_cast<int32_t *>(bud_smem));
+    const float *er = shared_er ? er_s : erank;
+    if (shared_er)
+        for (int u = tid; u < units; u += kBudThreads) er_s[u] = erank[u];
+    auto target = [&](int g) { return n_max * S - (int64_t)g * n * (n_max - avg); };   // t_g S
+    for (int g = tid; g < M; g += kBudThreads) rem_t[g] = M == 1 ? 0 : target(g) % S;
     __syncthreads();
-    // phase 2: largest remainders
-    for (int u = tid; u < units; u += kBudThreads) {
-        const int set_base = (u / n) * n;
-        const int64_t rem = rem_ws[u];
-        const int r = rank_ws[u];
+    // heads ahead of group g when the missing tokens are handed out: larger remainder, or the same and a better rank
+    for (int g = tid; g < M; g += kBudThreads) {
+        const int64_t rem = rem_t[g];
         int ahead = 0;
-        for (int j = 0; j < n; ++j) {
-            const int64_t rj = rem_ws[set_base + j];
-            ahead += (rj > rem) || (rj == rem && rank_ws[set_base + j] < r);
+        for (int o = 0; o < M; ++o) {
+            const int64_t ro = rem_t[o];
+            if (ro > rem || (ro == rem && o < g)) ahead += group_lo(o + 1, n, M) - group_lo(o, n, M);
         }
-        if (ahead < missing) budgets[u] += 1;
+        ahead_t[g] = ahead;
     }
     __syncthreads();
-    // phase 3: exclusive prefix sum over units, a block scan per 1024 units with a running carry
-    __shared__ int64_t scan[kBudThreads];
-    __shared__ int64_t carry;
-    if (tid == 0) { carry = 0; offsets[0] = 0; }
-    __syncthreads();
+    // budgets and their exclusive prefix sum over the units, 1024 units at a time
+    int64_t carry = 0;
+    if (tid == 0) offsets[0] = 0;
     for (int base = 0; base < units; base += kBudThreads) {
         const int u = base + tid;
-        scan[tid] = u < units ? (int64_t)budgets[u] : 0;
-        __syncthreads();
-        for (int o = 1; o < kBudThreads; o <<= 1) {
-            const int64_t add = tid >= o ? scan[tid - o] : 0;
-            __syncthreads();
-            scan[tid] += add;
-            __syncthreads();
+        int64_t budget = 0;
+        if (u < units) {
+            const int set_base = (u / n) * n;
+            const float e = er[u];
+            int r = 0;
+            for (int j = set_base; j < u; ++j) r += er[j] >= e;            // equal values: the lower index first
+            for (int j = u + 1; j < set_base + n; ++j) r += er[j] > e;
+            const uint64_t rm = (uint64_t)r * (uint64_t)M;
+            int g = rm >> 32 ? (int)(rm / (uint64_t)n) : (int)((uint32_t)rm / (uint32_t)n);
+            while (g + 1 < M && group_lo(g + 1, n, M) <= r) ++g;
+            while (g > 0 && group_lo(g, n, M) > r) --g;
+            budget = M == 1 ? avg : target(g) / S;
+            if (ahead_t[g] + r - group_lo(g, n, M) < sched.missing) budget += 1;
+            budgets[u] = (int32_t)budget;
         }
-        if (u < units) offsets[u + 1] = carry + scan[tid];
+        int64_t incl = budget;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t below = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += below;
+        }
+        if (lane == 31) warp_total[wid] = incl;
         __syncthreads();
-        if (tid == 0) carry += scan[kBudThreads - 1];
+        int64_t before = 0, all = warp_total[lane];
+        if (lane < wid) before = all;
+        before = warp_sum_i64(before);
+        all = warp_sum_i64(all);
+        if (u < units) offsets[u + 1] = carry + before + incl;
+        carry += all;
         __syncthreads();
     }
-    // phase 4: layer groups
-    if (layer_group && layer_ctx) {
+    // layer groups
+    if (layer_group && layer_ctx && bp.dn <= 0) {
+        for (int i = tid; i < B * L; i += kBudThreads) { layer_group[i] = 0; layer_ctx[i] = N; }
+    } else if (layer_group && layer_ctx) {
         for (int b = tid; b < B; b += kBudThreads) {
             int32_t *lg = layer_group + (size_t)b * L, *lc = layer_ctx + (size_t)b * L;
-            if (bp.dn <= 0) {
-                for (int l = 0; l < L; ++l) { lg[l] = 0; lc[l] = N; }
-                continue;
-            }
             int boundaries = 0;
             lg[0] = 0;
             double prev = 0.0;
@@ -146,8 +153,23 @@ int check_budget_params(const uncomp_shape &s, const uncomp_budget_params &bp) {
 cudaError_t launch_budgets(const Plan &p, const float *d_erank, const uncomp_budget_params &bp, int32_t *d_budgets,
                            int64_t *d_offsets, int32_t *d_layer_group, int32_t *d_layer_ctx, int32_t *d_rank,
                            int64_t *d_rem, cudaStream_t st) {
-    budgets_kernel<<<1, kBudThreads, 0, st>>>(d_erank, p.shape.B, p.shape.L, p.shape.H, p.shape.N, p.shape.w, bp,
-                                              d_budgets, d_offsets, d_layer_group, d_layer_ctx, d_rank, d_rem);
+    const int n = bp.scope ? p.shape.L * p.shape.H : p.shape.H, M = bp.M;
+    BudSched sched{0, 0};
+    int64_t floor_total = 0;
+    for (int g = 0; g < M; ++g) sched.S += (int64_t)(group_lo(g + 1, n, M) - group_lo(g, n, M)) * g;
+    for (int g = 0; g < M; ++g) {
+        const int64_t ng = group_lo(g + 1, n, M) - group_lo(g, n, M);
+        const int64_t fl = M == 1 ? bp.avg_budget
+                                  : (bp.n_max * sched.S - (int64_t)g * n * (bp.n_max - bp.avg_budget)) / sched.S;
+        floor_total += ng * fl;
+    }
+    sched.missing = (int)((int64_t)n * bp.avg_budget - floor_total);
+    const size_t smem = (M <= kBudShared ? (size_t)M * 12 : 0) + (p.units <= kBudShared ? (size_t)p.units * 4 : 0);
+    static bool done[64] = {};
+    cudaError_t e = allow_dynamic_smem((const void *)budgets_kernel, kBudShared * 16, done);
+    if (e != cudaSuccess) return e;
+    budgets_kernel<<<1, kBudThreads, smem, st>>>(d_erank, p.shape.B, p.shape.L, p.shape.H, p.shape.N, p.shape.w, bp, sched,
+                                                 d_budgets, d_offsets, d_layer_group, d_layer_ctx, d_rank, d_rem);
     return cudaGetLastError();
 }
 

@@ -2,12 +2,10 @@
 // the tokens with the highest cumulative window attention are kept within the head's budget; the w
 // window tokens are part of the budget).
 //
-// One CTA of 1024 threads per unit.
 //   1. pooled[j] = max / mean of raw over the pool window clipped to the prefix (written out: it is the
 //      `d_scores` output of the pass).
-//   2. Radix select of the k-th largest pooled score, k = budget - w, on the order-preserving 32-bit
-//      image of the float: three histogram passes (11 + 11 + 10 bits) give the exact threshold T, the
-//      number of scores above it and how many scores equal to T are still needed.
+//   2. the k-th largest pooled score, k = budget - w, on the order-preserving 32-bit image of the float: the exact
+//      threshold T, the number of scores above it and how many scores equal to T are still needed.
 //   3. Ordered compaction: each warp owns a contiguous segment; ballots and population counts give every
 //      kept position its output slot, so the kept positions come out ascending, and among scores equal to
 //      T the lowest positions win.  The window positions follow.
@@ -82,102 +80,9 @@ __device__ void find_bin(SelSmem &S, int nbins, int kr, int tid) {
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(kSelThreads) pool_select_kernel(const float *__restrict__ raw,
-                                                                 float *__restrict__ pooled, int P, int w,
-                                                                 int pool_kernel, int pool_mode,
-                                                                 const int32_t *__restrict__ budgets,
-                                                                 const int64_t *__restrict__ offsets,
-                                                                 int units, int32_t *__restrict__ indices,
-                                                                 uint32_t *__restrict__ status) {
-    __shared__ SelSmem S;
-    const int u = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const float *r = raw + (size_t)u * P;
-    float *s = pooled + (size_t)u * P;
-
-    // ---- 1. pooling ------------------------------------------------------------------------------
-    const int half = pool_kernel >> 1;
-    for (int j = tid; j < P; j += kSelThreads) {
-        const int lo = max(0, j - half), hi = min(P - 1, j + half);
-        float acc = pool_mode ? 0.f : r[lo];
-        for (int t = lo; t <= hi; ++t) acc = pool_mode ? acc + r[t] : fmaxf(acc, r[t]);
-        s[j] = pool_mode ? acc / (float)(hi - lo + 1) : acc;
-    }
-    const Slab slab = slab_of(budgets, offsets, units, u, P, w, tid == 0, status);
-    const int k = slab.k;
-    int32_t *out = indices + slab.begin;
-    for (int i = tid; i < slab.wn; i += kSelThreads)
-            if (UNCOMP_INDEX_OK(k + i, slab.seg, status)) out[k + i] = P + i;
-    for (int64_t i = tid; i < slab.fill; i += kSelThreads)
-            if (UNCOMP_INDEX_OK(k + slab.wn + i, slab.seg, status)) out[k + slab.wn + i] = P + w - 1;
-    if (k == 0) return;   // uniform over the CTA
-    __syncthreads();      // pooled scores of this unit are visible to the whole CTA
-
-    // ---- 2. threshold ----------------------------------------------------------------------------
-    uint32_t prefix = 0;      // bits of the threshold fixed so far
-    int kr = k;               // rank still to resolve inside the current bin
-    if (k < P) {
-#pragma unroll 1
-        for (int pass = 0; pass < 3; ++pass) {
-            const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
-            const int nbits = pass == 2 ? 10 : 11;
-            const int nbins = 1 << nbits;
-            const uint32_t himask = pass == 0 ? 0u : (0xffffffffu << (shift + nbits));
-            for (int b = tid; b < 2048; b += kSelThreads) S.hist[b] = 0;
-            __syncthreads();
-            for (int j = tid; j < P; j += kSelThreads) {
-                const uint32_t v = ordered_bits(s[j]);
-                if ((v & himask) == prefix && UNCOMP_INDEX_OK((v >> shift) & (nbins - 1), 2048, status))
-                    atomicAdd(&S.hist[(v >> shift) & (nbins - 1)], 1);
-            }
-            __syncthreads();
-            find_bin(S, nbins, kr, tid);
-            prefix |= (uint32_t)S.bin << shift;
-            kr -= S.above;
-            __syncthreads();
-        }
-    }
-    // k >= P keeps every prefix position: threshold below everything
-    const uint32_t T = k < P ? prefix : 0u;
-    const int need_eq = k < P ? kr : P;   // scores equal to T that are still kept (lowest positions first)
-
-    // ---- 3. ordered compaction -------------------------------------------------------------------
-    const int seg = ((P + kSelWarps - 1) / kSelWarps + 31) & ~31;
-    const int j0 = min(P, wid * seg), j1 = min(P, j0 + seg);
-    int cg = 0, ce = 0;
-    for (int j = j0 + lane; j < j1; j += 32) {
-        const uint32_t v = ordered_bits(s[j]);
-        cg += v > T;
-        ce += v == T;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        cg += __shfl_xor_sync(0xffffffffu, cg, o);
-        ce += __shfl_xor_sync(0xffffffffu, ce, o);
-    }
-    if (lane == 0) { S.warp_gt[wid] = cg; S.warp_eq[wid] = ce; }
-    __syncthreads();
-    int gt_run = 0, eq_run = 0;
-    for (int x = 0; x < wid; ++x) { gt_run += S.warp_gt[x]; eq_run += S.warp_eq[x]; }
-    const unsigned lt = (1u << lane) - 1u;
-    for (int jb = j0; jb < j1; jb += 32) {
-        const int j = jb + lane;
-        const uint32_t v = j < j1 ? ordered_bits(s[j]) : 0u;
-        const bool gt = j < j1 && v > T;
-        const bool eq = j < j1 && v == T;
-        const unsigned mg = __ballot_sync(0xffffffffu, gt), me = __ballot_sync(0xffffffffu, eq);
-        const int gtb = gt_run + __popc(mg & lt);
-        const int eqb = eq_run + __popc(me & lt);
-        if ((gt || (eq && eqb < need_eq)) && UNCOMP_INDEX_OK(gtb + min(eqb, need_eq), k, status))
-            out[gtb + min(eqb, need_eq)] = j;
-        gt_run += __popc(mg);
-        eq_run += __popc(me);
-    }
-}
-
-// The same selection with a unit spread over a cluster of 8 CTAs, for calls with few units (a layer of one sequence,
-// the hidden-state eviction with one unit per sequence), where one CTA per unit would leave most SMs idle.  CTA r of
-// the cluster owns the r-th eighth of the positions; histograms and counts are combined through distributed shared
-// memory by CTA 0 and read back by the others.  The result is identical to the single-CTA kernel.
+// ---- longer prefixes: radix select of the pooled scores in global memory ------------------------------------------
+// A cluster of 8 CTAs per unit.  CTA r owns the r-th eighth of the positions; histograms and counts are combined through
+// distributed shared memory by CTA 0 and read back by the others.
 constexpr int kSelCluster = 8;
 
 __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kSelThreads)
@@ -297,20 +202,350 @@ pool_select_cluster_kernel(const float *__restrict__ raw, float *__restrict__ po
     cluster.sync();       // no CTA leaves while another may still read its shared memory
 }
 
+// ---- prefixes up to 262144 positions: keys in shared memory --------------------------------------------------------
+// A unit is a CTA of 1024 threads (up to 32768 positions) or a cluster of 2, 4 or 8; a warp owns NBK x 128 consecutive
+// positions, a lane 4 consecutive ones of every 128.  The pooled scores replace the raw ones in shared memory as
+// order-preserving integers.  The threshold comes from
+// histograms of 2048 bins over the range the keys really span (not over their leading bits: scores share most of those,
+// and the shared-memory atomics of a warp would meet in a few bins), then over the chosen bin, at most three times.  One
+// cluster barrier per histogram: every CTA adds up all of them, the next pass uses another array.
+// Bound by shared-memory atomics, barriers and, with many units, issue.  256 units of 32704 positions / 1024 of 3704 / 8
+// of 6969: radix select that read the pooled scores from global memory three times with 20 barriers a pass 75 / 61 / 23 us,
+// keys in registers and a search bit by bit with counts (no atomics, 20 to 30 rounds) 163 / 74 / 25 us, this 65 / 50 / 15 us
+// (128 of 131008: 133 us, was 201).
+constexpr int kKeyThreads = 1024;
+constexpr int kKeyWarps = kKeyThreads / 32;
+constexpr int kKeyMaxCluster = 8;
+constexpr int kKeyHalo = 32;                             // pool windows reach at most 31 positions beyond a CTA's share
+constexpr int kKeyBins = 2 * kKeyThreads;
+enum { kPoolAny, kPoolNone, kPoolMax7 };
+
+template <int NBK> struct KeySmem {
+    float raw[2 * kKeyHalo + kKeyWarps * NBK * 128];     // this CTA's raw scores with their neighbours, later its keys
+    int hist[3][kKeyBins];
+    unsigned slot[2][2][kKeyMaxCluster];                 // [exchange][value][CTA of the cluster]
+    unsigned warp_a[kKeyWarps], warp_b[kKeyWarps];
+    int warp_sum[kKeyWarps];
+    int bin, above, in_bin;
+};
+
+template <int NBK, int POOL>
+__global__ void __launch_bounds__(kKeyThreads, NBK <= 4 ? 2 : 1)
+pool_select_keys_kernel(const float *__restrict__ raw, float *__restrict__ pooled, int P, int w, int pool_kernel, int pool_mode,
+                        const int32_t *__restrict__ budgets, const int64_t *__restrict__ offsets, int units,
+                        int32_t *__restrict__ indices, uint32_t *__restrict__ status) {
+    namespace cg = cooperative_groups;
+    constexpr int kShare = kKeyWarps * NBK * 128, kWarpShare = NBK * 128;
+    extern __shared__ __align__(16) unsigned char key_smem[];
+    KeySmem<NBK> &S = *reinterpret_cast<KeySmem<NBK> *>(key_smem);
+    cg::cluster_group cluster = cg::this_cluster();
+    const int ctas = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int u = blockIdx.x / ctas, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const float *r = raw + (size_t)u * P;
+    float *s = pooled + (size_t)u * P;
+    const int p0 = rank * kShare;                        // S.raw[i] is position p0 - kKeyHalo + i
+    const int half = pool_kernel >> 1;
+    if (ctas > 1) cluster.barrier_arrive();              // waited for before anybody's shared memory is touched
+
+    // ---- 1. raw scores to shared memory, pooled scores out and, as keys, in their place ---------------------
+    const float outside = pool_mode ? 0.f : -INFINITY;
+    constexpr int kVec = (kShare + 2 * kKeyHalo) / 4;
+    if ((reinterpret_cast<uintptr_t>(r) & 15u) == 0) {
+#pragma unroll 4
+        for (int i = tid; i < kVec; i += kKeyThreads) {
+            const int j = p0 - kKeyHalo + 4 * i;
+            float4 x = make_float4(outside, outside, outside, outside);
+            if (j >= 0 && j + 3 < P) x = __ldg(reinterpret_cast<const float4 *>(r + j));
+            else if (j >= 0 && j < P) {
+                x.x = r[j];
+                if (j + 1 < P) x.y = r[j + 1];
+                if (j + 2 < P) x.z = r[j + 2];
+            }
+            reinterpret_cast<float4 *>(S.raw)[i] = x;
+        }
+    } else {
+#pragma unroll 8
+        for (int i = tid; i < kShare + 2 * kKeyHalo; i += kKeyThreads) {
+            const int j = p0 - kKeyHalo + i;
+            S.raw[i] = j >= 0 && j < P ? __ldg(r + j) : outside;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 3 * kKeyBins / kKeyThreads; ++i) (&S.hist[0][0])[tid + i * kKeyThreads] = 0;
+    const Slab slab = slab_of(budgets, offsets, units, u, P, w, tid == 0 && rank == 0, status);
+    const int k = slab.k;
+    int32_t *out = indices + slab.begin;
+    if (rank == 0) {
+        for (int i = tid; i < slab.wn; i += kKeyThreads)
+            if (UNCOMP_INDEX_OK(k + i, slab.seg, status)) out[k + i] = P + i;
+        for (int64_t i = tid; i < slab.fill; i += kKeyThreads)
+            if (UNCOMP_INDEX_OK(k + slab.wn + i, slab.seg, status)) out[k + slab.wn + i] = P + w - 1;
+    }
+    __syncthreads();
+    const int at0 = wid * kWarpShare + lane * 4, j0 = p0 + at0;        // block b: 128 b further
+    float *mine = S.raw + kKeyHalo + at0;
+    const bool vec = (reinterpret_cast<uintptr_t>(s) & 15u) == 0;
+    uint32_t hi = 0u, lo = 0xffffffffu;
+    auto finish = [&](int b, const float4 &o) {          // pooled scores out, keys in place; 0 beyond the prefix
+        const int j = j0 + 128 * b;
+        if (vec && j + 3 < P) {
+            *reinterpret_cast<float4 *>(s + j) = o;
+        } else {
+            if (j < P) s[j] = o.x;
+            if (j + 1 < P) s[j + 1] = o.y;
+            if (j + 2 < P) s[j + 2] = o.z;
+            if (j + 3 < P) s[j + 3] = o.w;
+        }
+        uint4 key = make_uint4(ordered_bits(o.x), ordered_bits(o.y), ordered_bits(o.z), ordered_bits(o.w));
+        if (j + 3 < P) {
+            hi = max(max(hi, max(key.x, key.y)), max(key.z, key.w));
+            lo = min(min(lo, min(key.x, key.y)), min(key.z, key.w));
+        } else {
+            if (j < P) { hi = max(hi, key.x); lo = min(lo, key.x); } else key.x = 0u;
+            if (j + 1 < P) { hi = max(hi, key.y); lo = min(lo, key.y); } else key.y = 0u;
+            if (j + 2 < P) { hi = max(hi, key.z); lo = min(lo, key.z); } else key.z = 0u;
+            key.w = 0u;
+        }
+        *reinterpret_cast<uint4 *>(mine + 128 * b) = key;
+    };
+    if (POOL == kPoolMax7) {
+        // the neighbours that other warps overwrite are taken before anybody writes
+        const float4 left = *reinterpret_cast<const float4 *>(mine - 4);                       // lane 0 uses it
+        const float4 right = *reinterpret_cast<const float4 *>(mine + 128 * (NBK - 1) + 4);    // lane 31 uses it
+        __syncthreads();
+        float4 m = *reinterpret_cast<const float4 *>(mine);
+        float py = left.y, pz = left.z, pw = left.w;     // raw scores left of the lane's first position
+#pragma unroll
+        for (int b = 0; b < NBK; ++b) {
+            const float4 next = b + 1 < NBK ? *reinterpret_cast<const float4 *>(mine + 128 * (b + 1)) : right;
+            // right of the lane: the next lane's, for lane 31 the first of the next 128
+            float ax = __shfl_up_sync(0xffffffffu, m.y, 1), ay = __shfl_up_sync(0xffffffffu, m.z, 1), az = __shfl_up_sync(0xffffffffu, m.w, 1);
+            const float nx = b + 1 < NBK ? __shfl_sync(0xffffffffu, next.x, 0) : right.x;
+            const float ny = b + 1 < NBK ? __shfl_sync(0xffffffffu, next.y, 0) : right.y;
+            const float nz = b + 1 < NBK ? __shfl_sync(0xffffffffu, next.z, 0) : right.z;
+            float zx = __shfl_down_sync(0xffffffffu, m.x, 1), zy = __shfl_down_sync(0xffffffffu, m.y, 1), zz = __shfl_down_sync(0xffffffffu, m.z, 1);
+            if (lane == 0) { ax = py; ay = pz; az = pw; }
+            if (lane == 31) { zx = nx; zy = ny; zz = nz; }
+            py = __shfl_sync(0xffffffffu, m.y, 31);
+            pz = __shfl_sync(0xffffffffu, m.z, 31);
+            pw = __shfl_sync(0xffffffffu, m.w, 31);
+            const float mid = fmaxf(fmaxf(m.x, m.y), fmaxf(m.z, m.w));
+            const float4 o = make_float4(fmaxf(mid, fmaxf(ax, fmaxf(ay, az))), fmaxf(mid, fmaxf(fmaxf(ay, az), zx)),
+                                         fmaxf(mid, fmaxf(az, fmaxf(zx, zy))), fmaxf(mid, fmaxf(zx, fmaxf(zy, zz))));
+            finish(b, o);
+            m = next;
+        }
+    } else if (POOL == kPoolNone) {
+#pragma unroll
+        for (int b = 0; b < NBK; ++b) finish(b, *reinterpret_cast<const float4 *>(mine + 128 * b));
+    } else {
+        auto pooled_at = [&](int at, int j) {
+            const float *x = S.raw + kKeyHalo + at;
+            float acc;
+            if (pool_mode) {
+                const int lo_j = max(0, j - half), hi_j = min(P - 1, j + half);
+                acc = 0.f;
+                for (int t = lo_j; t <= hi_j; ++t) acc += x[t - j];
+                return acc / (float)(hi_j - lo_j + 1);
+            }
+            acc = x[-half];
+            for (int t = 1 - half; t <= half; ++t) acc = fmaxf(acc, x[t]);
+            return acc;
+        };
+        for (int i = tid; i < kShare; i += kKeyThreads)
+            if (p0 + i < P) s[p0 + i] = pooled_at(i, p0 + i);
+        __syncthreads();                                 // nobody reads raw scores any more; s is visible to the CTA
+#pragma unroll 1
+        for (int b = 0; b < NBK; ++b) {
+            const int j = j0 + 128 * b;
+            finish(b, make_float4(j < P ? s[j] : 0.f, j + 1 < P ? s[j + 1] : 0.f, j + 2 < P ? s[j + 2] : 0.f, j + 3 < P ? s[j + 3] : 0.f));
+        }
+    }
+    if (ctas > 1) cluster.barrier_wait();
+    if (k == 0) return;                                  // uniform over the cluster, nobody has touched a peer's memory
+
+    // From here on a thread reads only the keys it has written.
+    auto keys = [&](int b) { return *reinterpret_cast<const uint4 *>(mine + 128 * b); };
+
+    // ---- 2. threshold ------------------------------------------------------------------------------
+    uint32_t T = 0;
+    bool all_equal_kept = k >= P;                        // every key that equals T is kept
+    if (k < P) {
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        if (lane == 0) { S.warp_a[wid] = hi; S.warp_b[wid] = lo; }
+        __syncthreads();
+        hi = __reduce_max_sync(0xffffffffu, S.warp_a[lane]);
+        lo = __reduce_min_sync(0xffffffffu, S.warp_b[lane]);
+        if (ctas > 1) {
+            if (tid < ctas) {
+                KeySmem<NBK> *R = cluster.map_shared_rank(&S, tid);
+                R->slot[0][0][rank] = hi;
+                R->slot[0][1][rank] = lo;
+            }
+            cluster.sync();
+            for (int c = 0; c < ctas; ++c) { hi = max(hi, S.slot[0][0][c]); lo = min(lo, S.slot[0][1][c]); }
+        }
+        int kr = k;                                      // rank to resolve inside [lo, lo + width)
+        uint32_t width = hi - lo;                        // first as the largest distance
+        int shift = max(0, 21 - __clz((int)width));      // 11 bits of it
+        if (width == 0u) { T = lo; __syncthreads(); }    // all keys equal; warp_a is written again below
+#pragma unroll 1
+        for (int pass = 0; width != 0u; ++pass) {
+            int *hist = S.hist[pass];
+            const uint32_t last = pass == 0 ? width : width - 1;      // largest distance from lo that counts
+#pragma unroll
+            for (int b = 0; b < NBK; ++b) {
+                const uint4 key = keys(b);
+                const uint32_t d[4] = {key.x - lo, key.y - lo, key.z - lo, key.w - lo};
+                const int left = P - (j0 + 128 * b);     // of the four, those before the prefix' end
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (d[c] <= last && c < left && UNCOMP_INDEX_OK(d[c] >> shift, kKeyBins, status)) atomicAdd(&hist[d[c] >> shift], 1);
+            }
+            if (ctas > 1) cluster.sync();                // every histogram of the cluster is complete
+            else __syncthreads();
+            // bins from the top: this thread has bins b0 and b0 - 1
+            const int b0 = kKeyBins - 1 - 2 * tid;
+            int h0 = 0, h1 = 0;
+            for (int c = 0; c < ctas; ++c) {
+                const int2 h = *reinterpret_cast<const int2 *>(&(ctas > 1 ? cluster.map_shared_rank(&S, c) : &S)->hist[pass][b0 - 1]);
+                h0 += h.y;
+                h1 += h.x;
+            }
+            int incl = h0 + h1;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int below = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += below;
+            }
+            if (lane == 31) S.warp_sum[wid] = incl;
+            __syncthreads();
+            const int excl = incl - h0 - h1 + __reduce_add_sync(0xffffffffu, lane < wid ? S.warp_sum[lane] : 0);
+            if (excl < kr && kr <= excl + h0) { S.bin = b0; S.above = excl; S.in_bin = h0; }
+            else if (excl + h0 < kr && kr <= excl + h0 + h1) { S.bin = b0 - 1; S.above = excl + h0; S.in_bin = h1; }
+            __syncthreads();
+            lo += (uint32_t)S.bin << shift;
+            kr -= S.above;
+            T = lo;
+            all_equal_kept = S.in_bin == kr;             // the whole bin is kept: T is its lower end
+            if (all_equal_kept || shift == 0) break;
+            width = 1u << shift;
+            shift = max(0, shift - 11);
+            __syncthreads();                             // bin, above and in_bin are read before the next pass writes them
+        }
+    }
+
+    // ---- 3. ordered compaction: counts of the lower CTAs, then of the lower warps ------------------------
+    // kept: above T (low half of a count), equal to T (high half); when all equal ones are kept they count as above
+    auto is_above = [&](uint32_t x) { return all_equal_kept ? x >= T : x > T; };
+    unsigned cnt = 0;
+#pragma unroll
+    for (int b = 0; b < NBK; ++b) {
+        const uint4 key = keys(b);
+        const int left = P - (j0 + 128 * b);
+        cnt += (is_above(key.x) && 0 < left) + (is_above(key.y) && 1 < left) + (is_above(key.z) && 2 < left) + (is_above(key.w) && 3 < left);
+        if (!all_equal_kept) cnt += ((key.x == T && 0 < left) + (key.y == T && 1 < left) + (key.z == T && 2 < left) + (key.w == T && 3 < left)) << 16;
+    }
+    unsigned gt = __reduce_add_sync(0xffffffffu, cnt & 0xffffu), eq = __reduce_add_sync(0xffffffffu, cnt >> 16);
+    if (lane == 0) { S.warp_a[wid] = gt; S.warp_b[wid] = eq; }
+    __syncthreads();
+    unsigned gt_run = __reduce_add_sync(0xffffffffu, lane < wid ? S.warp_a[lane] : 0u);
+    unsigned eq_run = __reduce_add_sync(0xffffffffu, lane < wid ? S.warp_b[lane] : 0u);
+    unsigned gt_all = __reduce_add_sync(0xffffffffu, S.warp_a[lane]);
+    if (ctas > 1) {
+        const unsigned eq_all = __reduce_add_sync(0xffffffffu, S.warp_b[lane]);
+        if (tid < ctas) {
+            KeySmem<NBK> *R = cluster.map_shared_rank(&S, tid);
+            R->slot[1][0][rank] = gt_all;
+            R->slot[1][1][rank] = eq_all;
+        }
+        cluster.sync();                                  // also the last access to a peer's memory
+        gt_all = 0;
+        for (int c = 0; c < ctas; ++c) {
+            gt_all += S.slot[1][0][c];
+            if (c < rank) { gt_run += S.slot[1][0][c]; eq_run += S.slot[1][1][c]; }
+        }
+    }
+    const unsigned need_eq = all_equal_kept ? 0u : (unsigned)k - gt_all;
+#pragma unroll
+    for (int b = 0; b < NBK; ++b) {
+        const uint4 kv = keys(b);
+        const uint32_t key[4] = {kv.x, kv.y, kv.z, kv.w};
+        const int j = j0 + 128 * b, left = P - j;
+        unsigned own = 0;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            own += is_above(key[c]) && c < left;
+            if (!all_equal_kept) own += (key[c] == T && c < left) << 16;
+        }
+        if (!__any_sync(0xffffffffu, own != 0u)) continue;
+        unsigned incl = own;                             // 128 of each at most: the halves do not meet
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned below = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += below;
+        }
+        const unsigned total = __shfl_sync(0xffffffffu, incl, 31);
+        unsigned g = gt_run + ((incl - own) & 0xffffu), e = eq_run + ((incl - own) >> 16);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const bool is_gt = is_above(key[c]) && c < left, is_eq = !all_equal_kept && key[c] == T && c < left;
+            const unsigned at = g + min(e, need_eq);
+            if ((is_gt || (is_eq && e < need_eq)) && UNCOMP_INDEX_OK(at, k, status)) out[at] = j + c;
+            g += is_gt;
+            e += is_eq;
+        }
+        gt_run += total & 0xffffu;
+        eq_run += total >> 16;
+    }
+}
+
+template <int NBK, int POOL>
+cudaError_t launch_keys(const Plan &p, int ctas, const float *d_raw, float *d_pooled, int pool_kernel, int pool_mode,
+                        const int32_t *d_budgets, const int64_t *d_offsets, int32_t *d_indices, uint32_t *d_status, cudaStream_t st) {
+    static bool done[64] = {};
+    cudaError_t e = allow_dynamic_smem((const void *)pool_select_keys_kernel<NBK, POOL>, sizeof(KeySmem<NBK>), done);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = ctas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(p.units * ctas);
+    cfg.blockDim = dim3(kKeyThreads);
+    cfg.dynamicSmemBytes = sizeof(KeySmem<NBK>);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = ctas > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, pool_select_keys_kernel<NBK, POOL>, d_raw, d_pooled, p.prefix, p.shape.w, pool_kernel, pool_mode,
+                              d_budgets, d_offsets, p.units, d_indices, d_status);
+}
+
+template <int POOL>
+cudaError_t launch_keys_nbk(const Plan &p, int n, int ctas, const float *d_raw, float *d_pooled, int pool_kernel, int pool_mode,
+                            const int32_t *d_budgets, const int64_t *d_offsets, int32_t *d_indices, uint32_t *d_status, cudaStream_t st) {
+    const auto f = n > 4 * ctas ? launch_keys<8, POOL> : n > 2 * ctas ? launch_keys<4, POOL> : n > ctas ? launch_keys<2, POOL> : launch_keys<1, POOL>;
+    return f(p, ctas, d_raw, d_pooled, pool_kernel, pool_mode, d_budgets, d_offsets, d_indices, d_status, st);
+}
+
 cudaError_t launch_pool_select(const Plan &p, const float *d_raw, float *d_pooled, int pool_kernel, int pool_mode,
                                const int32_t *d_budgets, const int64_t *d_offsets, int32_t *d_indices,
                                uint32_t *d_status, cudaStream_t st) {
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (p.units * kSelCluster <= 2 * sms && p.prefix >= 4096)      // few units: a cluster of CTAs per unit
+    // 4096 positions per CTA and block of keys.  One CTA per unit up to 32768 positions (a cluster barrier costs a
+    // microsecond), clusters beyond; shorter shares only while most of the GPU would idle.
+    const int n = (p.prefix + 4095) / 4096;
+    if (n > 64) {
         pool_select_cluster_kernel<<<p.units * kSelCluster, kSelThreads, 0, st>>>(
             d_raw, d_pooled, p.prefix, p.shape.w, pool_kernel, pool_mode, d_budgets, d_offsets, p.units, d_indices,
             d_status);
-    else
-        pool_select_kernel<<<p.units, kSelThreads, 0, st>>>(d_raw, d_pooled, p.prefix, p.shape.w, pool_kernel, pool_mode,
-                                                            d_budgets, d_offsets, p.units, d_indices, d_status);
-    return cudaGetLastError();
+        return cudaGetLastError();
+    }
+    int ctas = 1;
+    while (ctas < kKeyMaxCluster && (n > 8 * ctas || (n > 2 * ctas && (int64_t)p.units * ctas * 2 <= kTargetSms))) ctas *= 2;
+    const auto f = pool_kernel == 1 ? launch_keys_nbk<kPoolNone>
+                                    : pool_kernel == 7 && pool_mode == 0 ? launch_keys_nbk<kPoolMax7> : launch_keys_nbk<kPoolAny>;
+    return f(p, n, ctas, d_raw, d_pooled, pool_kernel, pool_mode, d_budgets, d_offsets, d_indices, d_status, st);
 }
 
 }  // namespace uncomp
