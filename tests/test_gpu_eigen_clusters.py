@@ -18,6 +18,9 @@ pytestmark = pytest.mark.gpu
     (1, 75, 2100, 128),    # clusters of one, all eigenvalues
     (2, 74, 600, 32),      # 148 units, one and two partials
     (3, 50, 2, 32),        # two tokens: rank one after centring
+    (8, 37, 600, 32),      # 296 units: the last count of one kernel
+    (9, 33, 700, 32),      # 297 units: a second kernel for the last 64 steps, three of four warps in its last CTA idle
+    (10, 32, 300, 100),    # more eigenvalues than lanes there
 ])
 def test_cluster_sizes(L, H, N, k_trunc):
     from paper_2410_03090_b200 import binding as ub
