@@ -291,8 +291,7 @@ int uncomp_entropy(uncomp_ctx *ctx, const void *d_K, uncomp_strides sK, const un
     if (tensor_path && d_Qw) {
         // one sweep over K: Gram partials per scorer chunk and the scorer's row statistics
         const float sc = effective_scale(scale, p.shape.d);
-        e = launch_scores_tc(p, d_Qw, d_K, addr, sc, nullptr, reinterpret_cast<float *>(ctx->ws + p.off_stats_part),
-                             reinterpret_cast<float *>(ctx->ws + p.off_stats), nullptr,
+        e = launch_scores_tc(p, d_Qw, d_K, addr, sc, nullptr, reinterpret_cast<float *>(ctx->ws + p.off_stats_part), nullptr,
                              reinterpret_cast<float *>(partials), kScorePhaseStats, d_status, &ctx->tmaps, ctx->prof, st);
         if (e != cudaSuccess) return cuda_fail(ctx, e);
         parts = p.score_splits;
@@ -388,7 +387,7 @@ int uncomp_score_select(uncomp_ctx *ctx, const void *d_Qw, const void *d_K, unco
     cudaError_t e;
     if (tensor_path) {
         const int phases = (reuse || d_lse) ? kScorePhaseColsum : (kScorePhaseStats | kScorePhaseColsum);
-        e = launch_scores_tc(p, d_Qw, d_K, addr, scale, d_lse, stats_part, stats, raw, nullptr, phases, d_status,
+        e = launch_scores_tc(p, d_Qw, d_K, addr, scale, d_lse, stats_part, raw, nullptr, phases, d_status,
                              &ctx->tmaps, ctx->prof, st);
     } else {
         e = launch_scores_simt(p, d_Qw, d_K, addr, scale, d_lse, stats_part, stats, raw, d_status, ctx->prof, st);
@@ -457,8 +456,7 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
         const UnitAddr addr = make_addr(p.shape, sK);
         ctx->stats_valid = 0;
         cudaError_t e = launch_scores_tc(p, d_Qw, d_K, addr, effective_scale(sparams->scale, p.shape.d), d_lse,
-                                         reinterpret_cast<float *>(ctx->ws + p.off_stats_part),
-                                         reinterpret_cast<float *>(ctx->ws + p.off_stats), raw, partials, kScorePhaseColsum,
+                                         reinterpret_cast<float *>(ctx->ws + p.off_stats_part), raw, partials, kScorePhaseColsum,
                                          d_status, &ctx->tmaps, ctx->prof, st);
         if (e != cudaSuccess) return cuda_fail(ctx, e);
         {
@@ -480,11 +478,10 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
         }
         if (e != cudaSuccess) return cuda_fail(ctx, e);
     } else if (tensor_path) {
-        // Gram + statistics sweep; then eigenvalues and budgets on a second stream beside the merge and the column
-        // sums: neither needs the other, only the selection needs both.  The eigenvalue kernel is a chain of
-        // dependent steps that leaves most of an SM idle; beside the column sums it costs little (measured against
-        // the staged order: 0.51 ms instead of 0.59 ms at 8K tokens, 1.88 instead of 1.93 ms at 32K tokens, no
-        // change with four 32K-token sequences).
+        // Gram + statistics sweep; then eigenvalues and budgets beside the column sums: neither needs the other, only the
+        // selection needs both.  The two cannot share an SM (registers), so which one is launched first matters: while all
+        // units are in work at once the eigenvalues are a chain on a few SMs and go first, on the caller's stream (one layer
+        // of 7001 tokens 138 us, 175 the other way round); with more units the column sums do (four 32K sequences 5.05 ms, 5.19).
         if (!d_K || !d_Qw || !d_entropy || !d_budgets || !d_offsets || !d_indices) return UNCOMP_E_NULL;
         if (!aligned16(d_K) || !aligned16(d_Qw)) return UNCOMP_E_ALIGN;
         rc = check_strides(p.shape, sK);
@@ -505,32 +502,35 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
         uint32_t *d_status = reinterpret_cast<uint32_t *>(ctx->ws + p.off_status);
         float *partials = reinterpret_cast<float *>(ctx->ws + p.off_gram);
         float *stats_part = reinterpret_cast<float *>(ctx->ws + p.off_stats_part);
-        float *stats = reinterpret_cast<float *>(ctx->ws + p.off_stats);
         float *raw = reinterpret_cast<float *>(ctx->ws + p.off_raw);
         float *pooled = d_scores ? d_scores : reinterpret_cast<float *>(ctx->ws + p.off_pooled);
         const UnitAddr addr = make_addr(p.shape, sK);
         const float sc = effective_scale(sparams->scale, p.shape.d);
         ctx->stats_valid = 0;
-        e = launch_scores_tc(p, d_Qw, d_K, addr, sc, nullptr, stats_part, stats, nullptr, partials, kScorePhaseStats,
+        e = launch_scores_tc(p, d_Qw, d_K, addr, sc, nullptr, stats_part, nullptr, partials, kScorePhaseStats,
                              d_status, &ctx->tmaps, ctx->prof, st);
+        const bool eigen_first = p.units <= 2 * kTargetSms;
+        cudaStream_t st_eigen = eigen_first ? st : ctx->side, st_sums = eigen_first ? ctx->side : st;
         if (e == cudaSuccess) e = cudaEventRecord(ctx->ev_fork, st);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0);
         if (e != cudaSuccess) return cuda_fail(ctx, e);
-        {
-            ProfScope ps(ctx->prof, kSlotEigen, ctx->side);
-            e = launch_eigen_f32(p, partials, p.score_splits, *eparams, d_entropy, d_erank, nullptr, d_status, ctx->side);
+        auto sums = [&] {
+            return launch_scores_tc(p, d_Qw, d_K, addr, sc, nullptr, stats_part, raw, nullptr, kScorePhaseColsum, d_status,
+                                    &ctx->tmaps, ctx->prof, st_sums);
+        };
+        if (!eigen_first) e = sums();
+        if (e == cudaSuccess) {
+            ProfScope ps(ctx->prof, kSlotEigen, st_eigen);
+            e = launch_eigen_f32(p, partials, p.score_splits, *eparams, d_entropy, d_erank, nullptr, d_status, st_eigen);
         }
-        if (e != cudaSuccess) return cuda_fail(ctx, e);
-        {
-            ProfScope ps(ctx->prof, kSlotBudgets, ctx->side);
+        if (e == cudaSuccess && eigen_first) e = sums();
+        if (e == cudaSuccess) {
+            ProfScope ps(ctx->prof, kSlotBudgets, st_eigen);
             e = launch_budgets(p, d_erank, *bparams, d_budgets, d_offsets, d_layer_group, d_layer_ctx,
                                reinterpret_cast<int32_t *>(ctx->ws + p.off_rank),
-                               reinterpret_cast<int64_t *>(ctx->ws + p.off_rem), ctx->side);
+                               reinterpret_cast<int64_t *>(ctx->ws + p.off_rem), st_eigen);
         }
         if (e == cudaSuccess) e = cudaEventRecord(ctx->ev_join, ctx->side);
-        if (e != cudaSuccess) return cuda_fail(ctx, e);
-        e = launch_scores_tc(p, d_Qw, d_K, addr, sc, nullptr, stats_part, stats, raw, nullptr, kScorePhaseColsum, d_status,
-                             &ctx->tmaps, ctx->prof, st);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ctx->ev_join, 0);
         if (e != cudaSuccess) return cuda_fail(ctx, e);
         {

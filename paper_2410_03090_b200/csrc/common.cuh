@@ -160,17 +160,12 @@ cudaError_t launch_budgets(const Plan &p, const float *d_erank, const uncomp_bud
 cudaError_t launch_scores_simt(const Plan &p, const void *dQw, const void *dK, const UnitAddr &addr, float scale,
                                const float *d_lse, float *d_stats_part, float *d_stats, float *d_raw,
                                uint32_t *d_status, Profiler *prof, cudaStream_t st);
-// Caller-supplied ln-sum-exp [units, rows] -> the merged statistics the column-sum kernels read: m' = lse * log2(e)
-// per row (log2_domain, tensor-core kernels) or the pair (lse, 1) (CUDA-core kernels).  A non-finite entry raises
-// UNCOMP_STATUS_NONFINITE and becomes +inf, so that its row adds nothing.
-cudaError_t launch_lse_import(const Plan &p, const float *d_lse, float *d_stats, bool log2_domain, uint32_t *d_status,
-                              cudaStream_t st);
 struct TmapCache;
 // phases: kScorePhaseStats (pass A; with d_gram_part != NULL the Gram partials of every (unit, scorer chunk) are
-// produced in the same sweep) and / or kScorePhaseColsum (merge, or the import of d_lse when given, + pass B).
+// produced in the same sweep) and / or kScorePhaseColsum (pass B, which merges the chunk statistics or takes d_lse).
 // kScorePhaseColsum alone with d_gram_part != NULL: pass B and the Gram partials from one sweep (needs d_lse).
 cudaError_t launch_scores_tc(const Plan &p, const void *dQw, const void *dK, const UnitAddr &addr, float scale,
-                             const float *d_lse, float *d_stats_part, float *d_stats, float *d_raw, float *d_gram_part,
+                             const float *d_lse, float *d_stats_part, float *d_raw, float *d_gram_part,
                              int phases, uint32_t *d_status, TmapCache *cache, Profiler *prof, cudaStream_t st);
 cudaError_t launch_pool_select(const Plan &p, const float *d_raw, float *d_pooled, int pool_kernel, int pool_mode,
                                const int32_t *d_budgets, const int64_t *d_offsets, int32_t *d_indices,

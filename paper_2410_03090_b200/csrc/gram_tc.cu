@@ -49,7 +49,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, int L, int H, int N, in
     GramSmemTail &T = *reinterpret_cast<GramSmemTail *>(ones + kOnesBytes);
 
     const int p = blockIdx.x, u = blockIdx.y;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // uniform for the compiler too
     const int h = u % H, l = (u / H) % L, b = u / (H * L);
     const int t0 = p * chunk;
     const int t1 = min(N, t0 + chunk);
@@ -102,7 +102,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, int L, int H, int N, in
         }
     } else if (warp == 5) {
         // ---------------- MMA issue ----------------
-        if (lane == 0) {
+        if (tc::elect_one()) {          // descriptors stay in uniform registers
             constexpr uint32_t idesc_g = tc::idesc_bf16_f32(128, 128, 1, 1);
             constexpr uint32_t idesc_s = tc::idesc_bf16_f32(128, 16, 1, 1);
             // descriptors: MN-major, 128-byte swizzle; feature halves kRegion apart (LBO), 8-token groups

@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(256) score_colsum_simt_kernel(const T *__restr
 }
 
 // one thread per (unit, row): the caller's natural-log sum of exponentials in place of pass A and the merge
-__global__ void lse_import_kernel(const float *__restrict__ lse, int units, int rows, int log2_domain,
+__global__ void lse_import_kernel(const float *__restrict__ lse, int units, int rows,
                                   float *__restrict__ stats, uint32_t *__restrict__ status) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= units * rows) return;
@@ -182,20 +182,8 @@ __global__ void lse_import_kernel(const float *__restrict__ lse, int units, int 
         atomicOr(status, (uint32_t)UNCOMP_STATUS_NONFINITE);
         v = INFINITY;                        // exp(s - inf) = 0: the row drops out of every column sum
     }
-    if (log2_domain) {
-        stats[(size_t)u * kMaxRows + r] = v * 1.4426950408889634f;
-    } else {
-        stats[((size_t)u * kMaxRows + r) * 2] = v;
-        stats[((size_t)u * kMaxRows + r) * 2 + 1] = 1.f;
-    }
-}
-
-cudaError_t launch_lse_import(const Plan &p, const float *d_lse, float *d_stats, bool log2_domain, uint32_t *d_status,
-                              cudaStream_t st) {
-    const int total = p.units * p.rows;
-    lse_import_kernel<<<(total + 255) / 256, 256, 0, st>>>(d_lse, p.units, p.rows, log2_domain ? 1 : 0, d_stats,
-                                                           d_status);
-    return cudaGetLastError();
+    stats[((size_t)u * kMaxRows + r) * 2] = v;
+    stats[((size_t)u * kMaxRows + r) * 2 + 1] = 1.f;
 }
 
 template <typename T>
@@ -211,8 +199,8 @@ static cudaError_t launch_scores_simt_t(const Plan &p, const T *dQw, const T *dK
     if (e != cudaSuccess) return e;
     if (d_lse) {
         ProfScope ps(prof, kSlotStatsMerge, st);
-        e = launch_lse_import(p, d_lse, d_stats, false, d_status, st);
-        if (e != cudaSuccess) return e;
+        const int total = p.units * p.rows;
+        lse_import_kernel<<<(total + 255) / 256, 256, 0, st>>>(d_lse, p.units, p.rows, d_stats, d_status);
     } else {
         const int row_blocks = (p.rows + kSB - 1) / kSB;
         dim3 gA(p.score_splits, row_blocks, p.units);

@@ -5,7 +5,7 @@
 //   pass A  S = Qw K^T with the window rows on the TMEM lanes (M = 128 rows, N = 128 tokens per MMA tile):
 //           a thread owns a row, so its running maximum and sum of exponentials are thread-local;
 //           every (unit, chunk) writes partial statistics (m, l) in the log2 domain;
-//   merge   partials combined in index order into m'_r = m_r + log2 l_r;
+//           pass B combines them in index order into m'_r = m_r + log2 l_r when it comes to a unit;
 //   pass B  operands swapped (M = 128 tokens on the lanes, N = 128 rows): a thread owns a token and adds
 //           2^(s c - m'_r) along its TMEM row; tokens of a warp are consecutive, the store is coalesced.
 // K tiles (128 tokens x 128 features, two 128B-swizzled boxes of 64 features) stream through a TMA ring;
@@ -161,6 +161,28 @@ __device__ __forceinline__ void load_columns(uint32_t taddr, uint32_t (&v)[NC]) 
 }
 }  // namespace
 
+// m'_r of row r of unit u in the log2 domain, for pass B: from the caller's log-sum-exp, or from the partial (m, l) of pass A,
+// combined in chunk order.  A non-finite log-sum-exp raises UNCOMP_STATUS_NONFINITE and its row adds nothing.
+__device__ __forceinline__ float row_norm(const float *__restrict__ stats, int parts, const float *__restrict__ lse, size_t u, int r,
+                                          int rows, uint32_t *status) {
+    if (lse) {
+        const float v = lse[u * rows + r];
+        if (isfinite(v)) return v * 1.4426950408889634f;
+        atomicOr(status, (uint32_t)UNCOMP_STATUS_NONFINITE);
+        return INFINITY;
+    }
+    const float2 *s = reinterpret_cast<const float2 *>(stats) + u * parts * kMaxRows + r;
+    float m = -INFINITY, l = 0.f;
+#pragma unroll 4
+    for (int p = 0; p < parts; ++p) m = fmaxf(m, s[(size_t)p * kMaxRows].x);
+#pragma unroll 4
+    for (int p = 0; p < parts; ++p) {
+        const float2 x = s[(size_t)p * kMaxRows];
+        if (x.x > -INFINITY) l += x.y * exp2f(x.x - m);
+    }
+    return m + log2f(l);
+}
+
 // MODE 0: pass A, 1: pass B, 2: pass A fused with the Gram stage, 3: pass B fused with it.
 // SPLIT 2 and 4 (MB = 1 only): at most 64 or 32 window rows.  A block of 128 rows would be mostly padding, and every
 // padded row costs as many exponentials as a real one.  Pass A keeps M = 128 but fills it with SPLIT copies of the rows;
@@ -170,7 +192,8 @@ template <int MB, int MODE, int SPLIT>
 __global__ void __launch_bounds__(kGramThreads, 1)
 score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant__ CUtensorMap tmapK, int L, int H,
                 int N, int w, int rows, int units, int chunk, int splits, float c_log2, float *__restrict__ stats_part,
-                const float *__restrict__ mprime, float *__restrict__ raw, float *__restrict__ gram_part,
+                const float *__restrict__ stats_in, int stats_splits, const float *__restrict__ lse, float *__restrict__ raw,
+                float *__restrict__ gram_part,
                 uint32_t *__restrict__ status) {
     constexpr bool PASS_B = MODE == 1 || MODE == 3, GRAM = MODE >= 2;
     // Accumulator buffers (128 TMEM columns each).  An accumulator holds one 128-row block of one tile; tile n (counted
@@ -474,7 +497,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
                 cur_u = u;
                 ++useq;
                 for (int r = threadIdx.x; r < MB * 128; r += kSoftThreads)
-                    mp[(useq & 1) * (MB * 128) + r] = r < rows ? -mprime[(size_t)u * kMaxRows + r] : -INFINITY;
+                    mp[(useq & 1) * (MB * 128) + r] =
+                        r < rows ? -row_norm(stats_in, stats_splits, lse, (size_t)u, r, rows, status) : -INFINITY;
                 all_soft_barrier();
             }
             const float *mpu = mp + (useq & 1) * (MB * 128);
@@ -584,22 +608,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
     if (warp == 17) tc::tmem_dealloc(tmem, 512);
 }
 
-// one thread per (unit, row): partial (m, l) in index order -> m' = m + log2 l
-__global__ void score_tc_merge_kernel(const float *__restrict__ stats_part, int units, int rows, int parts,
-                                      float *__restrict__ mprime) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= units * rows) return;
-    const int u = idx / rows, r = idx % rows;
-    float m = -INFINITY;
-    for (int p = 0; p < parts; ++p) m = fmaxf(m, stats_part[(((size_t)u * parts + p) * kMaxRows + r) * 2]);
-    float l = 0.f;
-    for (int p = 0; p < parts; ++p) {
-        const float *s = stats_part + (((size_t)u * parts + p) * kMaxRows + r) * 2;
-        if (s[0] > -INFINITY) l += s[1] * exp2f(s[0] - m);
-    }
-    mprime[(size_t)u * kMaxRows + r] = m + log2f(l);
-}
-
 template <int MB, int MODE, int SPLIT>
 static cudaError_t raise_smem_limit() {
     static bool done[64] = {};
@@ -608,7 +616,7 @@ static cudaError_t raise_smem_limit() {
 
 template <int MB, int SPLIT>
 static cudaError_t launch_scores_tc_mb(const Plan &p, const CUtensorMap &tq, const CUtensorMap &tk, float c_log2,
-                                       const float *d_lse, float *d_stats_part, float *d_mprime, float *d_raw,
+                                       const float *d_lse, float *d_stats_part, float *d_raw,
                                        float *d_gram_part, int phases, uint32_t *d_status, Profiler *prof,
                                        cudaStream_t st) {
     const uncomp_shape &s = p.shape;
@@ -625,60 +633,49 @@ static cudaError_t launch_scores_tc_mb(const Plan &p, const CUtensorMap &tq, con
         ProfScope ps(prof, d_gram_part ? kSlotGramStats : kSlotScoreStats, st);
         if (d_gram_part)
             score_tc_kernel<MB, 2, SPLIT><<<ctas(p.score_splits), kGramThreads, smem, st>>>(
-                tq, tk, s.L, s.H, s.N, s.w, p.rows, p.units, p.score_chunk, p.score_splits, c_log2, d_stats_part, nullptr, nullptr,
+                tq, tk, s.L, s.H, s.N, s.w, p.rows, p.units, p.score_chunk, p.score_splits, c_log2, d_stats_part, nullptr, 0, nullptr, nullptr,
                 d_gram_part, d_status);
         else
             score_tc_kernel<MB, 0, SPLIT><<<ctas(p.score_splits), kScoreThreads, smem, st>>>(
-                tq, tk, s.L, s.H, s.N, s.w, p.rows, p.units, p.score_chunk, p.score_splits, c_log2, d_stats_part, nullptr, nullptr,
+                tq, tk, s.L, s.H, s.N, s.w, p.rows, p.units, p.score_chunk, p.score_splits, c_log2, d_stats_part, nullptr, 0, nullptr, nullptr,
                 nullptr, d_status);
     }
     if (phases & kScorePhaseColsum) {
         const bool with_gram = (phases & kScorePhaseStats) == 0 && d_gram_part != nullptr;   // mode 3
-        {
-            ProfScope ps(prof, kSlotStatsMerge, st);
-            if (d_lse) {
-                e = launch_lse_import(p, d_lse, d_mprime, true, d_status, st);
-                if (e != cudaSuccess) return e;
-            } else {
-                const int total = p.units * p.rows;
-                score_tc_merge_kernel<<<(total + 255) / 256, 256, 0, st>>>(d_stats_part, p.units, p.rows,
-                                                                           p.score_splits, d_mprime);
-            }
-        }
         ProfScope ps(prof, with_gram ? kSlotGramColsum : kSlotScoreColsum, st);
         const int splitsB = (p.prefix + p.score_chunk - 1) / p.score_chunk;
         if (with_gram) {
             e = raise_smem_limit<MB, 3, SPLIT>();
             if (e != cudaSuccess) return e;
             score_tc_kernel<MB, 3, SPLIT><<<ctas(p.score_splits), kGramThreads, smem, st>>>(
-                tq, tk, s.L, s.H, s.N, s.w, p.rows, p.units, p.score_chunk, p.score_splits, c_log2, nullptr, d_mprime, d_raw,
-                d_gram_part, d_status);
+                tq, tk, s.L, s.H, s.N, s.w, p.rows, p.units, p.score_chunk, p.score_splits, c_log2, nullptr, d_stats_part, p.score_splits, d_lse,
+                d_raw, d_gram_part, d_status);
             return cudaGetLastError();
         }
         e = raise_smem_limit<MB, 1, SPLIT>();
         if (e != cudaSuccess) return e;
         score_tc_kernel<MB, 1, SPLIT><<<ctas(splitsB), kScoreThreads, smem, st>>>(tq, tk, s.L, s.H, s.N, s.w, p.rows, p.units,
-                                                                                 p.score_chunk, splitsB, c_log2, nullptr, d_mprime,
-                                                                                 d_raw, nullptr, d_status);
+                                                                                 p.score_chunk, splitsB, c_log2, nullptr, d_stats_part,
+                                                                                 p.score_splits, d_lse, d_raw, nullptr, d_status);
     }
     return cudaGetLastError();
 }
 
 cudaError_t launch_scores_tc(const Plan &p, const void *dQw, const void *dK, const UnitAddr &addr, float scale,
-                             const float *d_lse, float *d_stats_part, float *d_stats, float *d_raw, float *d_gram_part,
+                             const float *d_lse, float *d_stats_part, float *d_raw, float *d_gram_part,
                              int phases, uint32_t *d_status, TmapCache *cache, Profiler *prof, cudaStream_t st) {
     CUtensorMap tq, tk;
     cudaError_t e = cached_scorer_maps(cache, p, addr, dQw, dK, kTile, &tq, &tk);
     if (e != cudaSuccess) return e;
     const float c_log2 = scale * 1.4426950408889634f;
     const int MB = (p.rows + 127) / 128;
-    if (p.rows <= 32) return launch_scores_tc_mb<1, 4>(p, tq, tk, c_log2, d_lse, d_stats_part, d_stats, d_raw, d_gram_part, phases, d_status, prof, st);
-    if (p.rows <= 64) return launch_scores_tc_mb<1, 2>(p, tq, tk, c_log2, d_lse, d_stats_part, d_stats, d_raw, d_gram_part, phases, d_status, prof, st);
+    if (p.rows <= 32) return launch_scores_tc_mb<1, 4>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
+    if (p.rows <= 64) return launch_scores_tc_mb<1, 2>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
     switch (MB) {
-        case 1: return launch_scores_tc_mb<1, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_stats, d_raw, d_gram_part, phases, d_status, prof, st);
-        case 2: return launch_scores_tc_mb<2, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_stats, d_raw, d_gram_part, phases, d_status, prof, st);
-        case 3: return launch_scores_tc_mb<3, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_stats, d_raw, d_gram_part, phases, d_status, prof, st);
-        default: return launch_scores_tc_mb<4, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_stats, d_raw, d_gram_part, phases, d_status, prof, st);
+        case 1: return launch_scores_tc_mb<1, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
+        case 2: return launch_scores_tc_mb<2, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
+        case 3: return launch_scores_tc_mb<3, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
+        default: return launch_scores_tc_mb<4, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
     }
 }
 

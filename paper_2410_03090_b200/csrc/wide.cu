@@ -121,7 +121,7 @@ gram_wide_kernel(const __grid_constant__ CUtensorMap tmap, int N, int nblk, int 
         }
     }
     const bool diag = I == J;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // uniform for the compiler too
     const int t0 = blockIdx.y * chunk, t1 = min(N, t0 + chunk);
     const int ntiles = (t1 - t0 + kWTok - 1) / kWTok;
 
@@ -176,7 +176,7 @@ gram_wide_kernel(const __grid_constant__ CUtensorMap tmap, int N, int nblk, int 
             }
         }
     } else if (warp == 5) {
-        if (lane == 0) {
+        if (tc::elect_one()) {          // descriptors stay in uniform registers
             constexpr uint32_t idesc = DUAL ? tc::idesc_bf16_f32(128, 256, 0, 0) : tc::idesc_bf16_f32(128, 256, 1, 1);
             // MN-major, 128-byte swizzle: 64-feature regions kWRegion apart (LBO), 8-token groups 1024 B apart
             // (SBO); 16 tokens further = 2048 B = +128 in the 16-byte address field.  K-major: 8-row groups 1024 B
