@@ -20,8 +20,8 @@
 // the product takes 17 us of fp32 multiply-adds at n = 4096.  The counts are bound by issue and the fp64 units (190
 // instructions per row for two shifts).
 // Convergence is tested, not assumed: T_m contains T_{m-64}, so by interlacing the i-th eigenvalue has moved by less than
-// delta over the last two blocks exactly if T_{m-64} has i eigenvalues above lambda_i - delta (one more elimination per
-// eigenvalue, delta = 1e-7 of the largest).  What has not converged gets twice as many steps, in a second and a third
+// delta over the last two blocks exactly if T_{m-64} has i eigenvalues above lambda_i - delta (delta = 1e-7 of the
+// largest; its pivots are the first ones of T, so one of the last round's shifts tells).  What has not converged gets twice as many steps, in a second and a third
 // launch; they leave at once when there is nothing to do.  Nothing converged after that, a block that loses rank, or
 // a cluster as large as the block (an eigenvalue that may have higher multiplicity than the block can show): the caller's
 // full reduction runs instead.
@@ -423,6 +423,7 @@ __global__ void __launch_bounds__(kLT, 1) lanczos_kernel(const float *__restrict
 
 // ---------------------------------------------------------------------------------------- eigenvalues of T
 constexpr int kBT = 128;                          // 4 warps, two shifts each: 8 shifts per CTA
+constexpr int kBandLead = 64;                     // rows that the leading block of the interlacing check lacks
 constexpr int kBandCluster = 4;
 constexpr int kCtaShifts = kBT / 16;
 constexpr int kShifts = kBandCluster * kCtaShifts;   // 32 shifts per round
@@ -436,7 +437,7 @@ struct BandSmem {
     double red[kBT / 32];
 };
 
-// Negative pivots of T - x, rows 0 .. m - 1, by half a warp per shift.  Lane i of the half-warp holds the window rows
+// Negative pivots of T - x, rows 0 .. m - 1 (in lead: rows 0 .. m - kBandLead - 1), by half a warp per shift.  Lane i of the half-warp holds the window rows
 // that are i and i + 16 modulo 32; register j is the column j places behind the pivot, so the window moves along by
 // writing a multiply-add one register further down.  At row r the lane that owns it publishes the row; row and column
 // r + 32 enter in its place.  Entries of a row at earlier columns are never read.
@@ -444,7 +445,7 @@ struct BandSmem {
 // per warp the shared-memory pipe was the limit: 740 cycles per row at 8 shifts per SM, now 570).  The next pivot is
 // updated first, so its reciprocal is ready when the row is.
 __device__ __forceinline__ int band_count(const double *__restrict__ T, int m, double x, double tiny, double *row,
-                                          double (*ring)[kKryBand]) {
+                                          double (*ring)[kKryBand], int &lead) {
     const int lane = threadIdx.x & 31, h = lane & 15;
     double a[2][kB];
     // the first 32 columns: column c holds rows c - o
@@ -482,6 +483,7 @@ __device__ __forceinline__ int band_count(const double *__restrict__ T, int m, d
     __syncwarp();
     fetch(kB);
     for (int r0 = 0; r0 < m; r0 += kB) {
+        if (r0 == m - kBandLead) lead = count;
 #pragma unroll
         for (int w = 0; w < 2; ++w) {
 #pragma unroll 1
@@ -570,36 +572,39 @@ band_eigen_kernel(const float *__restrict__ C, int n, int k, int q, int max_iter
     const int idx = m - 1 - t;                    // ascending index of the t-th largest
     double lo = -1e-6 * bound, hi = bound * (1.0 + 1e-9);        // count(lo) <= idx < count(hi)
     const int rounds = max_iters > 0 ? max_iters : 8;
-    int it = 0;
-    for (; it < rounds && hi - lo > tol; ++it) {
-        const double step = (hi - lo) / (double)(kShifts + 1);
+    // Interlacing: T without its last rows has more than t eigenvalues above lam - delta, or the eigenvalue has not
+    // settled.  The pivots of a leading block are the first pivots of T, so the last round's last shift, moved to just
+    // above lo - delta, answers it on the way (a count of its own cost 70 us).
+    const double delta = 1e-7 * bound;
+    bool last = false;
+    for (int it = 0; it < rounds && !last; ++it) {
+        last = hi - lo <= tol * (double)kShifts || it == rounds - 1;
+        const int shifts = last ? kShifts - 1 : kShifts;
+        const double step = (hi - lo) / (double)(shifts + 1);
         const int own = tid >> 4, p = rank * kCtaShifts + own;
-        const int c = band_count(T, m, lo + step * (double)(p + 1), tiny, S.row[own], S.ring[wid]);
+        int lead = 0;
+        const double x = p < shifts ? lo + step * (double)(p + 1) : hi - delta;
+        const int c = band_count(T, m, x, tiny, S.row[own], S.ring[wid], lead);
+        if (p == shifts && (lane & 15) == 0) B.state[8 + t] = (m - kBandLead) - lead >= t + 1 ? 1 : 0;
         if ((lane & 15) < kBandCluster) cluster.map_shared_rank(&S, lane & 15)->count[it & 1][p] = c;
         cluster.sync();
         // the shifts whose count is still <= idx come first
-        const unsigned below = __ballot_sync(0xffffffffu, S.count[it & 1][lane] <= idx);
-        const int nb = below == 0xffffffffu ? kShifts : __ffs(~below) - 1;
-        const double nl = nb > 0 ? lo + step * (double)nb : lo, nh = nb < kShifts ? lo + step * (double)(nb + 1) : hi;
+        int nb = 0;
+#pragma unroll
+        for (int g0 = 0; g0 < kShifts; g0 += 32)
+            nb += __popc(__ballot_sync(0xffffffffu, g0 + lane < shifts && S.count[it & 1][g0 + lane] <= idx));
+        const double nl = nb > 0 ? lo + step * (double)nb : lo, nh = nb < shifts ? lo + step * (double)(nb + 1) : hi;
         lo = nl;
         hi = nh;
     }
-    const double lam = 0.5 * (lo + hi);
-    if (rank == 0 && wid == 0) {
-        // interlacing: T_{m-64} has more than t eigenvalues above lam - delta, or the eigenvalue has not settled
-        const double delta = 1e-7 * bound;
-        const int below = band_count(T, m - 64, lam - delta, tiny, S.row[lane >> 4], S.ring[0]);
-        if (lane == 0) {
-            const int above = (m - 64) - below;
-            B.state[8 + t] = above >= t + 1 ? 1 : 0;
-            B.lam[t] = lam;
-            if (hi - lo > tol) atomicOr(status, (uint32_t)UNCOMP_STATUS_NOT_CONVERGED);
-            if (t == 0) {
-                double sum = 0.0;
+    if (rank == 0 && tid == 0) {
+        B.lam[t] = 0.5 * (lo + hi);
+        if (hi - lo > tol) atomicOr(status, (uint32_t)UNCOMP_STATUS_NOT_CONVERGED);
+        if (t == 0) {
+            double sum = 0.0;
 #pragma unroll
-                for (int w = 0; w < kBT / 32; ++w) sum += S.red[w];
-                B.lam[k] = sum;
-            }
+            for (int w = 0; w < kBT / 32; ++w) sum += S.red[w];
+            B.lam[k] = sum;
         }
     }
     cluster.sync();                               // nobody leaves while another may still write its counts
