@@ -8,13 +8,14 @@
 //                       what is left, normalised.  Partial products of the CTAs meet in global memory and are summed in
 //                       fp64 in a fixed order, two grid barriers per pass.  The coefficients make up the projected
 //                       matrix T, block tridiagonal with upper triangular couplings: half-bandwidth 32 exactly.
+//   band_coarse_kernel  the spectrum's bound, and negative pivots of T - x at 1024 shifts that all eigenvalues share.
 //   band_eigen_kernel   a cluster of four CTAs per wanted eigenvalue, 32 shifts at a time, 33-fold per round: a warp
 //                       eliminates T - x row by row in fp64 (the trailing 32 x 32 window in its registers) and counts
 //                       negative pivots.
 //
 // Why: the reduction column by column sweeps the whole trailing matrix n times (33 ms at n = 4096), although only k of n
 // eigenvalues are wanted; here a step of 32 vectors reads the matrix once and 8 to 32 steps suffice (8192 x 4096 hidden
-// states with a decaying spectrum, k = 32: 8 steps, 0.9 ms, and the counts 0.55 ms; an isotropic matrix, the slowest to
+// states with a decaying spectrum, k = 32: 8 steps, 0.95 ms, and the counts 0.42 ms, 0.54 with no shared round; an isotropic matrix, the slowest to
 // converge, takes 32).  Accuracy is that of fp32 products summed in fp32 / fp64, as before.
 // What bounds it: about 70 us of every step are grid barriers, sums over the CTAs and the two factorisations, whatever n;
 // the product takes 17 us of fp32 multiply-adds at n = 4096.  The counts are bound by issue and the fp64 units (190
@@ -428,6 +429,9 @@ constexpr int kBandCluster = 4;
 constexpr int kCtaShifts = kBT / 16;
 constexpr int kShifts = kBandCluster * kCtaShifts;   // 32 shifts per round
 
+constexpr int kCoarseCtas = 128;                  // below the number of SMs: a CTA of the counts fills one
+constexpr int kCoarse = kCoarseCtas * kCtaShifts; // shifts of the first round, for all eigenvalues together
+
 constexpr int kRing = 8;                          // columns of T on their way per warp
 
 struct BandSmem {
@@ -536,16 +540,25 @@ __device__ __forceinline__ int band_count(const double *__restrict__ T, int m, d
     return count;
 }
 
-__global__ void __cluster_dims__(kBandCluster, 1, 1) __launch_bounds__(kBT, 1)
-band_eigen_kernel(const float *__restrict__ C, int n, int k, int q, int max_iters, KrylovBuffers B, uint32_t *__restrict__ status) {
-    namespace cg = cooperative_groups;
+__device__ __forceinline__ double band_low(double bound) { return -1e-6 * bound; }
+__device__ __forceinline__ double band_high(double bound) { return bound * (1.0 + 1e-9); }
+
+// What the coarse round leaves for the eigenvalues, in the scratch of the products.
+struct BandCoarse {
+    double bound, trace;
+    int count[kCoarse];
+};
+
+// The first round of the bisection: the bracket is the same for all eigenvalues, so they share 1024 shifts, eight per
+// SM (what a round costs anyway), instead of 32 each: five rounds to the tolerance instead of six.
+__global__ void __launch_bounds__(kBT, 1)
+band_coarse_kernel(const float *__restrict__ C, int n, int q, KrylovBuffers B) {
     __shared__ BandSmem S;
-    cg::cluster_group cluster = cg::this_cluster();
-    const int t = blockIdx.x / kBandCluster, rank = (int)cluster.block_rank();
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, m = q * kB;
-    // state[0] is q only if the Lanczos launch before this one ran; flags and eigenvalues are read by the NEXT launch
+    // state[0] is q only if the Lanczos launch before this one ran
     if (B.state[1] || B.state[0] != q) return;    // uniform over the grid
     const double *T = B.T;
+    BandCoarse *out = reinterpret_cast<BandCoarse *>(B.part);
     // Gershgorin bound of the spectrum (entries (i, c), i <= c, in column c) and the trace of the whole matrix
     double g = 0.0, tr = 0.0;
     for (int c = tid; c < m; c += kBT) {
@@ -554,24 +567,64 @@ band_eigen_kernel(const float *__restrict__ C, int n, int k, int q, int max_iter
         for (int o = 1; o <= kB && c + o < m; ++o) s += fabs(__ldg(T + (size_t)(c + o) * kKryBand + o));
         g = fmax(g, s);
     }
-    if (t == 0 && rank == 0)
+    if (blockIdx.x == 0)
         for (int i = tid; i < n; i += kBT) tr += (double)C[(size_t)i * n + i];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) g = fmax(g, __shfl_xor_sync(0xffffffffu, g, o));
     tr = warp_sum(tr);
     if (lane == 0) S.red[wid] = g;
     __syncthreads();
-    double bound = 0.0;
+    double bound = 1e-280;
 #pragma unroll
     for (int w = 0; w < kBT / 32; ++w) bound = fmax(bound, S.red[w]);
     __syncthreads();
     if (lane == 0) S.red[wid] = tr;
     __syncthreads();
-    bound = fmax(bound, 1e-280);
-    const double tiny = bound * 1e-19, tol = bound * 1e-9;
+    const double lo = band_low(bound), hi = band_high(bound);
+    const int own = tid >> 4, p = blockIdx.x * kCtaShifts + own;
+    int lead = 0;
+    const int c = band_count(T, m, lo + (hi - lo) / (double)(kCoarse + 1) * (double)(p + 1), bound * 1e-19, S.row[own],
+                             S.ring[wid], lead);
+    if ((lane & 15) == 0) out->count[p] = c;
+    if (blockIdx.x == 0 && tid == 0) {
+        double sum = 0.0;
+#pragma unroll
+        for (int w = 0; w < kBT / 32; ++w) sum += S.red[w];
+        out->bound = bound;
+        out->trace = sum;
+    }
+}
+
+__global__ void __cluster_dims__(kBandCluster, 1, 1) __launch_bounds__(kBT, 1)
+band_eigen_kernel(int k, int q, int max_iters, KrylovBuffers B, uint32_t *__restrict__ status) {
+    namespace cg = cooperative_groups;
+    __shared__ BandSmem S;
+    __shared__ int s_first;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int t = blockIdx.x / kBandCluster, rank = (int)cluster.block_rank();
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, m = q * kB;
+    // flags and eigenvalues are read by the NEXT launch
+    if (B.state[1] || B.state[0] != q) return;    // uniform over the grid
+    const double *T = B.T;
+    const BandCoarse *in = reinterpret_cast<const BandCoarse *>(B.part);
+    const double bound = in->bound, tiny = bound * 1e-19, tol = bound * 1e-9;
     const int idx = m - 1 - t;                    // ascending index of the t-th largest
-    double lo = -1e-6 * bound, hi = bound * (1.0 + 1e-9);        // count(lo) <= idx < count(hi)
-    const int rounds = max_iters > 0 ? max_iters : 8;
+    double lo = band_low(bound), hi = band_high(bound);          // count(lo) <= idx < count(hi)
+    if (tid == 0) s_first = kCoarse;
+    __syncthreads();
+    int first = kCoarse;                          // the first coarse shift above the eigenvalue
+    for (int p = tid; p < kCoarse; p += kBT)
+        if (in->count[p] > idx) first = min(first, p);
+    atomicMin(&s_first, first);
+    __syncthreads();
+    first = s_first;
+    {
+        const double step = (hi - lo) / (double)(kCoarse + 1);
+        const double nl = first > 0 ? lo + step * (double)first : lo, nh = first < kCoarse ? lo + step * (double)(first + 1) : hi;
+        lo = nl;
+        hi = nh;
+    }
+    const int rounds = max_iters > 0 ? max(max_iters - 1, 1) : 7;
     // Interlacing: T without its last rows has more than t eigenvalues above lam - delta, or the eigenvalue has not
     // settled.  The pivots of a leading block are the first pivots of T, so the last round's last shift, moved to just
     // above lo - delta, answers it on the way (a count of its own cost 70 us).
@@ -600,12 +653,7 @@ band_eigen_kernel(const float *__restrict__ C, int n, int k, int q, int max_iter
     if (rank == 0 && tid == 0) {
         B.lam[t] = 0.5 * (lo + hi);
         if (hi - lo > tol) atomicOr(status, (uint32_t)UNCOMP_STATUS_NOT_CONVERGED);
-        if (t == 0) {
-            double sum = 0.0;
-#pragma unroll
-            for (int w = 0; w < kBT / 32; ++w) sum += S.red[w];
-            B.lam[k] = sum;
-        }
+        if (t == 0) B.lam[k] = in->trace;
     }
     cluster.sync();                               // nobody leaves while another may still write its counts
 }
@@ -628,7 +676,8 @@ cudaError_t launch_krylov(const float *C, int n, int k, int max_iters, const Kry
                         (void *)&bar, (void *)&d_status};
         e = cudaLaunchCooperativeKernel((const void *)lanczos_kernel, dim3(n / kB), dim3(kLT), args, sizeof(LanczosSmem), st);
         if (e != cudaSuccess) return e;
-        band_eigen_kernel<<<k * kBandCluster, kBT, 0, st>>>(C, n, k, q, max_iters, b, d_status);
+        band_coarse_kernel<<<kCoarseCtas, kBT, 0, st>>>(C, n, q, b);
+        band_eigen_kernel<<<k * kBandCluster, kBT, 0, st>>>(k, q, max_iters, b, d_status);
         if (q >= most || ++launch >= 3) break;
         q0 = q;
         q = min(most, 2 * q);
