@@ -479,9 +479,9 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
         if (e != cudaSuccess) return cuda_fail(ctx, e);
     } else if (tensor_path) {
         // Gram + statistics sweep; then eigenvalues and budgets beside the column sums: neither needs the other, only the
-        // selection needs both.  The two cannot share an SM (registers), so which one is launched first matters: while all
-        // units are in work at once the eigenvalues are a chain on a few SMs and go first, on the caller's stream (one layer
-        // of 7001 tokens 138 us, 175 the other way round); with more units the column sums do (four 32K sequences 5.05 ms, 5.19).
+        // selection needs both.  The two cannot share an SM (registers), so which one is launched first matters: with few
+        // units the eigenvalues are a chain on a few SMs and have to go first (one layer of 7001 tokens 138 us, 175 the other
+        // way round); with many the order makes no difference (1024 units of 3712 tokens 820 and 825 us, of 32K 5.03 ms both).
         if (!d_K || !d_Qw || !d_entropy || !d_budgets || !d_offsets || !d_indices) return UNCOMP_E_NULL;
         if (!aligned16(d_K) || !aligned16(d_Qw)) return UNCOMP_E_ALIGN;
         rc = check_strides(p.shape, sK);
@@ -509,29 +509,25 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
         ctx->stats_valid = 0;
         e = launch_scores_tc(p, d_Qw, d_K, addr, sc, nullptr, stats_part, nullptr, partials, kScorePhaseStats,
                              d_status, &ctx->tmaps, ctx->prof, st);
-        const bool eigen_first = p.units <= 2 * kTargetSms;
-        cudaStream_t st_eigen = eigen_first ? st : ctx->side, st_sums = eigen_first ? ctx->side : st;
         if (e == cudaSuccess) e = cudaEventRecord(ctx->ev_fork, st);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0);
         if (e != cudaSuccess) return cuda_fail(ctx, e);
-        auto sums = [&] {
-            return launch_scores_tc(p, d_Qw, d_K, addr, sc, nullptr, stats_part, raw, nullptr, kScorePhaseColsum, d_status,
-                                    &ctx->tmaps, ctx->prof, st_sums);
-        };
-        if (!eigen_first) e = sums();
-        if (e == cudaSuccess) {
-            ProfScope ps(ctx->prof, kSlotEigen, st_eigen);
-            e = launch_eigen_f32(p, partials, p.score_splits, *eparams, d_entropy, d_erank, nullptr, d_status, st_eigen);
+        {
+            ProfScope ps(ctx->prof, kSlotEigen, st);
+            e = launch_eigen_f32(p, partials, p.score_splits, *eparams, d_entropy, d_erank, nullptr, d_status, st);
         }
-        if (e == cudaSuccess && eigen_first) e = sums();
+        if (e == cudaSuccess)
+            e = launch_scores_tc(p, d_Qw, d_K, addr, sc, nullptr, stats_part, raw, nullptr, kScorePhaseColsum, d_status,
+                                 &ctx->tmaps, ctx->prof, ctx->side);
         if (e == cudaSuccess) {
-            ProfScope ps(ctx->prof, kSlotBudgets, st_eigen);
+            ProfScope ps(ctx->prof, kSlotBudgets, st);
             e = launch_budgets(p, d_erank, *bparams, d_budgets, d_offsets, d_layer_group, d_layer_ctx,
                                reinterpret_cast<int32_t *>(ctx->ws + p.off_rank),
-                               reinterpret_cast<int64_t *>(ctx->ws + p.off_rem), st_eigen);
+                               reinterpret_cast<int64_t *>(ctx->ws + p.off_rem), st);
         }
-        if (e == cudaSuccess) e = cudaEventRecord(ctx->ev_join, ctx->side);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ctx->ev_join, 0);
+        cudaError_t join = cudaEventRecord(ctx->ev_join, ctx->side);       // after an error too: the side stream may hold work
+        if (join == cudaSuccess) join = cudaStreamWaitEvent(st, ctx->ev_join, 0);
+        if (e == cudaSuccess) e = join;
         if (e != cudaSuccess) return cuda_fail(ctx, e);
         {
             ProfScope ps(ctx->prof, kSlotPoolSelect, st);
