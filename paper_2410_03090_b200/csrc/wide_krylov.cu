@@ -20,12 +20,17 @@
 // What bounds it: about 70 us of every step are grid barriers, sums over the CTAs and the two factorisations, whatever n;
 // the product takes 17 us of fp32 multiply-adds at n = 4096.  The counts are bound by issue and the fp64 units (190
 // instructions per row for two shifts).
-// Convergence is tested, not assumed: T_m contains T_{m-64}, so by interlacing the i-th eigenvalue has moved by less than
-// delta over the last two blocks exactly if T_{m-64} has i eigenvalues above lambda_i - delta (delta = 1e-7 of the
-// largest; its pivots are the first ones of T, so one of the last round's shifts tells).  What has not converged gets twice as many steps, in a second and a third
-// launch; they leave at once when there is nothing to do.  Nothing converged after that, a block that loses rank, or
-// a cluster as large as the block (an eigenvalue that may have higher multiplicity than the block can show): the caller's
-// full reduction runs instead.
+// Convergence is tested by how far an eigenvalue still moves: T_m contains T_{m-64}, so by interlacing the i-th eigenvalue
+// has moved by less than delta over the last two blocks exactly if T_{m-64} has i eigenvalues above lambda_i - delta (its
+// pivots are the first ones of T, so one of the last round's shifts tells).  delta is 2e-6 of the eigenvalue itself (1e-7 of
+// the bound at most, 1e-11 at least), not of the largest one: with one direction 1e5 times the rest the others may be off by
+// per cents and still move by less than 1e-7 of the largest.  A movement is not a bound of the error; the error is smaller
+// than the last movement as long as the steps converge at least as fast as before, which block Lanczos does (isotropic
+// matrices of n = 1024, the slowest: movements of 4e-3, 1e-5, 1e-9 over two blocks left errors of 4e-4, 1e-7 and less).
+// What has not settled gets twice as many steps, in a second and a third launch; they leave at once when there is
+// nothing to do.  Not settled after that, a block that loses rank, a cluster as large as the block (an eigenvalue that may
+// have higher multiplicity than the block can show), or wanted eigenvalues further apart than kKryMaxRatio: the
+// caller's full reduction runs instead.
 #include <cooperative_groups.h>
 
 #include "grid_barrier.cuh"
@@ -343,7 +348,8 @@ __global__ void __launch_bounds__(kLT, 1) lanczos_kernel(const float *__restrict
                                                         uint32_t *__restrict__ status) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LanczosSmem &S = *reinterpret_cast<LanczosSmem *>(smem_raw);
-    if (B.state[1] || (q_begin > 0 && krylov_done(B.state, B.lam, k))) return;      // the same answer in every CTA
+    if (B.state[1]) return;                       // the same answers in every CTA
+    if (q_begin > 0 && (krylov_too_graded(B.lam, k) || krylov_done(B.state, B.lam, k))) return;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, r0 = blockIdx.x * kB;
     const size_t block = (size_t)kB * n, part_stride = (size_t)part_blocks * kB * kB;
     float *part = B.part + (size_t)blockIdx.x * part_stride;
@@ -543,9 +549,26 @@ __device__ __forceinline__ int band_count(const double *__restrict__ T, int m, d
 __device__ __forceinline__ double band_low(double bound) { return -1e-6 * bound; }
 __device__ __forceinline__ double band_high(double bound) { return bound * (1.0 + 1e-9); }
 
+// To how much an eigenvalue of at least `lo` is bracketed: 2e-8 of itself, but no finer than 1e-13 and no coarser than 1e-9
+// of the spectrum's bound.  It has settled when it moved by less than kSettled times that over the last two blocks.
+constexpr double kSettled = 100.0;
+__device__ __forceinline__ double band_tolerance(double lo, double bound) {
+    return fmin(fmax(2e-8 * lo, 1e-13 * bound), 1e-9 * bound);
+}
+
+// The shared shifts, ascending: kCoarseLow of constant ratio up to 5 % of the bound, where the tolerance becomes a share
+// of the eigenvalue itself, and equally spaced from there.  Both spacings are what four rounds bring to the tolerance
+// (32 times 33^3 of it: 1.15e-3 of the bound, 2.3 % of the shift); below 6.6e-4 of the bound it takes two or three more.
+constexpr int kCoarseLow = 194;
+__device__ __forceinline__ double coarse_shift(int p, double bound) {
+    if (p < kCoarseLow) return 0.05 * bound * exp(-0.02245 * (double)(kCoarseLow - 1 - p));
+    return bound * (0.05 + 0.95 / (double)(kCoarse - kCoarseLow + 1) * (double)(p - kCoarseLow + 1));
+}
+
 // What the coarse round leaves for the eigenvalues, in the scratch of the products.
 struct BandCoarse {
     double bound, trace;
+    double shift[kCoarse];
     int count[kCoarse];
 };
 
@@ -580,12 +603,14 @@ band_coarse_kernel(const float *__restrict__ C, int n, int q, KrylovBuffers B) {
     __syncthreads();
     if (lane == 0) S.red[wid] = tr;
     __syncthreads();
-    const double lo = band_low(bound), hi = band_high(bound);
     const int own = tid >> 4, p = blockIdx.x * kCtaShifts + own;
+    const double x = coarse_shift(p, bound);
     int lead = 0;
-    const int c = band_count(T, m, lo + (hi - lo) / (double)(kCoarse + 1) * (double)(p + 1), bound * 1e-19, S.row[own],
-                             S.ring[wid], lead);
-    if ((lane & 15) == 0) out->count[p] = c;
+    const int c = band_count(T, m, x, bound * 1e-19, S.row[own], S.ring[wid], lead);
+    if ((lane & 15) == 0) {
+        out->shift[p] = x;
+        out->count[p] = c;
+    }
     if (blockIdx.x == 0 && tid == 0) {
         double sum = 0.0;
 #pragma unroll
@@ -607,7 +632,7 @@ band_eigen_kernel(int k, int q, int max_iters, KrylovBuffers B, uint32_t *__rest
     if (B.state[1] || B.state[0] != q) return;    // uniform over the grid
     const double *T = B.T;
     const BandCoarse *in = reinterpret_cast<const BandCoarse *>(B.part);
-    const double bound = in->bound, tiny = bound * 1e-19, tol = bound * 1e-9;
+    const double bound = in->bound, tiny = bound * 1e-19;
     const int idx = m - 1 - t;                    // ascending index of the t-th largest
     double lo = band_low(bound), hi = band_high(bound);          // count(lo) <= idx < count(hi)
     if (tid == 0) s_first = kCoarse;
@@ -618,25 +643,20 @@ band_eigen_kernel(int k, int q, int max_iters, KrylovBuffers B, uint32_t *__rest
     atomicMin(&s_first, first);
     __syncthreads();
     first = s_first;
-    {
-        const double step = (hi - lo) / (double)(kCoarse + 1);
-        const double nl = first > 0 ? lo + step * (double)first : lo, nh = first < kCoarse ? lo + step * (double)(first + 1) : hi;
-        lo = nl;
-        hi = nh;
-    }
-    const int rounds = max_iters > 0 ? max(max_iters - 1, 1) : 7;
-    // Interlacing: T without its last rows has more than t eigenvalues above lam - delta, or the eigenvalue has not
-    // settled.  The pivots of a leading block are the first pivots of T, so the last round's last shift, moved to just
-    // above lo - delta, answers it on the way (a count of its own cost 70 us).
-    const double delta = 1e-7 * bound;
+    if (first > 0) lo = in->shift[first - 1];
+    if (first < kCoarse) hi = in->shift[first];
+    // max_iters counts 257-fold rounds, as in the full reduction; these are 33-fold after the coarse 1025 intervals
+    const int rounds = max_iters > 0 ? min(max((8 * max_iters - 6) / 5, 1), 7) : 7;
+    double tol = 0.0;
     bool last = false;
     for (int it = 0; it < rounds && !last; ++it) {
+        tol = band_tolerance(lo, bound);
         last = hi - lo <= tol * (double)kShifts || it == rounds - 1;
         const int shifts = last ? kShifts - 1 : kShifts;
         const double step = (hi - lo) / (double)(shifts + 1);
         const int own = tid >> 4, p = rank * kCtaShifts + own;
         int lead = 0;
-        const double x = p < shifts ? lo + step * (double)(p + 1) : hi - delta;
+        const double x = p < shifts ? lo + step * (double)(p + 1) : hi - kSettled * tol;
         const int c = band_count(T, m, x, tiny, S.row[own], S.ring[wid], lead);
         if (p == shifts && (lane & 15) == 0) B.state[8 + t] = (m - kBandLead) - lead >= t + 1 ? 1 : 0;
         if ((lane & 15) < kBandCluster) cluster.map_shared_rank(&S, lane & 15)->count[it & 1][p] = c;

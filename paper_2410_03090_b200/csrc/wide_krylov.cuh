@@ -25,9 +25,17 @@ constexpr int kKryBand = 34;
 constexpr int kKryStateInts = 8 + kKryMaxK;
 constexpr int kKryMaxLaunches = 4;
 
+// Largest ratio of the k wanted eigenvalues.  Rounding of the product is a share of the largest one; relative to the
+// eigenvalue itself (root mean square over 32, six matrices each, n = 512 to 2048) it comes to 0.4e-6 to 0.9e-6 at ratios
+// up to 1000 and 1.0e-6 at 3000, as in the full reduction, but 3.6e-6 to 7.3e-6 at 30000 where the reduction has 2.9e-6 to
+// 5.7e-6: beyond this the reduction runs.
+constexpr double kKryMaxRatio = 4096.0;
+
+__device__ __forceinline__ bool krylov_too_graded(const double *lam, int k) { return !(lam[0] <= kKryMaxRatio * lam[k - 1]); }
+
 // true when all k eigenvalues have converged (every kernel behind the first asks this before it does anything)
 __device__ __forceinline__ bool krylov_done(const int *state, const double *lam, int k) {
-    if (state[1]) return false;
+    if (state[1] || krylov_too_graded(lam, k)) return false;
     for (int i = 0; i < k; ++i)
         if (!state[8 + i]) return false;
     // a block of 32 start vectors shows an eigenvalue at most 32 times: a cluster of that size may be larger

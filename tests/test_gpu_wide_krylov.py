@@ -1,8 +1,10 @@
 """Wide entropy where a few eigenvalues of a large matrix come from block Lanczos: the edges of its range, slow
 convergence (a second and third launch), and the inputs that must end in the full reduction, against the oracle."""
+import numpy as np
 import pytest
 import torch
 
+import oracle
 import test_gpu_wide as tw
 
 pytestmark = pytest.mark.gpu
@@ -47,3 +49,44 @@ def test_multiple_eigenvalues_rank_loss_and_zero():
     ent, er = ub.uncomp_entropy_wide(ctx, torch.ones(1, 1024, 512, dtype=torch.bfloat16, device="cuda"), 32)
     torch.cuda.synchronize()
     assert ub.uncomp_status(ctx) == 0 and float(ent[0]) == 0.0 and float(er[0]) == 1.0
+
+
+@pytest.mark.parametrize("N,D,strength,k", [
+    (3000, 1024, 1e2, 32),     # few enough orders apart for block Lanczos
+    (3000, 1024, 1e5, 64),
+    (3000, 1024, 1e6, 32),     # movements of 1e-7 of the largest say nothing about the others
+    (8192, 4096, 1e5, 32),
+])
+def test_one_dominating_direction_leaves_the_others_exact(N, D, strength, k):
+    """Isotropic hidden states and one direction that is `strength` times stronger: every eigenvalue held to its own size.
+    The tensor cores add one product of 16 tokens after another, m of them per partial Gram matrix, each sum good to 2^-24:
+    at most m 2^-24 of every eigenvalue; and the rounding of the strongest direction's part of the entries,
+    sqrt(m) 2^-24 lam_0 / n each and without a pattern, times 6 for 1e6 entries."""
+    from paper_2410_03090_b200 import binding as ub
+    g = torch.Generator(device="cuda").manual_seed(N + D + k)
+    one = torch.nn.functional.normalize(torch.randn(1, D, generator=g, device="cuda"), dim=1)
+    X = torch.randn(N, D, generator=g, device="cuda") + strength ** 0.5 * torch.randn(N, 1, generator=g, device="cuda") * one
+    X = X.to(torch.bfloat16)[None]
+    ctx = ub.Context(ub.make_shape(1, 1, 1, 1, 256, 128, 8, "bf16"))
+    ent, _, spec = ub.uncomp_entropy_wide(ctx, X, k, spectrum=True)
+    torch.cuda.synchronize()
+    assert ub.uncomp_status(ctx) == 0
+    H, _, lam = oracle.entropy_wide(X[0].double().cpu().numpy(), k, True, 0, return_spectrum=True)
+    lam = lam[:k]
+    pairs = (D // 256) * (D // 256 + 1) // 2
+    chunks = min(-(-296 // pairs), -(-N // 512))
+    m = -(-N // chunks) / 16
+    rel = np.abs(spec[0].cpu().numpy() - lam) / lam
+    bound = 2.0 ** -24 * (m + 6 * m ** 0.5 * lam[0] / (D * lam))
+    assert (rel <= bound).all(), (rel.max(), bound[rel.argmax()], lam[0] / lam[-1])
+    assert abs(float(ent[0]) - H) <= 1e-5
+
+
+def test_few_rounds_are_reported():
+    from paper_2410_03090_b200 import binding as ub
+    X = tw._matrix(1, 1300, 512, 60, 0.1, seed=1)
+    ctx = ub.Context(ub.make_shape(1, 1, 1, 1, 256, 128, 8, "bf16"))
+    ub.uncomp_entropy_wide(ctx, X, 32, max_iters=1)
+    assert ub.uncomp_status(ctx) & 1
+    ub.uncomp_entropy_wide(ctx, X, 32, max_iters=6)          # 257^6 > 1e13
+    assert ub.uncomp_status(ctx) == 0
