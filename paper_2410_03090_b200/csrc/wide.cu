@@ -702,7 +702,10 @@ cudaError_t launch_entropy_wide(const void *d_X, int64_t sN, int N, int D, const
     double *lam = (double *)(scratch + w.off_lam);
     int *kry = nullptr;
     // A few of the eigenvalues of a large matrix: block Lanczos.  What follows leaves at once when it has converged.
-    if (krylov_applies(w.Dt, kf)) {
+    int resident = 0;
+    if (krylov_steps(w.Dt) > 0) err = krylov_resident(resident);
+    if (err != cudaSuccess) return err;
+    if (krylov_applies(w.Dt, kf, resident)) {
         ProfScope ps(prof, kSlotWideKrylov, st);
         KrylovBuffers b;
         b.Q = (float *)(scratch + w.off_Q);

@@ -679,14 +679,25 @@ band_eigen_kernel(int k, int q, int max_iters, KrylovBuffers B, uint32_t *__rest
 }
 }  // namespace
 
-bool krylov_applies(int n, int k) { return n >= kKryMinN && k <= kKryMaxK && krylov_steps(n) >= (k <= 32 ? 8 : 10); }
+bool krylov_applies(int n, int k, int ctas) {
+    return n >= kKryMinN && k <= kKryMaxK && krylov_steps(n) >= (k <= 32 ? 8 : 10) && n / kB <= ctas;
+}
+
+cudaError_t krylov_resident(int &ctas) {
+    static bool done[64] = {};
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaError_t e = allow_dynamic_smem((const void *)lanczos_kernel, sizeof(LanczosSmem), done);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lanczos_kernel, kLT, sizeof(LanczosSmem));
+    ctas = sms * per_sm;
+    return e;
+}
 int krylov_steps(int n) { return n < kKryMinN ? 0 : min(kKryMaxSteps, (n - 128) / kB); }
 
 cudaError_t launch_krylov(const float *C, int n, int k, int max_iters, const KrylovBuffers &b, uint32_t *d_status,
                           cudaStream_t st) {
-    static bool done[64] = {};
-    cudaError_t e = allow_dynamic_smem((const void *)lanczos_kernel, sizeof(LanczosSmem), done);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
     const int most = krylov_steps(n);
     int part_blocks = most + 3, q0 = 0, q = k <= 32 ? 8 : 10, launch = 0;
     while (true) {

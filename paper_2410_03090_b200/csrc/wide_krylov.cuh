@@ -44,7 +44,9 @@ __device__ __forceinline__ bool krylov_done(const int *state, const double *lam,
     return true;
 }
 
-bool krylov_applies(int n, int k);
+// `ctas`: how many CTAs of the Lanczos kernel the device holds at once (they wait for one another, n / 32 of them)
+bool krylov_applies(int n, int k, int ctas);
+cudaError_t krylov_resident(int &ctas);
 int krylov_steps(int n);             // blocks the buffers hold besides the first
 cudaError_t launch_krylov(const float *C, int n, int k, int max_iters, const KrylovBuffers &b, uint32_t *d_status, cudaStream_t st);
 
