@@ -28,6 +28,24 @@ def test_cluster_steps(caps, G, dtype, full):
     assert ub.uncomp_status(ctx) == 0
 
 
+@pytest.mark.parametrize("G,dtype", [(1, "bf16"), (2, "bf16"), (4, "bf16"), (8, "bf16"), (16, "bf16"), (1, "fp32"), (16, "fp32")])
+@pytest.mark.parametrize("full", [True, False])
+def test_three_launches_beyond_shared_memory(G, dtype, full):
+    """Eight CTAs hold 200 KB of logits each: 51200 / G entries, less the padding.  The three launches beyond that, evicting
+    and appending, beside a unit of one chunk and one of a single row."""
+    from paper_2410_03090_b200 import binding as ub
+    cap = 8 * 51200 // G + 8
+    caps = np.array([1, cap, 1023])
+    lens = caps.copy() if full else np.maximum(0, caps - 2)
+    N = max(cap + 64, 150000)
+    ctx = ub.Context(ub.make_shape(1, 1, 3, 3 * G, N, 128, 32, dtype))
+    st = td.State(1, 1, 3, 3 * G, dtype, caps, lens, seed=G, start_pos=cap + 500)
+    ub.uncomp_profile_enable(ctx, True)
+    td._step_and_check(ub, ctx, st, cap, protect=1)
+    launches = {name: n for name, (_, n) in ub.uncomp_profile_read(ctx).items() if n}
+    assert launches == {"decode_logits": 1, "decode_accumulate": 1, "decode_commit": 1}
+
+
 @pytest.mark.parametrize("units", [147, 296, 297, 600])
 def test_cluster_choice_by_units(units):
     from paper_2410_03090_b200 import binding as ub

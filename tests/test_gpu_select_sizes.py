@@ -56,6 +56,21 @@ def test_ties(P, budget):
     _select(ub, P, 2, budget, 1, 0, ties=True)
 
 
+@pytest.mark.parametrize("P,budget,pk,pm,ties", [
+    (262144, 3000, 7, 0, False),       # the longest prefix whose keys fit the shared memory of a cluster
+    (262145, 3000, 7, 0, False),       # one more: radix select over global memory
+    (262147, 2, 1, 0, False),          # one position
+    (263000, 262999, 7, 0, False),     # all but two
+    (263000, 263001, 63, 0, False),    # all
+    (270001, 20000, 63, 1, False),     # mean pool
+    (270001, 40000, 1, 0, True),       # the threshold among equal scores
+    (270001, 9000, 7, 0, True),
+])
+def test_beyond_the_keys_in_shared_memory(P, budget, pk, pm, ties):
+    from paper_2410_03090_b200 import binding as ub
+    _select(ub, P, 2, budget, pk, pm, ties=ties, seed=P + budget)
+
+
 @pytest.mark.parametrize("L,H,M,scope", [(1, 7, 3, 0), (80, 64, 5000, 1), (80, 64, 100, 1), (33, 32, 32, 0), (3, 8, 1, 1)])
 def test_budget_tables(L, H, M, scope):
     from paper_2410_03090_b200 import binding as ub
