@@ -18,6 +18,7 @@
 // k / 16); inside the groups nothing is masked: reflectors and products are zero there.  With the matrix in shared
 // memory, one warp forming the reflector and a warp per row for the product, 8 units took 543 us; now 166 us.
 #include "common.cuh"
+#include "newton.cuh"
 
 namespace uncomp {
 
@@ -43,22 +44,6 @@ struct EigenSmem {
     int cnt[kCoarse + 2];
     int flags[2];
 };
-
-// reciprocal and square root in fp64 from the hardware approximations and Newton steps
-__device__ __forceinline__ double recip_newton(double d) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    r = fma(r, fma(-d, r, 1.0), r);
-    return fma(r, fma(-d, r, 1.0), r);
-}
-__device__ __forceinline__ double sqrt_newton(double x) {
-    double r;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    r = fma(0.5 * r, fma(-x * r, r, 1.0), r);
-    r = fma(0.5 * r, fma(-x * r, r, 1.0), r);
-    const double s = x * r;
-    return fma(0.5 * r, fma(-s, s, x), s);
-}
 
 // number of eigenvalues of the normalised tridiagonal matrix that are < x
 __device__ __noinline__ int sturm_count_robust(const double2 *de, double x) {

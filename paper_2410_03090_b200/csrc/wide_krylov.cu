@@ -34,6 +34,7 @@
 #include <cooperative_groups.h>
 
 #include "grid_barrier.cuh"
+#include "newton.cuh"
 #include "wide_krylov.cuh"
 
 namespace uncomp {
@@ -243,14 +244,6 @@ __device__ __forceinline__ void reduce_slice(LanczosSmem &S, const KrylovBuffers
     }
 }
 
-// reciprocal in fp64 from the hardware's 20-bit approximation and two Newton steps
-__device__ __forceinline__ double recip64(double d) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    r = fma(r, fma(-d, r, 1.0), r);
-    return fma(r, fma(-d, r, 1.0), r);
-}
-
 // G = L D L^T by elimination beside the identity; Rinv = L^-T D^-1/2 and R = D^1/2 L^T, so that W Rinv has orthonormal
 // columns and W = (W Rinv) R.  Thread: column tid mod 64 of [G | I], eight rows in registers; a step publishes pivot row
 // and pivot column, one barrier each.  A pivot that has lost all of its column's norm marks the block as broken.
@@ -279,7 +272,7 @@ __device__ __forceinline__ void factorise(LanczosSmem &S, const double *G, float
         const double d = row[s], u = row[col];
         const bool ok = d > 1e-14 * top;
         if (!ok && tid == 0) S.bad = 1;
-        const double inv = ok ? recip64(d) : 0.0, f = -u * inv;
+        const double inv = ok ? recip_newton(d) : 0.0, f = -u * inv;
 #pragma unroll
         for (int q = s >> 2; q < kB / 4; ++q)
             if (rq + 4 * q > s) v[q] = fma(column[8 * rq + q], f, v[q]);
@@ -471,7 +464,7 @@ __device__ __forceinline__ int band_count(const double *__restrict__ T, int m, d
         }
     int count = 0;
     auto pivot = [&](double d) { return fabs(d) < tiny ? -tiny : d; };
-    double d = pivot(__shfl_sync(0xffffffffu, a[0][0], lane & 16)), inv = recip64(d);
+    double d = pivot(__shfl_sync(0xffffffffu, a[0][0], lane & 16)), inv = recip_newton(d);
     // column r + 32 enters at row r; eight columns are on their way to the warp's ring (a row takes less time than L2)
     auto load = [&](int c) {
         if (c < m) {
@@ -521,7 +514,7 @@ __device__ __forceinline__ int band_count(const double *__restrict__ T, int m, d
                     // the next pivot: row r + 1
                     const double dn = s < 15 ? a[w][0] : a[1 - w][0];
                     d = pivot(__shfl_sync(0xffffffffu, dn, (lane & 16) + ((s + 1) & 15)));
-                    inv = recip64(d);
+                    inv = recip_newton(d);
                     a[0][1] = fma(l0, u.y, a[0][2]);
                     a[1][1] = fma(l1, u.y, a[1][2]);
                 }
