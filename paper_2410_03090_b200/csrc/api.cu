@@ -431,9 +431,7 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
     const Plan &p = ctx->plan;
     const bool tensor_path = p.shape.dtype == UNCOMP_BF16 && !ctx->force_simt;
     int rc;
-    if (d_lse && tensor_path) {
-        // One sweep over K: the window scores (the caller brings the row normalisers) and the Gram partials of the
-        // entropy stage come out of the same kernel; then eigenvalues, budgets, selection, gather.
+    if (tensor_path) {                        // the staged calls below check for themselves
         if (!d_K || !d_Qw || !d_entropy || !d_budgets || !d_offsets || !d_indices) return UNCOMP_E_NULL;
         if (!aligned16(d_K) || !aligned16(d_Qw) || (reinterpret_cast<uintptr_t>(d_lse) & 3u)) return UNCOMP_E_ALIGN;
         rc = check_strides(p.shape, sK);
@@ -448,6 +446,10 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
         rc = check_budget_params(p.shape, *bparams);
         if (rc != UNCOMP_OK) return rc;
         if ((d_layer_group == nullptr) != (d_layer_ctx == nullptr)) return UNCOMP_E_NULL;
+    }
+    if (d_lse && tensor_path) {
+        // One sweep over K: the window scores (the caller brings the row normalisers) and the Gram partials of the
+        // entropy stage come out of the same kernel; then eigenvalues, budgets, selection, gather.
         cudaStream_t st = static_cast<cudaStream_t>(stream);
         uint32_t *d_status = reinterpret_cast<uint32_t *>(ctx->ws + p.off_status);
         float *partials = reinterpret_cast<float *>(ctx->ws + p.off_gram);
@@ -482,20 +484,6 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
         // selection needs both.  The two cannot share an SM (registers), so which one is launched first matters: with few
         // units the eigenvalues are a chain on a few SMs and have to go first (one layer of 7001 tokens 138 us, 175 the other
         // way round); with many the order makes no difference (1024 units of 3712 tokens 820 and 825 us, of 32K 5.03 ms both).
-        if (!d_K || !d_Qw || !d_entropy || !d_budgets || !d_offsets || !d_indices) return UNCOMP_E_NULL;
-        if (!aligned16(d_K) || !aligned16(d_Qw)) return UNCOMP_E_ALIGN;
-        rc = check_strides(p.shape, sK);
-        if (rc != UNCOMP_OK) return rc;
-        if (eparams->k_trunc < 1 || eparams->max_iters < 0 || (eparams->center != 0 && eparams->center != 1) ||
-            (eparams->norm != 0 && eparams->norm != 1))
-            return UNCOMP_E_PARAM;
-        if (sparams->pool_kernel < 1 || sparams->pool_kernel > 63 || (sparams->pool_kernel & 1) == 0 ||
-            (sparams->pool_mode != 0 && sparams->pool_mode != 1) || !(sparams->scale >= 0.f) || isinf(sparams->scale))
-            return UNCOMP_E_PARAM;
-        if (bparams->scope != 0 && bparams->scope != 1) return UNCOMP_E_PARAM;
-        rc = check_budget_params(p.shape, *bparams);
-        if (rc != UNCOMP_OK) return rc;
-        if ((d_layer_group == nullptr) != (d_layer_ctx == nullptr)) return UNCOMP_E_NULL;
         cudaStream_t st = static_cast<cudaStream_t>(stream);
         cudaError_t e = ensure_side_stream(ctx);
         if (e != cudaSuccess) return cuda_fail(ctx, e);
@@ -536,14 +524,13 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
         }
         if (e != cudaSuccess) return cuda_fail(ctx, e);
     } else {
-        // the four calls back to back; bf16 keys without normalisers take the fused Gram + statistics sweep
-        const bool fuse = tensor_path && !d_lse;
-        rc = uncomp_entropy(ctx, d_K, sK, eparams, fuse ? d_Qw : nullptr, sparams->scale, d_entropy, d_erank, nullptr, stream);
+        // CUDA-core kernels: the calls back to back, nothing to fuse
+        rc = uncomp_entropy(ctx, d_K, sK, eparams, nullptr, sparams->scale, d_entropy, d_erank, nullptr, stream);
         if (rc != UNCOMP_OK) return rc;
         rc = uncomp_assign_budgets(ctx, d_erank, bparams, d_budgets, d_offsets, d_layer_group, d_layer_ctx, stream);
         if (rc != UNCOMP_OK) return rc;
         uncomp_score_params sp = *sparams;
-        sp.reuse_stats = fuse ? 1 : 0;
+        sp.reuse_stats = 0;
         rc = uncomp_score_select(ctx, d_Qw, d_K, sK, d_lse, d_budgets, d_offsets, &sp, d_scores, d_indices, stream);
         if (rc != UNCOMP_OK) return rc;
     }

@@ -101,19 +101,9 @@ __device__ __forceinline__ bool elect_one() {
 }
 
 // ---- MMA ------------------------------------------------------------------------------------------
-// D[tmem] (+)= A[smem] * B[smem]; issued by ONE thread.
-__device__ __forceinline__ void mma_f16_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                           uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// Same MMA with the descriptors given as 32-bit halves.  The upper half of a shared-memory descriptor
-// (stride offset, version, swizzle mode) is the same for every tile of a kernel and the lower half only
-// changes in its address field, so the issuing thread advances a descriptor with ONE 32-bit add instead of
+// D[tmem] (+)= A[smem] * B[smem]; issued by ONE thread.  The descriptors are given as 32-bit halves: the upper
+// half of a shared-memory descriptor (stride offset, version, swizzle mode) is the same for every tile of a kernel
+// and the lower half only changes in its address field, so the issuing thread advances a descriptor with ONE 32-bit add instead of
 // rebuilding 64 bits: that thread's serial instruction stream is what paces the tensor pipe.
 __device__ __forceinline__ void mma_f16_ss_lohi(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi,
                                                 uint32_t idesc, uint32_t accumulate) {

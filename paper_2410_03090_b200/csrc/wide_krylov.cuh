@@ -23,7 +23,6 @@ struct KrylovBuffers {
 };
 constexpr int kKryBand = 34;
 constexpr int kKryStateInts = 8 + kKryMaxK;
-constexpr int kKryMaxLaunches = 4;
 
 // Largest ratio of the k wanted eigenvalues.  Rounding of the product is a share of the largest one; relative to the
 // eigenvalue itself (root mean square over 32, six matrices each, n = 512 to 2048) it comes to 0.4e-6 to 0.9e-6 at ratios
