@@ -641,10 +641,9 @@ band_eigen_kernel(int k, int q, int max_iters, KrylovBuffers B, uint32_t *__rest
     if (first < kCoarse) hi = in->shift[first];
     // max_iters counts 257-fold rounds, as in the full reduction; these are 33-fold after the coarse 1025 intervals
     const int rounds = max_iters > 0 ? min(max((8 * max_iters - 6) / 5, 1), 7) : 7;
-    double tol = 0.0;
     bool last = false;
     for (int it = 0; it < rounds && !last; ++it) {
-        tol = band_tolerance(lo, bound);
+        const double tol = band_tolerance(lo, bound);
         last = hi - lo <= tol * (double)kShifts || it == rounds - 1;
         const int shifts = last ? kShifts - 1 : kShifts;
         const double step = (hi - lo) / (double)(shifts + 1);
@@ -666,7 +665,7 @@ band_eigen_kernel(int k, int q, int max_iters, KrylovBuffers B, uint32_t *__rest
     }
     if (rank == 0 && tid == 0) {
         B.lam[t] = 0.5 * (lo + hi);
-        if (hi - lo > tol) atomicOr(status, (uint32_t)UNCOMP_STATUS_NOT_CONVERGED);
+        if (hi - lo > band_tolerance(lo, bound)) atomicOr(status, (uint32_t)UNCOMP_STATUS_NOT_CONVERGED);
         if (t == 0) B.lam[k] = in->trace;
     }
     cluster.sync();                               // nobody leaves while another may still write its counts
