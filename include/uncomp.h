@@ -97,7 +97,7 @@ void uncomp_destroy(uncomp_ctx *ctx);
  * bf16 input: Gram matrix on the tensor cores with fp32 accumulation, chunk partials added in fp64, then
  * an fp32 Householder tridiagonalisation held in registers and a Sturm-count multi-section for the k
  * largest eigenvalues (bracketed to 2e-8 of the spectral radius; the fp32 reduction is good to about
- * 1e-7).  fp32 input: Gram matrix and eigenvalues in fp64 throughout (Householder in shared memory,
+ * 1e-7).  fp32 input: Gram matrix and eigenvalues in fp64 throughout (Householder in registers,
  * brackets to 1e-13 of the spectral radius).  max_iters bounds the multi-section rounds (0 = the default
  * of the path, 10 or 14); a unit that has not reached its tolerance by then sets
  * UNCOMP_STATUS_NOT_CONVERGED and still writes its current estimate.
@@ -385,8 +385,10 @@ int uncomp_prepare_groups(uncomp_ctx *ctx, const float *d_erank, int32_t S, int3
  * uncomp_entropy_wide -- Section 3.1 Eq. 1 for token vectors x_i in R^D with D beyond a head (the hidden
  * states of a layer, D = 4096, or the heads of a layer side by side), Lemma 2 and Section 3.2: the same
  * H_k and erank_k as uncomp_entropy, of `count` matrices X_i [N, D] (bf16; the context must be a bf16
- * one).  The D x D scatter matrix is formed on the tensor cores, tridiagonalised in fp32 by one
- * cooperative kernel that spans the GPU and its k largest eigenvalues are found in fp64 (Sturm counts).
+ * one).  The D x D scatter matrix is formed on the tensor cores.  Up to 64 eigenvalues of a matrix of 384
+ * and more come from block Lanczos in fp32 and Sturm counts in fp64 of what it projects to; all others, and
+ * what does not settle there, from a tridiagonalisation in fp32 and Sturm counts in fp64.  Both are
+ * cooperative kernels that span the GPU.  max_iters counts rounds of 256 points per eigenvalue (0 = 8).
  *
  * d_X            in   matrix i starts at element i * stride_matrix; token rows stride_row elements apart
  *                     (stride_row >= D, both strides multiples of 8 elements), features contiguous
@@ -397,7 +399,7 @@ int uncomp_prepare_groups(uncomp_ctx *ctx, const float *d_erank, int32_t S, int3
  *                     matrices are processed one after the other and share it
  * d_entropy      out  [count] float;  d_erank out [count] float, may be NULL
  * d_spectrum     out  [count, min(k_trunc, D)] double, the largest eigenvalues, descending; may be NULL
- * The cooperative kernel needs the GPU to itself while it runs: launching it on a device whose SMs are
+ * A cooperative kernel needs the GPU to itself while it runs: launching it on a device whose SMs are
  * held by another long-running kernel delays it, it never deadlocks (its grid barrier gives up after a
  * bounded number of polls and raises UNCOMP_STATUS_TIMEOUT).
  * ------------------------------------------------------------------------------------------------- */

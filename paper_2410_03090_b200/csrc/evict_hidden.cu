@@ -7,12 +7,13 @@
 // the lower position), indices ascending; rows of the hidden-state matrix X [N, D] are gathered.
 //
 // The last token has one query row per head, so this is matrix-vector work bound by reading K once:
-//   1. logits kernel   grid (token chunks, B*H): half a warp owns a token and reads its 128-feature key row
-//                      as one coalesced line; the G dot products of its KV head against the query vectors
-//                      (pre-scaled to the log2 domain) are summed over the lanes by a transposing butterfly;
-//                      logits go to scratch, each chunk leaves (max, sum of 2^(x - max)) per query head;
+//   1. logits kernel   grid (token chunks, B*H).  bf16: the warp-level tensor-core instruction on 16 key rows at a time,
+//                      both operands straight from 16-byte loads.  fp32: half a warp owns a token and reads its
+//                      128-feature key row as one coalesced line; the G dot products of its KV head against the query
+//                      vectors (pre-scaled to the log2 domain) are summed over the lanes by a transposing butterfly.
+//                      Logits go to scratch, each chunk leaves (max, sum of 2^(x - max)) per query head;
 //   2. scores kernel   merges the chunk statistics per head (fixed order) and adds 2^(x - m'_h) over heads;
-//   3. selection       the radix select of select.cu with one unit per sequence;
+//   3. selection       the one of select.cu (histograms over keys in shared memory) with one unit per sequence;
 //   4. row gather      a warp per kept row, 16-byte vectors, any row width that is a multiple of 16 bytes.
 #include "common.cuh"
 

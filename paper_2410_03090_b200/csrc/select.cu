@@ -80,7 +80,7 @@ __device__ void find_bin(SelSmem &S, int nbins, int kr, int tid) {
     __syncthreads();
 }
 
-// ---- longer prefixes: radix select of the pooled scores in global memory ------------------------------------------
+// ---- prefixes beyond 262144: radix select of the pooled scores in global memory -----------------------------------
 // A cluster of 8 CTAs per unit.  CTA r owns the r-th eighth of the positions; histograms and counts are combined through
 // distributed shared memory by CTA 0 and read back by the others.
 constexpr int kSelCluster = 8;
@@ -218,6 +218,10 @@ constexpr int kKeyWarps = kKeyThreads / 32;
 constexpr int kKeyMaxCluster = 8;
 constexpr int kKeyHalo = 32;                             // pool windows reach at most 31 positions beyond a CTA's share
 constexpr int kKeyBins = 2 * kKeyThreads;
+// How the scores are pooled: width 1 takes them as they are; the 7-wide maximum, what the pass defaults to, from the four
+// scores of a lane and shuffles; any other width by a loop per position.  256 units of 32704 positions / 1024 of 3704 / 8 of
+// 6969: 53 / 41 / 15 us, 66 / 50 / 17 us, and by the loop 77 / 54 / 17 us for a maximum over 5, 82 / 54 / 18 over 9, 141 /
+// 72 / 23 over 63.
 enum { kPoolAny, kPoolNone, kPoolMax7 };
 
 template <int NBK> struct KeySmem {
@@ -229,6 +233,8 @@ template <int NBK> struct KeySmem {
     int bin, above, in_bin;
 };
 
+// Two CTAs per SM up to four blocks of keys: with many units one CTA's barriers hide behind the other.  That bound leaves
+// 32 registers and spills 36 to 64 bytes of a thread, also in calls whose few units leave the second place empty.
 template <int NBK, int POOL>
 __global__ void __launch_bounds__(kKeyThreads, NBK <= 4 ? 2 : 1)
 pool_select_keys_kernel(const float *__restrict__ raw, float *__restrict__ pooled, int P, int w, int pool_kernel, int pool_mode,

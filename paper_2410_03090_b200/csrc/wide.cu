@@ -8,12 +8,15 @@
 //                        (64-feature boxes, 128B swizzle); both MMA operands are read MN-major, two
 //                        M = 128, N = 256 accumulators fill the 512 TMEM columns; partial blocks to scratch;
 //   3. assemble          C = G - s s^T / N (fp64 subtraction), stored as a full symmetric fp32 matrix;
-//   4. tridiagonalise    Householder on the whole GPU: one cooperative launch, rows of the trailing matrix
-//                        spread over all warps, ONE grid barrier per column.  The rank-2 update of column k
-//                        is applied while the matrix is swept for the matrix-vector product of column k + 1,
-//                        so the matrix (64 MB at D = 4096, resident in L2) is read and written once per column;
-//   5. eigenvalues       Sturm-count 256-section (fp64), one CTA per wanted eigenvalue of the tridiagonal
-//                        matrix, then H_k and erank_k.
+//   4. eigenvalues       up to 64 of a matrix of 384 and more: block Lanczos and Sturm counts of the projected band
+//                        matrix (wide_krylov.cu), 35 ms -> 1.4 ms at D = 4096, k = 32.  What that does not take or leaves
+//                        unsettled goes through the two steps of the full reduction, whose kernels otherwise leave at once:
+//                        - Householder on the whole GPU: one cooperative launch, rows of the trailing matrix spread over all
+//                          warps, ONE grid barrier per column.  The rank-2 update of column k is applied while the matrix
+//                          is swept for the matrix-vector product of column k + 1, so the matrix (64 MB at D = 4096,
+//                          resident in L2) is read and written once per column;
+//                        - Sturm-count 256-section (fp64), one CTA per wanted eigenvalue of the tridiagonal matrix;
+//   5. entropy           H_k and erank_k.
 // When the matrix has fewer tokens than features (N < D) the same non-zero eigenvalues are taken from the N x N
 // matrix of the centred rows' inner products, (x_i - mean) . (x_j - mean) = G'_ij - g_i - g_j + mean . mean with
 // G' = X X^T and g = X mean: the Gram kernel then contracts over features (both operands K-major, a CTA owns a
@@ -300,7 +303,7 @@ __global__ void __launch_bounds__(256) wide_rowdot_kernel(const __nv_bfloat16 *_
     if (lane == 0) g[row < N ? row : Dt] = acc;
 }
 
-// ------------------------------------------------------------------------------------- 4. tridiagonalisation
+// ------------------------------------------------------------------------------ 4. full reduction: tridiagonal form
 constexpr int kTriThreads = 1024;
 constexpr int kTriWarps = kTriThreads / 32;
 
@@ -478,7 +481,7 @@ __global__ void __launch_bounds__(kTriThreads, 1) l2_sweep_kernel(float *__restr
     }
 }
 
-// --------------------------------------------------------------------------------- 5. eigenvalues, entropy
+// -------------------------------------------------------------------- 4., 5. its eigenvalues; entropy of either route
 constexpr int kSturmThreads = 256;
 constexpr int kSturmMaxK = 256;
 

@@ -15,11 +15,14 @@
 //
 // Why: the reduction column by column sweeps the whole trailing matrix n times (33 ms at n = 4096), although only k of n
 // eigenvalues are wanted; here a step of 32 vectors reads the matrix once and 8 to 32 steps suffice (8192 x 4096 hidden
-// states with a decaying spectrum, k = 32: 8 steps, 0.95 ms, and the counts 0.42 ms, 0.54 with no shared round; an isotropic matrix, the slowest to
-// converge, takes 32).  Accuracy is that of fp32 products summed in fp32 / fp64, as before.
+// states with a decaying spectrum, k = 32: 8 steps, 0.93 ms, and the counts 0.44 ms, 0.1 more with no shared round; an
+// isotropic matrix, the slowest to converge, takes 32).  Accuracy is that of fp32 products summed in fp32 / fp64, as in the
+// reduction.
 // What bounds it: about 70 us of every step are grid barriers, sums over the CTAs and the two factorisations, whatever n;
-// the product takes 17 us of fp32 multiply-adds at n = 4096.  The counts are bound by issue and the fp64 units (190
-// instructions per row for two shifts).
+// the product takes 17 us of fp32 multiply-adds at n = 4096.  The counts are bound by the latency of one warp: eight shifts
+// per SM are one warp per scheduler, which issues every 3.4 cycles (1.4 of them wait for results of fixed latency, 0.3 for
+// shared memory, 0.3 for columns of T, 0.2 at branches); 29 % of the issue slots, 23 % of the fp64 pipe and, next in line,
+// 52 % of the shared-memory pipe are used, which is why a second warp per scheduler did not pay.
 // Convergence is tested by how far an eigenvalue still moves: T_m contains T_{m-64}, so by interlacing the i-th eigenvalue
 // has moved by less than delta over the last two blocks exactly if T_{m-64} has i eigenvalues above lambda_i - delta (its
 // pivots are the first ones of T, so one of the last round's shifts tells).  delta is 2e-6 of the eigenvalue itself (1e-7 of
@@ -672,6 +675,10 @@ band_eigen_kernel(int k, int q, int max_iters, KrylovBuffers B, uint32_t *__rest
 }
 }  // namespace
 
+// More than kKryMaxK = 64 eigenvalues go to the reduction: the range that the tests hold against the oracle, not where the
+// two sides meet.  That depends on the spectrum: 8192 x 4096 with 256 strong directions takes 2.2 ms here at k = 64, 5.0 at
+// 128, 11.5 at 256, the reduction 35.8 whatever k; an isotropic matrix of n = 2048 12.8 ms at k = 64 against 11.3.
+// kKryMinN: at n = 384 the buffers just hold the eight steps of k <= 32.
 bool krylov_applies(int n, int k, int ctas) {
     return n >= kKryMinN && k <= kKryMaxK && krylov_steps(n) >= (k <= 32 ? 8 : 10) && n / kB <= ctas;
 }
@@ -692,6 +699,10 @@ cudaError_t launch_krylov(const float *C, int n, int k, int max_iters, const Kry
                           cudaStream_t st) {
     cudaError_t e = cudaSuccess;
     const int most = krylov_steps(n);
+    // Steps at first, and twice as many whenever some eigenvalue has not settled.  Nine spectra (256 strong directions, power
+    // laws, exponential, 50 and 600 directions, isotropic; n = 1024 to 4096), k = 32, all nine together: from 6 steps 28.8 ms,
+    // from 8 26.6, 10 32.1, 12 27.0, 16 32.8.  k = 64, the six of them that end here: from 8 29.8 ms, 10 24.8, 12 22.9,
+    // 16 26.3; 10 is the best of the two with 256 strong directions (2.2 and 1.7 ms against 2.6 and 2.1 from 12).
     int part_blocks = most + 3, q0 = 0, q = k <= 32 ? 8 : 10, launch = 0;
     while (true) {
         unsigned *bar = b.bar + launch;

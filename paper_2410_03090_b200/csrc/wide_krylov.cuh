@@ -18,16 +18,16 @@ struct KrylovBuffers {
     double *G;           // [1024] Gram matrix of the new block
     double *T;           // [32 steps + 32][kKryBand] projected matrix, column c: entry (c - o, c) at [c][o], o <= 32
     double *lam;         // [k + 1] eigenvalues descending, then the trace
-    int *state;          // [0] steps in Q, [1] broken, [2] first unconverged count; [8 ..] converged, one per eigenvalue
+    int *state;          // [0] steps in Q, [1] broken, [2] all settled (set by the reduction's kernel); [8 ..] settled, each
     unsigned *bar;       // grid barrier counters, one per launch, zero at the start
 };
 constexpr int kKryBand = 34;
 constexpr int kKryStateInts = 8 + kKryMaxK;
 
-// Largest ratio of the k wanted eigenvalues.  Rounding of the product is a share of the largest one; relative to the
-// eigenvalue itself (root mean square over 32, six matrices each, n = 512 to 2048) it comes to 0.4e-6 to 0.9e-6 at ratios
-// up to 1000 and 1.0e-6 at 3000, as in the full reduction, but 3.6e-6 to 7.3e-6 at 30000 where the reduction has 2.9e-6 to
-// 5.7e-6: beyond this the reduction runs.
+// Largest ratio of the k wanted eigenvalues.  Rounding of the product is a share of the largest one.  Relative to the
+// eigenvalue itself (root mean square over 32, six matrices each, n = 1024 and 2048) it comes to 0.4e-6 to 0.7e-6 at ratios
+// up to 1000 and 1.0e-6 to 1.2e-6 at 3000, as in the full reduction, but 2.8e-6 to 7.3e-6 at 30000, where the reduction has
+// 2.2e-6 to 5.7e-6: beyond this the reduction runs.
 constexpr double kKryMaxRatio = 4096.0;
 
 __device__ __forceinline__ bool krylov_too_graded(const double *lam, int k) { return !(lam[0] <= kKryMaxRatio * lam[k - 1]); }
