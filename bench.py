@@ -31,7 +31,7 @@ if ROOT not in sys.path:
 # recorded beside them: when the file has changed since the capture, the bench prints null instead.
 NCU_COUNTERS = {
     "source": "paper_2410_03090_b200/csrc/scores_tc.cu",
-    "sha256": "0f8501a15275a1bda302b234570cbaa2347548619910feb2a96519c8045d572d",
+    "sha256": "0e2c45c81c8ffff40991394f6f22e53355b5a0b799a041c1ef1e5f0eb831fbc4",
     "capture": "ncu --set full, one launch per kernel, c3 scaled to N 16384 x 10 layers; summary in profiles/",
     "kernels": {
         "gram_score_stats": {"dram_bytes_per_unit_token": (344.463872e6 + 29.947904e6) / (80 * 16384),

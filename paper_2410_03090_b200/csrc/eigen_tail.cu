@@ -5,8 +5,8 @@
 // i = lane / 8 holds the 128 entries M[i + 4 a][4 t + 32 j + e], a < 16, j < 2, e < 4, as packed pairs), so a step needs
 // no block barrier, and eight units share an SM where the whole matrix allows two.  The steps are the first kernel's
 // (one exchange through shared memory, the rank-2 update one step late) with a warp barrier.
-// Bound by the chain of a step (three shuffle reductions, a square root, a reciprocal) while a unit has an SM
-// sub-partition for itself, by issue with two warps on it.
+// Bound by the chain of a step (three shuffle reductions, a square root, a reciprocal); two warps per SM sub-partition, what
+// the registers admit, use half of its issue slots (1024 units: 49 %, an instruction of a warp every 3.4 cycles).
 #include "eigen_common.cuh"
 
 namespace uncomp {

@@ -15,7 +15,7 @@ namespace uncomp {
 // fp32 keys.  Grid: (units x 10 tile pairs I <= J of 32 x 32 entries, token chunks): the symmetric half, and enough CTAs
 // for calls of few units and few tokens (one CTA per unit and chunk took 126 us for 8 units of 512 tokens, this 17 us).
 // A quarter of the CTA takes every fourth token; a thread owns 4 x 4 entries, so four 16-byte loads feed 16 fp64
-// multiply-adds, which bound it.
+// multiply-adds.  Those loads bound it: shared memory at 77 % of its rate, the fp64 pipe at 23 %.
 __global__ void __launch_bounds__(256) gram_f64_kernel(const float *__restrict__ K, UnitAddr addr, int N, int chunk,
                                                       double *__restrict__ partials, int P) {
     constexpr int TT = 32;

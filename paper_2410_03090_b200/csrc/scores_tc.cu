@@ -29,9 +29,11 @@
 // tile paced the kernel).
 // Mode 3 is pass B with the Gram stage folded in the same way, for callers who bring the row normalisers (their
 // prefill attention kernel's log-sum-exp): entropy stage and scores from ONE sweep over K.
-// What bounds it: power.  With keys streaming and the tensor pipe busy the SM clock falls from 1.9 to 1.2 - 1.6 GHz; a
-// micro-benchmark of the same MMAs, TMA loads and exponentials without any hand-over takes 1,180 cycles = 0.95 us per tile
-// of one row block, modes 2 and 3 take about 1.1 us.  Two row blocks are bound by the exponential unit (2,048 cycles).
+// What bounds it.  In single passes the exponential unit, 66 % (mode 2) and 76 % (mode 1) busy, and the queue in front of it
+// (two row blocks need 2,048 cycles of it per tile).  Repeated for more than half a second, power: 985 W, and the clock falls
+// from 1.965 to 1.75 (8192 and 131072 tokens), 1.57 (32768) or 1.40 GHz (4 x 32768); a micro-benchmark of the same MMAs, TMA
+// loads and exponentials without any hand-over takes 1,180 cycles per tile of one row block, 0.95 us at such a clock, and
+// modes 2 and 3 take about 1.1 us.
 // Every wait is bounded; a timeout raises UNCOMP_STATUS_TIMEOUT and the CTA drains and exits.
 #include "tc_common.cuh"
 
