@@ -53,6 +53,7 @@ __global__ void __launch_bounds__(kBudThreads) budgets_kernel(const float *__res
     float *er_s = reinterpret_cast<float *>(shared_tab ? reinterpret_cast<int32_t *>(bud_smem + M) + M
                                                        : reinterpret_cast<int32_t *>(bud_smem));
     const float *er = shared_er ? er_s : erank;
+    chain_wait();
     if (shared_er)
         for (int u = tid; u < units; u += kBudThreads) er_s[u] = erank[u];
     auto target = [&](int g) { return n_max * S - (int64_t)g * n * (n_max - avg); };   // t_g S
@@ -168,9 +169,9 @@ cudaError_t launch_budgets(const Plan &p, const float *d_erank, const uncomp_bud
     static bool done[64] = {};
     cudaError_t e = allow_dynamic_smem((const void *)budgets_kernel, kBudShared * 16, done);
     if (e != cudaSuccess) return e;
-    budgets_kernel<<<1, kBudThreads, smem, st>>>(d_erank, p.shape.B, p.shape.L, p.shape.H, p.shape.N, p.shape.w, bp, sched,
-                                                 d_budgets, d_offsets, d_layer_group, d_layer_ctx, d_rank, d_rem);
-    return cudaGetLastError();
+    return launch_kernel(budgets_kernel, LaunchShape{dim3(1), kBudThreads, smem, 1, true}, st, d_erank, p.shape.B, p.shape.L,
+                         p.shape.H, p.shape.N, p.shape.w, bp, sched, d_budgets, d_offsets, d_layer_group, d_layer_ctx, d_rank,
+                         d_rem);
 }
 
 }  // namespace uncomp

@@ -25,6 +25,7 @@ __global__ void __launch_bounds__(256) compact_kernel(const unsigned char *__res
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    chain_wait();
     const int64_t total = offsets[units];
     const int sub = lane / LANES_PER_ROW, vec = lane % LANES_PER_ROW;
     for (int64_t t0 = warp * 32; t0 < total; t0 += nwarps * 32) {
@@ -68,16 +69,10 @@ cudaError_t launch_compact(const Plan &p, const void *dK, const void *dV, const 
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int grid = sms * 8;
-    if (p.shape.dtype == UNCOMP_FP32)
-        compact_kernel<512><<<grid, 256, 0, st>>>((const unsigned char *)dK, (const unsigned char *)dV, aK, aV,
-                                                  p.units, p.shape.N, 4, d_indices, d_offsets, (unsigned char *)dKc,
-                                                  (unsigned char *)dVc, d_status);
-    else
-        compact_kernel<256><<<grid, 256, 0, st>>>((const unsigned char *)dK, (const unsigned char *)dV, aK, aV,
-                                                  p.units, p.shape.N, 2, d_indices, d_offsets, (unsigned char *)dKc,
-                                                  (unsigned char *)dVc, d_status);
-    return cudaGetLastError();
+    const bool f32 = p.shape.dtype == UNCOMP_FP32;
+    return launch_kernel(f32 ? compact_kernel<512> : compact_kernel<256>, LaunchShape{dim3(sms * 8), 256, 0, 1, true}, st,
+                         (const unsigned char *)dK, (const unsigned char *)dV, aK, aV, p.units, p.shape.N, f32 ? 4 : 2,
+                         d_indices, d_offsets, (unsigned char *)dKc, (unsigned char *)dVc, d_status);
 }
 
 }  // namespace uncomp

@@ -518,6 +518,7 @@ __global__ void __launch_bounds__(kDecThreads, 3) decode_step_kernel(DecArgs a, 
     cg::cluster_group cluster = cg::this_cluster();
     const int ctas = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
     const int u = blockIdx.x / ctas, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    chain_wait();
     // the new token's row and position are not needed before the end: on their way from the start
     constexpr int kVecs = kD * (int)sizeof(T) / 16;      // 16-byte vectors per row
     int4 fresh = make_int4(0, 0, 0, 0);
@@ -660,18 +661,7 @@ cudaError_t launch_step(const DecArgs &a, const StepArgs &b, int units, int ctas
     static bool done[64] = {};
     cudaError_t e = allow_dynamic_smem((const void *)decode_step_kernel<G, T>, kStepSmem, done);
     if (e != cudaSuccess) return e;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = ctas;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(units * ctas);
-    cfg.blockDim = dim3(kDecThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = ctas > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, decode_step_kernel<G, T>, a, b);
+    return launch_kernel(decode_step_kernel<G, T>, LaunchShape{dim3(units * ctas), kDecThreads, smem, (unsigned)ctas, true}, st, a, b);
 }
 template <typename T>
 cudaError_t launch_step_g(const DecArgs &a, const StepArgs &b, int units, int ctas, size_t smem, cudaStream_t st) {

@@ -248,6 +248,7 @@ eigen_entropy_kernel(const PartialT *__restrict__ partials, int P, int N, int k_
     const int row0 = tid >> 4, t = tid & 15;
     constexpr int len = n * n + n;
     const PartialT *base = partials + (size_t)u * P * len;
+    chain_wait();
 
     // ---- 1. assemble C in registers ----------------------------------------------------------------
     if (tid < n) {
@@ -439,16 +440,12 @@ cudaError_t launch_gram_reduce(const Plan &p, const void *d_partials, double *d_
 cudaError_t launch_eigen_entropy(const Plan &p, const void *d_partials, const uncomp_entropy_params &ep,
                                  float *d_entropy, float *d_erank, double *d_spectrum, uint32_t *d_status,
                                  cudaStream_t st) {
-    if (p.shape.dtype == UNCOMP_FP32) {
-        eigen_entropy_kernel<double><<<p.units, kEigThreads, 0, st>>>(
-            (const double *)d_partials, p.gram_splits, p.shape.N, ep.k_trunc, ep.center, ep.norm, ep.max_iters,
-            d_entropy, d_erank, d_spectrum, d_status);
-    } else {
-        eigen_entropy_kernel<float><<<p.units, kEigThreads, 0, st>>>(
-            (const float *)d_partials, p.gram_splits, p.shape.N, ep.k_trunc, ep.center, ep.norm, ep.max_iters,
-            d_entropy, d_erank, d_spectrum, d_status);
-    }
-    return cudaGetLastError();
+    const LaunchShape shape{dim3(p.units), kEigThreads, 0, 1, true};
+    if (p.shape.dtype == UNCOMP_FP32)
+        return launch_kernel(eigen_entropy_kernel<double>, shape, st, (const double *)d_partials, p.gram_splits, p.shape.N,
+                             ep.k_trunc, ep.center, ep.norm, ep.max_iters, d_entropy, d_erank, d_spectrum, d_status);
+    return launch_kernel(eigen_entropy_kernel<float>, shape, st, (const float *)d_partials, p.gram_splits, p.shape.N, ep.k_trunc,
+                         ep.center, ep.norm, ep.max_iters, d_entropy, d_erank, d_spectrum, d_status);
 }
 
 }  // namespace uncomp

@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(kEvThreads) last_token_logits_kernel(
     const int c = blockIdx.x, bh = blockIdx.y, b = bh / H, h = bh % H;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, hw = lane >> 4, sub = lane & 15;
     const int Hq = H * G;
+    chain_wait();
     for (int e = tid; e < G * kD; e += kEvThreads)
         qs[e / kD][e % kD] = to_float(qlast[((size_t)b * Hq + (size_t)h * G) * kD + e]) * c_log2;
     __syncthreads();
@@ -179,6 +180,7 @@ __global__ void __launch_bounds__(kEvThreads) last_token_logits_mma_kernel(
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, gid = lane >> 2, tig = lane & 3;
     const int Hq = H * G;
     const __nv_bfloat16 *qb = qlast + ((size_t)b * Hq + (size_t)h * G) * kD;
+    chain_wait();
     uint32_t bq[NB][16];
 #pragma unroll
     for (int nb = 0; nb < NB; ++nb) {
@@ -278,6 +280,7 @@ __global__ void __launch_bounds__(kEvThreads) last_token_scores_kernel(
     extern __shared__ float mprime[];   // [Hq]
     const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
     const int j = blockIdx.x * kEvThreads + tid;
+    chain_wait();
     for (int h = tid >> 5; h < Hq; h += kEvThreads / 32) {
         const float2 *p = reinterpret_cast<const float2 *>(stats_part) + ((size_t)b * Hq + h) * chunks;
         float m = -1e30f, l = 0.f;
@@ -324,6 +327,7 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const unsigned char *_
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    chain_wait();
     for (int64_t t = warp; t < rows_total; t += nwarps) {
         const int64_t b = t / n_keep;
         if (!UNCOMP_INDEX_OK(idx[t], N, status)) continue;
@@ -337,28 +341,28 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const unsigned char *_
 template <typename T>
 cudaError_t launch_logits(int G, dim3 grid, cudaStream_t st, const T *q, const T *K, int H, int64_t sB, int64_t sH,
                           int64_t sN, int N, int chunk, int chunks, float c_log2, float *logits, float *stats) {
+    const LaunchShape shape{grid, kEvThreads, 0, 1, true};
     switch (G) {
-        case 1: last_token_logits_kernel<T, 1><<<grid, kEvThreads, 0, st>>>(q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats); break;
-        case 2: last_token_logits_kernel<T, 2><<<grid, kEvThreads, 0, st>>>(q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats); break;
-        case 4: last_token_logits_kernel<T, 4><<<grid, kEvThreads, 0, st>>>(q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats); break;
-        case 8: last_token_logits_kernel<T, 8><<<grid, kEvThreads, 0, st>>>(q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats); break;
-        case 16: last_token_logits_kernel<T, 16><<<grid, kEvThreads, 0, st>>>(q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats); break;
+        case 1: return launch_kernel(last_token_logits_kernel<T, 1>, shape, st, q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats);
+        case 2: return launch_kernel(last_token_logits_kernel<T, 2>, shape, st, q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats);
+        case 4: return launch_kernel(last_token_logits_kernel<T, 4>, shape, st, q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats);
+        case 8: return launch_kernel(last_token_logits_kernel<T, 8>, shape, st, q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats);
+        case 16: return launch_kernel(last_token_logits_kernel<T, 16>, shape, st, q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 cudaError_t launch_logits_mma(int G, dim3 grid, cudaStream_t st, const __nv_bfloat16 *q, const __nv_bfloat16 *K, int H,
                               int64_t sB, int64_t sH, int64_t sN, int N, int chunk, int chunks, float c_log2,
                               float *logits, float *stats) {
+    const LaunchShape shape{grid, kEvThreads, 0, 1, true};
     switch (G) {
-        case 1: last_token_logits_mma_kernel<1><<<grid, kEvThreads, 0, st>>>(q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats); break;
-        case 2: last_token_logits_mma_kernel<2><<<grid, kEvThreads, 0, st>>>(q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats); break;
-        case 4: last_token_logits_mma_kernel<4><<<grid, kEvThreads, 0, st>>>(q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats); break;
-        case 8: last_token_logits_mma_kernel<8><<<grid, kEvThreads, 0, st>>>(q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats); break;
-        case 16: last_token_logits_mma_kernel<16><<<grid, kEvThreads, 0, st>>>(q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats); break;
+        case 1: return launch_kernel(last_token_logits_mma_kernel<1>, shape, st, q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats);
+        case 2: return launch_kernel(last_token_logits_mma_kernel<2>, shape, st, q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats);
+        case 4: return launch_kernel(last_token_logits_mma_kernel<4>, shape, st, q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats);
+        case 8: return launch_kernel(last_token_logits_mma_kernel<8>, shape, st, q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats);
+        case 16: return launch_kernel(last_token_logits_mma_kernel<16>, shape, st, q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 }  // namespace
 
@@ -388,8 +392,9 @@ cudaError_t launch_evict_hidden(const Plan &p, const void *d_qlast, const void *
     {
         ProfScope ps(prof, kSlotEvictScores, st);
         dim3 grid((s.N - 1 + kEvThreads - 1) / kEvThreads, s.B);
-        last_token_scores_kernel<<<grid, kEvThreads, s.Hq * sizeof(float), st>>>(d_logits, d_stats, s.B, s.Hq, s.N, chunks,
-                                                                                n_keep, d_raw, d_budgets, d_offsets);
+        e = launch_kernel(last_token_scores_kernel, LaunchShape{grid, kEvThreads, s.Hq * sizeof(float), 1, true}, st, d_logits, d_stats, s.B,
+                          s.Hq, s.N, chunks, n_keep, d_raw, d_budgets, d_offsets);
+        if (e != cudaSuccess) return e;
     }
     {
         // the selection kernel with one unit per sequence, a window of one (the last position), no pooling
@@ -398,7 +403,7 @@ cudaError_t launch_evict_hidden(const Plan &p, const void *d_qlast, const void *
         q.units = s.B;
         q.prefix = s.N - 1;
         q.shape.w = 1;
-        e = launch_pool_select(q, d_raw, d_scores, 1, 0, d_budgets, d_offsets, d_indices, d_status, st);
+        e = launch_pool_select(q, d_raw, d_scores, 1, 0, d_budgets, d_offsets, d_indices, true, d_status, st);
         if (e != cudaSuccess) return e;
     }
     {
@@ -406,10 +411,10 @@ cudaError_t launch_evict_hidden(const Plan &p, const void *d_qlast, const void *
         int dev = 0, sms = 148;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        gather_rows_kernel<<<sms * 8, 256, 0, st>>>((const unsigned char *)d_X, d_indices, (int64_t)s.B * n_keep, n_keep,
-                                                    s.N, row_bytes, (unsigned char *)d_Xout, d_status);
+        e = launch_kernel(gather_rows_kernel, LaunchShape{dim3(sms * 8), 256, 0, 1, true}, st, (const unsigned char *)d_X, d_indices,
+                          (int64_t)s.B * n_keep, n_keep, s.N, row_bytes, (unsigned char *)d_Xout, d_status);
     }
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace uncomp

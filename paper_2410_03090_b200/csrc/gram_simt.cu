@@ -46,6 +46,7 @@ __global__ void __launch_bounds__(256) gram_f64_kernel(const float *__restrict__
             *reinterpret_cast<double2 *>(dst + 2) = make_double2((double)pre[i].z, (double)pre[i].w);
         }
     };
+    chain_wait();
     double acc[4][4], colsum = 0.0;
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -145,8 +146,8 @@ __global__ void __launch_bounds__(256) gram_simt_kernel(const T *__restrict__ K,
 
 cudaError_t launch_gram_simt(const Plan &p, const void *dK, const UnitAddr &addr, void *d_partials, cudaStream_t st) {
     if (p.shape.dtype == UNCOMP_FP32) {
-        gram_f64_kernel<<<dim3(10 * p.units, p.gram_splits), 256, 0, st>>>((const float *)dK, addr, p.shape.N, p.gram_chunk,
-                                                                         (double *)d_partials, p.gram_splits);
+        return launch_kernel(gram_f64_kernel, LaunchShape{dim3(10 * p.units, p.gram_splits), 256, 0, 1, true}, st, (const float *)dK, addr,
+                             p.shape.N, p.gram_chunk, (double *)d_partials, p.gram_splits);
     } else {
         dim3 grid(p.gram_splits, p.units);
         gram_simt_kernel<__nv_bfloat16, float><<<grid, 256, 0, st>>>((const __nv_bfloat16 *)dK, addr, p.shape.N,

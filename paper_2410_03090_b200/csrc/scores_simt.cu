@@ -57,6 +57,7 @@ __global__ void __launch_bounds__(256) score_stats_simt_kernel(const T *__restri
     const int rows = G * w, P = N - w;
     const T *Qu = Qw + (size_t)u * rows * kD;   // [G, w, d] of this unit: its G query heads are adjacent
     const T *Ku = K + addr.base(u);
+    chain_wait();
     load_rows(qs, Qu, kD, rb * kSB, rows, tid);
 
     float m_run[4], l_run[4];
@@ -113,6 +114,7 @@ __global__ void score_stats_merge_kernel(const float *__restrict__ stats_part, i
                                          float *__restrict__ stats) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= units * rows) return;
+    chain_wait();
     const int u = idx / rows, r = idx % rows;
     float m = -INFINITY;
     for (int c = 0; c < splits; ++c) m = fmaxf(m, stats_part[(((size_t)u * splits + c) * kMaxRows + r) * 2]);
@@ -141,6 +143,7 @@ __global__ void __launch_bounds__(256) score_colsum_simt_kernel(const T *__restr
     const T *Qu = Qw + (size_t)u * rows * kD;
     const T *Ku = K + addr.base(u);
     const int t = tile * kSB;
+    chain_wait();
     load_rows(ks, Ku, addr.sN, t, P, tid);
     float col[4] = {0.f, 0.f, 0.f, 0.f};
     for (int rb = 0; rb * kSB < rows; ++rb) {
@@ -176,6 +179,7 @@ __global__ void lse_import_kernel(const float *__restrict__ lse, int units, int 
                                   float *__restrict__ stats, uint32_t *__restrict__ status) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= units * rows) return;
+    chain_wait();
     const int u = idx / rows, r = idx % rows;
     float v = lse[idx];
     if (!isfinite(v)) {
@@ -200,27 +204,27 @@ static cudaError_t launch_scores_simt_t(const Plan &p, const T *dQw, const T *dK
     if (d_lse) {
         ProfScope ps(prof, kSlotStatsMerge, st);
         const int total = p.units * p.rows;
-        lse_import_kernel<<<(total + 255) / 256, 256, 0, st>>>(d_lse, p.units, p.rows, d_stats, d_status);
+        e = launch_kernel(lse_import_kernel, LaunchShape{dim3((total + 255) / 256), 256, 0, 1, true}, st, d_lse, p.units, p.rows, d_stats,
+                          d_status);
     } else {
         const int row_blocks = (p.rows + kSB - 1) / kSB;
         dim3 gA(p.score_splits, row_blocks, p.units);
         {
             ProfScope ps(prof, kSlotScoreStats, st);
-            score_stats_simt_kernel<T><<<gA, 256, smemA, st>>>(dQw, dK, addr, p.shape.N, p.shape.w, p.G, p.score_chunk,
-                                                               p.score_splits, scale, d_stats_part);
+            e = launch_kernel(score_stats_simt_kernel<T>, LaunchShape{gA, 256, smemA, 1, true}, st, dQw, dK, addr, p.shape.N, p.shape.w,
+                              p.G, p.score_chunk, p.score_splits, scale, d_stats_part);
         }
+        if (e != cudaSuccess) return e;
         const int total = p.units * p.rows;
         ProfScope ps(prof, kSlotStatsMerge, st);
-        score_stats_merge_kernel<<<(total + 255) / 256, 256, 0, st>>>(d_stats_part, p.units, p.rows, p.score_splits,
-                                                                      d_stats);
+        e = launch_kernel(score_stats_merge_kernel, LaunchShape{dim3((total + 255) / 256), 256, 0, 1, true}, st, d_stats_part, p.units,
+                          p.rows, p.score_splits, d_stats);
     }
+    if (e != cudaSuccess) return e;
     dim3 gB((p.prefix + kSB - 1) / kSB, p.units);
-    {
-        ProfScope ps(prof, kSlotScoreColsum, st);
-        score_colsum_simt_kernel<T><<<gB, 256, smemB, st>>>(dQw, dK, addr, p.shape.N, p.shape.w, p.G, scale, d_stats,
-                                                            d_raw);
-    }
-    return cudaGetLastError();
+    ProfScope ps(prof, kSlotScoreColsum, st);
+    return launch_kernel(score_colsum_simt_kernel<T>, LaunchShape{gB, 256, smemB, 1, true}, st, dQw, dK, addr, p.shape.N, p.shape.w, p.G,
+                         scale, d_stats, d_raw);
 }
 
 cudaError_t launch_scores_simt(const Plan &p, const void *dQw, const void *dK, const UnitAddr &addr, float scale,

@@ -270,6 +270,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = T.tmem_base;
+    chain_wait();               // barriers, TMEM and descriptors are ready by then
 
     if (warp == 16) {
         // ---------------- TMA producer: runs ahead into the next items ----------------
@@ -619,7 +620,7 @@ static cudaError_t raise_smem_limit() {
 template <int MB, int SPLIT>
 static cudaError_t launch_scores_tc_mb(const Plan &p, const CUtensorMap &tq, const CUtensorMap &tk, float c_log2,
                                        const float *d_lse, float *d_stats_part, float *d_raw,
-                                       float *d_gram_part, int phases, uint32_t *d_status, Profiler *prof,
+                                       float *d_gram_part, int phases, bool chained, uint32_t *d_status, Profiler *prof,
                                        cudaStream_t st) {
     const uncomp_shape &s = p.shape;
     const int smem = score_smem(MB);
@@ -629,55 +630,48 @@ static cudaError_t launch_scores_tc_mb(const Plan &p, const CUtensorMap &tq, con
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // one CTA per SM, each with an equal share of the (unit, chunk) items
     auto ctas = [&](int splits) { return (unsigned)min((int64_t)sms, (int64_t)p.units * splits); };
+    auto launch = [&](auto kernel, int splits, int threads, float *stats_out, const float *stats_in, int stats_splits, const float *lse,
+                      float *raw, float *gram) {
+        return launch_kernel(kernel, LaunchShape{dim3(ctas(splits)), (unsigned)threads, (size_t)smem, 1, chained}, st, tq, tk, s.L, s.H,
+                             s.N, s.w, p.rows, p.units, p.score_chunk, splits, c_log2, stats_out, stats_in, stats_splits, lse, raw,
+                             gram, d_status);
+    };
     if (phases & kScorePhaseStats) {
         e = d_gram_part ? raise_smem_limit<MB, 2, SPLIT>() : raise_smem_limit<MB, 0, SPLIT>();
         if (e != cudaSuccess) return e;
         ProfScope ps(prof, d_gram_part ? kSlotGramStats : kSlotScoreStats, st);
-        if (d_gram_part)
-            score_tc_kernel<MB, 2, SPLIT><<<ctas(p.score_splits), kGramThreads, smem, st>>>(
-                tq, tk, s.L, s.H, s.N, s.w, p.rows, p.units, p.score_chunk, p.score_splits, c_log2, d_stats_part, nullptr, 0, nullptr, nullptr,
-                d_gram_part, d_status);
-        else
-            score_tc_kernel<MB, 0, SPLIT><<<ctas(p.score_splits), kScoreThreads, smem, st>>>(
-                tq, tk, s.L, s.H, s.N, s.w, p.rows, p.units, p.score_chunk, p.score_splits, c_log2, d_stats_part, nullptr, 0, nullptr, nullptr,
-                nullptr, d_status);
+        e = launch(d_gram_part ? score_tc_kernel<MB, 2, SPLIT> : score_tc_kernel<MB, 0, SPLIT>, p.score_splits,
+                   d_gram_part ? kGramThreads : kScoreThreads, d_stats_part, nullptr, 0, nullptr, nullptr, d_gram_part);
+        if (e != cudaSuccess) return e;
     }
     if (phases & kScorePhaseColsum) {
         const bool with_gram = (phases & kScorePhaseStats) == 0 && d_gram_part != nullptr;   // mode 3
         ProfScope ps(prof, with_gram ? kSlotGramColsum : kSlotScoreColsum, st);
         const int splitsB = (p.prefix + p.score_chunk - 1) / p.score_chunk;
-        if (with_gram) {
-            e = raise_smem_limit<MB, 3, SPLIT>();
-            if (e != cudaSuccess) return e;
-            score_tc_kernel<MB, 3, SPLIT><<<ctas(p.score_splits), kGramThreads, smem, st>>>(
-                tq, tk, s.L, s.H, s.N, s.w, p.rows, p.units, p.score_chunk, p.score_splits, c_log2, nullptr, d_stats_part, p.score_splits, d_lse,
-                d_raw, d_gram_part, d_status);
-            return cudaGetLastError();
-        }
-        e = raise_smem_limit<MB, 1, SPLIT>();
+        e = with_gram ? raise_smem_limit<MB, 3, SPLIT>() : raise_smem_limit<MB, 1, SPLIT>();
         if (e != cudaSuccess) return e;
-        score_tc_kernel<MB, 1, SPLIT><<<ctas(splitsB), kScoreThreads, smem, st>>>(tq, tk, s.L, s.H, s.N, s.w, p.rows, p.units,
-                                                                                 p.score_chunk, splitsB, c_log2, nullptr, d_stats_part,
-                                                                                 p.score_splits, d_lse, d_raw, nullptr, d_status);
+        e = launch(with_gram ? score_tc_kernel<MB, 3, SPLIT> : score_tc_kernel<MB, 1, SPLIT>, with_gram ? p.score_splits : splitsB,
+                   with_gram ? kGramThreads : kScoreThreads, nullptr, d_stats_part, p.score_splits, d_lse, d_raw,
+                   with_gram ? d_gram_part : nullptr);
     }
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_scores_tc(const Plan &p, const void *dQw, const void *dK, const UnitAddr &addr, float scale,
                              const float *d_lse, float *d_stats_part, float *d_raw, float *d_gram_part,
-                             int phases, uint32_t *d_status, TmapCache *cache, Profiler *prof, cudaStream_t st) {
+                             int phases, bool chained, uint32_t *d_status, TmapCache *cache, Profiler *prof, cudaStream_t st) {
     CUtensorMap tq, tk;
     cudaError_t e = cached_scorer_maps(cache, p, addr, dQw, dK, kTile, &tq, &tk);
     if (e != cudaSuccess) return e;
     const float c_log2 = scale * 1.4426950408889634f;
     const int MB = (p.rows + 127) / 128;
-    if (p.rows <= 32) return launch_scores_tc_mb<1, 4>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
-    if (p.rows <= 64) return launch_scores_tc_mb<1, 2>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
+    if (p.rows <= 32) return launch_scores_tc_mb<1, 4>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, chained, d_status, prof, st);
+    if (p.rows <= 64) return launch_scores_tc_mb<1, 2>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, chained, d_status, prof, st);
     switch (MB) {
-        case 1: return launch_scores_tc_mb<1, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
-        case 2: return launch_scores_tc_mb<2, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
-        case 3: return launch_scores_tc_mb<3, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
-        default: return launch_scores_tc_mb<4, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
+        case 1: return launch_scores_tc_mb<1, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, chained, d_status, prof, st);
+        case 2: return launch_scores_tc_mb<2, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, chained, d_status, prof, st);
+        case 3: return launch_scores_tc_mb<3, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, chained, d_status, prof, st);
+        default: return launch_scores_tc_mb<4, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, chained, d_status, prof, st);
     }
 }
 
