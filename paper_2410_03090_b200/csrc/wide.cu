@@ -46,6 +46,7 @@ __global__ void __launch_bounds__(256) wide_colsum_kernel(const __nv_bfloat16 *_
     const int per = (N + kColChunks - 1) / kColChunks;
     const int t0 = c * per, t1 = min(N, t0 + per);
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    chain_wait();
     if (f < D) {
         for (int t = t0 + warp; t < t1; t += 32) {
             uint2 x[4];
@@ -76,6 +77,7 @@ __global__ void __launch_bounds__(256) wide_colsum_reduce_kernel(const double *_
                                                                 double *__restrict__ s) {
     const int f = blockIdx.x * 256 + threadIdx.x;
     if (f >= D) return;
+    chain_wait();
     double acc = 0.0;
     for (int c = 0; c < kColChunks; ++c) acc += part[(size_t)c * D + f];
     s[f] = acc;
@@ -146,6 +148,7 @@ gram_wide_kernel(const __grid_constant__ CUtensorMap tmap, int N, int nblk, int 
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = T.tmem_base;
+    chain_wait();
 
     if (warp == 4) {
         if (lane == 0) {
@@ -247,6 +250,7 @@ __global__ void __launch_bounds__(256) wide_assemble_kernel(const float *__restr
                                                             int nblk, int Dt, int N, int center,
                                                             const double *__restrict__ v, float *__restrict__ C) {
     __shared__ float tile[32][33];
+    chain_wait();
     int I = 0, J = 0;
     {
         int rem = blockIdx.x;
@@ -294,6 +298,7 @@ __global__ void __launch_bounds__(256) wide_rowdot_kernel(const __nv_bfloat16 *_
                                                          const double *__restrict__ s, double *__restrict__ g) {
     const int lane = threadIdx.x & 31, row = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (row > N) return;                                  // warp N computes mean . mean
+    chain_wait();
     double acc = 0.0;
     for (int f = lane; f < D; f += 32) {
         const double m = s[f] / (double)N;
@@ -340,7 +345,7 @@ __global__ void __launch_bounds__(kTriThreads, 1) tridiag_wide_kernel(float *__r
                                                                      unsigned *bar, int *kry, const double *lam, int k_wanted,
                                                                      uint32_t *__restrict__ status) {
     extern __shared__ float sm[];
-    if (kry && krylov_done(kry, lam, k_wanted)) {          // the same answer in every CTA
+    if (kry && krylov_done(kry, lam, k_wanted)) {          // the same answer in every warp
         if (blockIdx.x == 0 && threadIdx.x == 0) kry[2] = 1;
         return;
     }
@@ -504,6 +509,7 @@ __device__ int sturm_count_wide(const double *__restrict__ a, const double *__re
 __global__ void __launch_bounds__(kSturmThreads) sturm_wide_kernel(const double *__restrict__ a, const double *__restrict__ e,
                                                                   int D, int k, int max_iters, const int *kry, double *__restrict__ lam_out,
                                                                   uint32_t *__restrict__ status) {
+    chain_wait();
     if (kry && kry[2]) return;                             // set by the launch before this one
     __shared__ double redlo[kSturmThreads / 32], redhi[kSturmThreads / 32], redtr[kSturmThreads / 32];
     __shared__ int redc[kSturmThreads / 32];
@@ -574,6 +580,7 @@ __global__ void __launch_bounds__(32) wide_entropy_kernel(const double *__restri
                                                          float *__restrict__ H_out, float *__restrict__ erank_out,
                                                          double *__restrict__ spectrum) {
     const int lane = threadIdx.x;
+    chain_wait();
     double denom = 0.0;
     if (norm == 0) {
         for (int i = lane; i < kf; i += 32) denom += fmax(lam[i], 0.0);
@@ -671,8 +678,10 @@ cudaError_t launch_entropy_wide(const void *d_X, int64_t sN, int N, int D, const
     if (err != cudaSuccess) return err;
     {
         ProfScope ps(prof, kSlotWideGram, st);
-        wide_colsum_kernel<<<dim3((D + 127) / 128, kColChunks), 256, 0, st>>>(X, sN, N, D, colpart);
-        wide_colsum_reduce_kernel<<<(D + 255) / 256, 256, 0, st>>>(colpart, D, s);
+        err = launch_kernel(wide_colsum_kernel, LaunchShape{dim3((D + 127) / 128, kColChunks), 256, 0, 1, false}, st, X, sN, N, D, colpart);
+        if (err != cudaSuccess) return err;
+        err = launch_kernel(wide_colsum_reduce_kernel, LaunchShape{dim3((D + 255) / 256), 256, 0, 1, true}, st, colpart, D, s);
+        if (err != cudaSuccess) return err;
         CUtensorMap tmap;
         uint64_t dims[3] = {(uint64_t)D, (uint64_t)N, 1};
         uint64_t str[2] = {(uint64_t)sN * 2, (uint64_t)sN * 2 * (uint64_t)N};
@@ -682,23 +691,25 @@ cudaError_t launch_entropy_wide(const void *d_X, int64_t sN, int N, int D, const
         if (w.dual) {
             err = cudaFuncSetAttribute(gram_wide_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmem);
             if (err != cudaSuccess) return err;
-            gram_wide_kernel<true><<<dim3(w.pairs, w.chunks), kWThreads, kWSmem, st>>>(tmap, D, w.nblk, w.chunk, part, d_status);
-            wide_rowdot_kernel<<<(N + 1 + 7) / 8, 256, 0, st>>>(X, sN, N, D, w.Dt, s, g);
+            err = launch_kernel(gram_wide_kernel<true>, LaunchShape{dim3(w.pairs, w.chunks), kWThreads, kWSmem, 1, true}, st, tmap, D, w.nblk,
+                                w.chunk, part, d_status);
+            if (err != cudaSuccess) return err;
+            err = launch_kernel(wide_rowdot_kernel, LaunchShape{dim3((N + 1 + 7) / 8), 256, 0, 1, true}, st, X, sN, N, D, w.Dt, s, g);
         } else {
             err = cudaFuncSetAttribute(gram_wide_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmem);
             if (err != cudaSuccess) return err;
-            gram_wide_kernel<false><<<dim3(w.pairs, w.chunks), kWThreads, kWSmem, st>>>(tmap, N, w.nblk, w.chunk, part, d_status);
+            err = launch_kernel(gram_wide_kernel<false>, LaunchShape{dim3(w.pairs, w.chunks), kWThreads, kWSmem, 1, true}, st, tmap, N, w.nblk,
+                                w.chunk, part, d_status);
         }
+        if (err != cudaSuccess) return err;
     }
     {
         ProfScope ps(prof, kSlotWideAssemble, st);
         const unsigned tiles = (kWBlock / 32) * (kWBlock / 32);
-        if (w.dual)
-            wide_assemble_kernel<true><<<dim3(w.pairs, tiles), 256, 0, st>>>(part, w.pairs, w.chunks, w.nblk, w.Dt, N, ep.center, g, C);
-        else
-            wide_assemble_kernel<false><<<dim3(w.pairs, tiles), 256, 0, st>>>(part, w.pairs, w.chunks, w.nblk, w.Dt, N, ep.center, s, C);
+        err = launch_kernel(w.dual ? wide_assemble_kernel<true> : wide_assemble_kernel<false>,
+                            LaunchShape{dim3(w.pairs, tiles), 256, 0, 1, true}, st, part, w.pairs, w.chunks, w.nblk, w.Dt, N, (int)ep.center,
+                            w.dual ? g : s, C);
     }
-    err = cudaGetLastError();
     if (err != cudaSuccess) return err;
     const int k = ep.k_trunc < D ? ep.k_trunc : D;                // entries of the outputs
     const int kf = k < w.Dt ? k : w.Dt;                           // eigenvalues the matrix can have; the rest are zero
@@ -716,6 +727,7 @@ cudaError_t launch_entropy_wide(const void *d_X, int64_t sN, int N, int D, const
         b.H = (float *)(scratch + w.off_H);
         b.G = (double *)(scratch + w.off_G);
         b.T = (double *)(scratch + w.off_T);
+        b.Trev = (double *)part;              // the Gram partials have been consumed; they take 750 KB at least, this 350 at most
         b.lam = lam;
         b.state = kry = (int *)(scratch + w.off_state);
         b.bar = bar + 8;
@@ -745,10 +757,12 @@ cudaError_t launch_entropy_wide(const void *d_X, int64_t sN, int N, int D, const
     }
     {
         ProfScope ps(prof, kSlotWideSturm, st);
-        sturm_wide_kernel<<<kf, kSturmThreads, 0, st>>>(a, e, w.Dt, kf, ep.max_iters, kry, lam, d_status);
-        wide_entropy_kernel<<<1, 32, 0, st>>>(lam, k, kf, ep.norm, d_entropy, d_erank, d_spectrum);
+        err = launch_kernel(sturm_wide_kernel, LaunchShape{dim3(kf), kSturmThreads, 0, 1, true}, st, a, e, w.Dt, kf, (int)ep.max_iters, kry, lam,
+                            d_status);
+        if (err != cudaSuccess) return err;
+        err = launch_kernel(wide_entropy_kernel, LaunchShape{dim3(1), 32, 0, 1, true}, st, lam, k, kf, (int)ep.norm, d_entropy, d_erank, d_spectrum);
     }
-    return cudaGetLastError();
+    return err;
 }
 
 }  // namespace uncomp

@@ -17,6 +17,7 @@ struct KrylovBuffers {
     float *H;            // [steps][1024] their sums
     double *G;           // [1024] Gram matrix of the new block
     double *T;           // [32 steps + 32][kKryBand] projected matrix, column c: entry (c - o, c) at [c][o], o <= 32
+    double *Trev;        // [the same] row r: entry (r, r + o) at [r][o]; read backwards, the columns of T reversed
     double *lam;         // [k + 1] eigenvalues descending, then the trace
     int *state;          // [0] steps in Q, [1] broken, [2] all settled (set by the reduction's kernel); [8 ..] settled, each
     unsigned *bar;       // grid barrier counters, one per launch, zero at the start
@@ -32,15 +33,15 @@ constexpr double kKryMaxRatio = 4096.0;
 
 __device__ __forceinline__ bool krylov_too_graded(const double *lam, int k) { return !(lam[0] <= kKryMaxRatio * lam[k - 1]); }
 
-// true when all k eigenvalues have converged (every kernel behind the first asks this before it does anything)
+// true when all k eigenvalues have converged (every kernel behind the first asks this before it does anything).  Called by
+// whole warps, the answer is the same in all of them.
 __device__ __forceinline__ bool krylov_done(const int *state, const double *lam, int k) {
-    if (state[1] || krylov_too_graded(lam, k)) return false;
-    for (int i = 0; i < k; ++i)
-        if (!state[8 + i]) return false;
+    const int lane = threadIdx.x & 31;
+    bool ok = !state[1] && !krylov_too_graded(lam, k);
+    for (int i = lane; i < k; i += 32) ok = ok && state[8 + i];
     // a block of 32 start vectors shows an eigenvalue at most 32 times: a cluster of that size may be larger
-    for (int i = 0; i + kKryBlock <= k - 1; ++i)
-        if (lam[i] - lam[i + kKryBlock - 1] <= 1e-6 * lam[0]) return false;
-    return true;
+    for (int i = lane; i + kKryBlock <= k - 1; i += 32) ok = ok && lam[i] - lam[i + kKryBlock - 1] > 1e-6 * lam[0];
+    return __all_sync(0xffffffffu, ok);
 }
 
 // `ctas`: how many CTAs of the Lanczos kernel the device holds at once (they wait for one another, n / 32 of them)

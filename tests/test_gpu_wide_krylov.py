@@ -82,6 +82,28 @@ def test_one_dominating_direction_leaves_the_others_exact(N, D, strength, k):
     assert abs(float(ent[0]) - H) <= 1e-5
 
 
+@pytest.mark.parametrize("rank,noise,k", [(50, 0.1, 32), (50, 0.003, 32), (33, 0.02, 33), (256, 0.02, 64)])
+def test_blocks_that_lose_most_of_their_norm(rank, noise, k):
+    """A few strong directions over noise of 1e-2 to 1e-5 of their variance: once they are in the basis, a block keeps so
+    little that its Gram matrix cannot be had by subtraction (a third pass), and what is left is close to rounding.  Bound:
+    m 2^-24 of every eigenvalue for the tensor cores' sums (see above) and 4e-6 for the reduction in fp32."""
+    from paper_2410_03090_b200 import binding as ub
+    N, D = 3000, 1024
+    g = torch.Generator(device="cuda").manual_seed(rank)
+    W = torch.randn(rank, D, generator=g, device="cuda") * torch.linspace(2, 0.5, rank, device="cuda")[:, None]
+    X = torch.randn(N, rank, generator=g, device="cuda") @ W + noise * torch.randn(N, D, generator=g, device="cuda")
+    X = X.to(torch.bfloat16)[None]
+    ctx = ub.Context(ub.make_shape(1, 1, 1, 1, 256, 128, 8, "bf16"))
+    ent, _, spec = ub.uncomp_entropy_wide(ctx, X, k, spectrum=True)
+    torch.cuda.synchronize()
+    assert ub.uncomp_status(ctx) == 0
+    H, _, lam = oracle.entropy_wide(X[0].double().cpu().numpy(), k, True, 0, return_spectrum=True)
+    lam = lam[:k]
+    rel = np.abs(spec[0].cpu().numpy() - lam) / lam
+    assert (rel <= 600 / 16 * 2.0 ** -24 + 4e-6 * max(1.0, lam[0] / lam[-1] / 500)).all(), (rel.max(), lam[0] / lam[-1])
+    assert abs(float(ent[0]) - H) <= 1e-5
+
+
 def test_few_rounds_are_reported():
     from paper_2410_03090_b200 import binding as ub
     X = tw._matrix(1, 1300, 512, 60, 0.1, seed=1)
