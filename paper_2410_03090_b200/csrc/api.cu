@@ -309,7 +309,7 @@ int uncomp_entropy(uncomp_ctx *ctx, const void *d_K, uncomp_strides sK, const un
     {
         ProfScope ps(ctx->prof, kSlotEigen, st);
         if (tensor_path)
-            e = launch_eigen_f32(p, partials, parts, *params, d_entropy, d_erank, d_spectrum, d_status, st);
+            e = launch_eigen_f32(p, partials, parts, d_Qw != nullptr, *params, d_entropy, d_erank, d_spectrum, d_status, st);
         else
             e = launch_eigen_entropy(p, partials, *params, d_entropy, d_erank, d_spectrum, d_status, st);
     }
@@ -463,7 +463,7 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
         if (e != cudaSuccess) return cuda_fail(ctx, e);
         {
             ProfScope ps(ctx->prof, kSlotEigen, st);
-            e = launch_eigen_f32(p, partials, p.score_splits, *eparams, d_entropy, d_erank, nullptr, d_status, st);
+            e = launch_eigen_f32(p, partials, p.score_splits, true, *eparams, d_entropy, d_erank, nullptr, d_status, st);
         }
         if (e != cudaSuccess) return cuda_fail(ctx, e);
         {
@@ -502,7 +502,7 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
         if (e != cudaSuccess) return cuda_fail(ctx, e);
         {
             ProfScope ps(ctx->prof, kSlotEigen, st);
-            e = launch_eigen_f32(p, partials, p.score_splits, *eparams, d_entropy, d_erank, nullptr, d_status, st);
+            e = launch_eigen_f32(p, partials, p.score_splits, true, *eparams, d_entropy, d_erank, nullptr, d_status, st);
         }
         if (e == cudaSuccess)
             e = launch_scores_tc(p, d_Qw, d_K, addr, sc, nullptr, stats_part, raw, nullptr, kScorePhaseColsum, false, d_status,

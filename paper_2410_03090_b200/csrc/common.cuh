@@ -34,6 +34,12 @@ struct Plan {
 
 Plan make_plan(const uncomp_shape &s);
 
+// Place of the 16-byte vector (row r, columns 4 c4 .. 4 c4 + 3) in a Gram partial of the scorer: the vectors of four rows lie
+// side by side, so that a warp that holds a row per lane (as TMEM hands it out) stores 64-byte pieces, eight cache lines an
+// instruction, and a warp of the eigenvalue kernel reads four rows x 128 bytes as one run.  Row by row a store touched 32
+// lines, and the 128 x 128 block took 4,000 cycles of an item whose tiles take 25,000.
+__host__ __device__ __forceinline__ int gram_vec4(int r, int c4) { return ((r >> 2) * (kD / 4) + c4) * 4 + (r & 3); }
+
 struct UnitAddr {
     int L, H;
     int64_t sB, sL, sH, sN;
@@ -190,7 +196,8 @@ cudaError_t launch_eigen_entropy(const Plan &p, const void *d_partials, const un
 // The partials are scratch of the eigenvalue stage: overwritten.
 cudaError_t launch_eigen_tail(int units, float *d_partials, int partials_per_unit, const uncomp_entropy_params &ep,
                               float *d_entropy, float *d_erank, double *d_spectrum, uint32_t *d_status, cudaStream_t st);
-cudaError_t launch_eigen_f32(const Plan &p, void *d_partials, int partials_per_unit, const uncomp_entropy_params &ep,
+// tiled: the partials' matrices are laid out by gram_vec4 (the scorer's), else row by row
+cudaError_t launch_eigen_f32(const Plan &p, void *d_partials, int partials_per_unit, bool tiled, const uncomp_entropy_params &ep,
                              float *d_entropy, float *d_erank, double *d_spectrum, uint32_t *d_status, cudaStream_t st);
 cudaError_t launch_gram_reduce(const Plan &p, const void *d_partials, double *d_out, cudaStream_t st);
 int check_budget_params(const uncomp_shape &s, const uncomp_budget_params &bp);

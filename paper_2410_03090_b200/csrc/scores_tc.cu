@@ -568,10 +568,10 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
                     tc::tc_fence_before();
                     __syncwarp();
                     if (lane == 0) tc::mbar_arrive(tc::smem_u32(&T.gdrained));
-                    float4 *dst = reinterpret_cast<float4 *>(out + (size_t)lane_row * kD + cb * 32);
+                    float4 *dst = reinterpret_cast<float4 *>(out) + gram_vec4(lane_row, cb * 8);
 #pragma unroll
                     for (int q4 = 0; q4 < 8; ++q4)
-                        dst[q4] = make_float4(__uint_as_float(r[4 * q4]), __uint_as_float(r[4 * q4 + 1]),
+                        dst[4 * q4] = make_float4(__uint_as_float(r[4 * q4]), __uint_as_float(r[4 * q4 + 1]),
                                               __uint_as_float(r[4 * q4 + 2]), __uint_as_float(r[4 * q4 + 3]));
                 }
             }
