@@ -14,26 +14,29 @@
 // One CTA per SM works through its share of the (unit, token chunk) items.  The TMA producer runs ahead into the next item,
 // so a CTA's pipeline fills once and not once per item (a CTA per item spent 8,000 of 38,000 cycles on a 3712-token unit
 // before its first tile arrived and 6,000 after its last).
-// Warps 0-15 softmax in two groups of eight that take alternate token tiles (so the four
+// Warps 0-15 softmax in two groups of eight that take alternate 128-row blocks or token tiles (so the four
 // warps of an SM sub-partition are in different phases: while one group waits for its accumulator, the
 // other keeps the exponential unit busy); inside a group warp % 4 selects the TMEM lane quarter and bit 2
 // of the warp index the 64-column half of an accumulator.  Warp 16 is the TMA producer, warp 17 allocates
 // TMEM and issues the MMAs: one ELECTED lane (elect.sync lets the compiler keep descriptors in uniform registers; with
 // `lane == 0` an MMA took 130 cycles to issue, twice what the tensor pipe needs for it, and paced the kernel).  The
-// 128-column accumulators form one ring that both groups draw from in order
-// (block = one 128-row block of one tile): four buffers in modes 0 and 1, three in modes 2 and 3.
+// 128-column accumulators are four buffers in modes 0 and 1, two in modes 2 and 3.
 // Mode 2 of the kernel is pass A with the Gram stage folded in: the K tile that is in shared memory for
 // Qw K^T is also the MN-major operand of G += K_tile^T K_tile, so the entropy stage costs no second sweep
-// over K.  The Gram block takes the last 128 TMEM columns; the column sums s = K^T 1 are added up by two
-// extra warps (18, 19) that read the tile from shared memory as well (from global memory, 3,000 cycles of latency per
-// tile paced the kernel).
+// over K.  The column sums s = K^T 1 come out of the same MMAs, as 16 more columns whose operand is ones.  (Two warps that
+// read the tile from shared memory once more took a sixth of what the MMAs and TMA leave of its bandwidth: 256 units of 8192
+// tokens 128.5 us, now 123; 1024 of 3712 205, now 190; of 32768 2052, now 1995; 256 of 32768 with two row blocks 833, now
+// 803.  From global memory, 3,000 cycles of latency per tile paced the kernel.)  The errors are those of the warps' fp32 sums:
+// entropies of keys with means of 0, 1, 10 and 100 times their spread are as far from 64 bits as before.
 // Mode 3 is pass B with the Gram stage folded in the same way, for callers who bring the row normalisers (their
 // prefill attention kernel's log-sum-exp): entropy stage and scores from ONE sweep over K.
-// What bounds it.  In single passes the exponential unit, 66 % (mode 2) and 76 % (mode 1) busy, and the queue in front of it
-// (two row blocks need 2,048 cycles of it per tile).  Repeated for more than half a second, power: 985 W, and the clock falls
-// from 1.965 to 1.75 (8192 and 131072 tokens), 1.57 (32768) or 1.40 GHz (4 x 32768); a micro-benchmark of the same MMAs, TMA
-// loads and exponentials without any hand-over takes 1,180 cycles per tile of one row block, 0.95 us at such a clock, and
-// modes 2 and 3 take about 1.1 us.
+// What bounds it.  The clock that power allows, 1.6 to 1.7 GHz from the first pass on (four row blocks 1.83), repeated for more
+// than half a second 1.75 (8192 and 131072 tokens), 1.57 (32768) or 1.40 GHz (4 x 32768) at 985 W; and at that clock, with two
+// row blocks or more, the exponential unit, 75 % (mode 2) and 80 % (mode 1) busy: 2,700 and 2,540 cycles per tile of two row
+// blocks, which need 2,048 of it.  The exponential loops alone keep it 97 % busy with two warps per scheduler.  Letting the
+// groups take turns on it (named barriers) was slower (1,600 cycles per block against 1,300), three accumulators beside the
+// Gram block and blocks by tile in pass A were the same.  One row block: shared memory (the MMAs read 128 bytes per cycle, which
+// is all it has) and, in mode 1, HBM (5.4 TB/s).
 // Every wait is bounded; a timeout raises UNCOMP_STATUS_TIMEOUT and the CTA drains and exits.
 #include "tc_common.cuh"
 
@@ -45,22 +48,63 @@ constexpr int kHalfBytes = 128 * 128;            // 64 features x 128 rows/token
 constexpr int kBlockBytes = 2 * kHalfBytes;      // one K tile or one block of 128 query rows
 constexpr int kNB = 4;                           // accumulator buffers (x 128 TMEM columns = all 512)
 constexpr int kSoftThreads = 512;
-constexpr int kScoreThreads = kSoftThreads + 64;  // modes 0 and 1
-constexpr int kGramThreads = kScoreThreads + 64;  // mode 2: two more warps for the column sums
+constexpr int kScoreThreads = kSoftThreads + 64;
+// The compiler may use 96 registers, as if there were two more warps.  With the 112 that 576 threads leave it puts the
+// loads of the normalisers elsewhere: column sums of 1024 units of 32768 tokens 1865 us against 1600 (88 registers 1763, 80
+// 1823).
+constexpr int kBoundThreads = kScoreThreads + 64;
 constexpr int kMaxStages = 4;
 
 struct ScoreTail {
     uint64_t full[kMaxStages], empty[kMaxStages], qfull[2], qempty[2], tfull[2 * kNB], tempty[kNB], gfull, gdrained;
     uint32_t tmem_base;
-    float sum_xch[2][kD];  // hand-over of the second column-sum warp (modes 2 and 3)
 };
 
 __host__ __device__ constexpr int score_stages(int MB) { return MB <= 2 ? 4 : (MB == 3 ? 3 : 2); }
 __host__ __device__ constexpr int query_buffers(int MB) { return MB == 1 ? 2 : 1; }
-__host__ __device__ constexpr int score_smem(int MB) {
-    return 1024 + query_buffers(MB) * MB * kBlockBytes + score_stages(MB) * kBlockBytes + 2 * MB * 128 * 4 + 2 * 4 * 128 * 4 +
-           4 * MB * 128 * 8 + (int)sizeof(ScoreTail);
+
+// Places in shared memory, in halves (16 KB: 64 features of a K tile or of 128 query rows).  Without the Gram stage: queries, then
+// stages.  With it (modes 2 and 3) half kOnesHalf is filled with ones, and the halves of stage s lie at kOnesHalf - 2 x and
+// kOnesHalf - x, so that to the tensor core, which finds the 64-feature regions of an MN-major operand at equal distances, the
+// ones are features 128 .. of every tile: N = 144 instead of 128 columns give the Gram block and, in the last 16, the column
+// sums.  x = 1, 3, 4, 5 keeps all of them apart; the queries take what is left.
+constexpr int kOnesHalf = 12;
+__host__ __device__ constexpr int stage_x(int s) { return s + 1 + (s != 0); }
+template <bool GRAM> __host__ __device__ constexpr int stage_half(int MB, int s, int h) {
+    return GRAM ? kOnesHalf - (2 - h) * stage_x(s) : 2 * (query_buffers(MB) * MB + s) + h;
 }
+// the i-th half that no stage takes
+__host__ __device__ constexpr int free_half(int MB, int i) {
+    return MB <= 2 ? i + (i > 1) + (i > 2) : (MB == 3 ? i + (i > 3) + (i > 4) : i + (i > 5));
+}
+constexpr bool halves_apart(int MB) {
+    bool taken[kOnesHalf + 1] = {}, ok = true;
+    for (int s = 0; s < score_stages(MB); ++s)
+        for (int h = 0; h < 2; ++h) {
+            const int at = stage_half<true>(MB, s, h);
+            ok = ok && at >= 0 && at < kOnesHalf && !taken[at];
+            taken[at] = true;
+        }
+    for (int i = 0; i < 2 * query_buffers(MB) * MB; ++i) {
+        const int at = free_half(MB, i);
+        ok = ok && at >= 0 && at < kOnesHalf && !taken[at];
+        taken[at] = true;
+    }
+    return ok;
+}
+static_assert(halves_apart(1) && halves_apart(2) && halves_apart(3) && halves_apart(4), "every half has one owner");
+template <bool GRAM> __host__ __device__ constexpr int query_half(int MB, int buf, int mb, int h) {
+    return GRAM ? free_half(MB, 2 * (buf * MB + mb) + h) : 2 * (buf * MB + mb) + h;
+}
+__host__ __device__ constexpr int score_halves(int MB, bool gram) {
+    return gram ? kOnesHalf + 1 : 2 * (query_buffers(MB) * MB + score_stages(MB));
+}
+// pass B: normalisers of two units and column sums; pass A: statistics to be merged
+__host__ __device__ constexpr int score_smem(int MB, int mode) {
+    return 1024 + score_halves(MB, mode >= 2) * kHalfBytes + (mode == 1 || mode == 3 ? 2 * MB * 128 * 4 + 2 * 4 * 128 * 4 : 4 * MB * 128 * 8) +
+           (int)sizeof(ScoreTail);
+}
+static_assert(score_smem(4, 2) <= 227 * 1024 && score_smem(4, 0) <= 227 * 1024, "shared memory of one CTA");
 
 __device__ __forceinline__ float ex2(float x) {
     float y;
@@ -69,20 +113,6 @@ __device__ __forceinline__ float ex2(float x) {
 }
 __device__ __forceinline__ void all_soft_barrier() { asm volatile("bar.sync 3, 512;" ::: "memory"); }
 __device__ __forceinline__ void group_barrier(int g) { asm volatile("bar.sync %0, 256;" ::"r"(1 + g) : "memory"); }
-__device__ __forceinline__ void sum_warps_barrier() { asm volatile("bar.sync 4, 64;" ::: "memory"); }
-__device__ __forceinline__ float bf16_lo(uint32_t x) { return __uint_as_float(x << 16); }
-__device__ __forceinline__ float bf16_hi(uint32_t x) { return __uint_as_float(x & 0xffff0000u); }
-__device__ __forceinline__ void add_bf16x8(f32x2 (&acc)[4], const uint4 &x) {
-    acc[0] = add2(acc[0], pack2(bf16_lo(x.x), bf16_hi(x.x)));
-    acc[1] = add2(acc[1], pack2(bf16_lo(x.y), bf16_hi(x.y)));
-    acc[2] = add2(acc[2], pack2(bf16_lo(x.z), bf16_hi(x.z)));
-    acc[3] = add2(acc[3], pack2(bf16_lo(x.w), bf16_hi(x.w)));
-}
-__device__ __forceinline__ uint4 ld_shared16(uint32_t addr) {
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
-    return v;
-}
 __device__ __forceinline__ float max3(float a, float b, float c) {
     float d;
     asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
@@ -191,31 +221,34 @@ __device__ __forceinline__ float row_norm(const float *__restrict__ stats, int p
 // the lanes of a copy take their own part of the tile's tokens.  Pass B takes N = 128 / SPLIT instead of 128.  (Copies of
 // 16 rows were no faster: the keys' bandwidth and the Gram MMAs bound it then.)
 template <int MB, int MODE, int SPLIT>
-__global__ void __launch_bounds__(kGramThreads, 1)
+__global__ void __launch_bounds__(kBoundThreads, 1)
 score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant__ CUtensorMap tmapK, int L, int H,
                 int N, int w, int rows, int units, int chunk, int splits, float c_log2, float *__restrict__ stats_part,
                 const float *__restrict__ stats_in, int stats_splits, const float *__restrict__ lse, float *__restrict__ raw,
                 float *__restrict__ gram_part,
                 uint32_t *__restrict__ status) {
-    constexpr bool PASS_B = MODE == 1 || MODE == 3, GRAM = MODE >= 2;
-    // Accumulator buffers (128 TMEM columns each).  An accumulator holds one 128-row block of one tile; tile n (counted
-    // over everything the CTA does) belongs to softmax group n & 1.  Modes 0 and 1: four buffers, two owned by each group,
-    // which it fills alternately (so each group runs up to two blocks ahead, independent of the other).  Modes 2 and 3:
-    // the Gram block leaves room for three, which form one ring in issue order.
-    constexpr int NB = GRAM ? 3 : kNB;
-    // Modes 2 and 3: "block q is ready" is signalled on barrier q % (2 NB).  A softmax group that waits for the first block
-    // of its next tile may get there before the other group's block q - NB has completed, and with one barrier per
-    // buffer the parity of that unfinished phase could not be told from the one waited for.  The user of barrier
-    // q % (2 NB) before block q is block q - 2 NB, which lies in a tile this group has already consumed (2 NB > MB).
-    // Modes 0 and 1 need no such care: a group only ever waits on its own buffers.
-    constexpr int NF = 2 * NB;
-    // block (tile n, mb) -> buffer, ready barrier and its parity, and the drain phase the MMA thread waits for
+    constexpr bool PASS_B = MODE == 1 || MODE == 3, GRAM = MODE >= 2, RING = MODE != 1;
+    // Accumulator buffers (128 TMEM columns each).  An accumulator holds one 128-row block of one tile; blocks are counted over
+    // everything the CTA does, block (tile n, mb) is number n MB + mb.
+    // RING: the buffers are used in the order of the blocks.  Pass A: blocks go to the two softmax groups in turn, whichever
+    // tile they belong to, so both groups always have one (four buffers without the Gram stage, two beside it: an accumulator is
+    // free again as soon as its values are in registers, a third made no difference).
+    // Pass B: a token's sum takes all blocks of its tile, so tile n belongs to group n & 1.  Mode 1: four buffers, two owned
+    // by each group, which it fills alternately (so each group runs up to two blocks ahead, independent of the other).
+    constexpr int NB = GRAM ? 2 : kNB;
+    // RING: "block q is ready" is signalled on barrier q % NF.  A softmax group that waits for its next block may get
+    // there before the blocks in between have completed, and the parity of an unfinished phase could not be told from the one
+    // waited for: the user of the barrier before, block q - NF, must not lie behind the last block this group has consumed,
+    // which is q - MB - 1 at the earliest.
+    constexpr int NF = RING ? 2 * kNB : kNB;
+    static_assert(!RING || NF > MB, "see above");
+    // block -> buffer, ready barrier and its parity, and the drain phase the MMA thread waits for
     // (-1: the buffer has not been used yet)
-    auto item_buf = [](int n, int mb) { return GRAM ? (n * MB + mb) % NB : 2 * (n & 1) + (((n >> 1) * MB + mb) & 1); };
-    auto item_ready_bar = [](int n, int mb) { return GRAM ? (n * MB + mb) % NF : 2 * (n & 1) + (((n >> 1) * MB + mb) & 1); };
-    auto item_ready_parity = [](int n, int mb) { return GRAM ? ((n * MB + mb) / NF) & 1 : ((((n >> 1) * MB + mb) >> 1) & 1); };
-    auto item_drain_phase = [](int n, int mb) { return GRAM ? (n * MB + mb) / NB - 1 : ((((n >> 1) * MB + mb) >> 1) - 1); };
-    constexpr uint32_t kGramCol = 384;               // TMEM columns of the Gram block (modes 2 and 3)
+    auto item_buf = [](int n, int mb) { return RING ? (n * MB + mb) % NB : 2 * (n & 1) + (((n >> 1) * MB + mb) & 1); };
+    auto item_ready_bar = [](int n, int mb) { return RING ? (n * MB + mb) % NF : 2 * (n & 1) + (((n >> 1) * MB + mb) & 1); };
+    auto item_ready_parity = [](int n, int mb) { return RING ? ((n * MB + mb) / NF) & 1 : ((((n >> 1) * MB + mb) >> 1) & 1); };
+    auto item_drain_phase = [](int n, int mb) { return RING ? (n * MB + mb) / NB - 1 : ((((n >> 1) * MB + mb) >> 1) - 1); };
+    constexpr uint32_t kGramCol = NB * 128;          // TMEM columns of the Gram block (modes 2 and 3): 128 and 16 of column sums
     constexpr int kRows = 128 / SPLIT;               // rows of a copy (pass A), columns of an accumulator (pass B)
     constexpr int NC = 64 / SPLIT;                   // logits a thread takes from an accumulator
     static_assert(kRows >= 32, "a TMEM load has one address per warp: a warp belongs to one copy");
@@ -225,12 +258,17 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
     const uint32_t raw_addr = tc::smem_u32(smem_raw);
     const uint32_t pad = (1024u - (raw_addr & 1023u)) & 1023u;
     unsigned char *smem = smem_raw + pad;
-    const uint32_t q_addr = raw_addr + pad;
-    const uint32_t k_addr = q_addr + QB * MB * kBlockBytes;
-    float *mp = reinterpret_cast<float *>(smem + (QB * MB + S) * kBlockBytes);     // [2][MB * 128], by unit
-    float *colsum = mp + 2 * MB * 128;                                             // [2][4][128]
-    float2 *merge = reinterpret_cast<float2 *>(colsum + 2 * 4 * 128);              // [4][MB * 128]
-    ScoreTail &T = *reinterpret_cast<ScoreTail *>(merge + 4 * MB * 128);
+    const uint32_t base = raw_addr + pad;
+    auto stage_addr = [&](int st, int h) { return base + (uint32_t)(stage_half<GRAM>(MB, st, h) * kHalfBytes); };
+    auto query_addr = [&](int buf, int mb, int h) {
+        const int at = QB == 2 && buf ? query_half<GRAM>(MB, 1, mb, h) : query_half<GRAM>(MB, 0, mb, h);
+        return base + (uint32_t)(at * kHalfBytes);
+    };
+    unsigned char *behind = smem + score_halves(MB, GRAM) * kHalfBytes;
+    float *mp = reinterpret_cast<float *>(behind);                                 // pass B: [2][MB * 128], by unit
+    float *colsum = mp + 2 * MB * 128;                                             // pass B: [2][4][128]
+    float2 *merge = reinterpret_cast<float2 *>(behind);                            // pass A: [4][MB * 128]
+    ScoreTail &T = *reinterpret_cast<ScoreTail *>(behind + (PASS_B ? 2 * MB * 128 * 4 + 2 * 4 * 128 * 4 : 4 * MB * 128 * 8));
 
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int P = N - w;
@@ -246,7 +284,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             tc::mbar_init(tc::smem_u32(&T.full[s]), 1);
-            tc::mbar_init(tc::smem_u32(&T.empty[s]), GRAM ? 3 : 1);     // the MMAs and the two column-sum warps
+            tc::mbar_init(tc::smem_u32(&T.empty[s]), 1);
         }
         for (int q = 0; q < QB; ++q) {
             tc::mbar_init(tc::smem_u32(&T.qfull[q]), 1);
@@ -257,6 +295,11 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
         for (int i = 0; i < 2 * kNB; ++i) tc::mbar_init(tc::smem_u32(&T.tfull[i]), 1);
         for (int i = 0; i < kNB; ++i) tc::mbar_init(tc::smem_u32(&T.tempty[i]), kSoftThreads / 64);   // the 8 warps of one group
         tc::fence_mbar_init();
+    }
+    if (GRAM) {                                        // ones; what the tensor core reads goes through the asynchronous proxy
+        uint4 *ones = reinterpret_cast<uint4 *>(smem + kOnesHalf * kHalfBytes);
+        for (int i = threadIdx.x; i < kHalfBytes / 16; i += kScoreThreads) ones[i] = make_uint4(0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u);
+        tc::fence_proxy_async();
     }
     if (warp == 17) {
         tc::tmem_alloc(tc::smem_u32(&T.tmem_base), 512);
@@ -286,9 +329,9 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
                 tc::mbar_expect_tx(bar, MB * kCopies * (kBlockBytes / SPLIT));
                 for (int mb = 0; mb < MB; ++mb)
                     for (int cp = 0; cp < kCopies; ++cp) {
-                        const uint32_t dst = q_addr + ((useq % QB) * MB + mb) * kBlockBytes + cp * (kHalfBytes / SPLIT);
-                        tc::tma_load_3d(dst, &tmapQ, bar, 0, mb * 128, cur_u);
-                        tc::tma_load_3d(dst + kHalfBytes, &tmapQ, bar, 64, mb * 128, cur_u);
+                        const uint32_t at = cp * (kHalfBytes / SPLIT);
+                        tc::tma_load_3d(query_addr(useq % QB, mb, 0) + at, &tmapQ, bar, 0, mb * 128, cur_u);
+                        tc::tma_load_3d(query_addr(useq % QB, mb, 1) + at, &tmapQ, bar, 64, mb * 128, cur_u);
                     }
                 q_pending = false;
                 ++q_sent;
@@ -320,10 +363,9 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
                         if (!ok) break;
                     }
                     const uint32_t bar = tc::smem_u32(&T.full[s]);
-                    const uint32_t dst = k_addr + s * kBlockBytes;
                     tc::mbar_expect_tx(bar, kBlockBytes);
-                    tc::tma_load_5d(dst, &tmapK, bar, 0, t0 + i * kTile, h, l, b);
-                    tc::tma_load_5d(dst + kHalfBytes, &tmapK, bar, 64, t0 + i * kTile, h, l, b);
+                    tc::tma_load_5d(stage_addr(s, 0), &tmapK, bar, 0, t0 + i * kTile, h, l, b);
+                    tc::tma_load_5d(stage_addr(s, 1), &tmapK, bar, 64, t0 + i * kTile, h, l, b);
                     if (q_pending && q_free()) send_q();
                 }
             }
@@ -340,13 +382,9 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
         if (tc::elect_one()) {
             constexpr uint32_t idesc = tc::idesc_bf16_f32(128, PASS_B ? kRows : 128, 0, 0);
             // descriptors: K-major, 128-byte swizzle, 8-row groups 1024 B apart.  Only the address field
-            // (16-byte units) of the lower half changes: +2 per 16 features inside a 128-byte row, +1024 for
-            // the second 64-feature half.
-            const uint64_t d0 = tc::smem_desc_sw128(q_addr, 16, 1024);
-            const uint32_t dhi = tc::desc_hi(d0), q_lo0 = tc::desc_lo(d0);
-            const uint32_t k_lo0 = tc::desc_lo(tc::smem_desc_sw128(k_addr, 16, 1024));
-            const uint64_t gd = tc::smem_desc_sw128(k_addr, kHalfBytes, 1024);
-            const uint32_t g_lo0 = tc::desc_lo(gd), g_hi = tc::desc_hi(gd);
+            // (16-byte units) of the lower half changes: +2 per 16 features inside a 128-byte row.
+            auto half_desc = [](uint32_t addr) { return tc::desc_lo(tc::smem_desc_sw128(addr, 16, 1024)); };
+            const uint32_t dhi = tc::desc_hi(tc::smem_desc_sw128(base, 16, 1024));
             int n = 0, useq = -1, cur_u = -1, iseq = 0, item_start = 0;
             bool ok = true;
             bool have_tile = false, have_buf = false;   // known of the next tile before this one's Gram MMAs are issued
@@ -358,20 +396,20 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
             constexpr int kLag = MB == 1 ? 0 : 1;
             int g_done = 0;                    // tiles whose Gram MMAs are issued (and whose stage is released)
             auto issue_gram = [&]() {
-                constexpr uint32_t idesc_g = tc::idesc_bf16_f32(128, 128, 1, 1);
+                constexpr uint32_t idesc_g = tc::idesc_bf16_f32(128, 144, 1, 1);
                 const int t = g_done, sg = t % S;
                 if (t == item_start && iseq > 0) {      // the softmax warps have read the item before
                     ok = tc::mbar_wait(tc::smem_u32(&T.gdrained), (iseq - 1) & 1, status);
                     tc::tc_fence_after();
                     if (!ok) return;
                 }
-                const uint32_t g_lo = g_lo0 + (uint32_t)(sg * (kBlockBytes >> 4));
+                const uint32_t g_lo = tc::desc_lo(tc::smem_desc_sw128(stage_addr(sg, 0), (uint32_t)(stage_x(sg) * kHalfBytes), 1024));
 #pragma unroll
                 for (int k = 0; k < kTile / 16; ++k) {
-                    // the same stage read MN-major (feature halves kHalfBytes apart, 8-token groups 1024 B
+                    // the same stage read MN-major (feature halves and the ones equally far apart, 8-token groups 1024 B
                     // apart); 16 tokens further = +128 address units
                     const uint32_t acc = (t > item_start || k > 0) ? 1u : 0u;
-                    tc::mma_f16_ss_lohi(tmem + kGramCol, g_lo + k * 128, g_lo + k * 128, g_hi, idesc_g, acc);
+                    tc::mma_f16_ss_lohi(tmem + kGramCol, g_lo + k * 128, g_lo + k * 128, dhi, idesc_g, acc);
                 }
                 tc::mma_commit(tc::smem_u32(&T.empty[sg]));
                 ++g_done;
@@ -385,13 +423,12 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
                     ok = tc::mbar_wait(tc::smem_u32(&T.qfull[useq % QB]), (useq / QB) & 1, status);
                 }
                 const bool leaves_q = !more || (j + 1) / splits != u;      // the unit's last item of this CTA
-                const uint32_t q_lo = q_lo0 + (uint32_t)((useq % QB) * MB * (kBlockBytes >> 4));
                 item_start = n;
                 for (int i = 0; i < ntiles && ok; ++i, ++n) {
                     const int s = n % S;
                     if (!have_tile) ok = tc::mbar_wait(tc::smem_u32(&T.full[s]), (n / S) & 1, status);
                     if (!ok) break;
-                    const uint32_t k_lo = k_lo0 + (uint32_t)(s * (kBlockBytes >> 4));
+                    const uint32_t k_lo[2] = {half_desc(stage_addr(s, 0)), half_desc(stage_addr(s, 1))};
 #pragma unroll
                     for (int mb = 0; mb < MB; ++mb) {
                         // the block's buffer must have been drained of its previous block
@@ -407,12 +444,12 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
                         if (!ok) break;
                         tc::tc_fence_after();
                         const uint32_t d_tmem = tmem + buf * 128;
-                        const uint32_t qb_lo = q_lo + (uint32_t)(mb * (kBlockBytes >> 4));
+                        const uint32_t q_lo[2] = {half_desc(query_addr(useq % QB, mb, 0)), half_desc(query_addr(useq % QB, mb, 1))};
 #pragma unroll
                         for (int k = 0; k < 8; ++k) {
-                            const uint32_t off = (uint32_t)(k >> 2) * (kHalfBytes >> 4) + (uint32_t)(k & 3) * 2;
-                            if (PASS_B) tc::mma_f16_ss_lohi(d_tmem, k_lo + off, qb_lo + off, dhi, idesc, k > 0);
-                            else tc::mma_f16_ss_lohi(d_tmem, qb_lo + off, k_lo + off, dhi, idesc, k > 0);
+                            const uint32_t kd = k_lo[k >> 2] + (k & 3) * 2, qd = q_lo[k >> 2] + (k & 3) * 2;
+                            if (PASS_B) tc::mma_f16_ss_lohi(d_tmem, kd, qd, dhi, idesc, k > 0);
+                            else tc::mma_f16_ss_lohi(d_tmem, qd, kd, dhi, idesc, k > 0);
                         }
                         tc::mma_commit(tc::smem_u32(&T.tfull[item_ready_bar(n, mb)]));
                     }
@@ -431,55 +468,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
                     while (ok && g_done < n) issue_gram();
                     if (ok) tc::mma_commit(tc::smem_u32(&T.gfull));
                     ++iseq;
-                }
-            }
-        }
-    } else if (warp >= 18) {
-        // ---------------- column sums s = K^T 1 (modes 2 and 3) ----------------
-        // Two warps read every tile from its stage, beside the MMAs, and hand the stage back like the MMA thread does.  A
-        // lane owns one 16-byte chunk (8 features) of the row and one of four row phases; its rows are added in
-        // increasing order, the phases in a fixed order below.
-        if (GRAM) {
-            const int sw = warp - 18, ch = lane & 15, phase = 2 * sw + (lane >> 4);
-            // row phase + 4 q of the swizzled half: chunk c sits at c ^ (row & 7)
-            const uint32_t at0 = k_addr + (uint32_t)(ch >> 3) * kHalfBytes + phase * 128, c8 = ch & 7;
-            const uint32_t even = at0 + ((c8 ^ phase) << 4), odd = at0 + 512 + ((c8 ^ (phase + 4)) << 4);
-            bool ok = true;                            // after a timeout the warp only keeps its barrier
-            int n = 0;
-            for (int j = first; j < last_item; ++j) {
-                const int ntiles = tiles_of(j);
-                f32x2 acc2[4] = {0ull, 0ull, 0ull, 0ull};
-                for (int i = 0; i < ntiles && ok; ++i, ++n) {
-                    const int s = n % S;
-                    ok = tc::mbar_wait(tc::smem_u32(&T.full[s]), (n / S) & 1, status);
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (!ok) break;
-#pragma unroll 1
-                    for (int q = 0; q < 4; ++q) {
-                        uint4 x[8];
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) x[e] = ld_shared16((e & 1 ? odd : even) + s * kBlockBytes + (q * 4 + (e >> 1)) * 1024);
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) add_bf16x8(acc2, x[e]);
-                    }
-                    __syncwarp();
-                    if (lane == 0) tc::mbar_arrive(tc::smem_u32(&T.empty[s]));
-                }
-                float acc[8];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) unpack2(acc2[e], acc[2 * e], acc[2 * e + 1]);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], 16);   // phases 2 sw, 2 sw + 1
-                float *xch = T.sum_xch[j & 1];         // the array of item j - 2 has been read: the barrier of j - 1 is past
-                if (sw == 1 && lane < 16) {
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) xch[ch * 8 + e] = acc[e];
-                }
-                sum_warps_barrier();
-                if (sw == 0 && lane < 16 && ok) {
-                    float *out = gram_part + (size_t)j * (kD * kD + kD) + kD * kD;
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) out[ch * 8 + e] = acc[e] + xch[ch * 8 + e];
                 }
             }
         }
@@ -509,12 +497,13 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
 #pragma unroll
             for (int mb = 0; mb < MB; ++mb) { m_run[mb] = -INFINITY; l_run[mb] = 0.f; }
 
-            for (int i = group ^ (n0 & 1); i < ntiles; i += 2) {    // this group's tiles
+            for (int i = PASS_B ? group ^ (n0 & 1) : 0; i < ntiles; i += PASS_B ? 2 : 1) {    // pass B: this group's tiles
                 const int n = n0 + i, tile_t0 = t0 + i * kTile;
                 const bool masked = tile_t0 + kTile > P;            // uniform over the CTA
                 float acc = 0.f;
 #pragma unroll
                 for (int mb = 0; mb < MB; ++mb) {
+                    if (!PASS_B && ((n * MB + mb) & 1) != group) continue;            // pass A: this group's blocks
                     const int buf = item_buf(n, mb);
                     uint32_t v[NC];
                     if (!dead) {
@@ -562,12 +551,15 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
                     tc::tc_fence_after();
                     const int cb = warp >> 2;
                     float *out = gram_part + (size_t)j * (kD * kD + kD);
-                    uint32_t r[32];
-                    tc::tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + kGramCol + cb * 32, r);
+                    const uint32_t rows_at = tmem + ((uint32_t)(quarter * 32) << 16) + kGramCol;
+                    uint32_t r[32], sum = 0u;
+                    tc::tmem_ld32(rows_at + cb * 32, r);
+                    if (cb == 0) sum = tc::tmem_ld1(rows_at + 128);
                     tc::tmem_ld_wait();
                     tc::tc_fence_before();
                     __syncwarp();
                     if (lane == 0) tc::mbar_arrive(tc::smem_u32(&T.gdrained));
+                    if (cb == 0) out[kD * kD + lane_row] = __uint_as_float(sum);
                     float4 *dst = reinterpret_cast<float4 *>(out) + gram_vec4(lane_row, cb * 8);
 #pragma unroll
                     for (int q4 = 0; q4 < 8; ++q4)
@@ -614,7 +606,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
 template <int MB, int MODE, int SPLIT>
 static cudaError_t raise_smem_limit() {
     static bool done[64] = {};
-    return allow_dynamic_smem((const void *)score_tc_kernel<MB, MODE, SPLIT>, score_smem(MB), done);
+    return allow_dynamic_smem((const void *)score_tc_kernel<MB, MODE, SPLIT>, score_smem(MB, MODE), done);
 }
 
 template <int MB, int SPLIT>
@@ -623,16 +615,15 @@ static cudaError_t launch_scores_tc_mb(const Plan &p, const CUtensorMap &tq, con
                                        float *d_gram_part, int phases, bool chained, uint32_t *d_status, Profiler *prof,
                                        cudaStream_t st) {
     const uncomp_shape &s = p.shape;
-    const int smem = score_smem(MB);
     cudaError_t e = cudaSuccess;
     int dev = 0, sms = kTargetSms;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // one CTA per SM, each with an equal share of the (unit, chunk) items
     auto ctas = [&](int splits) { return (unsigned)min((int64_t)sms, (int64_t)p.units * splits); };
-    auto launch = [&](auto kernel, int splits, int threads, float *stats_out, const float *stats_in, int stats_splits, const float *lse,
+    auto launch = [&](auto kernel, int mode, int splits, float *stats_out, const float *stats_in, int stats_splits, const float *lse,
                       float *raw, float *gram) {
-        return launch_kernel(kernel, LaunchShape{dim3(ctas(splits)), (unsigned)threads, (size_t)smem, 1, chained}, st, tq, tk, s.L, s.H,
+        return launch_kernel(kernel, LaunchShape{dim3(ctas(splits)), kScoreThreads, (size_t)score_smem(MB, mode), 1, chained}, st, tq, tk, s.L, s.H,
                              s.N, s.w, p.rows, p.units, p.score_chunk, splits, c_log2, stats_out, stats_in, stats_splits, lse, raw,
                              gram, d_status);
     };
@@ -640,8 +631,7 @@ static cudaError_t launch_scores_tc_mb(const Plan &p, const CUtensorMap &tq, con
         e = d_gram_part ? raise_smem_limit<MB, 2, SPLIT>() : raise_smem_limit<MB, 0, SPLIT>();
         if (e != cudaSuccess) return e;
         ProfScope ps(prof, d_gram_part ? kSlotGramStats : kSlotScoreStats, st);
-        e = launch(d_gram_part ? score_tc_kernel<MB, 2, SPLIT> : score_tc_kernel<MB, 0, SPLIT>, p.score_splits,
-                   d_gram_part ? kGramThreads : kScoreThreads, d_stats_part, nullptr, 0, nullptr, nullptr, d_gram_part);
+        e = launch(d_gram_part ? score_tc_kernel<MB, 2, SPLIT> : score_tc_kernel<MB, 0, SPLIT>, d_gram_part ? 2 : 0, p.score_splits, d_stats_part, nullptr, 0, nullptr, nullptr, d_gram_part);
         if (e != cudaSuccess) return e;
     }
     if (phases & kScorePhaseColsum) {
@@ -650,8 +640,8 @@ static cudaError_t launch_scores_tc_mb(const Plan &p, const CUtensorMap &tq, con
         const int splitsB = (p.prefix + p.score_chunk - 1) / p.score_chunk;
         e = with_gram ? raise_smem_limit<MB, 3, SPLIT>() : raise_smem_limit<MB, 1, SPLIT>();
         if (e != cudaSuccess) return e;
-        e = launch(with_gram ? score_tc_kernel<MB, 3, SPLIT> : score_tc_kernel<MB, 1, SPLIT>, with_gram ? p.score_splits : splitsB,
-                   with_gram ? kGramThreads : kScoreThreads, nullptr, d_stats_part, p.score_splits, d_lse, d_raw,
+        e = launch(with_gram ? score_tc_kernel<MB, 3, SPLIT> : score_tc_kernel<MB, 1, SPLIT>, with_gram ? 3 : 1,
+                   with_gram ? p.score_splits : splitsB, nullptr, d_stats_part, p.score_splits, d_lse, d_raw,
                    with_gram ? d_gram_part : nullptr);
     }
     return e;
