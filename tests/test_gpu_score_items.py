@@ -48,3 +48,21 @@ def test_items(L, H, G, w, N):
         assert bool((o.scores >= 0).all()) and bool((o.entropy >= 0).all())
         parity.check_scores(wl, K, Qw, o.scores, units)
         parity.check_entropy(wl, K, o.entropy, o.erank, units)
+
+
+@pytest.mark.parametrize("G,w,N", [(4, 8, 700), (1, 64, 641), (4, 32, 1300), (5, 40, 900), (6, 64, 769), (8, 64, 640)])
+def test_column_sums_of_keys_with_a_mean(G, w, N):
+    """Keys whose mean is ten times their spread: the covariance is what the subtraction of the column sums leaves, so the
+    entropy only agrees when the sums come out of the same tiles as the Gram matrix, every feature in its place."""
+    from paper_2410_03090_b200.compress import CompressionPass
+    avg = w + 20
+    wl = replace(synth.WORKLOADS["c2"], L=20, H=2, Hq=2 * G, N=N, w=w, avg_budget=avg, M=1, n_max=avg, seed=7)
+    K, V, Qw = synth.generate(wl, "cuda")
+    K = (K.float() + 10 * torch.linspace(-1, 2, wl.d, device="cuda").roll(G)).to(torch.bfloat16)
+    cp = CompressionPass(wl, "cuda")
+    for out in (lambda: cp.run(K, V, Qw), lambda: cp.run_one_call(K, V, Qw, lse=_lse(wl, K, Qw))):
+        cp.out.entropy.fill_(-1)
+        o = out()
+        torch.cuda.synchronize()
+        assert cp.status() == 0
+        parity.check_entropy(wl, K, o.entropy, o.erank, [0, 17, wl.units - 1])
