@@ -30,10 +30,9 @@ constexpr int kCoarse = 2 * kEigThreads;
 constexpr int n = kD;
 
 struct EigenSmem {
-    double x[n];      // row k of the matrix, zero up to the diagonal
-    double x1[n];     // row k + 1
-    double v[n];      // reflector
-    double p[n];      // beta A v
+    double x[2][n];   // row k + 1 before the update of step k
+    double v[2][n];   // the step's reflector
+    double p[2][n];   // minus the product of the matrix and the reflector
     double part[kEigWarps];
     double sd[n];     // column sums
     double dd[n];
@@ -112,58 +111,78 @@ __device__ __forceinline__ void sturm_count(const double2 *de, const double (&x)
         if (p1[c] == 0.0) count[c] = sturm_count_robust(de, x[c]);
 }
 
-// Row of the matrix to shared memory by the 16 lanes that hold it, zero up to column `upto`.
-template <int J>
-__device__ __forceinline__ void publish_row(const double (&row)[8], double *dst, int t, int upto) {
+__device__ __forceinline__ double sum16(double v) {   // over the 16 lanes that share a row
 #pragma unroll
-    for (int j = J; j < 4; ++j) {
-        const int c = 32 * j + 2 * t;
-        double a = row[2 * j], b = row[2 * j + 1];
-        if (j <= J + 1) {                              // groups that can hold columns up to k + 1
-            if (c <= upto) a = 0.0;
-            if (c + 1 <= upto) b = 0.0;
-        }
-        *reinterpret_cast<double2 *>(dst + c) = make_double2(a, b);
-    }
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
-// ... and its diagonal entry
+
+// 8 columns of a row vector, 32 (q / 2) + 2 t + q % 2, to shared memory
 template <int J>
-__device__ __forceinline__ void publish_diagonal(const double (&row)[8], double *dst, int t, int k) {
+__device__ __forceinline__ void publish(const double (&row)[8], double *dst, int t) {
 #pragma unroll
-    for (int j = J; j < 4 && j <= J + 1; ++j) {
-        if (32 * j + 2 * t == k) *dst = row[2 * j];
-        if (32 * j + 2 * t + 1 == k) *dst = row[2 * j + 1];
-    }
+    for (int j = J; j < 4; ++j) *reinterpret_cast<double2 *>(dst + 32 * j + 2 * t) = make_double2(row[2 * j], row[2 * j + 1]);
 }
+
+// What a thread carries from step to step: the pending rank-2 update (v and -w for its columns and for its rows) and the row x
+// the next reflector is made of, zero up to the diagonal.
+struct Carry {
+    double vc[8], wc[8], xc[8], vr[8], wr[8];
+    double x0;         // entry k + 1 of x
+};
 
 // Householder steps k = 16 KA .. 16 KA + 15 (stopping at n - 3); row groups (16 rows) below KA and column groups (32
 // columns) below J are done.
 template <int KA>
-__device__ __forceinline__ void householder_block(double (&A)[8][8], EigenSmem &S, int lane, int warp) {
-    constexpr int J = KA >> 1, KN = KA < 7 ? KA + 1 : 7;
+__device__ __forceinline__ void householder_block(double (&A)[8][8], Carry &R, EigenSmem &S, int lane, int warp) {
+    constexpr int J = KA >> 1, JN = J < 3 ? J + 1 : 3, KN = KA < 7 ? KA + 1 : 7;
+    constexpr bool kOdd = (KA & 1) != 0 && KA < 7;     // the block's end is also the end of a column group
     const int i = 2 * warp + (lane >> 4), t = lane & 15;
-    const int mine = i + 16 * (t >> 1);                // the row this lane finishes: 2 lanes share it
 #pragma unroll 1
     for (int kt = 0; kt < 16; ++kt) {
         const int k = 16 * KA + kt;
         if (KA == 7 && k > n - 3) break;
-        // ---- norm of x; y = A x meanwhile ----
-        const double x0 = S.x[k + 1];
-        double sig;
-        {
-            const double2 a = *reinterpret_cast<const double2 *>(S.x + 4 * lane), b = *reinterpret_cast<const double2 *>(S.x + 4 * lane + 2);
-            sig = fma(a.x, a.x, a.y * a.y) + fma(b.x, b.x, b.y * b.y);
-        }
+        const bool end = KA < 7 && kt == 15;
+        // ---- norm of x; meanwhile the pending update of step k - 1 and A x ----
+        double sq[2] = {R.xc[2 * J] * R.xc[2 * J], R.xc[2 * J + 1] * R.xc[2 * J + 1]};
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sig += __shfl_xor_sync(0xffffffffu, sig, o);
+        for (int q = 2 * J + 2; q < 8; ++q) sq[q & 1] = fma(R.xc[q], R.xc[q], sq[q & 1]);
+        const double sig = sum16(sq[0] + sq[1]);
         double y[8];
 #pragma unroll
         for (int a = 0; a < 8; ++a) y[a] = 0.0;
 #pragma unroll
-        for (int j = J; j < 4; ++j) {
-            const double2 x = *reinterpret_cast<const double2 *>(S.x + 32 * j + 2 * t);
+        for (int a = KA; a < 8; ++a) {
 #pragma unroll
-            for (int a = KA; a < 8; ++a) y[a] = fma(A[a][2 * j], x.x, fma(A[a][2 * j + 1], x.y, y[a]));
+            for (int q = 2 * J; q < 8; ++q) A[a][q] = fma(R.vr[a], R.wc[q], fma(R.wr[a], R.vc[q], A[a][q]));
+#pragma unroll
+            for (int q = 2 * J; q < 8; ++q) y[a] = fma(A[a][q], R.xc[q], y[a]);
+        }
+        // ---- -p = -beta A v, v = x - alpha e_{k+1}: the product starts from x, what alpha adds sits in one group ----
+        double *xs = S.x[k & 1], *ps = S.p[k & 1], *vs = S.v[k & 1];
+        const bool flat = !(sig > 1e-290);             // the row is reduced already: beta = 0
+        const double root = sqrt_newton(sig);
+        const double minus_alpha = flat ? -R.x0 : (R.x0 >= 0.0 ? root : -root);
+        const double minus_beta = flat ? 0.0 : -recip_newton(fma(fabs(R.x0), root, sig));         // -2 / (v^T v)
+        const double vk = R.x0 + minus_alpha;          // v_{k+1}
+        if (threadIdx.x == 0) S.ee[k] = -minus_alpha;
+        if (kOdd && end) {                             // column k + 1 is the first of the next group
+            const double d0 = t == 0 ? minus_alpha : 0.0;
+#pragma unroll
+            for (int a = KA; a < 8; ++a) y[a] = fma(A[a][2 * JN], d0, y[a]);
+            R.xc[2 * JN] += d0;
+        } else {
+            const int at = k + 1 - 32 * J - 2 * t;
+            const double d0 = at == 0 ? minus_alpha : 0.0, d1 = at == 1 ? minus_alpha : 0.0;
+#pragma unroll
+            for (int a = KA; a < 8; ++a) y[a] = fma(A[a][2 * J], d0, fma(A[a][2 * J + 1], d1, y[a]));
+            R.xc[2 * J] += d0;
+            R.xc[2 * J + 1] += d1;
+        }
+        if (i == ((k + 1) & 15)) {                     // 16 lanes of one warp
+            if (end) publish<J>(A[KN], xs, t);
+            else publish<J>(A[KA], xs, t);
+            publish<J>(R.xc, vs, t);
         }
         // over the 16 lanes of a row: three transposing levels and a plain one; lane t ends up with row group t / 2
         const bool up8 = (t & 8) != 0, up4 = (t & 4) != 0, up2 = (t & 2) != 0;
@@ -180,60 +199,50 @@ __device__ __forceinline__ void householder_block(double (&A)[8][8], EigenSmem &
         }
         double z = (up2 ? s2[1] : s2[0]) + __shfl_xor_sync(0xffffffffu, up2 ? s2[0] : s2[1], 2);
         z += __shfl_xor_sync(0xffffffffu, z, 1);
-        // ---- v = x - alpha e_{k+1}; p = beta A v = beta (y - alpha A e_{k+1}), and column k + 1 is row k + 1 ----
-        double alpha = x0, beta = 0.0;
-        if (sig > 1e-290) {                            // otherwise the row is reduced already: beta = 0
-            const double root = sqrt_newton(sig);
-            alpha = x0 >= 0.0 ? -root : root;
-            beta = recip_newton(fma(fabs(x0), root, sig));            // 2 / (v^T v)
-        }
-        const double v = mine > k + 1 ? S.x[mine] : (mine == k + 1 ? x0 - alpha : 0.0);
-        const double p = mine > k ? beta * fma(-alpha, S.x1[mine], z) : 0.0;
-        double s = v * p;
-#pragma unroll
-        for (int o = 2; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) S.part[warp] = s;
-        if ((t & 1) == 0) { S.v[mine] = v; S.p[mine] = p; }
-        if (mine == k + 1 && (t & 1) == 0) S.ee[k] = alpha;
+        if ((t & 1) == 0 && (t >> 1) >= KA) ps[i + 16 * (t >> 1)] = minus_beta * z;
         __syncthreads();
-        // ---- kk = beta/2 v^T p; A -= v p^T + (p - 2 kk v) v^T ----
-        double q[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-        for (int w = 0; w < kEigWarps; w += 4) {
-            const double2 a = *reinterpret_cast<const double2 *>(S.part + w), b = *reinterpret_cast<const double2 *>(S.part + w + 2);
-            q[0] += a.x; q[1] += a.y; q[2] += b.x; q[3] += b.y;
-        }
-        const double kk = beta * ((q[0] + q[1]) + (q[2] + q[3]));     // 2 kk
-        double nv[8], nf[8];
-#pragma unroll
-        for (int a = KA; a < 8; ++a) {
-            const double vr = S.v[i + 16 * a];
-            nv[a] = -vr;
-            nf[a] = fma(kk, vr, -S.p[i + 16 * a]);
-        }
+        // ---- -w = -p + (beta/2 v^T p) v, then row k + 1 after this step's update: the next x ----
 #pragma unroll
         for (int j = J; j < 4; ++j) {
-            const double2 vc = *reinterpret_cast<const double2 *>(S.v + 32 * j + 2 * t), pc = *reinterpret_cast<const double2 *>(S.p + 32 * j + 2 * t);
+            const double2 q = *reinterpret_cast<const double2 *>(ps + 32 * j + 2 * t);
+            R.wc[2 * j] = q.x;
+            R.wc[2 * j + 1] = q.y;
+            R.vc[2 * j] = R.xc[2 * j];
+            R.vc[2 * j + 1] = R.xc[2 * j + 1];
+        }
+        double dot[2] = {R.vc[2 * J] * R.wc[2 * J], R.vc[2 * J + 1] * R.wc[2 * J + 1]};
 #pragma unroll
-            for (int a = KA; a < 8; ++a) {
-                A[a][2 * j] = fma(nv[a], pc.x, fma(nf[a], vc.x, A[a][2 * j]));
-                A[a][2 * j + 1] = fma(nv[a], pc.y, fma(nf[a], vc.y, A[a][2 * j + 1]));
+        for (int q = 2 * J + 2; q < 8; ++q) dot[q & 1] = fma(R.vc[q], R.wc[q], dot[q & 1]);
+        const double kk = 0.5 * minus_beta * sum16(dot[0] + dot[1]);            // beta/2 v^T p
+        const double wk = fma(kk, vk, ps[k + 1]);
+        if (threadIdx.x == 0) S.dd[k + 1] = fma(2.0 * vk, wk, xs[k + 1]);
+#pragma unroll
+        for (int j = J; j < 4; ++j) {
+            const double2 row = *reinterpret_cast<const double2 *>(xs + 32 * j + 2 * t);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int q = 2 * j + e;
+                R.wc[q] = fma(kk, R.vc[q], R.wc[q]);
+                R.xc[q] = fma(vk, R.wc[q], fma(wk, R.vc[q], e ? row.y : row.x));
             }
         }
-        // ---- rows k + 1 and k + 2 for the next step ----
-        if (i == ((k + 1) & 15)) {
-            if (KA == 7 || kt < 15) {
-                publish_row<J>(A[KA], S.x, t, k + 1);
-                publish_diagonal<J>(A[KA], &S.dd[k + 1], t, k + 1);
-            } else {
-                publish_row<J>(A[KN], S.x, t, k + 1);
-                publish_diagonal<J>(A[KN], &S.dd[k + 1], t, k + 1);
-            }
-        } else if (i == ((k + 2) & 15)) {
-            if (KA == 7 || kt < 14) publish_row<J>(A[KA], S.x1, t, -1);
-            else publish_row<J>(A[KN], S.x1, t, -1);
+        {                                              // columns up to k + 1 are zero
+            const int at = k + 1 - 32 * J - 2 * t;
+            if (at >= 0) R.xc[2 * J] = 0.0;
+            if (at >= 1) R.xc[2 * J + 1] = 0.0;
+            if (kOdd && end && t == 0) R.xc[2 * JN] = 0.0;
         }
-        __syncthreads();
+        {                                              // entry k + 2 of the new x for everybody
+            const int c = k + 2;
+            const bool next = kOdd && kt >= 14;        // it lies in the next column group
+            const double lo = next ? R.xc[2 * JN] : R.xc[2 * J], hi = next ? R.xc[2 * JN + 1] : R.xc[2 * J + 1];
+            R.x0 = __shfl_sync(0xffffffffu, (c & 1) ? hi : lo, (lane & 16) + ((c >> 1) & 15));
+        }
+#pragma unroll
+        for (int a = KA; a < 8; ++a) {
+            R.vr[a] = vs[i + 16 * a];
+            R.wr[a] = fma(kk, R.vr[a], ps[i + 16 * a]);
+        }
     }
 }
 }  // namespace
@@ -292,33 +301,36 @@ eigen_entropy_kernel(const PartialT *__restrict__ partials, int P, int N, int k_
     }
     d = warp_sum(d);
     if (lane == 0) S.part[wid] = d;
-    if (row0 == 0) {
-        publish_row<0>(A[0], S.x, t, 0);
-        if (t == 0) S.dd[0] = A[0][0];
-    } else if (row0 == 1) {
-        publish_row<0>(A[0], S.x1, t, -1);
-    }
+    if (row0 == 0) publish<0>(A[0], S.x[1], t);
     __syncthreads();
     if (tid == 0) {
         double s = 0.0;
         for (int w = 0; w < kEigWarps; ++w) s += S.part[w];
         S.trace = s;
     }
-    __syncthreads();                                   // the first step overwrites S.part
 
     // ---- 2. Householder tridiagonalisation ---------------------------------------------------------
-    householder_block<0>(A, S, lane, wid);
-    householder_block<1>(A, S, lane, wid);
-    householder_block<2>(A, S, lane, wid);
-    householder_block<3>(A, S, lane, wid);
-    householder_block<4>(A, S, lane, wid);
-    householder_block<5>(A, S, lane, wid);
-    householder_block<6>(A, S, lane, wid);
-    householder_block<7>(A, S, lane, wid);
-    if (tid == 0) {                                    // the last 2 x 2 block was published by step n - 3
-        S.ee[n - 2] = S.x[n - 1];
-        S.dd[n - 1] = S.x1[n - 1];
-        S.ee[n - 1] = 0.0;
+    {
+        Carry R;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            R.vc[q] = R.wc[q] = R.vr[q] = R.wr[q] = 0.0;
+            R.xc[q] = S.x[1][32 * (q >> 1) + 2 * t + (q & 1)];
+        }
+        R.x0 = S.x[1][1];
+        if (tid == 0) S.dd[0] = S.x[1][0];
+        if (t == 0) R.xc[0] = 0.0;
+        householder_block<0>(A, R, S, lane, wid);
+        householder_block<1>(A, R, S, lane, wid);
+        householder_block<2>(A, R, S, lane, wid);
+        householder_block<3>(A, R, S, lane, wid);
+        householder_block<4>(A, R, S, lane, wid);
+        householder_block<5>(A, R, S, lane, wid);
+        householder_block<6>(A, R, S, lane, wid);
+        householder_block<7>(A, R, S, lane, wid);
+        if (tid == 0) { S.ee[n - 2] = R.x0; S.ee[n - 1] = 0.0; }
+        if (row0 == 15 && t == 15)                     // entry (127, 127) after the last update
+            S.dd[n - 1] = fma(R.vr[7], R.wc[7], fma(R.wr[7], R.vc[7], A[7][7]));
     }
     __syncthreads();
 
@@ -398,20 +410,26 @@ eigen_entropy_kernel(const PartialT *__restrict__ partials, int P, int N, int k_
     __syncthreads();
 
     // ---- 4. entropy -----------------------------------------------------------------------------
-    if (tid == 0) {
-        double total = 0.0;
-        if (norm) total = S.trace;
-        else for (int i = 0; i < k; ++i) total += S.lam[i] > 0.0 ? S.lam[i] : 0.0;
+    if (wid == 0) {      // lane i takes eigenvalues i, i + 32, ...; fixed-order butterfly sums
+        double total = S.trace;
+        if (!norm) {
+            total = 0.0;
+            for (int i = lane; i < k; i += 32) total += S.lam[i] > 0.0 ? S.lam[i] : 0.0;
+            total = warp_sum(total);
+        }
         double h = 0.0;
         if (total > 0.0) {
-            for (int i = 0; i < k; ++i) {
+            for (int i = lane; i < k; i += 32) {
                 const double p = (S.lam[i] > 0.0 ? S.lam[i] : 0.0) / total;
                 if (p > 0.0) h -= p * log(p);
             }
         }
-        entropy[u] = (float)h;
-        if (erank) erank[u] = (float)exp(h);
-        if (S.flags[0]) atomicOr(status, UNCOMP_STATUS_NOT_CONVERGED);
+        h = warp_sum(h);
+        if (lane == 0) {
+            entropy[u] = (float)h;
+            if (erank) erank[u] = (float)exp(h);
+            if (S.flags[0]) atomicOr(status, UNCOMP_STATUS_NOT_CONVERGED);
+        }
     }
     if (spectrum && tid < k) spectrum[(size_t)u * k + tid] = S.lam[tid];
 }
