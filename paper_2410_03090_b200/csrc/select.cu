@@ -219,6 +219,7 @@ constexpr int kKeyWarps = kKeyThreads / 32;
 constexpr int kKeyMaxCluster = 8;
 constexpr int kKeyHalo = 32;                             // pool windows reach at most 31 positions beyond a CTA's share
 constexpr int kKeyBins = 2 * kKeyThreads;
+constexpr int kCandidates = 256;                         // keys ranked against one another instead of by another histogram
 // How the scores are pooled: width 1 takes them as they are; the 7-wide maximum, what the pass defaults to, from the four
 // scores of a lane and shuffles; any other width by a loop per position.  256 units of 32704 positions / 1024 of 3704 / 8 of
 // 6969: 53 / 41 / 15 us, 66 / 50 / 17 us, and by the loop 77 / 54 / 17 us for a maximum over 5, 82 / 54 / 18 over 9, 141 /
@@ -231,8 +232,22 @@ template <int NBK> struct KeySmem {
     unsigned slot[2][2][kKeyMaxCluster];                 // [exchange][value][CTA of the cluster]
     unsigned warp_a[kKeyWarps], warp_b[kKeyWarps];
     int warp_sum[kKeyWarps];
-    int bin, above, in_bin;
+    uint4 above_bits[kKeyWarps * NBK], equal_bits[kKeyWarps * NBK];      // of 128 positions: bit l of word c is position 4 l + c
+    uint32_t threshold;
+    int bin, above, in_bin, candidates, all_equal;
 };
+
+// bit i of a byte to bit 4 i
+__device__ __forceinline__ uint32_t spread4(uint32_t x) {
+    x = (x | (x << 12)) & 0x000f000fu;
+    x = (x | (x << 6)) & 0x03030303u;
+    return (x | (x << 3)) & 0x11111111u;
+}
+// the 32 positions 32 g .. 32 g + 31 of 128, in their order
+__device__ __forceinline__ uint32_t in_order(const uint4 &w, int g) {
+    const int s = 8 * g;
+    return spread4((w.x >> s) & 255u) | spread4((w.y >> s) & 255u) << 1 | spread4((w.z >> s) & 255u) << 2 | spread4((w.w >> s) & 255u) << 3;
+}
 
 // Two CTAs per SM up to four blocks of keys: with many units one CTA's barriers hide behind the other.  That bound leaves
 // 32 registers and spills 36 to 64 bytes of a thread, also in calls whose few units leave the second place empty.
@@ -258,18 +273,21 @@ pool_select_keys_kernel(const float *__restrict__ raw, float *__restrict__ poole
     // ---- 1. raw scores to shared memory, pooled scores out and, as keys, in their place ---------------------
     const float outside = pool_mode ? 0.f : -INFINITY;
     constexpr int kVec = (kShare + 2 * kKeyHalo) / 4;
-    if ((reinterpret_cast<uintptr_t>(r) & 15u) == 0) {
+    if ((reinterpret_cast<uintptr_t>(r) & 15u) == 0) {               // asynchronous copies: all on their way at once
 #pragma unroll 4
         for (int i = tid; i < kVec; i += kKeyThreads) {
             const int j = p0 - kKeyHalo + 4 * i;
-            float4 x = make_float4(outside, outside, outside, outside);
-            if (j >= 0 && j + 3 < P) x = __ldg(reinterpret_cast<const float4 *>(r + j));
-            else if (j >= 0 && j < P) {
-                x.x = r[j];
-                if (j + 1 < P) x.y = r[j + 1];
-                if (j + 2 < P) x.z = r[j + 2];
+            if (j >= 0 && j + 3 < P) {
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(S.raw + 4 * i)), "l"(r + j) : "memory");
+            } else {
+                float4 x = make_float4(outside, outside, outside, outside);
+                if (j >= 0 && j < P) {
+                    x.x = r[j];
+                    if (j + 1 < P) x.y = r[j + 1];
+                    if (j + 2 < P) x.z = r[j + 2];
+                }
+                reinterpret_cast<float4 *>(S.raw)[i] = x;
             }
-            reinterpret_cast<float4 *>(S.raw)[i] = x;
         }
     } else {
 #pragma unroll 8
@@ -289,6 +307,8 @@ pool_select_keys_kernel(const float *__restrict__ raw, float *__restrict__ poole
         for (int64_t i = tid; i < slab.fill; i += kKeyThreads)
             if (UNCOMP_INDEX_OK(k + slab.wn + i, slab.seg, status)) out[k + slab.wn + i] = P + w - 1;
     }
+    if (tid == 0) S.candidates = 0;
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     const int at0 = wid * kWarpShare + lane * 4, j0 = p0 + at0;        // block b: 128 b further
     float *mine = S.raw + kKeyHalo + at0;
@@ -438,74 +458,108 @@ pool_select_keys_kernel(const float *__restrict__ raw, float *__restrict__ poole
             T = lo;
             all_equal_kept = S.in_bin == kr;             // the whole bin is kept: T is its lower end
             if (all_equal_kept || shift == 0) break;
+            if (ctas == 1 && S.in_bin <= kCandidates) {
+                // few keys are left in the bin: they are collected, and each is ranked against all of them
+                uint32_t *list = reinterpret_cast<uint32_t *>(S.hist[2]);
+                const int m = S.in_bin;
+#pragma unroll 1
+                for (int b = 0; b < NBK; ++b) {
+                    const uint4 kv = keys(b);
+                    const uint32_t key[4] = {kv.x, kv.y, kv.z, kv.w};
+                    const int left = P - (j0 + 128 * b);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        if ((key[c] - lo) >> shift == 0u && c < left) {
+                            const int at = atomicAdd(&S.candidates, 1);
+                            if (UNCOMP_INDEX_OK(at, kCandidates, status)) list[at] = key[c];
+                        }
+                }
+                __syncthreads();
+                if (tid < m) {
+                    const uint32_t own = list[tid];
+                    int above = 0, equal = 0;
+#pragma unroll 4
+                    for (int i = 0; i < m; ++i) {
+                        const uint32_t x = list[i];
+                        above += x > own;
+                        equal += x == own;
+                    }
+                    if (above < kr && kr <= above + equal) {      // the same for all keys equal to it
+                        S.threshold = own;
+                        S.all_equal = kr == above + equal;
+                    }
+                }
+                __syncthreads();
+                T = S.threshold;
+                all_equal_kept = S.all_equal != 0;
+                break;
+            }
             width = 1u << shift;
             shift = max(0, shift - 11);
             __syncthreads();                             // bin, above and in_bin are read before the next pass writes them
         }
     }
 
-    // ---- 3. ordered compaction: counts of the lower CTAs, then of the lower warps ------------------------
-    // kept: above T (low half of a count), equal to T (high half); when all equal ones are kept they count as above
+    // ---- 3. ordered compaction ---------------------------------------------------------------------------
+    // kept: above T, and of those equal to T the first; when all equal ones are kept they count as above.  The warps leave a bit
+    // per position; then a thread has 32 consecutive positions, so one scan of the block gives every thread its first
+    // slot.  (A scan per 128 positions took 15,000 cycles of a unit of 32768.)
     auto is_above = [&](uint32_t x) { return all_equal_kept ? x >= T : x > T; };
-    unsigned cnt = 0;
 #pragma unroll
     for (int b = 0; b < NBK; ++b) {
         const uint4 key = keys(b);
         const int left = P - (j0 + 128 * b);
-        cnt += (is_above(key.x) && 0 < left) + (is_above(key.y) && 1 < left) + (is_above(key.z) && 2 < left) + (is_above(key.w) && 3 < left);
-        if (!all_equal_kept) cnt += ((key.x == T && 0 < left) + (key.y == T && 1 < left) + (key.z == T && 2 < left) + (key.w == T && 3 < left)) << 16;
+        const uint4 above = make_uint4(__ballot_sync(0xffffffffu, is_above(key.x) && 0 < left), __ballot_sync(0xffffffffu, is_above(key.y) && 1 < left),
+                                       __ballot_sync(0xffffffffu, is_above(key.z) && 2 < left), __ballot_sync(0xffffffffu, is_above(key.w) && 3 < left));
+        if (lane == 0) S.above_bits[wid * NBK + b] = above;
+        if (!all_equal_kept) {
+            const uint4 equal = make_uint4(__ballot_sync(0xffffffffu, key.x == T && 0 < left), __ballot_sync(0xffffffffu, key.y == T && 1 < left),
+                                           __ballot_sync(0xffffffffu, key.z == T && 2 < left), __ballot_sync(0xffffffffu, key.w == T && 3 < left));
+            if (lane == 0) S.equal_bits[wid * NBK + b] = equal;
+        }
     }
-    unsigned gt = __reduce_add_sync(0xffffffffu, cnt & 0xffffu), eq = __reduce_add_sync(0xffffffffu, cnt >> 16);
-    if (lane == 0) { S.warp_a[wid] = gt; S.warp_b[wid] = eq; }
     __syncthreads();
-    unsigned gt_run = __reduce_add_sync(0xffffffffu, lane < wid ? S.warp_a[lane] : 0u);
-    unsigned eq_run = __reduce_add_sync(0xffffffffu, lane < wid ? S.warp_b[lane] : 0u);
-    unsigned gt_all = __reduce_add_sync(0xffffffffu, S.warp_a[lane]);
+    constexpr int kGroups = 4 * kKeyWarps * NBK;         // of 32 positions, at most one per thread
+    uint32_t above = 0u, equal = 0u;
+    if (tid < kGroups) {
+        above = in_order(S.above_bits[tid >> 2], tid & 3);
+        if (!all_equal_kept) equal = in_order(S.equal_bits[tid >> 2], tid & 3);
+    }
+    const unsigned own = __popc(above) | (unsigned)__popc(equal) << 16;         // 32768 of each at most
+    unsigned incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned below = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += below;
+    }
+    if (lane == 31) S.warp_a[wid] = incl;
+    __syncthreads();
+    const unsigned warp_all = S.warp_a[lane];
+    const unsigned before = __reduce_add_sync(0xffffffffu, lane < wid ? warp_all : 0u) + incl - own;
+    const unsigned all = __reduce_add_sync(0xffffffffu, warp_all);
+    unsigned g = before & 0xffffu, e = before >> 16, gt_all = all & 0xffffu;
     if (ctas > 1) {
-        const unsigned eq_all = __reduce_add_sync(0xffffffffu, S.warp_b[lane]);
         if (tid < ctas) {
             KeySmem<NBK> *R = cluster.map_shared_rank(&S, tid);
             R->slot[1][0][rank] = gt_all;
-            R->slot[1][1][rank] = eq_all;
+            R->slot[1][1][rank] = all >> 16;
         }
         cluster.sync();                                  // also the last access to a peer's memory
         gt_all = 0;
         for (int c = 0; c < ctas; ++c) {
             gt_all += S.slot[1][0][c];
-            if (c < rank) { gt_run += S.slot[1][0][c]; eq_run += S.slot[1][1][c]; }
+            if (c < rank) { g += S.slot[1][0][c]; e += S.slot[1][1][c]; }
         }
     }
     const unsigned need_eq = all_equal_kept ? 0u : (unsigned)k - gt_all;
-#pragma unroll
-    for (int b = 0; b < NBK; ++b) {
-        const uint4 kv = keys(b);
-        const uint32_t key[4] = {kv.x, kv.y, kv.z, kv.w};
-        const int j = j0 + 128 * b, left = P - j;
-        unsigned own = 0;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            own += is_above(key[c]) && c < left;
-            if (!all_equal_kept) own += (key[c] == T && c < left) << 16;
-        }
-        if (!__any_sync(0xffffffffu, own != 0u)) continue;
-        unsigned incl = own;                             // 128 of each at most: the halves do not meet
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned below = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += below;
-        }
-        const unsigned total = __shfl_sync(0xffffffffu, incl, 31);
-        unsigned g = gt_run + ((incl - own) & 0xffffu), e = eq_run + ((incl - own) >> 16);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const bool is_gt = is_above(key[c]) && c < left, is_eq = !all_equal_kept && key[c] == T && c < left;
-            const unsigned at = g + min(e, need_eq);
-            if ((is_gt || (is_eq && e < need_eq)) && UNCOMP_INDEX_OK(at, k, status)) out[at] = j + c;
-            g += is_gt;
-            e += is_eq;
-        }
-        gt_run += total & 0xffffu;
-        eq_run += total >> 16;
+    const int j = p0 + 32 * tid;
+    for (uint32_t rest = above | equal; rest != 0u; rest &= rest - 1u) {
+        const int bit = __ffs(rest) - 1;
+        const bool is_gt = (above >> bit) & 1u;
+        const unsigned at = g + min(e, need_eq);
+        if ((is_gt || e < need_eq) && UNCOMP_INDEX_OK(at, k, status)) out[at] = j + bit;
+        g += is_gt;
+        e += !is_gt;
     }
 }
 
