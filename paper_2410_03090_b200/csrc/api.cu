@@ -36,6 +36,14 @@ Plan make_plan(const uncomp_shape &s) {
         int want = (target_ctas + p.units - 1) / p.units;
         int most = (s.N + 1023) / 1024;
         int P = want < 1 ? 1 : (want > most ? most : want);
+        // fp32 keys: ten CTAs per unit and chunk, a sequence of short steps each; while they leave SMs idle up to four chunks of
+        // 128 tokens or more (8 units of 512 tokens: 20.7 us with one, 18.1 with two, 15.4 with four, and 2 more for the
+        // eigenvalues to add them up)
+        if (s.dtype == UNCOMP_FP32) {
+            const int idle = 3 * kTargetSms / (10 * p.units);
+            const int finer = idle > 4 ? 4 : idle, least = (s.N + 127) / 128;
+            if (P < (finer < least ? finer : least)) P = finer < least ? finer : least;
+        }
         int chunk = (int)align_up((size_t)(s.N + P - 1) / P, 128);
         p.gram_chunk = chunk;
         p.gram_splits = (s.N + chunk - 1) / chunk;

@@ -28,6 +28,7 @@ constexpr int kEigWarps = kEigThreads / 32;
 constexpr int kTeamThreads = 128;
 constexpr int kCoarse = 2 * kEigThreads;
 constexpr int n = kD;
+template <typename T> struct __align__(2 * sizeof(T)) Pair { T x, y; };
 
 struct EigenSmem {
     double x[2][n];   // row k + 1 before the update of step k
@@ -274,11 +275,12 @@ eigen_entropy_kernel(const PartialT *__restrict__ partials, int P, int N, int k_
     for (int p = 0; p < P; ++p) {
 #pragma unroll
         for (int a = 0; a < 8; ++a) {
-            const PartialT *row = base + (size_t)p * len + (row0 + 16 * a) * n + 2 * t;
+            const Pair<PartialT> *row = reinterpret_cast<const Pair<PartialT> *>(base + (size_t)p * len + (row0 + 16 * a) * n + 2 * t);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                A[a][2 * j] += (double)row[32 * j];
-                A[a][2 * j + 1] += (double)row[32 * j + 1];
+                const Pair<PartialT> x = row[16 * j];
+                A[a][2 * j] += (double)x.x;
+                A[a][2 * j + 1] += (double)x.y;
             }
         }
     }

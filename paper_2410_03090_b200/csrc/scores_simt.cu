@@ -14,8 +14,23 @@ namespace uncomp {
 constexpr int kSB = 64;   // rows and tokens per block of logits
 constexpr int kKPad = kD + 1;
 
-template <typename T>
-__device__ __forceinline__ void load_rows(float (*dst)[kKPad], const T *src, int64_t row_stride, int first, int limit,
+// 64 rows of 128 features; rows are 16-byte aligned.  All of a thread's loads are in flight together (one by one they took
+// a third of the statistics' 12 us at 8 units of 512 tokens, now 9; column sums 10.3, now 8.8).
+__device__ __forceinline__ void load_rows(float (*dst)[kKPad], const float *src, int64_t row_stride, int first, int limit,
+                                          int tid) {
+    float4 v[kSB * kD / 4 / 256];
+#pragma unroll
+    for (int i = 0; i < kSB * kD / 4 / 256; ++i) {
+        const int row = first + (tid >> 5) + 8 * i;
+        v[i] = row < limit ? *reinterpret_cast<const float4 *>(src + (int64_t)row * row_stride + 4 * (tid & 31)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int i = 0; i < kSB * kD / 4 / 256; ++i) {
+        float *d = dst[(tid >> 5) + 8 * i] + 4 * (tid & 31);
+        d[0] = v[i].x; d[1] = v[i].y; d[2] = v[i].z; d[3] = v[i].w;
+    }
+}
+__device__ __forceinline__ void load_rows(float (*dst)[kKPad], const __nv_bfloat16 *src, int64_t row_stride, int first, int limit,
                                           int tid) {
     for (int e = tid; e < kSB * kD; e += 256) {
         const int r = e >> 7, c = e & 127;
