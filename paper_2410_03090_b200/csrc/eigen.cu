@@ -5,18 +5,23 @@
 //      dropped for the uncentred variant).  Eq. 1 without its 1/(N-1), which cancels in step 4.
 //   2. Householder reduction of the 128 x 128 symmetric C to tridiagonal form, C in registers: lane t = lane & 15 of row
 //      group i = 2 warp + lane / 16 holds the 64 entries C[i + 16 a][32 j + 2 t + e], a < 8, j < 4, e < 2.
-//   3. The k largest eigenvalues by Sturm-count multi-section: a coarse round of 512 points, then 4 lanes per eigenvalue
-//      evaluate the division-free three-term recurrence of the characteristic polynomials at 8 interior points, so the
-//      bracket shrinks 9-fold per round.  The recurrence is rescaled against underflow.
+//   3. The k largest eigenvalues by Sturm-count multi-section: a coarse round shared by all, then a team of lanes per
+//      eigenvalue evaluates the division-free three-term recurrence of the characteristic polynomials at one interior point
+//      each (8 lanes: 9-fold per round).  The recurrence is rescaled against underflow.  Few units: steps 3 and 4 are a
+//      kernel of their own, where a cluster of CTAs shares the eigenvalues of a unit in larger teams.
 //   4. p_i = lambda_i / sum (over the k kept, or the whole trace), H_k = -sum p_i ln p_i, erank_k = exp H_k.
 //
-// What bounds it: the chain of a step (a norm, a square root, a reciprocal, four shuffle reductions of two words a level,
-// two barriers) and, while the matrix is large, the fp64 units (192 multiply-adds per thread and full step).  Shared
+// What bounds it: the chain of a step (a norm, a square root, a reciprocal, three shuffle reductions of two words a level,
+// a barrier) and, while the matrix is large, the fp64 units (192 multiply-adds per thread and full step).  Shared
 // memory delivers 128 bytes per cycle whatever the lanes have in common, so a layout with few columns per thread matters
 // more than few shuffles: four lanes per row and 32 columns each took 4400 cycles per full step, 512 threads with 8 columns
-// 3100, this form 2500.  Row and column groups that are done drop out of the code (the step loop is unrolled over
+// 3100, this form 2370, 1000 where almost nothing is left to
+// update.  Row and column groups that are done drop out of the code (the step loop is unrolled over
 // k / 16); inside the groups nothing is masked: reflectors and products are zero there.  With the matrix in shared
-// memory, one warp forming the reflector and a warp per row for the product, 8 units took 543 us; now 166 us.
+// memory, one warp forming the reflector and a warp per row for the product, 8 units took 543 us; now 140 (113 and 15 for the
+// eigenvalues with a kernel of their own).
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 #include "newton.cuh"
 
@@ -24,9 +29,8 @@ namespace uncomp {
 
 namespace {
 constexpr int kEigThreads = 256;
+constexpr int kValueThreads = 128;   // of a CTA of the eigenvalue kernel
 constexpr int kEigWarps = kEigThreads / 32;
-constexpr int kTeamThreads = 128;
-constexpr int kCoarse = 2 * kEigThreads;
 constexpr int n = kD;
 template <typename T> struct __align__(2 * sizeof(T)) Pair { T x, y; };
 
@@ -36,13 +40,20 @@ struct EigenSmem {
     double p[2][n];   // minus the product of the matrix and the reflector
     double part[kEigWarps];
     double sd[n];     // column sums
+    double trace;
+};
+struct ValueSmem {
     double dd[n];
     double ee[n];     // ee[i] couples i and i+1
     double2 de[n];    // (diagonal, -coupling^2) of the scaled matrix, the coupling to the entry before
     double lam[n];
-    double scale, trace;
-    int cnt[kCoarse + 2];
-    int flags[2];
+    double scale;
+    int cnt[2 * kEigThreads + 2];
+    int not_converged;
+};
+// What the first kernel leaves for the eigenvalue kernel of few units, over the unit's own first partial, which it has consumed.
+struct EigenBand64 {
+    double dd[n], ee[n], trace;
 };
 
 // number of eigenvalues of the normalised tridiagonal matrix that are < x
@@ -66,50 +77,84 @@ __device__ __noinline__ int sturm_count_robust(const double2 *de, double x) {
     }
     return count;
 }
-// The same for NP points without a branch per step: sign bits are shifted into a word and the changes counted 32 at a
-// time, the pair is brought back near 1 every 8 steps (a step shrinks it by at most 2^-60 or so).  A zero between non-zero
-// neighbours adds one change whichever sign it gets; a zero that stays zero to the end is recounted.
+// factor that brings |p| back near 1 (a power of two; p below 2^-831 is raised by 2^832)
+__device__ __forceinline__ double rescale_of(double p) {
+    const int ex = max(__double2hiint(p) & 0x7ff00000, 0x0c000000);
+    return __hiloint2double(0x7fe00000 - ex, 0);
+}
+// The same for NP points without a branch per step, from both ends at once (half the chain): p over the leading, q over the
+// trailing 64 rows.  With F = p_64 q_64 - e^2 p_63 q_63 (the whole determinant, e couples the halves) the count is the sign
+// changes of p up to p_64, those of q up to q_63, and one more when F and p_64 q_63 differ in sign.  Sign bits are shifted
+// into a word and the changes counted 32 at a time, the pairs are brought back near 1 every 8 steps (a step shrinks them by
+// at most 2^-60 or so).  A zero adds one change whichever sign it gets as long as the coupling behind it is not zero;
+// otherwise F is zero and the point is recounted.  Bound by the fp64 units and by the sign words (a funnel shift costs as
+// much as an fp64 operation): with the next eight rows loaded ahead 8 warps take 3300 cycles (3900 from one end, 4 warps of
+// two points).
 template <int NP>
 __device__ __forceinline__ void sturm_count(const double2 *de, const double (&x)[NP], int (&count)[NP]) {
-    double p0[NP], p1[NP];
-    uint32_t last[NP];
+    double p0[NP], p1[NP], q0[NP], q1[NP], me2 = 0.0;
+    uint32_t lastp[NP], lastq[NP];
+    double2 fn[8], gn[8];
 #pragma unroll
-    for (int c = 0; c < NP; ++c) { p0[c] = 0.0; p1[c] = 1.0; count[c] = 0; last[c] = 0u; }
-#pragma unroll 1
-    for (int w = 0; w < n / 32; ++w) {
-        uint32_t m[NP];
+    for (int i = 0; i < 8; ++i) { fn[i] = de[i]; gn[i] = de[n - 1 - i]; }
 #pragma unroll
-        for (int c = 0; c < NP; ++c) m[c] = 0u;
+    for (int c = 0; c < NP; ++c) { p0[c] = q0[c] = 0.0; p1[c] = q1[c] = 1.0; count[c] = 0; lastp[c] = lastq[c] = 0u; }
 #pragma unroll 1
-        for (int i0 = 0; i0 < 32; i0 += 8) {
+    for (int w = 0; w < 2; ++w) {
+        uint32_t mp[NP], mq[NP];
+#pragma unroll
+        for (int c = 0; c < NP; ++c) mp[c] = mq[c] = 0u;
+#pragma unroll 1
+        for (int i0 = w * 32; i0 < w * 32 + 32; i0 += 8) {
+            double2 f[8], g[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {              // the next eight entries are on their way
+                f[i] = fn[i];
+                g[i] = gn[i];
+                fn[i] = de[(i0 + 8 + i) & (n - 1)];
+                gn[i] = de[(n - 1 - i0 - 8 - i) & (n - 1)];
+            }
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                const double2 q = de[w * 32 + i0 + i];
 #pragma unroll
                 for (int c = 0; c < NP; ++c) {
-                    const double pn = fma(q.x - x[c], p1[c], q.y * p0[c]);
+                    const double pn = fma(f[i].x - x[c], p1[c], f[i].y * p0[c]), qn = fma(g[i].x - x[c], q1[c], me2 * q0[c]);
                     p0[c] = p1[c];
                     p1[c] = pn;
-                    m[c] = __funnelshift_l((uint32_t)__double2hiint(pn), m[c], 1);
+                    q0[c] = q1[c];
+                    q1[c] = qn;
+                    mp[c] = __funnelshift_l((uint32_t)__double2hiint(pn), mp[c], 1);
+                    mq[c] = __funnelshift_l((uint32_t)__double2hiint(qn), mq[c], 1);
                 }
+                me2 = g[i].y;                          // couples row 127 - i0 - i to the one before
             }
 #pragma unroll
             for (int c = 0; c < NP; ++c) {
-                const int ex = max(__double2hiint(p1[c]) & 0x7ff00000, 0x0c000000);     // at least 2^-831
-                const double s = __hiloint2double(0x7fe00000 - ex, 0);
-                p0[c] *= s;
-                p1[c] *= s;
+                const double sp = rescale_of(p1[c]), sq = rescale_of(q1[c]);
+                p0[c] *= sp;
+                p1[c] *= sp;
+                q0[c] *= sq;
+                q1[c] *= sq;
             }
         }
 #pragma unroll
         for (int c = 0; c < NP; ++c) {
-            count[c] += __popc(m[c] ^ ((m[c] >> 1) | (last[c] << 31)));
-            last[c] = m[c] & 1u;
+            const uint32_t up = mp[c] ^ ((mp[c] >> 1) | (lastp[c] << 31));
+            uint32_t dn = mq[c] ^ ((mq[c] >> 1) | (lastq[c] << 31));
+            if (w == 1) dn &= ~1u;                     // q_64 belongs to F
+            count[c] += __popc(up) + __popc(dn);
+            lastp[c] = mp[c] & 1u;
+            lastq[c] = w == 0 ? mq[c] & 1u : (mq[c] >> 1) & 1u;
         }
     }
 #pragma unroll
-    for (int c = 0; c < NP; ++c)
-        if (p1[c] == 0.0) count[c] = sturm_count_robust(de, x[c]);
+    for (int c = 0; c < NP; ++c) {                     // me2: -e^2 between rows 63 and 64
+        // the larger of a pair near 1: neither product leaves the range
+        const double sp = rescale_of(fmax(fabs(p0[c]), fabs(p1[c]))), sq = rescale_of(fmax(fabs(q0[c]), fabs(q1[c])));
+        const double F = fma(p1[c] * sp, q1[c] * sq, me2 * (p0[c] * sp) * (q0[c] * sq));
+        count[c] += (int)(((uint32_t)__double2hiint(F) >> 31) ^ lastp[c] ^ lastq[c]);
+        if (F == 0.0 || !isfinite(F)) count[c] = sturm_count_robust(de, x[c]);
+    }
 }
 
 __device__ __forceinline__ double sum16(double v) {   // over the 16 lanes that share a row
@@ -135,7 +180,7 @@ struct Carry {
 // Householder steps k = 16 KA .. 16 KA + 15 (stopping at n - 3); row groups (16 rows) below KA and column groups (32
 // columns) below J are done.
 template <int KA>
-__device__ __forceinline__ void householder_block(double (&A)[8][8], Carry &R, EigenSmem &S, int lane, int warp) {
+__device__ __forceinline__ void householder_block(double (&A)[8][8], Carry &R, EigenSmem &S, ValueSmem &F, int lane, int warp) {
     constexpr int J = KA >> 1, JN = J < 3 ? J + 1 : 3, KN = KA < 7 ? KA + 1 : 7;
     constexpr bool kOdd = (KA & 1) != 0 && KA < 7;     // the block's end is also the end of a column group
     const int i = 2 * warp + (lane >> 4), t = lane & 15;
@@ -166,7 +211,7 @@ __device__ __forceinline__ void householder_block(double (&A)[8][8], Carry &R, E
         const double minus_alpha = flat ? -R.x0 : (R.x0 >= 0.0 ? root : -root);
         const double minus_beta = flat ? 0.0 : -recip_newton(fma(fabs(R.x0), root, sig));         // -2 / (v^T v)
         const double vk = R.x0 + minus_alpha;          // v_{k+1}
-        if (threadIdx.x == 0) S.ee[k] = -minus_alpha;
+        if (threadIdx.x == 0) F.ee[k] = -minus_alpha;
         if (kOdd && end) {                             // column k + 1 is the first of the next group
             const double d0 = t == 0 ? minus_alpha : 0.0;
 #pragma unroll
@@ -216,7 +261,7 @@ __device__ __forceinline__ void householder_block(double (&A)[8][8], Carry &R, E
         for (int q = 2 * J + 2; q < 8; ++q) dot[q & 1] = fma(R.vc[q], R.wc[q], dot[q & 1]);
         const double kk = 0.5 * minus_beta * sum16(dot[0] + dot[1]);            // beta/2 v^T p
         const double wk = fma(kk, vk, ps[k + 1]);
-        if (threadIdx.x == 0) S.dd[k + 1] = fma(2.0 * vk, wk, xs[k + 1]);
+        if (threadIdx.x == 0) F.dd[k + 1] = fma(2.0 * vk, wk, xs[k + 1]);
 #pragma unroll
         for (int j = J; j < 4; ++j) {
             const double2 row = *reinterpret_cast<const double2 *>(xs + 32 * j + 2 * t);
@@ -246,18 +291,138 @@ __device__ __forceinline__ void householder_block(double (&A)[8][8], Carry &R, E
         }
     }
 }
+
+// Steps 3 and 4 of unit u, its tridiagonal matrix in S.dd and S.ee, by a block of NT threads; TEAM lanes look for an eigenvalue.
+// CLUSTER: the CTAs of the cluster share the eigenvalues, the first of them collects.
+template <int NT, int TEAM, bool CLUSTER>
+__device__ __forceinline__ void finish_unit64(ValueSmem &S, int u, double trace, int k_trunc, int norm, int max_iters,
+                                              float *__restrict__ entropy, float *__restrict__ erank,
+                                              double *__restrict__ spectrum, uint32_t *__restrict__ status) {
+    constexpr int kCoarse = 2 * NT;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    double *lam = S.lam;
+    int *not_converged = &S.not_converged, rank = 0, ctas = 1;
+    if constexpr (CLUSTER) {
+        cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+        rank = (int)cluster.block_rank();
+        ctas = (int)cluster.num_blocks();
+        lam = cluster.map_shared_rank(S.lam, 0);
+        not_converged = cluster.map_shared_rank(&S.not_converged, 0);
+        cluster.sync();                                // the first CTA runs and has cleared its flag
+    }
+    // ---- 3. k largest eigenvalues by multi-section ------------------------------------------------
+    if (wid == 0) {
+        double rad = 0.0;   // Gershgorin radius as the scale
+        for (int i = lane; i < n; i += 32) {
+            const double left = i > 0 ? fabs(S.ee[i - 1]) : 0.0;
+            const double right = i < n - 1 ? fabs(S.ee[i]) : 0.0;
+            rad = fmax(rad, fabs(S.dd[i]) + left + right);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) rad = fmax(rad, __shfl_xor_sync(0xffffffffu, rad, o));
+        if (lane == 0) S.scale = rad > 0.0 ? rad : 1.0;
+    }
+    __syncthreads();
+    const double scale = S.scale, inv_scale = 1.0 / scale;
+    if (tid < n) {
+        const double e = tid > 0 ? S.ee[tid - 1] * inv_scale : 0.0;
+        S.de[tid] = make_double2(S.dd[tid] * inv_scale, -e * e);
+    }
+    __syncthreads();
+
+    // coarse round: counts at 2 NT interior points of [lo0, hi0], shared by all eigenvalues (C is positive semi-definite:
+    // what rounding leaves below lo0 is a zero eigenvalue)
+    const double lo0 = -0x1p-10, hi0 = 1.0 + 0x1p-40, step0 = (hi0 - lo0) / (double)(kCoarse + 1);
+    {
+        const double x[2] = {lo0 + step0 * (double)(2 * tid + 1), lo0 + step0 * (double)(2 * tid + 2)};
+        int c[2];
+        sturm_count<2>(S.de, x, c);
+        S.cnt[2 * tid + 1] = c[0];
+        S.cnt[2 * tid + 2] = c[1];
+    }
+    if (tid == 0) { S.cnt[0] = 0; S.cnt[kCoarse + 1] = n; }
+    __syncthreads();
+
+    // Teams of TEAM lanes, a point each, refine one eigenvalue.  A round is at least 9-fold and there is one more than asked
+    // for: at least what as many rounds give after a coarse round of 512 points.
+    static_assert(TEAM >= 8 && 9 * kCoarse >= 512, "");
+    const int k = min(k_trunc, n);
+    const int iters = (max_iters > 0 ? max_iters : 14) + 1;
+    const double tol = 1e-13;
+    const int sub = tid % TEAM, team0 = lane & ~(TEAM - 1);
+    const unsigned team_mask = (0xffffffffu >> (32 - TEAM)) << team0;
+    for (int j0 = rank * (NT / TEAM); j0 < k; j0 += ctas * (NT / TEAM)) {
+        const int j = j0 + tid / TEAM;              // this team looks for the j-th largest
+        const bool active = j < k;
+        const int idx = n - 1 - (active ? j : 0);   // its 0-based rank from below
+        int lo_i = 0, hi_i = kCoarse + 1;       // cnt[lo_i] <= idx < cnt[hi_i]
+        while (hi_i - lo_i > 1) {
+            const int mid = (lo_i + hi_i) >> 1;
+            if (S.cnt[mid] > idx) hi_i = mid; else lo_i = mid;
+        }
+        double lo = lo0 + step0 * (double)lo_i, hi = lo0 + step0 * (double)hi_i;
+        for (int it = 0; it < iters; ++it) {
+            const double width = (hi - lo) * (1.0 / (TEAM + 1));
+            const bool done = hi - lo <= tol;
+            if (__all_sync(0xffffffffu, done)) break;
+            const double x[1] = {lo + width * (double)(sub + 1)};
+            int c[1];
+            sturm_count<1>(S.de, x, c);
+            const unsigned above = (__ballot_sync(0xffffffffu, c[0] > idx) & team_mask) >> team0;
+            if (!done) {
+                const int f = above ? __ffs(above) - 1 : TEAM;          // first of the points above the eigenvalue
+                const double base_lo = lo;
+                if (f < TEAM) hi = base_lo + width * (double)(f + 1);
+                if (f > 0) lo = base_lo + width * (double)f;
+            }
+        }
+        if (active && sub == 0) {
+            lam[j] = 0.5 * (lo + hi) * scale;
+            if (hi - lo > tol) atomicOr(not_converged, 1);
+        }
+    }
+    if constexpr (CLUSTER) {
+        cooperative_groups::this_cluster().sync();
+        if (rank != 0) return;
+    } else __syncthreads();
+
+    // ---- 4. entropy -----------------------------------------------------------------------------
+    if (wid == 0) {      // lane i takes eigenvalues i, i + 32, ...; fixed-order butterfly sums
+        double total = trace;
+        if (!norm) {
+            total = 0.0;
+            for (int i = lane; i < k; i += 32) total += S.lam[i] > 0.0 ? S.lam[i] : 0.0;
+            total = warp_sum(total);
+        }
+        double h = 0.0;
+        if (total > 0.0) {
+            for (int i = lane; i < k; i += 32) {
+                const double p = (S.lam[i] > 0.0 ? S.lam[i] : 0.0) / total;
+                if (p > 0.0) h -= p * log(p);
+            }
+        }
+        h = warp_sum(h);
+        if (lane == 0) {
+            entropy[u] = (float)h;
+            if (erank) erank[u] = (float)exp(h);
+            if (S.not_converged) atomicOr(status, UNCOMP_STATUS_NOT_CONVERGED);
+        }
+    }
+    if (spectrum && tid < k) spectrum[(size_t)u * k + tid] = S.lam[tid];
+}
 }  // namespace
 
 template <typename PartialT>
 __global__ void __launch_bounds__(kEigThreads, 1)
-eigen_entropy_kernel(const PartialT *__restrict__ partials, int P, int N, int k_trunc, int center, int norm,
+eigen_entropy_kernel(PartialT *partials, int P, bool hand_over, int N, int k_trunc, int center, int norm,
                      int max_iters, float *__restrict__ entropy, float *__restrict__ erank,
                      double *__restrict__ spectrum, uint32_t *__restrict__ status) {
     __shared__ EigenSmem S;
+    __shared__ ValueSmem F;
     const int u = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int row0 = tid >> 4, t = tid & 15;
     constexpr int len = n * n + n;
-    const PartialT *base = partials + (size_t)u * P * len;
+    PartialT *base = partials + (size_t)u * P * len;
     chain_wait();
 
     // ---- 1. assemble C in registers ----------------------------------------------------------------
@@ -266,7 +431,7 @@ eigen_entropy_kernel(const PartialT *__restrict__ partials, int P, int N, int k_
         for (int p = 0; p < P; ++p) s += (double)base[(size_t)p * len + n * n + tid];
         S.sd[tid] = s;
     }
-    if (tid == 0) S.flags[0] = 0;
+    if (tid == 0) F.not_converged = 0;
     double A[8][8];
 #pragma unroll
     for (int a = 0; a < 8; ++a)
@@ -320,120 +485,45 @@ eigen_entropy_kernel(const PartialT *__restrict__ partials, int P, int N, int k_
             R.xc[q] = S.x[1][32 * (q >> 1) + 2 * t + (q & 1)];
         }
         R.x0 = S.x[1][1];
-        if (tid == 0) S.dd[0] = S.x[1][0];
+        if (tid == 0) F.dd[0] = S.x[1][0];
         if (t == 0) R.xc[0] = 0.0;
-        householder_block<0>(A, R, S, lane, wid);
-        householder_block<1>(A, R, S, lane, wid);
-        householder_block<2>(A, R, S, lane, wid);
-        householder_block<3>(A, R, S, lane, wid);
-        householder_block<4>(A, R, S, lane, wid);
-        householder_block<5>(A, R, S, lane, wid);
-        householder_block<6>(A, R, S, lane, wid);
-        householder_block<7>(A, R, S, lane, wid);
-        if (tid == 0) { S.ee[n - 2] = R.x0; S.ee[n - 1] = 0.0; }
+        householder_block<0>(A, R, S, F, lane, wid);
+        householder_block<1>(A, R, S, F, lane, wid);
+        householder_block<2>(A, R, S, F, lane, wid);
+        householder_block<3>(A, R, S, F, lane, wid);
+        householder_block<4>(A, R, S, F, lane, wid);
+        householder_block<5>(A, R, S, F, lane, wid);
+        householder_block<6>(A, R, S, F, lane, wid);
+        householder_block<7>(A, R, S, F, lane, wid);
+        if (tid == 0) { F.ee[n - 2] = R.x0; F.ee[n - 1] = 0.0; }
         if (row0 == 15 && t == 15)                     // entry (127, 127) after the last update
-            S.dd[n - 1] = fma(R.vr[7], R.wc[7], fma(R.wr[7], R.vc[7], A[7][7]));
+            F.dd[n - 1] = fma(R.vr[7], R.wc[7], fma(R.wr[7], R.vc[7], A[7][7]));
     }
     __syncthreads();
 
-    // ---- 3. k largest eigenvalues by multi-section ------------------------------------------------
-    if (wid == 0) {
-        double rad = 0.0;   // Gershgorin radius as the scale
-        for (int i = lane; i < n; i += 32) {
-            const double left = i > 0 ? fabs(S.ee[i - 1]) : 0.0;
-            const double right = i < n - 1 ? fabs(S.ee[i]) : 0.0;
-            rad = fmax(rad, fabs(S.dd[i]) + left + right);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) rad = fmax(rad, __shfl_xor_sync(0xffffffffu, rad, o));
-        if (lane == 0) S.scale = rad > 0.0 ? rad : 1.0;
+    if (hand_over) {
+        EigenBand64 *out = reinterpret_cast<EigenBand64 *>(base);
+        if (tid < n) { out->dd[tid] = F.dd[tid]; out->ee[tid] = F.ee[tid]; }
+        if (tid == 0) out->trace = S.trace;
+        return;
     }
-    __syncthreads();
-    const double scale = S.scale, inv_scale = 1.0 / scale;
-    if (tid < n) {
-        const double e = tid > 0 ? S.ee[tid - 1] * inv_scale : 0.0;
-        S.de[tid] = make_double2(S.dd[tid] * inv_scale, -e * e);
-    }
-    __syncthreads();
+    finish_unit64<kEigThreads, 8, false>(F, u, S.trace, k_trunc, norm, max_iters, entropy, erank, spectrum, status);
+}
 
-    // coarse round: counts at 512 interior points of [lo0, hi0], shared by all eigenvalues (C is positive semi-definite:
-    // what rounding leaves below lo0 is a zero eigenvalue)
-    const double lo0 = -0x1p-10, hi0 = 1.0 + 0x1p-40, step0 = (hi0 - lo0) / (double)(kCoarse + 1);
-    {
-        const double x[2] = {lo0 + step0 * (double)(2 * tid + 1), lo0 + step0 * (double)(2 * tid + 2)};
-        int c[2];
-        sturm_count<2>(S.de, x, c);
-        S.cnt[2 * tid + 1] = c[0];
-        S.cnt[2 * tid + 2] = c[1];
-    }
-    if (tid == 0) { S.cnt[0] = 0; S.cnt[kCoarse + 1] = n; }
+// Steps 3 and 4 of few units: a cluster of 8, 4 or 2 CTAs per unit.
+template <int TEAM>
+__global__ void __launch_bounds__(kValueThreads)
+eigen_values64_kernel(const char *__restrict__ partials, int64_t unit_stride, int k_trunc, int norm, int max_iters,
+                      float *__restrict__ entropy, float *__restrict__ erank, double *__restrict__ spectrum, uint32_t *__restrict__ status) {
+    __shared__ ValueSmem F;
+    const int u = blockIdx.x / cooperative_groups::this_cluster().num_blocks(), tid = threadIdx.x;
+    chain_wait();
+    const EigenBand64 &E = *reinterpret_cast<const EigenBand64 *>(partials + u * unit_stride);
+    F.dd[tid] = E.dd[tid];
+    F.ee[tid] = E.ee[tid];
+    if (tid == 0) F.not_converged = 0;
     __syncthreads();
-
-    // teams of 4 lanes, two points each, refine one eigenvalue: 9-fold per round.  128 threads keep the fp64 units busy;
-    // with more, the broadcast loads of the matrix would be the limit.
-    const int k = min(k_trunc, n);
-    const int iters = max_iters > 0 ? max_iters : 14;
-    const double tol = 1e-13;
-    const int sub = tid & 3;
-    const unsigned team_mask = 0xfu << (lane & 28);
-    for (int j0 = 0; tid < kTeamThreads && j0 < k; j0 += kTeamThreads / 4) {
-        const int j = j0 + (tid >> 2);              // this team looks for the j-th largest
-        const bool active = j < k;
-        const int idx = n - 1 - (active ? j : 0);   // its 0-based rank from below
-        int lo_i = 0, hi_i = kCoarse + 1;       // cnt[lo_i] <= idx < cnt[hi_i]
-        while (hi_i - lo_i > 1) {
-            const int mid = (lo_i + hi_i) >> 1;
-            if (S.cnt[mid] > idx) hi_i = mid; else lo_i = mid;
-        }
-        double lo = lo0 + step0 * (double)lo_i, hi = lo0 + step0 * (double)hi_i;
-        for (int it = 0; it < iters; ++it) {
-            const double width = (hi - lo) * (1.0 / 9.0);
-            const bool done = hi - lo <= tol;
-            if (__all_sync(0xffffffffu, done)) break;
-            const double x[2] = {lo + width * (double)(2 * sub + 1), lo + width * (double)(2 * sub + 2)};
-            int c[2];
-            sturm_count<2>(S.de, x, c);
-            const unsigned above_a = (__ballot_sync(0xffffffffu, c[0] > idx) & team_mask) >> (lane & 28);
-            const unsigned above_b = (__ballot_sync(0xffffffffu, c[1] > idx) & team_mask) >> (lane & 28);
-            if (!done) {
-                // first of the 8 points above the eigenvalue (points 2 s + 1 and 2 s + 2 sit in lane s)
-                const int fa = above_a ? 2 * (__ffs(above_a) - 1) : 8, fb = above_b ? 2 * (__ffs(above_b) - 1) + 1 : 8;
-                const int f = min(fa, fb);
-                const double base_lo = lo;
-                if (f < 8) hi = base_lo + width * (double)(f + 1);
-                if (f > 0) lo = base_lo + width * (double)f;
-            }
-        }
-        if (active && sub == 0) {
-            S.lam[j] = 0.5 * (lo + hi) * scale;
-            if (hi - lo > tol) atomicOr(&S.flags[0], 1);
-        }
-    }
-    __syncthreads();
-
-    // ---- 4. entropy -----------------------------------------------------------------------------
-    if (wid == 0) {      // lane i takes eigenvalues i, i + 32, ...; fixed-order butterfly sums
-        double total = S.trace;
-        if (!norm) {
-            total = 0.0;
-            for (int i = lane; i < k; i += 32) total += S.lam[i] > 0.0 ? S.lam[i] : 0.0;
-            total = warp_sum(total);
-        }
-        double h = 0.0;
-        if (total > 0.0) {
-            for (int i = lane; i < k; i += 32) {
-                const double p = (S.lam[i] > 0.0 ? S.lam[i] : 0.0) / total;
-                if (p > 0.0) h -= p * log(p);
-            }
-        }
-        h = warp_sum(h);
-        if (lane == 0) {
-            entropy[u] = (float)h;
-            if (erank) erank[u] = (float)exp(h);
-            if (S.flags[0]) atomicOr(status, UNCOMP_STATUS_NOT_CONVERGED);
-        }
-    }
-    if (spectrum && tid < k) spectrum[(size_t)u * k + tid] = S.lam[tid];
+    finish_unit64<kValueThreads, TEAM, true>(F, u, E.trace, k_trunc, norm, max_iters, entropy, erank, spectrum, status);
 }
 
 // Sum of the chunk partials of every unit in chunk order: out[u] = [G (d*d) | s (d)] in fp64.
@@ -457,15 +547,27 @@ cudaError_t launch_gram_reduce(const Plan &p, const void *d_partials, double *d_
     return cudaGetLastError();
 }
 
-cudaError_t launch_eigen_entropy(const Plan &p, const void *d_partials, const uncomp_entropy_params &ep,
-                                 float *d_entropy, float *d_erank, double *d_spectrum, uint32_t *d_status,
-                                 cudaStream_t st) {
+cudaError_t launch_eigen_entropy(const Plan &p, void *d_partials, const uncomp_entropy_params &ep, float *d_entropy, float *d_erank,
+                                 double *d_spectrum, uint32_t *d_status, cudaStream_t st) {
+    // Few units: the eigenvalues in a kernel of their own, a cluster of CTAs per unit, while each CTA has an SM to itself.
+    // In the first kernel they take 28 us of one SM per unit, here 15 with eight CTAs of 128 threads (19 with 256 threads: two
+    // warps share a sub-partition's fp64 unit); passes of 8 / 32 / 64 units of 512 tokens 198 -> 186, 241 -> 232, 294 -> 287 us.
+    int ctas = 1;
+    while (ctas < 8 && p.units * ctas * 2 <= kTargetSms) ctas *= 2;
+    const bool wide = p.shape.dtype == UNCOMP_FP32;    // fp64 partials
     const LaunchShape shape{dim3(p.units), kEigThreads, 0, 1, true};
-    if (p.shape.dtype == UNCOMP_FP32)
-        return launch_kernel(eigen_entropy_kernel<double>, shape, st, (const double *)d_partials, p.gram_splits, p.shape.N,
-                             ep.k_trunc, ep.center, ep.norm, ep.max_iters, d_entropy, d_erank, d_spectrum, d_status);
-    return launch_kernel(eigen_entropy_kernel<float>, shape, st, (const float *)d_partials, p.gram_splits, p.shape.N, ep.k_trunc,
-                         ep.center, ep.norm, ep.max_iters, d_entropy, d_erank, d_spectrum, d_status);
+    cudaError_t e;
+    if (wide)
+        e = launch_kernel(eigen_entropy_kernel<double>, shape, st, (double *)d_partials, p.gram_splits, ctas > 1, p.shape.N,
+                          ep.k_trunc, ep.center, ep.norm, ep.max_iters, d_entropy, d_erank, d_spectrum, d_status);
+    else
+        e = launch_kernel(eigen_entropy_kernel<float>, shape, st, (float *)d_partials, p.gram_splits, ctas > 1, p.shape.N, ep.k_trunc,
+                          ep.center, ep.norm, ep.max_iters, d_entropy, d_erank, d_spectrum, d_status);
+    if (e != cudaSuccess || ctas == 1) return e;
+    const int64_t stride = (int64_t)p.gram_splits * (n * n + n) * (wide ? sizeof(double) : sizeof(float));
+    return launch_kernel(ctas == 8 ? eigen_values64_kernel<16> : eigen_values64_kernel<8>,
+                         LaunchShape{dim3(p.units * ctas), kValueThreads, 0, (unsigned)ctas, true}, st, (const char *)d_partials, stride,
+                         ep.k_trunc, ep.norm, ep.max_iters, d_entropy, d_erank, d_spectrum, d_status);
 }
 
 }  // namespace uncomp

@@ -248,7 +248,7 @@ eigen_tail_kernel(const float *__restrict__ partials, int64_t unit_stride, int u
         }
     }
     __syncwarp();
-    finish_unit<32>(S, u, lane, true, E.trace, k_trunc, norm, max_iters, entropy, erank, spectrum, status);
+    finish_unit<32, 1, false>(S, u, lane, true, E.trace, k_trunc, norm, max_iters, entropy, erank, spectrum, status);
 }
 
 cudaError_t launch_eigen_tail(int units, float *d_partials, int partials_per_unit, const uncomp_entropy_params &ep,

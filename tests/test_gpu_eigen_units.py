@@ -1,0 +1,34 @@
+"""Eigenvalues over the numbers of units at which the split of a unit over CTAs changes, against fp64 on the CPU."""
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("units", [1, 18, 19, 37, 38, 74, 75])
+def test_spectrum_over_unit_counts(units, dtype):
+    from paper_2410_03090_b200 import binding as ub
+
+    N = 160
+    torch.manual_seed(units)
+    K = torch.randn(1, units, 1, N, 128, device="cuda") * torch.logspace(0, -2, 128, device="cuda")
+    K = K.to(torch.float32 if dtype == "fp32" else torch.bfloat16)
+    X = K[0, :, 0].double().cpu()
+    X = X - X.mean(1, keepdim=True)
+    want = torch.linalg.eigvalsh(X.transpose(1, 2) @ X).flip(1).clamp(min=0)
+    ctx = ub.Context(ub.make_shape(1, units, 1, 1, N, 128, 32, dtype))
+    for k in (1, 33, 128):
+        spectrum = torch.empty(1, units, 1, k, dtype=torch.float64, device="cuda")
+        ent, erank = ub.uncomp_entropy(ctx, K, k, spectrum=spectrum)
+        assert ub.uncomp_status(ctx) == 0
+        lam = spectrum[0, :, 0].cpu()
+        # brackets of 1e-13 (fp32 keys) and 2e-8 of the Gershgorin radius, at most three times the largest eigenvalue of a
+        # tridiagonal matrix; the reductions: 128 steps of 2^-53 and, with the fp32 partials, of 2^-24
+        bound = 3e-13 + 128 * 2.0 ** -53 if dtype == "fp32" else 6e-8 + 128 * 2.0 ** -24
+        assert float(((lam - want[:, :k]).abs() / want[:, :1]).max()) < bound
+        p = want[:, :k] / want[:, :k].sum(1, keepdim=True)
+        H = -(p * p.clamp(min=1e-300).log()).sum(1)
+        assert float((ent[0, :, 0].double().cpu() - H).abs().max()) < 1e-4
+        assert torch.allclose(erank, ent.exp(), rtol=1e-5)
