@@ -12,7 +12,8 @@
 // groups (remainder, heads ahead of the group) and a head's rank inside its group; S and the number of missing tokens
 // come from the host; ranks are counted in shared memory; the prefix sum is one of warps.  With 64-bit divisions in every
 // thread, remainders compared head by head in global memory and a scan with 20 barriers 256 units took 15 us
-// (of which 9 are the launch and its event records), now 11.
+// (of which 9 are the launch and its event records), now 11.  The table of the groups is made before the effective ranks are
+// there: the kernels of the eigenvalues let this one start when all of theirs run (passes of few units 2.4 us shorter).
 #include "common.cuh"
 
 namespace uncomp {
@@ -53,9 +54,7 @@ __global__ void __launch_bounds__(kBudThreads) budgets_kernel(const float *__res
     float *er_s = reinterpret_cast<float *>(shared_tab ? reinterpret_cast<int32_t *>(bud_smem + M) + M
                                                        : reinterpret_cast<int32_t *>(bud_smem));
     const float *er = shared_er ? er_s : erank;
-    chain_wait();
-    if (shared_er)
-        for (int u = tid; u < units; u += kBudThreads) er_s[u] = erank[u];
+    if (!shared_tab) chain_wait();                     // the scratch may still be read
     auto target = [&](int g) { return n_max * S - (int64_t)g * n * (n_max - avg); };   // t_g S
     for (int g = tid; g < M; g += kBudThreads) rem_t[g] = M == 1 ? 0 : target(g) % S;
     __syncthreads();
@@ -70,6 +69,11 @@ __global__ void __launch_bounds__(kBudThreads) budgets_kernel(const float *__res
         ahead_t[g] = ahead;
     }
     __syncthreads();
+    chain_wait();                                      // what came before depends on the parameters alone
+    if (shared_er) {
+        for (int u = tid; u < units; u += kBudThreads) er_s[u] = erank[u];
+        __syncthreads();
+    }
     // budgets and their exclusive prefix sum over the units, 1024 units at a time
     int64_t carry = 0;
     if (tid == 0) offsets[0] = 0;

@@ -139,8 +139,11 @@ inline cudaError_t allow_dynamic_smem(const void *fn, size_t bytes, bool (&done)
 // take places early, and the kernels that fill the registers of an SM lost by it more than the launches cost.  Launches
 // with full serialization / signal at the start / at the end, back to back: fp32 pass of 512 tokens 251 / 248 / 232 us, one
 // layer of 7001 tokens 146 / 160 / 129, 256 units of 8192 tokens 427 / 453 / 414, 1024 of 3712 836 / 862 / 819, a decode
-// step on 256 caches of 410 rows 11.1 / 9.4 / 9.4.
+// step on 256 caches of 410 rows 11.1 / 9.4 / 9.4.  The exception are the kernels that end the eigenvalues of up to 296
+// units: next are the budgets, one CTA with work that depends on nothing (the table of the groups); a signal is no promise
+// about memory, chain_wait() still waits for the end.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_signal() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 struct LaunchShape {
     dim3 grid;

@@ -518,6 +518,7 @@ eigen_values64_kernel(const char *__restrict__ partials, int64_t unit_stride, in
     __shared__ ValueSmem F;
     const int u = blockIdx.x / cooperative_groups::this_cluster().num_blocks(), tid = threadIdx.x;
     chain_wait();
+    chain_signal();
     const EigenBand64 &E = *reinterpret_cast<const EigenBand64 *>(partials + u * unit_stride);
     F.dd[tid] = E.dd[tid];
     F.ee[tid] = E.ee[tid];
