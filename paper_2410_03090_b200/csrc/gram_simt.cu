@@ -13,9 +13,12 @@
 namespace uncomp {
 
 // fp32 keys.  Grid: (units x 10 tile pairs I <= J of 32 x 32 entries, token chunks): the symmetric half, and enough CTAs
-// for calls of few units and few tokens (one CTA per unit and chunk took 126 us for 8 units of 512 tokens, this 17 us).
+// for calls of few units and few tokens (one CTA per unit and chunk took 126 us for 8 units of 512 tokens, this 13 us).
 // A quarter of the CTA takes every fourth token; a thread owns 4 x 4 entries, so four 16-byte loads feed 16 fp64
-// multiply-adds.  Those loads bound it: shared memory at 77 % of its rate, the fp64 pipe at 23 %.
+// multiply-adds.  The columns are two neighbours in each half of the block: eight lanes read 128 contiguous bytes (four
+// neighbours are a two-way bank conflict and made shared memory the bound, at 77 % of its rate with the fp64 pipe at 23 %).
+// With the column sums spread over the warps: 8 units of 512 tokens 15.2 -> 12.8 us, the pass of 32 units of 8192 tokens
+// 926 -> 840.
 __global__ void __launch_bounds__(256) gram_f64_kernel(const float *__restrict__ K, UnitAddr addr, int N, int chunk,
                                                       double *__restrict__ partials, int P) {
     constexpr int TT = 32;
@@ -62,16 +65,16 @@ __global__ void __launch_bounds__(256) gram_f64_kernel(const float *__restrict__
         for (int k = 0; k < TT / 4; ++k) {
             const int tok = 4 * k + g;
             const double2 a0 = *reinterpret_cast<const double2 *>(tI + tok * 32 + 4 * ty), a1 = *reinterpret_cast<const double2 *>(tI + tok * 32 + 4 * ty + 2);
-            const double2 b0 = *reinterpret_cast<const double2 *>(tJ + tok * 32 + 4 * tx), b1 = *reinterpret_cast<const double2 *>(tJ + tok * 32 + 4 * tx + 2);
+            const double2 b0 = *reinterpret_cast<const double2 *>(tJ + tok * 32 + 2 * tx), b1 = *reinterpret_cast<const double2 *>(tJ + tok * 32 + 16 + 2 * tx);
             const double a[4] = {a0.x, a0.y, a1.x, a1.y}, c[4] = {b0.x, b0.y, b1.x, b1.y};
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], c[j], acc[i][j]);
         }
-        if (I == J && tid < 32) {
-#pragma unroll 8
-            for (int tok = 0; tok < TT; ++tok) colsum += tI[tok * 32 + tid];
+        if (I == J) {                                  // a warp per four tokens, a lane per column
+#pragma unroll
+            for (int i = 0; i < TT / 8; ++i) colsum += tI[((tid >> 5) * (TT / 8) + i) * 32 + (tid & 31)];
         }
         if (t + TT < t1) store(b ^ 1);
         __syncthreads();
@@ -80,7 +83,7 @@ __global__ void __launch_bounds__(256) gram_f64_kernel(const float *__restrict__
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) smem[(g * 32 + 4 * ty + i) * 32 + 4 * tx + j] = acc[i][j];
+        for (int j = 0; j < 4; ++j) smem[(g * 32 + 4 * ty + i) * 32 + 2 * tx + (j & 1) + 8 * (j & 2)] = acc[i][j];
     __syncthreads();
     double *out = partials + ((size_t)u * P + p) * (kD * kD + kD);
 #pragma unroll
@@ -90,7 +93,17 @@ __global__ void __launch_bounds__(256) gram_f64_kernel(const float *__restrict__
         out[(32 * I + i) * kD + 32 * J + j] = v;
         if (I != J) out[(32 * J + j) * kD + 32 * I + i] = v;
     }
-    if (I == J && tid < 32) out[kD * kD + 32 * I + tid] = colsum;
+    if (I == J) {
+        __syncthreads();
+        smem[tid] = colsum;
+        __syncthreads();
+        if (tid < 32) {
+            double sum = 0.0;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) sum += smem[32 * i + tid];
+            out[kD * kD + 32 * I + tid] = sum;
+        }
+    }
 }
 
 // Grid: (P token chunks, units).  A CTA of 256 threads streams its chunk in tiles of 32 tokens through shared memory;
