@@ -909,6 +909,7 @@ band_eigen_kernel(int k, int q, int max_iters, KrylovBuffers B, uint32_t *__rest
     chain_wait();
     // flags and eigenvalues are read by the NEXT launch
     if (B.state[1] || B.state[0] != q) return;    // uniform over the grid
+    cluster.barrier_arrive();                     // waited for before anybody's shared memory is written
     const double *T = B.T;
     const BandCoarse *in = reinterpret_cast<const BandCoarse *>(B.part);
     const double bound = in->bound, tiny = bound * 1e-19;
@@ -922,6 +923,7 @@ band_eigen_kernel(int k, int q, int max_iters, KrylovBuffers B, uint32_t *__rest
     atomicMin(&s_first, first);
     __syncthreads();
     first = s_first;
+    cluster.barrier_wait();                       // every CTA runs
     if (first > 0) lo = in->shift[first - 1];
     if (first < kCoarse) hi = in->shift[first];
     int c_lo = first > 0 ? in->count[first - 1] : 0, c_hi = first < kCoarse ? in->count[first] : m;
