@@ -31,15 +31,15 @@ if ROOT not in sys.path:
 # recorded beside them: when the file has changed since the capture, the bench prints null instead.
 NCU_COUNTERS = {
     "source": "paper_2410_03090_b200/csrc/scores_tc.cu",
-    "sha256": "0e2c45c81c8ffff40991394f6f22e53355b5a0b799a041c1ef1e5f0eb831fbc4",
+    "sha256": "63ec9cc4ca159417c73a7a1b5d6a6475d335ea14ff2ec4b43a4276ee1c29d6a2",
     "capture": "ncu --set full, one launch per kernel, c3 scaled to N 16384 x 10 layers; summary in profiles/",
     "kernels": {
-        "gram_score_stats": {"dram_bytes_per_unit_token": (344.463872e6 + 29.947904e6) / (80 * 16384),
-                             "tensor_pipe_pct": 48.3, "xu_pipe_pct": 65.9},
-        "score_colsum": {"dram_bytes_per_unit_token": (346.776320e6 + 8.228864e6) / (80 * 16384),
-                         "tensor_pipe_pct": 37.5, "xu_pipe_pct": 75.5},
-        "gram_score_colsum": {"dram_bytes_per_unit_token": (345.744640e6 + 34.919168e6) / (80 * 16384),
-                              "tensor_pipe_pct": 45.6, "xu_pipe_pct": 61.2},
+        "gram_score_stats": {"dram_bytes_per_unit_token": (344.470528e6 + 31.993088e6) / (80 * 16384),
+                             "tensor_pipe_pct": 53.9, "xu_pipe_pct": 70.6},
+        "score_colsum": {"dram_bytes_per_unit_token": (346.816000e6 + 11.107584e6) / (80 * 16384),
+                         "tensor_pipe_pct": 37.8, "xu_pipe_pct": 76.1},
+        "gram_score_colsum": {"dram_bytes_per_unit_token": (345.092096e6 + 34.181632e6) / (80 * 16384),
+                              "tensor_pipe_pct": 54.6, "xu_pipe_pct": 70.3},
     },
 }
 EXP_KERNELS = ("score_stats", "score_colsum", "gram_score_stats", "gram_score_colsum")
