@@ -697,6 +697,7 @@ __device__ __forceinline__ void band_sweep(BandWindow &W, int halves, const doub
         cp_wait<kRing - 1>();
         __syncwarp();
         fetch(kB);
+        __syncwarp();                             // row 0 loads column kB + kRing into the place of column kB
     }
 #pragma unroll 1
     for (int r0 = 0; r0 < 16 * halves; r0 += kB) {

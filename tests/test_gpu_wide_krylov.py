@@ -112,3 +112,18 @@ def test_few_rounds_are_reported():
     assert ub.uncomp_status(ctx) & 1
     ub.uncomp_entropy_wide(ctx, X, 32, max_iters=6)          # 257^6 > 1e13
     assert ub.uncomp_status(ctx) == 0
+
+
+@pytest.mark.parametrize("N,D,k", [(900, 384, 32), (1300, 1024, 64)])
+def test_repeated_calls_agree_bit_for_bit(N, D, k):
+    """The counts stream the band through small rings in shared memory, whose places are taken again as soon as a column has
+    been read: every call has to see the same columns."""
+    from paper_2410_03090_b200 import binding as ub
+    X = tw._matrix(1, N, D, 100, 0.1, seed=D)
+    ctx = ub.Context(ub.make_shape(1, 1, 1, 1, 256, 128, 8, "bf16"))
+    ent, _, spec = ub.uncomp_entropy_wide(ctx, X, k, spectrum=True)
+    for _ in range(60):
+        again, _, lam = ub.uncomp_entropy_wide(ctx, X, k, spectrum=True)
+        assert torch.equal(again, ent) and torch.equal(lam, spec)
+    assert ub.uncomp_status(ctx) == 0
+    tw._check(ub, X, k, 1, 0)
