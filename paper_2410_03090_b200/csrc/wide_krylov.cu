@@ -361,10 +361,12 @@ __device__ __forceinline__ void project_gram(LanczosSmem &S, const float *H, int
 }
 
 // S.gram = L D L^T by elimination beside the identity; Rinv = L^-T D^-1/2 and R = D^1/2 L^T, so that W Rinv has orthonormal
-// columns and W = (W Rinv) R.  Thread: column tid mod 64 of [G | I], eight rows in registers.  Two pivots at a time, by the
-// inverse of their 2 x 2 block: one barrier, one exchange and one reciprocal on the chain where single pivots take two (5.7
-// us, now 3.4).  `bad`: a pivot is below `share` of the bound of its row (its own entry of `before`, or the largest diagonal
-// entry without one).
+// columns and W = (W Rinv) R.  Thread: column tid mod 64 of [G | I], eight rows in registers.  Two pivots at a time: one
+// barrier, one exchange and one reciprocal on the chain where single pivots take two (5.7 us, now 3.4); the second pivot's
+// reciprocal comes from their determinant, but the rows are eliminated one after the other.  (With the inverse of the 2 x 2
+// block, whose entries grow with one over the ratio of its pivots, a block of which one direction is 1e10 times the others
+// lost the others, and matrices of rank 33 ended in the full reduction.)  False when a pivot is below `share` of the bound
+// of its row (its own entry of `before`, or the largest diagonal entry without one).
 __device__ __forceinline__ bool factorise(LanczosSmem &S, float (*R)[kB], const double *before, double share) {
     const int tid = threadIdx.x, col = tid & 63, rq = tid >> 6;
     double v[kB / 4], top = 0.0;
@@ -395,11 +397,14 @@ __device__ __forceinline__ bool factorise(LanczosSmem &S, float (*R)[kB], const 
         const bool ok = a > lim0 && det > lim1 * a;               // the same in every thread
         good = good && ok;
         const double ia = ok ? recip_newton(a) : 0.0, id = ok ? recip_newton(det) : 0.0;
-        const double f0 = -fma(c, u0, -b * u1) * id, f1 = -fma(a, u1, -b * u0) * id;
+        const double l = -b * ia, w1 = fma(l, u0, u1), f0 = -u0 * ia, f1 = -w1 * (a * id);      // w1: row s + 1 without row s
 #pragma unroll
         for (int q = s >> 2; q < kB / 4; ++q)
-            if (rq + 4 * q > s + 1) v[q] = fma(P[1][2 * kB + 8 * rq + q], f1, fma(P[0][2 * kB + 8 * rq + q], f0, v[q]));
-        if (rq == ((s + 1) & 3)) v[s >> 2] = fma(-b * ia, u0, v[s >> 2]);       // the second pivot's own row
+            if (rq + 4 * q > s + 1) {
+                const double p0 = P[0][2 * kB + 8 * rq + q];
+                v[q] = fma(fma(l, p0, P[1][2 * kB + 8 * rq + q]), f1, fma(p0, f0, v[q]));
+            }
+        if (rq == ((s + 1) & 3)) v[s >> 2] = w1;
         if (tid == s) S.diag[s] = a;
         if (tid == s + 1) S.diag[s + 1] = det * ia;
     }

@@ -127,3 +127,25 @@ def test_repeated_calls_agree_bit_for_bit(N, D, k):
         assert torch.equal(again, ent) and torch.equal(lam, spec)
     assert ub.uncomp_status(ctx) == 0
     tw._check(ub, X, k, 1, 0)
+
+
+def _lanczos_settled(ub, X, k):
+    """Correct, and without the full reduction: its kernels leave at once (some microseconds; 2.5 ms and more otherwise)."""
+    tw._check(ub, X, k, 1, 0)
+    ctx = ub.Context(ub.make_shape(1, 1, 1, 1, 256, 128, 8, "bf16"))
+    ub.uncomp_entropy_wide(ctx, X, k)
+    ub.uncomp_profile_enable(ctx, True)
+    ub.uncomp_entropy_wide(ctx, X, k)
+    ms, launches = ub.uncomp_profile_read(ctx)["wide_tridiag"]
+    assert ub.uncomp_status(ctx) == 0 and launches == 1 and ms < 0.5, ms
+
+
+@pytest.mark.parametrize("rank", [33, 34, 65])
+def test_rank_just_above_a_block(rank):
+    """The second or third block has one or two directions left and rounding, 1e-5 of them, in the others: its Gram matrix
+    has pivots of 1e-10 of its entries."""
+    from paper_2410_03090_b200 import binding as ub
+    g = torch.Generator(device="cuda").manual_seed(rank)
+    W = torch.randint(-1, 2, (rank, 1024), generator=g, device="cuda") * (torch.rand(rank, 1024, generator=g, device="cuda") < 8.0 / rank)
+    X = (torch.randint(-2, 3, (3000, rank), generator=g, device="cuda").float() @ (4.0 * W)).clamp(-250, 250)
+    _lanczos_settled(ub, X.to(torch.bfloat16)[None], 32)
