@@ -149,3 +149,14 @@ def test_rank_just_above_a_block(rank):
     W = torch.randint(-1, 2, (rank, 1024), generator=g, device="cuda") * (torch.rand(rank, 1024, generator=g, device="cuda") < 8.0 / rank)
     X = (torch.randint(-2, 3, (3000, rank), generator=g, device="cuda").float() @ (4.0 * W)).clamp(-250, 250)
     _lanczos_settled(ub, X.to(torch.bfloat16)[None], 32)
+
+
+@pytest.mark.parametrize("used,decay", [(48, 1.0), (80, 0.0), (130, 3.0), (200, 1.0), (300, 3.0)])
+def test_features_that_are_all_zero(used, decay):
+    """The rank is used up after a few blocks: what the next one keeps of its columns differs by 1e8 in length."""
+    from paper_2410_03090_b200 import binding as ub
+    g = torch.Generator(device="cuda").manual_seed(used)
+    X = torch.zeros(3000, 1024, device="cuda")
+    X[:, torch.randperm(1024, generator=g, device="cuda")[:used]] = (
+        6 * torch.randn(3000, used, generator=g, device="cuda") * torch.exp(-decay * torch.arange(used, device="cuda") / used)).round()
+    _lanczos_settled(ub, X.to(torch.bfloat16)[None], 32)
