@@ -65,7 +65,7 @@ struct LanczosSmem {
     };
     double piv[2][2][3 * kB];                     // two pivot rows (64 columns) and pivot columns of the factorisation
     double gram[kB * kB];                         // of the block before normalisation
-    float U[kB * kB], V[kB * kB];
+    double V[kB * kB];                            // of the second factorisation: R - I
     float tile[kCached][kB][kB];                  // this CTA's rows of the basis: tile[block][vector][row]
     float Wt[kB][kB + 4];                         // the CTA's rows of W, transposed: Wt[b][r]
     float Rinv[kB][kB];
@@ -330,11 +330,11 @@ __device__ __forceinline__ void load_gram(LanczosSmem &S, const double *G) {
 // H stays staged when one chunk holds it.
 __device__ __forceinline__ void project_gram(LanczosSmem &S, const float *H, int nq) {
     const int tid = threadIdx.x, part = tid >> 6, ty = (tid >> 3) & 7, tx = tid & 7;
-    float acc[4][4];
+    double acc[4][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
     for (int b0 = 0; b0 < nq; b0 += kHChunk) {
         const int nb = min(kHChunk, nq - b0);
         if (b0 > 0) __syncthreads();
@@ -342,11 +342,11 @@ __device__ __forceinline__ void project_gram(LanczosSmem &S, const float *H, int
 #pragma unroll 4
         for (int r = part; r < nb * kB; r += 4) {
             const float4 x = *reinterpret_cast<const float4 *>(S.H + r * kB + 4 * ty), y = *reinterpret_cast<const float4 *>(S.H + r * kB + 4 * tx);
-            const float xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
+            const double xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(xs[i], ys[j], acc[i][j]);
+                for (int j = 0; j < 4; ++j) acc[i][j] = fma(xs[i], ys[j], acc[i][j]);
         }
     }
     for (int p = 0; p < 4; ++p) {
@@ -354,7 +354,7 @@ __device__ __forceinline__ void project_gram(LanczosSmem &S, const float *H, int
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) S.gram[(4 * ty + i) * kB + 4 * tx + j] -= (double)acc[i][j];
+                for (int j = 0; j < 4; ++j) S.gram[(4 * ty + i) * kB + 4 * tx + j] -= acc[i][j];
         }
         __syncthreads();
     }
@@ -421,47 +421,61 @@ __device__ __forceinline__ bool factorise(LanczosSmem &S, float (*R)[kB], const 
     return true;
 }
 
-// The same for a Gram matrix within 1e-3 of the identity, I + E: with U = upper(E), the diagonal halved, R = I + U - upper(U^T U)
-// and Rinv = I - V + V V, V = R - I, up to E^3.  (What a block's first normalisation leaves is within 1e-4 of the identity as
-// a rule.)  Everything here is small against 1, so fp32 carries it.
+// The same for a Gram matrix within 1e-4 of the identity, I + E: with U = upper(E), the diagonal halved, R = I + U - upper(U^T U)
+// and Rinv = I - V + V V, V = R - I, up to E^3, which is 3e-8 at most.  (That is what a block's first normalisation leaves as
+// a rule.)  U and V^T take the place of the Gram matrix; a thread 2 x 2 entries, so that two loads of 16 bytes feed four
+// multiply-adds (1 x 4: 3 us more, shared memory).
 __device__ __forceinline__ bool nearly_orthonormal(LanczosSmem &S) {
     bool near = true;
-    for (int e = threadIdx.x; e < kB * kB; e += kLT) near = near && fabs(S.gram[e] - (e / kB == e % kB ? 1.0 : 0.0)) < 1e-3;
+    for (int e = threadIdx.x; e < kB * kB; e += kLT) near = near && fabs(S.gram[e] - (e / kB == e % kB ? 1.0 : 0.0)) < 1e-4;
     return __syncthreads_and(near) != 0;
 }
 __device__ __forceinline__ void factorise_near(LanczosSmem &S, float (*R)[kB]) {
-    const int tid = threadIdx.x, r = tid >> 3, c0 = 4 * (tid & 7);          // entries (r, c0 .. c0 + 3)
-    float *U = S.U;
+    const int tid = threadIdx.x, r0 = 2 * (tid >> 4), c0 = 2 * (tid & 15);  // entries (r0, c0) .. (r0 + 1, c0 + 1)
+    double *U = S.gram, *Vt = S.gram;
+    auto pair = [](const double *at) { return *reinterpret_cast<const double2 *>(at); };
+    double own[2][2], v[2][2] = {{0.0, 0.0}, {0.0, 0.0}}, w[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int c = c0 + j;
-        U[r * kB + c] = r < c ? (float)S.gram[r * kB + c] : (r == c ? (float)(0.5 * (S.gram[r * kB + c] - 1.0)) : 0.f);
-    }
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const int r = r0 + a, c = c0 + b;
+            own[a][b] = r < c ? U[r * kB + c] : (r == c ? 0.5 * (U[r * kB + c] - 1.0) : 0.0);
+            U[r * kB + c] = own[a][b];
+        }
     __syncthreads();
-    float v[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 8
-    for (int i = 0; i < kB; ++i) {                // U^T U
-        const float x = U[i * kB + r];
-        const float4 y = *reinterpret_cast<const float4 *>(U + i * kB + c0);
-        v[0] = fmaf(x, y.x, v[0]); v[1] = fmaf(x, y.y, v[1]); v[2] = fmaf(x, y.z, v[2]); v[3] = fmaf(x, y.w, v[3]);
+    if (c0 >= r0) {
+#pragma unroll 4
+        for (int i = 0; i <= r0 + 1; ++i) {       // U^T U
+            const double2 x = pair(U + i * kB + r0), y = pair(U + i * kB + c0);
+            v[0][0] = fma(x.x, y.x, v[0][0]); v[0][1] = fma(x.x, y.y, v[0][1]);
+            v[1][0] = fma(x.y, y.x, v[1][0]); v[1][1] = fma(x.y, y.y, v[1][1]);
+        }
     }
+    __syncthreads();                              // U has been read
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int c = c0 + j;
-        v[j] = r < c ? U[r * kB + c] - v[j] : (r == c ? U[r * kB + c] - 0.5f * v[j] : 0.f);
-        R[r][c] = v[j] + (r == c ? 1.f : 0.f);
-        S.V[r * kB + c] = v[j];
-    }
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const int r = r0 + a, c = c0 + b;
+            v[a][b] = r < c ? own[a][b] - v[a][b] : (r == c ? own[a][b] - 0.5 * v[a][b] : 0.0);
+            R[r][c] = (float)(v[a][b] + (r == c ? 1.0 : 0.0));
+            S.V[r * kB + c] = v[a][b];
+            Vt[c * kB + r] = v[a][b];
+        }
     __syncthreads();
-    float w[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 8
-    for (int i = 0; i < kB; ++i) {                // V V
-        const float x = S.V[r * kB + i];
-        const float4 y = *reinterpret_cast<const float4 *>(S.V + i * kB + c0);
-        w[0] = fmaf(x, y.x, w[0]); w[1] = fmaf(x, y.y, w[1]); w[2] = fmaf(x, y.z, w[2]); w[3] = fmaf(x, y.w, w[3]);
+    if (c0 >= r0) {
+#pragma unroll 4
+        for (int i = r0; i <= c0 + 1; ++i) {      // V V
+            const double2 x = pair(Vt + i * kB + r0), y = pair(S.V + i * kB + c0);
+            w[0][0] = fma(x.x, y.x, w[0][0]); w[0][1] = fma(x.x, y.y, w[0][1]);
+            w[1][0] = fma(x.y, y.x, w[1][0]); w[1][1] = fma(x.y, y.y, w[1][1]);
+        }
     }
 #pragma unroll
-    for (int j = 0; j < 4; ++j) S.Rinv[r][c0 + j] = w[j] - v[j] + (r == c0 + j ? 1.f : 0.f);
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) S.Rinv[r0 + a][c0 + b] = (float)(w[a][b] - v[a][b] + (r0 + a == c0 + b ? 1.0 : 0.0));
     __syncthreads();
 }
 
