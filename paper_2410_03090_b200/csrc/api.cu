@@ -277,6 +277,12 @@ static bool same_strides(const uncomp_strides &a, const uncomp_strides &b) {
     return a.sB == b.sB && a.sL == b.sL && a.sH == b.sH && a.sN == b.sN;
 }
 
+// More than 64 rounds of multi-section (9-fold at least) are as good as 64; the kernels calculate with the number.
+static uncomp_entropy_params bounded(uncomp_entropy_params p) {
+    if (p.max_iters > 64) p.max_iters = 64;
+    return p;
+}
+
 int uncomp_entropy(uncomp_ctx *ctx, const void *d_K, uncomp_strides sK, const uncomp_entropy_params *params,
                    const void *d_Qw, float scale, float *d_entropy, float *d_erank, double *d_spectrum,
                    void *stream) {
@@ -317,9 +323,9 @@ int uncomp_entropy(uncomp_ctx *ctx, const void *d_K, uncomp_strides sK, const un
     {
         ProfScope ps(ctx->prof, kSlotEigen, st);
         if (tensor_path)
-            e = launch_eigen_f32(p, partials, parts, d_Qw != nullptr, *params, d_entropy, d_erank, d_spectrum, d_status, st);
+            e = launch_eigen_f32(p, partials, parts, d_Qw != nullptr, bounded(*params), d_entropy, d_erank, d_spectrum, d_status, st);
         else
-            e = launch_eigen_entropy(p, partials, *params, d_entropy, d_erank, d_spectrum, d_status, st);
+            e = launch_eigen_entropy(p, partials, bounded(*params), d_entropy, d_erank, d_spectrum, d_status, st);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     return UNCOMP_OK;
@@ -471,7 +477,7 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
         if (e != cudaSuccess) return cuda_fail(ctx, e);
         {
             ProfScope ps(ctx->prof, kSlotEigen, st);
-            e = launch_eigen_f32(p, partials, p.score_splits, true, *eparams, d_entropy, d_erank, nullptr, d_status, st);
+            e = launch_eigen_f32(p, partials, p.score_splits, true, bounded(*eparams), d_entropy, d_erank, nullptr, d_status, st);
         }
         if (e != cudaSuccess) return cuda_fail(ctx, e);
         {
@@ -510,7 +516,7 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
         if (e != cudaSuccess) return cuda_fail(ctx, e);
         {
             ProfScope ps(ctx->prof, kSlotEigen, st);
-            e = launch_eigen_f32(p, partials, p.score_splits, true, *eparams, d_entropy, d_erank, nullptr, d_status, st);
+            e = launch_eigen_f32(p, partials, p.score_splits, true, bounded(*eparams), d_entropy, d_erank, nullptr, d_status, st);
         }
         if (e == cudaSuccess)
             e = launch_scores_tc(p, d_Qw, d_K, addr, sc, nullptr, stats_part, raw, nullptr, kScorePhaseColsum, false, d_status,
@@ -643,7 +649,7 @@ int uncomp_entropy_wide(uncomp_ctx *ctx, const void *d_X, int32_t count, int64_t
     const int k = params->k_trunc < D ? params->k_trunc : D;
     for (int i = 0; i < count; ++i) {
         const unsigned char *Xi = static_cast<const unsigned char *>(d_X) + (size_t)i * stride_matrix * 2;
-        cudaError_t e = launch_entropy_wide(Xi, stride_row, N, D, *params, static_cast<unsigned char *>(d_scratch),
+        cudaError_t e = launch_entropy_wide(Xi, stride_row, N, D, bounded(*params), static_cast<unsigned char *>(d_scratch),
                                             d_entropy + i, d_erank ? d_erank + i : nullptr,
                                             d_spectrum ? d_spectrum + (size_t)i * k : nullptr,
                                             reinterpret_cast<uint32_t *>(ctx->ws + ctx->plan.off_status), ctx->prof, st);

@@ -32,3 +32,19 @@ def test_spectrum_over_unit_counts(units, dtype):
         H = -(p * p.clamp(min=1e-300).log()).sum(1)
         assert float((ent[0, :, 0].double().cpu() - H).abs().max()) < 1e-4
         assert torch.allclose(erank, ent.exp(), rtol=1e-5)
+
+
+@pytest.mark.parametrize("dtype,units", [("fp32", 8), ("fp32", 80), ("bf16", 8), ("bf16", 80), ("bf16", 300)])
+@pytest.mark.parametrize("max_iters", [1 << 30, 2**31 - 1])
+def test_any_number_of_rounds(dtype, units, max_iters):
+    """As many rounds as fit the parameter: what the default gives, bit for bit."""
+    from paper_2410_03090_b200 import binding as ub
+
+    g = torch.Generator(device="cuda").manual_seed(units)
+    K = torch.randn(1, units, 1, 150, 128, generator=g, device="cuda").to(torch.float32 if dtype == "fp32" else torch.bfloat16)
+    ctx = ub.Context(ub.make_shape(1, units, 1, 1, 150, 128, 32, dtype))
+    spectra = [torch.empty(1, units, 1, 32, dtype=torch.float64, device="cuda") for _ in range(2)]
+    want = ub.uncomp_entropy(ctx, K, 32, spectrum=spectra[0])
+    got = ub.uncomp_entropy(ctx, K, 32, max_iters=max_iters, spectrum=spectra[1])
+    assert ub.uncomp_status(ctx) == 0
+    assert torch.equal(spectra[0], spectra[1]) and all(torch.equal(a, b) for a, b in zip(want, got))

@@ -114,6 +114,17 @@ def test_few_rounds_are_reported():
     assert ub.uncomp_status(ctx) == 0
 
 
+@pytest.mark.parametrize("k", [32, 65])                     # block Lanczos, and the full reduction
+@pytest.mark.parametrize("max_iters", [1 << 29, 2**31 - 1])
+def test_any_number_of_rounds(k, max_iters):
+    from paper_2410_03090_b200 import binding as ub
+    X = tw._matrix(1, 1300, 512, 60, 0.1, seed=1)
+    ctx = ub.Context(ub.make_shape(1, 1, 1, 1, 256, 128, 8, "bf16"))
+    want = ub.uncomp_entropy_wide(ctx, X, k, spectrum=True)
+    got = ub.uncomp_entropy_wide(ctx, X, k, max_iters=max_iters, spectrum=True)
+    assert ub.uncomp_status(ctx) == 0 and all(torch.equal(a, b) for a, b in zip(want, got))
+
+
 @pytest.mark.parametrize("N,D,k", [(900, 384, 32), (1300, 1024, 64)])
 def test_repeated_calls_agree_bit_for_bit(N, D, k):
     """The counts stream the band through small rings in shared memory, whose places are taken again as soon as a column has
