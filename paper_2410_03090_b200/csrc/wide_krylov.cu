@@ -847,7 +847,9 @@ __device__ __forceinline__ double band_high(double bound) { return bound * (1.0 
 // To how much an eigenvalue of at least `lo` is bracketed: 2e-8 of itself, but no finer than 1e-13 and no coarser than 1e-9
 // of the spectrum's bound.  It has settled when it moved by less than kSettled times that over the last two blocks.
 constexpr double kSettled = 100.0;
-constexpr int kBandRounds = 14;                   // six of equal spacing suffice
+// Rounds of equal spacing, 16-fold each: six between two shared shifts (2.3e-3 of the bound to 1e-9 of it, 4.6 % of a shift to
+// 2e-8), nine below the lowest of them (6.8e-4 of the bound to 1e-13), where an eigenvalue beyond the matrix's rank lies.
+constexpr int kBandRounds = 9;
 __device__ __forceinline__ double band_tolerance(double lo, double bound) {
     return fmin(fmax(2e-8 * lo, 1e-13 * bound), 1e-9 * bound);
 }
@@ -951,7 +953,8 @@ band_eigen_kernel(int k, int q, int max_iters, KrylovBuffers B, uint32_t *__rest
     const int rounds = max_iters > 0 ? min(max((8 * max_iters - 6) / 4, 1), kBandRounds) : kBandRounds;
     bool settled = false, done = false, guided = false;
     double guess = 0.0, width = 0.0;              // a guess of the eigenvalue, and the bracket it was made for
-    for (int it = 0; it < rounds && !done; ++it) {
+    // a guided round that has not earned as much as one of equal spacing does not count; one of those follows it
+    for (int it = 0, spent = 0; spent < rounds && !done; ++it) {
         const double tol = band_tolerance(lo, bound), step = (hi - lo) / (double)(kShifts + 1);
         // Shifts: equally spaced, or seven on either side of the guess at distances that grow from half the tolerance to a
         // quarter of the bracket, and the guess itself.
@@ -997,9 +1000,9 @@ band_eigen_kernel(int k, int q, int max_iters, KrylovBuffers B, uint32_t *__rest
         done = hi - lo <= band_tolerance(lo, bound);
         settled = count[kShifts] >= t + 1;
         // The next guess: inverse interpolation of the determinant through the four shifts around the eigenvalue, when it is
-        // the only one in the bracket and all four lie in the old bracket.  A guided round that has not earned as much as
-        // equal spacing would have is followed by one of equal spacing.
+        // the only one in the bracket and all four lie in the old bracket.
         const bool earned = hi - lo <= (1.0 / 16.0) * width;
+        spent += !guided || earned;
         const int i0 = min(max(nb - 2, 0), kShifts - 4);
         bool usable = c_hi - c_lo == 1 && (!guided || earned);
         double xs[4], fs[4];

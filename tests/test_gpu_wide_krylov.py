@@ -208,3 +208,14 @@ def test_errors_of_the_steps_alone(kind, N, D, k):
     share = rel / (2.0 ** -24 * (2 + lam[0] / lam))
     print(kind, N, D, k, "of the bound:", float(share.max()), float(rel.max()), float(lam[0] / lam[-1]))
     assert float(share.max()) <= 1
+
+
+@pytest.mark.parametrize("rank,noise,k", [(20, 0.0, 32), (31, 0.0, 32), (8, 1e-3, 32), (40, 1e-4, 64), (63, 0.0, 64), (20, 1e-2, 64)])
+def test_more_eigenvalues_than_the_matrix_has(rank, noise, k):
+    """The last ones are rounding, 1e-8 to 1e-14 of the bound and below the lowest shared shift, where the bracket needs the most
+    rounds: it closes within them, whoever supplies the eigenvalues."""
+    from paper_2410_03090_b200 import binding as ub
+    g = torch.Generator(device="cuda").manual_seed(rank + k)
+    X = torch.randn(2000, rank, generator=g, device="cuda").round() @ torch.randint(-2, 3, (rank, 768), generator=g, device="cuda").float()
+    X = X.clamp(-250, 250) + noise * torch.randn(2000, 768, generator=g, device="cuda")
+    tw._check(ub, X.to(torch.bfloat16)[None], k, 1, 0)
