@@ -306,7 +306,7 @@ int uncomp_entropy(uncomp_ctx *ctx, const void *d_K, uncomp_strides sK, const un
         // one sweep over K: Gram partials per scorer chunk and the scorer's row statistics
         const float sc = effective_scale(scale, p.shape.d);
         e = launch_scores_tc(p, d_Qw, d_K, addr, sc, nullptr, reinterpret_cast<float *>(ctx->ws + p.off_stats_part), nullptr,
-                             reinterpret_cast<float *>(partials), kScorePhaseStats, true, d_status, &ctx->tmaps, ctx->prof, st);
+                             reinterpret_cast<float *>(partials), kScorePhaseStats, d_status, &ctx->tmaps, ctx->prof, st);
         if (e != cudaSuccess) return cuda_fail(ctx, e);
         parts = p.score_splits;
         ctx->stats_valid = 1;
@@ -401,7 +401,7 @@ int uncomp_score_select(uncomp_ctx *ctx, const void *d_Qw, const void *d_K, unco
     cudaError_t e;
     if (tensor_path) {
         const int phases = (reuse || d_lse) ? kScorePhaseColsum : (kScorePhaseStats | kScorePhaseColsum);
-        e = launch_scores_tc(p, d_Qw, d_K, addr, scale, d_lse, stats_part, raw, nullptr, phases, true, d_status,
+        e = launch_scores_tc(p, d_Qw, d_K, addr, scale, d_lse, stats_part, raw, nullptr, phases, d_status,
                              &ctx->tmaps, ctx->prof, st);
     } else {
         e = launch_scores_simt(p, d_Qw, d_K, addr, scale, d_lse, stats_part, stats, raw, d_status, ctx->prof, st);
@@ -410,7 +410,7 @@ int uncomp_score_select(uncomp_ctx *ctx, const void *d_Qw, const void *d_K, unco
     {
         ProfScope ps(ctx->prof, kSlotPoolSelect, st);
         e = launch_pool_select(p, raw, pooled, params->pool_kernel, params->pool_mode, d_budgets, d_offsets,
-                               d_indices, true, d_status, st);
+                               d_indices, d_status, st);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     return UNCOMP_OK;
@@ -473,7 +473,7 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
         ctx->stats_valid = 0;
         cudaError_t e = launch_scores_tc(p, d_Qw, d_K, addr, effective_scale(sparams->scale, p.shape.d), d_lse,
                                          reinterpret_cast<float *>(ctx->ws + p.off_stats_part), raw, partials, kScorePhaseColsum,
-                                         true, d_status, &ctx->tmaps, ctx->prof, st);
+                                         d_status, &ctx->tmaps, ctx->prof, st);
         if (e != cudaSuccess) return cuda_fail(ctx, e);
         {
             ProfScope ps(ctx->prof, kSlotEigen, st);
@@ -490,7 +490,7 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
         {
             ProfScope ps(ctx->prof, kSlotPoolSelect, st);
             e = launch_pool_select(p, raw, pooled, sparams->pool_kernel, sparams->pool_mode, d_budgets, d_offsets,
-                                   d_indices, true, d_status, st);
+                                   d_indices, d_status, st);
         }
         if (e != cudaSuccess) return cuda_fail(ctx, e);
     } else if (tensor_path) {
@@ -510,7 +510,7 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
         const float sc = effective_scale(sparams->scale, p.shape.d);
         ctx->stats_valid = 0;
         e = launch_scores_tc(p, d_Qw, d_K, addr, sc, nullptr, stats_part, nullptr, partials, kScorePhaseStats,
-                             true, d_status, &ctx->tmaps, ctx->prof, st);
+                             d_status, &ctx->tmaps, ctx->prof, st);
         if (e == cudaSuccess) e = cudaEventRecord(ctx->ev_fork, st);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0);
         if (e != cudaSuccess) return cuda_fail(ctx, e);
@@ -519,7 +519,7 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
             e = launch_eigen_f32(p, partials, p.score_splits, true, bounded(*eparams), d_entropy, d_erank, nullptr, d_status, st);
         }
         if (e == cudaSuccess)
-            e = launch_scores_tc(p, d_Qw, d_K, addr, sc, nullptr, stats_part, raw, nullptr, kScorePhaseColsum, false, d_status,
+            e = launch_scores_tc(p, d_Qw, d_K, addr, sc, nullptr, stats_part, raw, nullptr, kScorePhaseColsum, d_status,
                                  &ctx->tmaps, ctx->prof, ctx->side);
         if (e == cudaSuccess) {
             ProfScope ps(ctx->prof, kSlotBudgets, st);
@@ -534,7 +534,7 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
         {
             ProfScope ps(ctx->prof, kSlotPoolSelect, st);
             e = launch_pool_select(p, raw, pooled, sparams->pool_kernel, sparams->pool_mode, d_budgets, d_offsets,
-                                   d_indices, false, d_status, st);
+                                   d_indices, d_status, st);
         }
         if (e != cudaSuccess) return cuda_fail(ctx, e);
     } else {

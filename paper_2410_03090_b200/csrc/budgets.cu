@@ -173,7 +173,7 @@ cudaError_t launch_budgets(const Plan &p, const float *d_erank, const uncomp_bud
     static bool done[64] = {};
     cudaError_t e = allow_dynamic_smem((const void *)budgets_kernel, kBudShared * 16, done);
     if (e != cudaSuccess) return e;
-    return launch_kernel(budgets_kernel, LaunchShape{dim3(1), kBudThreads, smem, 1, true}, st, d_erank, p.shape.B, p.shape.L,
+    return launch_kernel(budgets_kernel, LaunchShape{dim3(1), kBudThreads, smem, 1}, st, d_erank, p.shape.B, p.shape.L,
                          p.shape.H, p.shape.N, p.shape.w, bp, sched, d_budgets, d_offsets, d_layer_group, d_layer_ctx, d_rank,
                          d_rem);
 }

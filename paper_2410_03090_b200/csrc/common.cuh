@@ -141,7 +141,9 @@ inline cudaError_t allow_dynamic_smem(const void *fn, size_t bytes, bool (&done)
 // layer of 7001 tokens 146 / 160 / 129, 256 units of 8192 tokens 427 / 453 / 414, 1024 of 3712 836 / 862 / 819, a decode
 // step on 256 caches of 410 rows 11.1 / 9.4 / 9.4.  The exception are the kernels that end the eigenvalues of up to 296
 // units: next are the budgets, one CTA with work that depends on nothing (the table of the groups); a signal is no promise
-// about memory, chain_wait() still waits for the end.
+// about memory, chain_wait() still waits for the end.  All of this loosens the order behind the stream's previous kernel and
+// nothing else: copies, event waits and, in a captured graph, kernels of other branches are waited for as by any launch, so it
+// holds for the first kernel of a call, whatever the caller has put on the stream, and behind the library's own joins.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_signal() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -150,7 +152,6 @@ struct LaunchShape {
     unsigned block;
     size_t smem;
     unsigned cluster;    // CTAs per cluster
-    bool chained;        // false behind an event wait: the kernel has more than its stream to wait for
 };
 template <typename... P, typename... A>
 inline cudaError_t launch_kernel(void (*kernel)(P...), const LaunchShape &s, cudaStream_t st, A &&...args) {
@@ -161,10 +162,8 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), const LaunchShape &s, cud
     cfg.dynamicSmemBytes = s.smem;
     cfg.stream = st;
     cfg.attrs = attr;
-    if (s.chained) {
-        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
-    }
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
     if (s.cluster > 1) {
         attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
         attr[cfg.numAttrs].val.clusterDim.x = s.cluster;
@@ -217,9 +216,9 @@ struct TmapCache;
 // kScorePhaseColsum alone with d_gram_part != NULL: pass B and the Gram partials from one sweep (needs d_lse).
 cudaError_t launch_scores_tc(const Plan &p, const void *dQw, const void *dK, const UnitAddr &addr, float scale,
                              const float *d_lse, float *d_stats_part, float *d_raw, float *d_gram_part,
-                             int phases, bool chained, uint32_t *d_status, TmapCache *cache, Profiler *prof, cudaStream_t st);
+                             int phases, uint32_t *d_status, TmapCache *cache, Profiler *prof, cudaStream_t st);
 cudaError_t launch_pool_select(const Plan &p, const float *d_raw, float *d_pooled, int pool_kernel, int pool_mode,
-                               const int32_t *d_budgets, const int64_t *d_offsets, int32_t *d_indices, bool chained,
+                               const int32_t *d_budgets, const int64_t *d_offsets, int32_t *d_indices,
                                uint32_t *d_status, cudaStream_t st);
 int evict_chunks(const uncomp_shape &s);
 cudaError_t launch_evict_hidden(const Plan &p, const void *d_qlast, const void *d_K, int64_t sB, int64_t sH, int64_t sN,

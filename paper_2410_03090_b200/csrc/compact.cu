@@ -76,7 +76,7 @@ cudaError_t launch_compact(const Plan &p, const void *dK, const void *dV, const 
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const bool f32 = p.shape.dtype == UNCOMP_FP32;
-    return launch_kernel(f32 ? compact_kernel<512> : compact_kernel<256>, LaunchShape{dim3(sms * 8), 256, 0, 1, true}, st,
+    return launch_kernel(f32 ? compact_kernel<512> : compact_kernel<256>, LaunchShape{dim3(sms * 8), 256, 0, 1}, st,
                          (const unsigned char *)dK, (const unsigned char *)dV, aK, aV, p.units, p.shape.N, f32 ? 4 : 2,
                          d_indices, d_offsets, (unsigned char *)dKc, (unsigned char *)dVc, d_status);
 }

@@ -661,7 +661,7 @@ cudaError_t launch_step(const DecArgs &a, const StepArgs &b, int units, int ctas
     static bool done[64] = {};
     cudaError_t e = allow_dynamic_smem((const void *)decode_step_kernel<G, T>, kStepSmem, done);
     if (e != cudaSuccess) return e;
-    return launch_kernel(decode_step_kernel<G, T>, LaunchShape{dim3(units * ctas), kDecThreads, smem, (unsigned)ctas, true}, st, a, b);
+    return launch_kernel(decode_step_kernel<G, T>, LaunchShape{dim3(units * ctas), kDecThreads, smem, (unsigned)ctas}, st, a, b);
 }
 template <typename T>
 cudaError_t launch_step_g(const DecArgs &a, const StepArgs &b, int units, int ctas, size_t smem, cudaStream_t st) {

@@ -556,7 +556,7 @@ cudaError_t launch_eigen_entropy(const Plan &p, void *d_partials, const uncomp_e
     int ctas = 1;
     while (ctas < 8 && p.units * ctas * 2 <= kTargetSms) ctas *= 2;
     const bool wide = p.shape.dtype == UNCOMP_FP32;    // fp64 partials
-    const LaunchShape shape{dim3(p.units), kEigThreads, 0, 1, true};
+    const LaunchShape shape{dim3(p.units), kEigThreads, 0, 1};
     cudaError_t e;
     if (wide)
         e = launch_kernel(eigen_entropy_kernel<double>, shape, st, (double *)d_partials, p.gram_splits, ctas > 1, p.shape.N,
@@ -567,7 +567,7 @@ cudaError_t launch_eigen_entropy(const Plan &p, void *d_partials, const uncomp_e
     if (e != cudaSuccess || ctas == 1) return e;
     const int64_t stride = (int64_t)p.gram_splits * (n * n + n) * (wide ? sizeof(double) : sizeof(float));
     return launch_kernel(ctas == 8 ? eigen_values64_kernel<16> : eigen_values64_kernel<8>,
-                         LaunchShape{dim3(p.units * ctas), kValueThreads, 0, (unsigned)ctas, true}, st, (const char *)d_partials, stride,
+                         LaunchShape{dim3(p.units * ctas), kValueThreads, 0, (unsigned)ctas}, st, (const char *)d_partials, stride,
                          ep.k_trunc, ep.norm, ep.max_iters, d_entropy, d_erank, d_spectrum, d_status);
 }
 

@@ -254,7 +254,7 @@ eigen_tail_kernel(const float *__restrict__ partials, int64_t unit_stride, int u
 cudaError_t launch_eigen_tail(int units, float *d_partials, int partials_per_unit, const uncomp_entropy_params &ep,
                               float *d_entropy, float *d_erank, double *d_spectrum, uint32_t *d_status, cudaStream_t st) {
     const int64_t stride = (int64_t)partials_per_unit * (kD * kD + kD);
-    return launch_kernel(eigen_tail_kernel, LaunchShape{dim3((units + kT / 32 - 1) / (kT / 32)), kT, 0, 1, true}, st, d_partials, stride,
+    return launch_kernel(eigen_tail_kernel, LaunchShape{dim3((units + kT / 32 - 1) / (kT / 32)), kT, 0, 1}, st, d_partials, stride,
                          units, ep.k_trunc, ep.norm, ep.max_iters, d_entropy, d_erank, d_spectrum, d_status);
 }
 

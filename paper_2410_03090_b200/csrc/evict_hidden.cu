@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const unsigned char *_
 template <typename T>
 cudaError_t launch_logits(int G, dim3 grid, cudaStream_t st, const T *q, const T *K, int H, int64_t sB, int64_t sH,
                           int64_t sN, int N, int chunk, int chunks, float c_log2, float *logits, float *stats) {
-    const LaunchShape shape{grid, kEvThreads, 0, 1, true};
+    const LaunchShape shape{grid, kEvThreads, 0, 1};
     switch (G) {
         case 1: return launch_kernel(last_token_logits_kernel<T, 1>, shape, st, q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats);
         case 2: return launch_kernel(last_token_logits_kernel<T, 2>, shape, st, q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats);
@@ -354,7 +354,7 @@ cudaError_t launch_logits(int G, dim3 grid, cudaStream_t st, const T *q, const T
 cudaError_t launch_logits_mma(int G, dim3 grid, cudaStream_t st, const __nv_bfloat16 *q, const __nv_bfloat16 *K, int H,
                               int64_t sB, int64_t sH, int64_t sN, int N, int chunk, int chunks, float c_log2,
                               float *logits, float *stats) {
-    const LaunchShape shape{grid, kEvThreads, 0, 1, true};
+    const LaunchShape shape{grid, kEvThreads, 0, 1};
     switch (G) {
         case 1: return launch_kernel(last_token_logits_mma_kernel<1>, shape, st, q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats);
         case 2: return launch_kernel(last_token_logits_mma_kernel<2>, shape, st, q, K, H, sB, sH, sN, N, chunk, chunks, c_log2, logits, stats);
@@ -392,7 +392,7 @@ cudaError_t launch_evict_hidden(const Plan &p, const void *d_qlast, const void *
     {
         ProfScope ps(prof, kSlotEvictScores, st);
         dim3 grid((s.N - 1 + kEvThreads - 1) / kEvThreads, s.B);
-        e = launch_kernel(last_token_scores_kernel, LaunchShape{grid, kEvThreads, s.Hq * sizeof(float), 1, true}, st, d_logits, d_stats, s.B,
+        e = launch_kernel(last_token_scores_kernel, LaunchShape{grid, kEvThreads, s.Hq * sizeof(float), 1}, st, d_logits, d_stats, s.B,
                           s.Hq, s.N, chunks, n_keep, d_raw, d_budgets, d_offsets);
         if (e != cudaSuccess) return e;
     }
@@ -403,7 +403,7 @@ cudaError_t launch_evict_hidden(const Plan &p, const void *d_qlast, const void *
         q.units = s.B;
         q.prefix = s.N - 1;
         q.shape.w = 1;
-        e = launch_pool_select(q, d_raw, d_scores, 1, 0, d_budgets, d_offsets, d_indices, true, d_status, st);
+        e = launch_pool_select(q, d_raw, d_scores, 1, 0, d_budgets, d_offsets, d_indices, d_status, st);
         if (e != cudaSuccess) return e;
     }
     {
@@ -411,7 +411,7 @@ cudaError_t launch_evict_hidden(const Plan &p, const void *d_qlast, const void *
         int dev = 0, sms = 148;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        e = launch_kernel(gather_rows_kernel, LaunchShape{dim3(sms * 8), 256, 0, 1, true}, st, (const unsigned char *)d_X, d_indices,
+        e = launch_kernel(gather_rows_kernel, LaunchShape{dim3(sms * 8), 256, 0, 1}, st, (const unsigned char *)d_X, d_indices,
                           (int64_t)s.B * n_keep, n_keep, s.N, row_bytes, (unsigned char *)d_Xout, d_status);
     }
     return e;

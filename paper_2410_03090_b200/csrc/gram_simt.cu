@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(256) gram_simt_kernel(const T *__restrict__ K,
 
 cudaError_t launch_gram_simt(const Plan &p, const void *dK, const UnitAddr &addr, void *d_partials, cudaStream_t st) {
     if (p.shape.dtype == UNCOMP_FP32) {
-        return launch_kernel(gram_f64_kernel, LaunchShape{dim3(10 * p.units, p.gram_splits), 256, 0, 1, true}, st, (const float *)dK, addr,
+        return launch_kernel(gram_f64_kernel, LaunchShape{dim3(10 * p.units, p.gram_splits), 256, 0, 1}, st, (const float *)dK, addr,
                              p.shape.N, p.gram_chunk, (double *)d_partials, p.gram_splits);
     } else {
         dim3 grid(p.gram_splits, p.units);

@@ -231,26 +231,26 @@ static cudaError_t launch_scores_simt_t(const Plan &p, const T *dQw, const T *dK
     if (d_lse) {
         ProfScope ps(prof, kSlotStatsMerge, st);
         const int total = p.units * p.rows;
-        e = launch_kernel(lse_import_kernel, LaunchShape{dim3((total + 255) / 256), 256, 0, 1, true}, st, d_lse, p.units, p.rows, d_stats,
+        e = launch_kernel(lse_import_kernel, LaunchShape{dim3((total + 255) / 256), 256, 0, 1}, st, d_lse, p.units, p.rows, d_stats,
                           d_status);
     } else {
         const int row_blocks = (p.rows + kSB - 1) / kSB;
         dim3 gA(p.score_splits, row_blocks, p.units);
         {
             ProfScope ps(prof, kSlotScoreStats, st);
-            e = launch_kernel(score_stats_simt_kernel<T>, LaunchShape{gA, 256, smemA, 1, true}, st, dQw, dK, addr, p.shape.N, p.shape.w,
+            e = launch_kernel(score_stats_simt_kernel<T>, LaunchShape{gA, 256, smemA, 1}, st, dQw, dK, addr, p.shape.N, p.shape.w,
                               p.G, p.score_chunk, p.score_splits, scale, d_stats_part);
         }
         if (e != cudaSuccess) return e;
         const int total = p.units * p.rows;
         ProfScope ps(prof, kSlotStatsMerge, st);
-        e = launch_kernel(score_stats_merge_kernel, LaunchShape{dim3((total + 255) / 256), 256, 0, 1, true}, st, d_stats_part, p.units,
+        e = launch_kernel(score_stats_merge_kernel, LaunchShape{dim3((total + 255) / 256), 256, 0, 1}, st, d_stats_part, p.units,
                           p.rows, p.score_splits, d_stats);
     }
     if (e != cudaSuccess) return e;
     dim3 gB((p.prefix + kSB - 1) / kSB, p.units);
     ProfScope ps(prof, kSlotScoreColsum, st);
-    return launch_kernel(score_colsum_simt_kernel<T>, LaunchShape{gB, 256, smemB, 1, true}, st, dQw, dK, addr, p.shape.N, p.shape.w, p.G,
+    return launch_kernel(score_colsum_simt_kernel<T>, LaunchShape{gB, 256, smemB, 1}, st, dQw, dK, addr, p.shape.N, p.shape.w, p.G,
                          scale, d_stats, d_raw);
 }
 

@@ -612,7 +612,7 @@ static cudaError_t raise_smem_limit() {
 template <int MB, int SPLIT>
 static cudaError_t launch_scores_tc_mb(const Plan &p, const CUtensorMap &tq, const CUtensorMap &tk, float c_log2,
                                        const float *d_lse, float *d_stats_part, float *d_raw,
-                                       float *d_gram_part, int phases, bool chained, uint32_t *d_status, Profiler *prof,
+                                       float *d_gram_part, int phases, uint32_t *d_status, Profiler *prof,
                                        cudaStream_t st) {
     const uncomp_shape &s = p.shape;
     cudaError_t e = cudaSuccess;
@@ -623,7 +623,7 @@ static cudaError_t launch_scores_tc_mb(const Plan &p, const CUtensorMap &tq, con
     auto ctas = [&](int splits) { return (unsigned)min((int64_t)sms, (int64_t)p.units * splits); };
     auto launch = [&](auto kernel, int mode, int splits, float *stats_out, const float *stats_in, int stats_splits, const float *lse,
                       float *raw, float *gram) {
-        return launch_kernel(kernel, LaunchShape{dim3(ctas(splits)), kScoreThreads, (size_t)score_smem(MB, mode), 1, chained}, st, tq, tk, s.L, s.H,
+        return launch_kernel(kernel, LaunchShape{dim3(ctas(splits)), kScoreThreads, (size_t)score_smem(MB, mode), 1}, st, tq, tk, s.L, s.H,
                              s.N, s.w, p.rows, p.units, p.score_chunk, splits, c_log2, stats_out, stats_in, stats_splits, lse, raw,
                              gram, d_status);
     };
@@ -649,19 +649,19 @@ static cudaError_t launch_scores_tc_mb(const Plan &p, const CUtensorMap &tq, con
 
 cudaError_t launch_scores_tc(const Plan &p, const void *dQw, const void *dK, const UnitAddr &addr, float scale,
                              const float *d_lse, float *d_stats_part, float *d_raw, float *d_gram_part,
-                             int phases, bool chained, uint32_t *d_status, TmapCache *cache, Profiler *prof, cudaStream_t st) {
+                             int phases, uint32_t *d_status, TmapCache *cache, Profiler *prof, cudaStream_t st) {
     CUtensorMap tq, tk;
     cudaError_t e = cached_scorer_maps(cache, p, addr, dQw, dK, kTile, &tq, &tk);
     if (e != cudaSuccess) return e;
     const float c_log2 = scale * 1.4426950408889634f;
     const int MB = (p.rows + 127) / 128;
-    if (p.rows <= 32) return launch_scores_tc_mb<1, 4>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, chained, d_status, prof, st);
-    if (p.rows <= 64) return launch_scores_tc_mb<1, 2>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, chained, d_status, prof, st);
+    if (p.rows <= 32) return launch_scores_tc_mb<1, 4>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
+    if (p.rows <= 64) return launch_scores_tc_mb<1, 2>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
     switch (MB) {
-        case 1: return launch_scores_tc_mb<1, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, chained, d_status, prof, st);
-        case 2: return launch_scores_tc_mb<2, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, chained, d_status, prof, st);
-        case 3: return launch_scores_tc_mb<3, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, chained, d_status, prof, st);
-        default: return launch_scores_tc_mb<4, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, chained, d_status, prof, st);
+        case 1: return launch_scores_tc_mb<1, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
+        case 2: return launch_scores_tc_mb<2, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
+        case 3: return launch_scores_tc_mb<3, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
+        default: return launch_scores_tc_mb<4, 1>(p, tq, tk, c_log2, d_lse, d_stats_part, d_raw, d_gram_part, phases, d_status, prof, st);
     }
 }
 

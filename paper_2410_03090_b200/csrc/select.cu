@@ -565,32 +565,30 @@ pool_select_keys_kernel(const float *__restrict__ raw, float *__restrict__ poole
 
 template <int NBK, int POOL>
 cudaError_t launch_keys(const Plan &p, int ctas, const float *d_raw, float *d_pooled, int pool_kernel, int pool_mode,
-                        const int32_t *d_budgets, const int64_t *d_offsets, int32_t *d_indices, bool chained, uint32_t *d_status,
-                        cudaStream_t st) {
+                        const int32_t *d_budgets, const int64_t *d_offsets, int32_t *d_indices, uint32_t *d_status, cudaStream_t st) {
     static bool done[64] = {};
     cudaError_t e = allow_dynamic_smem((const void *)pool_select_keys_kernel<NBK, POOL>, sizeof(KeySmem<NBK>), done);
     if (e != cudaSuccess) return e;
     return launch_kernel(pool_select_keys_kernel<NBK, POOL>,
-                         LaunchShape{dim3(p.units * ctas), kKeyThreads, sizeof(KeySmem<NBK>), (unsigned)ctas, chained}, st, d_raw, d_pooled,
+                         LaunchShape{dim3(p.units * ctas), kKeyThreads, sizeof(KeySmem<NBK>), (unsigned)ctas}, st, d_raw, d_pooled,
                          p.prefix, p.shape.w, pool_kernel, pool_mode, d_budgets, d_offsets, p.units, d_indices, d_status);
 }
 
 template <int POOL>
 cudaError_t launch_keys_nbk(const Plan &p, int n, int ctas, const float *d_raw, float *d_pooled, int pool_kernel, int pool_mode,
-                            const int32_t *d_budgets, const int64_t *d_offsets, int32_t *d_indices, bool chained, uint32_t *d_status,
-                            cudaStream_t st) {
+                            const int32_t *d_budgets, const int64_t *d_offsets, int32_t *d_indices, uint32_t *d_status, cudaStream_t st) {
     const auto f = n > 4 * ctas ? launch_keys<8, POOL> : n > 2 * ctas ? launch_keys<4, POOL> : n > ctas ? launch_keys<2, POOL> : launch_keys<1, POOL>;
-    return f(p, ctas, d_raw, d_pooled, pool_kernel, pool_mode, d_budgets, d_offsets, d_indices, chained, d_status, st);
+    return f(p, ctas, d_raw, d_pooled, pool_kernel, pool_mode, d_budgets, d_offsets, d_indices, d_status, st);
 }
 
 cudaError_t launch_pool_select(const Plan &p, const float *d_raw, float *d_pooled, int pool_kernel, int pool_mode,
-                               const int32_t *d_budgets, const int64_t *d_offsets, int32_t *d_indices, bool chained,
+                               const int32_t *d_budgets, const int64_t *d_offsets, int32_t *d_indices,
                                uint32_t *d_status, cudaStream_t st) {
     // 4096 positions per CTA and block of keys.  One CTA per unit up to 32768 positions (a cluster barrier costs a
     // microsecond), clusters beyond; shorter shares only while most of the GPU would idle.
     const int n = (p.prefix + 4095) / 4096;
     if (n > 64) {
-        return launch_kernel(pool_select_cluster_kernel, LaunchShape{dim3(p.units * kSelCluster), kSelThreads, 0, 1, chained}, st,
+        return launch_kernel(pool_select_cluster_kernel, LaunchShape{dim3(p.units * kSelCluster), kSelThreads, 0, 1}, st,
                              d_raw, d_pooled, p.prefix, p.shape.w, pool_kernel, pool_mode, d_budgets, d_offsets, p.units,
                              d_indices, d_status);
     }
@@ -599,7 +597,7 @@ cudaError_t launch_pool_select(const Plan &p, const float *d_raw, float *d_poole
     while (ctas < kKeyMaxCluster && (n > 8 * ctas || (n > 4 && n > 2 * ctas && (int64_t)p.units * ctas * 2 <= kTargetSms))) ctas *= 2;
     const auto f = pool_kernel == 1 ? launch_keys_nbk<kPoolNone>
                                     : pool_kernel == 7 && pool_mode == 0 ? launch_keys_nbk<kPoolMax7> : launch_keys_nbk<kPoolAny>;
-    return f(p, n, ctas, d_raw, d_pooled, pool_kernel, pool_mode, d_budgets, d_offsets, d_indices, chained, d_status, st);
+    return f(p, n, ctas, d_raw, d_pooled, pool_kernel, pool_mode, d_budgets, d_offsets, d_indices, d_status, st);
 }
 
 }  // namespace uncomp

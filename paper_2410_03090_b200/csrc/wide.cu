@@ -678,9 +678,9 @@ cudaError_t launch_entropy_wide(const void *d_X, int64_t sN, int N, int D, const
     if (err != cudaSuccess) return err;
     {
         ProfScope ps(prof, kSlotWideGram, st);
-        err = launch_kernel(wide_colsum_kernel, LaunchShape{dim3((D + 127) / 128, kColChunks), 256, 0, 1, false}, st, X, sN, N, D, colpart);
+        err = launch_kernel(wide_colsum_kernel, LaunchShape{dim3((D + 127) / 128, kColChunks), 256, 0, 1}, st, X, sN, N, D, colpart);
         if (err != cudaSuccess) return err;
-        err = launch_kernel(wide_colsum_reduce_kernel, LaunchShape{dim3((D + 255) / 256), 256, 0, 1, true}, st, colpart, D, s);
+        err = launch_kernel(wide_colsum_reduce_kernel, LaunchShape{dim3((D + 255) / 256), 256, 0, 1}, st, colpart, D, s);
         if (err != cudaSuccess) return err;
         CUtensorMap tmap;
         uint64_t dims[3] = {(uint64_t)D, (uint64_t)N, 1};
@@ -691,14 +691,14 @@ cudaError_t launch_entropy_wide(const void *d_X, int64_t sN, int N, int D, const
         if (w.dual) {
             err = cudaFuncSetAttribute(gram_wide_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmem);
             if (err != cudaSuccess) return err;
-            err = launch_kernel(gram_wide_kernel<true>, LaunchShape{dim3(w.pairs, w.chunks), kWThreads, kWSmem, 1, true}, st, tmap, D, w.nblk,
+            err = launch_kernel(gram_wide_kernel<true>, LaunchShape{dim3(w.pairs, w.chunks), kWThreads, kWSmem, 1}, st, tmap, D, w.nblk,
                                 w.chunk, part, d_status);
             if (err != cudaSuccess) return err;
-            err = launch_kernel(wide_rowdot_kernel, LaunchShape{dim3((N + 1 + 7) / 8), 256, 0, 1, true}, st, X, sN, N, D, w.Dt, s, g);
+            err = launch_kernel(wide_rowdot_kernel, LaunchShape{dim3((N + 1 + 7) / 8), 256, 0, 1}, st, X, sN, N, D, w.Dt, s, g);
         } else {
             err = cudaFuncSetAttribute(gram_wide_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmem);
             if (err != cudaSuccess) return err;
-            err = launch_kernel(gram_wide_kernel<false>, LaunchShape{dim3(w.pairs, w.chunks), kWThreads, kWSmem, 1, true}, st, tmap, N, w.nblk,
+            err = launch_kernel(gram_wide_kernel<false>, LaunchShape{dim3(w.pairs, w.chunks), kWThreads, kWSmem, 1}, st, tmap, N, w.nblk,
                                 w.chunk, part, d_status);
         }
         if (err != cudaSuccess) return err;
@@ -707,7 +707,7 @@ cudaError_t launch_entropy_wide(const void *d_X, int64_t sN, int N, int D, const
         ProfScope ps(prof, kSlotWideAssemble, st);
         const unsigned tiles = (kWBlock / 32) * (kWBlock / 32);
         err = launch_kernel(w.dual ? wide_assemble_kernel<true> : wide_assemble_kernel<false>,
-                            LaunchShape{dim3(w.pairs, tiles), 256, 0, 1, true}, st, part, w.pairs, w.chunks, w.nblk, w.Dt, N, (int)ep.center,
+                            LaunchShape{dim3(w.pairs, tiles), 256, 0, 1}, st, part, w.pairs, w.chunks, w.nblk, w.Dt, N, (int)ep.center,
                             w.dual ? g : s, C);
     }
     if (err != cudaSuccess) return err;
@@ -757,10 +757,10 @@ cudaError_t launch_entropy_wide(const void *d_X, int64_t sN, int N, int D, const
     }
     {
         ProfScope ps(prof, kSlotWideSturm, st);
-        err = launch_kernel(sturm_wide_kernel, LaunchShape{dim3(kf), kSturmThreads, 0, 1, true}, st, a, e, w.Dt, kf, (int)ep.max_iters, kry, lam,
+        err = launch_kernel(sturm_wide_kernel, LaunchShape{dim3(kf), kSturmThreads, 0, 1}, st, a, e, w.Dt, kf, (int)ep.max_iters, kry, lam,
                             d_status);
         if (err != cudaSuccess) return err;
-        err = launch_kernel(wide_entropy_kernel, LaunchShape{dim3(1), 32, 0, 1, true}, st, lam, k, kf, (int)ep.norm, d_entropy, d_erank, d_spectrum);
+        err = launch_kernel(wide_entropy_kernel, LaunchShape{dim3(1), 32, 0, 1}, st, lam, k, kf, (int)ep.norm, d_entropy, d_erank, d_spectrum);
     }
     return err;
 }

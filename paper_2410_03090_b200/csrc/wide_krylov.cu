@@ -1069,9 +1069,9 @@ cudaError_t launch_krylov(const float *C, int n, int k, int max_iters, const Kry
                         (void *)&bar, (void *)&d_status};
         e = cudaLaunchCooperativeKernel((const void *)lanczos_kernel, dim3(n / kB), dim3(kLT), args, sizeof(LanczosSmem), st);
         if (e != cudaSuccess) return e;
-        e = launch_kernel(band_coarse_kernel, LaunchShape{dim3(kCoarseCtas), kBT, 0, 1, true}, st, C, n, q, b);
+        e = launch_kernel(band_coarse_kernel, LaunchShape{dim3(kCoarseCtas), kBT, 0, 1}, st, C, n, q, b);
         if (e != cudaSuccess) return e;
-        e = launch_kernel(band_eigen_kernel, LaunchShape{dim3(k * kBandCluster), kBT, 0, 1, true}, st, k, q, max_iters, b, d_status);
+        e = launch_kernel(band_eigen_kernel, LaunchShape{dim3(k * kBandCluster), kBT, 0, 1}, st, k, q, max_iters, b, d_status);
         if (e != cudaSuccess) return e;
         if (q >= most || ++launch >= 3) break;
         q0 = q;
