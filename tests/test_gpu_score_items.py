@@ -66,3 +66,35 @@ def test_column_sums_of_keys_with_a_mean(G, w, N):
         torch.cuda.synchronize()
         assert cp.status() == 0
         parity.check_entropy(wl, K, o.entropy, o.erank, [0, 17, wl.units - 1])
+
+
+@pytest.mark.parametrize("w,how", [(32, "statistics"), (64, "statistics"), (32, "lse")])
+@pytest.mark.parametrize("mean,whole", [(0, False), (1, False), (10, False), (100, False), (40, True), (100, True)])
+def test_column_sums_over_the_longest_chunks(w, how, mean, whole):
+    """Chunks of 8192 tokens, 512 additions into one accumulator, of keys with a mean of up to 100 times their spread, held to the
+    tolerance of the entropy.  Whole numbers around 40: every sum fits 24 bits, so the covariance is exact and the entropy is
+    good to the brackets of the eigenvalues (2e-8 of the largest, equal ones) and its own 24 bits."""
+    from paper_2410_03090_b200 import binding as ub
+    L, H, G, N, k = 32, 8, 4, 24576, 32
+    g = torch.Generator(device="cuda").manual_seed(w + mean)
+    K1 = torch.randn(H, N, 128, generator=g, device="cuda") * (1.0 if not whole else 1.5) + mean
+    K1 = (K1.round().clamp(mean - 4, mean + 4) if whole else K1).to(torch.bfloat16)
+    K = K1[None, None].expand(1, L, H, N, 128)
+    Qw = torch.randn(1, L, H * G, w, 128, generator=g, device="cuda").to(torch.bfloat16)
+    ctx = ub.Context(ub.make_shape(1, L, H, H * G, N, 128, w, "bf16"))
+    if how == "lse":
+        from paper_2410_03090_b200.compress import CompressionPass
+        wl = replace(synth.WORKLOADS["c2"], L=L, H=H, Hq=H * G, N=N, w=w, avg_budget=100, M=1, n_max=100)
+        cp = CompressionPass(wl, "cuda")
+        cp.run_one_call(K, K, Qw, lse=torch.full((1, L, H * G, w), 20.0 + mean, device="cuda"))
+        ent = cp.out.entropy
+        assert cp.status() == 0
+    else:
+        ent, _ = ub.uncomp_entropy(ctx, K, k, Qw=Qw)
+        assert ub.uncomp_status(ctx) == 0
+    X = K1.double() - K1.double().mean(1, keepdim=True)
+    lam = torch.linalg.eigvalsh(X.transpose(1, 2) @ X).flip(1)[:, :k]
+    p = lam / lam.sum(1, keepdim=True)
+    want = -(p * p.log()).sum(1)
+    err = float((ent[0].double() - want).abs().max())
+    assert err <= (1e-6 if whole and mean == 40 else parity.ENTROPY_RTOL * float(want.min()))
