@@ -391,8 +391,10 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmapQ, const __grid_constant
             // Modes 2 and 3: the Gram MMAs of a tile only have to be issued before its stage is handed back, so they
             // are deferred by up to one tile: the latency-critical QK^T MMAs never queue behind them, and while the
             // tensor pipe works on them this thread finds out about the next tile and accumulator.
-            // One 128-row block per tile: three accumulators are three tiles ahead, nothing waits behind the Gram MMAs, and
-            // issuing them at once frees the stage earlier (c4: 2204 -> 2126 us); with more blocks the lag pays (c3: 866 -> 838).
+            // One 128-row block per tile: little waits behind the Gram MMAs, and issuing them at once frees the stage earlier
+            // (1024 units of 3712 tokens 188 us, 196 with the lag; 256 of 8192 124 and 127).  With more blocks the lag pays: two
+            // in mode 3 751 us with it, 758 without (256 units of 32768), four in mode 2 725 and 730 (32 units of 131072), two in
+            // mode 2 756 both.
             constexpr int kLag = MB == 1 ? 0 : 1;
             int g_done = 0;                    // tiles whose Gram MMAs are issued (and whose stage is released)
             auto issue_gram = [&]() {
