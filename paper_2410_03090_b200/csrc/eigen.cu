@@ -377,7 +377,7 @@ __device__ __forceinline__ void finish_unit64(ValueSmem &S, int u, double trace,
             }
         }
         if (active && sub == 0) {
-            lam[j] = 0.5 * (lo + hi) * scale;
+            lam[j] = lo > 0.0 ? 0.5 * (lo + hi) * scale : 0.0;      // what cannot be told from zero is zero
             if (hi - lo > tol) atomicOr(not_converged, 1);
         }
     }

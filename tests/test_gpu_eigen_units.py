@@ -48,3 +48,29 @@ def test_any_number_of_rounds(dtype, units, max_iters):
     got = ub.uncomp_entropy(ctx, K, 32, max_iters=max_iters, spectrum=spectra[1])
     assert ub.uncomp_status(ctx) == 0
     assert torch.equal(spectra[0], spectra[1]) and all(torch.equal(a, b) for a, b in zip(want, got))
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("units", [4, 18, 37, 60, 74, 75, 300])
+def test_keys_without_any_spread(units, dtype):
+    """All zero, or the same row for every token: no eigenvalue, entropy 0 and effective rank 1, beside units like any other."""
+    from paper_2410_03090_b200 import binding as ub
+
+    N = 200
+    g = torch.Generator(device="cuda").manual_seed(units)
+    K = torch.randn(1, units, 1, N, 128, generator=g, device="cuda")
+    K[0, 1] = 0
+    K[0, 2] = torch.randint(-8, 9, (128,), generator=g, device="cuda").float()
+    K[0, units - 1] = 3.0
+    K = K.to(torch.float32 if dtype == "fp32" else torch.bfloat16)
+    Qw = torch.randn(1, units, 1, 32, 128, generator=g, device="cuda").to(K.dtype)
+    ctx = ub.Context(ub.make_shape(1, units, 1, 1, N, 128, 32, dtype))
+    for k in (1, 32, 128):
+        for center in (0, 1):
+            for norm in (0, 1):
+                for q in (None, Qw) if dtype == "bf16" else (None,):
+                    ent, erank = ub.uncomp_entropy(ctx, K, k, center, norm, Qw=q)
+                    assert ub.uncomp_status(ctx) == 0
+                    for u in (1, 2, units - 1):        # without centring a constant row is one direction: entropy 0 as well
+                        assert abs(float(ent[0, u, 0])) < 1e-4 and abs(float(erank[0, u, 0]) - 1) < 1e-4, (u, k, center, norm)
+                    assert k == 1 or float(ent[0, 0, 0]) > 1
