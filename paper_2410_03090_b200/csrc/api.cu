@@ -495,9 +495,10 @@ int uncomp_compress(uncomp_ctx *ctx, const void *d_K, const void *d_V, uncomp_st
         if (e != cudaSuccess) return cuda_fail(ctx, e);
     } else if (tensor_path) {
         // Gram + statistics sweep; then eigenvalues and budgets beside the column sums: neither needs the other, only the
-        // selection needs both.  The two cannot share an SM (registers), so which one is launched first matters: with few
-        // units the eigenvalues are a chain on a few SMs and have to go first (one layer of 7001 tokens 138 us, 175 the other
-        // way round); with many the order makes no difference (1024 units of 3712 tokens 820 and 825 us, of 32K 5.03 ms both).
+        // selection needs both.  The two cannot share an SM (registers).  With few units the eigenvalues are a chain on a few SMs
+        // that the column sums leave free, with many either fills the GPU in turn, so which one is launched first makes no
+        // difference (one layer of 7001 tokens 118.5 and 118.7 us, 1024 units of 32768 tokens 5.12 and 5.14 ms, 16 random
+        // shapes within 0.5 %).
         cudaStream_t st = static_cast<cudaStream_t>(stream);
         cudaError_t e = ensure_side_stream(ctx);
         if (e != cudaSuccess) return cuda_fail(ctx, e);

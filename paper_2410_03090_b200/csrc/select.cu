@@ -212,8 +212,8 @@ pool_select_cluster_kernel(const float *__restrict__ raw, float *__restrict__ po
 // cluster barrier per histogram: every CTA adds up all of them, the next pass uses another array.
 // Bound by shared-memory atomics, barriers and, with many units, issue.  256 units of 32704 positions / 1024 of 3704 / 8
 // of 6969: radix select that read the pooled scores from global memory three times with 20 barriers a pass 75 / 61 / 23 us,
-// keys in registers and a search bit by bit with counts (no atomics, 20 to 30 rounds) 163 / 74 / 25 us, this 65 / 50 / 15 us
-// (128 of 131008: 133 us, was 201).
+// keys in registers and a search bit by bit with counts (no atomics, 20 to 30 rounds) 163 / 74 / 25 us, this 39 / 36 / 14 us
+// (128 of 131008: 101 us, was 201).
 constexpr int kKeyThreads = 1024;
 constexpr int kKeyWarps = kKeyThreads / 32;
 constexpr int kKeyMaxCluster = 8;
@@ -222,8 +222,8 @@ constexpr int kKeyBins = 2 * kKeyThreads;
 constexpr int kCandidates = 256;                         // keys ranked against one another instead of by another histogram
 // How the scores are pooled: width 1 takes them as they are; the 7-wide maximum, what the pass defaults to, from the four
 // scores of a lane and shuffles; any other width by a loop per position.  256 units of 32704 positions / 1024 of 3704 / 8 of
-// 6969: 53 / 41 / 15 us, 66 / 50 / 17 us, and by the loop 77 / 54 / 17 us for a maximum over 5, 82 / 54 / 18 over 9, 141 /
-// 72 / 23 over 63.
+// 6969: 33 / 31 / 13 us, 39 / 36 / 14 us, and by the loop 55 / 45 / 17 us for a maximum over 5, 54 / 44 / 17 over 9, 119 /
+// 72 / 25 over 63.
 enum { kPoolAny, kPoolNone, kPoolMax7 };
 
 template <int NBK> struct KeySmem {
@@ -584,8 +584,9 @@ cudaError_t launch_keys_nbk(const Plan &p, int n, int ctas, const float *d_raw, 
 cudaError_t launch_pool_select(const Plan &p, const float *d_raw, float *d_pooled, int pool_kernel, int pool_mode,
                                const int32_t *d_budgets, const int64_t *d_offsets, int32_t *d_indices,
                                uint32_t *d_status, cudaStream_t st) {
-    // 4096 positions per CTA and block of keys.  One CTA per unit up to 32768 positions (a cluster barrier costs a
-    // microsecond), clusters beyond; shorter shares only while most of the GPU would idle.
+    // 4096 positions per CTA and block of keys.  One CTA per unit up to 16384 positions (a cluster barrier costs a microsecond:
+    // 16 units of 16000 positions 17 us on one CTA, 20 on two), and up to 32768 unless most of the GPU would idle (8 units of
+    // 32768: 23 us on one or two, 21 on four); clusters beyond.
     const int n = (p.prefix + 4095) / 4096;
     if (n > 64) {
         return launch_kernel(pool_select_cluster_kernel, LaunchShape{dim3(p.units * kSelCluster), kSelThreads, 0, 1}, st,
@@ -593,7 +594,6 @@ cudaError_t launch_pool_select(const Plan &p, const float *d_raw, float *d_poole
                              d_indices, d_status);
     }
     int ctas = 1;
-    // (16 units of 16000 positions 17 us on one CTA, 20 on two; 8 of 32768 23 on one or two, 21 on four)
     while (ctas < kKeyMaxCluster && (n > 8 * ctas || (n > 4 && n > 2 * ctas && (int64_t)p.units * ctas * 2 <= kTargetSms))) ctas *= 2;
     const auto f = pool_kernel == 1 ? launch_keys_nbk<kPoolNone>
                                     : pool_kernel == 7 && pool_mode == 0 ? launch_keys_nbk<kPoolMax7> : launch_keys_nbk<kPoolAny>;

@@ -9,7 +9,7 @@
 //                        M = 128, N = 256 accumulators fill the 512 TMEM columns; partial blocks to scratch;
 //   3. assemble          C = G - s s^T / N (fp64 subtraction), stored as a full symmetric fp32 matrix;
 //   4. eigenvalues       up to 64 of a matrix of 384 and more: block Lanczos and Sturm counts of the projected band
-//                        matrix (wide_krylov.cu), 35 ms -> 1.4 ms at D = 4096, k = 32.  What that does not take or leaves
+//                        matrix (wide_krylov.cu), 35 ms -> 1.2 ms at D = 4096, k = 32.  What that does not take or leaves
 //                        unsettled goes through the two steps of the full reduction, whose kernels otherwise leave at once:
 //                        - Householder on the whole GPU: one cooperative launch, rows of the trailing matrix spread over all
 //                          warps, ONE grid barrier per column.  The rank-2 update of column k is applied while the matrix

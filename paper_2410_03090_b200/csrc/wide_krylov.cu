@@ -16,11 +16,11 @@
 //
 // Why: the reduction column by column sweeps the whole trailing matrix n times (33 ms at n = 4096), although only k of n
 // eigenvalues are wanted; here a step of 32 vectors reads the matrix once and 8 to 32 steps suffice (8192 x 4096 hidden
-// states with a decaying spectrum, k = 32: 8 steps, 0.68 ms, and the counts 0.29 ms; an isotropic matrix, the slowest to
+// states with a decaying spectrum, k = 32: 8 steps, 0.69 ms, and the counts 0.29 ms; an isotropic matrix, the slowest to
 // converge, takes 32).  Accuracy is that of fp32 products summed in fp32 / fp64, as in the reduction.
-// What bounds it, n = 4096, 84 us a step: the product 34 (1 MB per CTA from L2, 24 us without any arithmetic, and multiply-adds,
-// 21 us at the 100 per SM and cycle that an outer product in registers reaches), seven grid barriers and what they wait for 9,
-// sums over the CTAs 6, the two factorisations 8 and 4, H^T H 4, partial products 7, updates 7.  Three passes, sums with one
+// What bounds it, n = 4096, 85 us a step: the product 34 (1 MB per CTA from L2, 24 us without any arithmetic, and multiply-adds,
+// 21 us at the 100 per SM and cycle that an outer product in registers reaches), five grid barriers and what they wait for 9,
+// sums over the CTAs 6, the two factorisations 8 and 4, H^T H 5, partial products 7, updates 7.  Three passes, sums with one
 // load in flight, all of T by one CTA and smaller register tiles took 114.  The counts are bound by the latency of one warp
 // per scheduler (an instruction every 3.4 cycles); two warps per scheduler take 1000 cycles per row instead of 570 (8 x 8
 // tiles of the window in place of two rows per lane: 1200), so rows are saved by eliminating from both ends and rounds by
@@ -1034,9 +1034,11 @@ band_eigen_kernel(int k, int q, int max_iters, KrylovBuffers B, uint32_t *__rest
 }  // namespace
 
 // More than kKryMaxK = 64 eigenvalues go to the reduction: the range that the tests hold against the oracle, not where the
-// two sides meet.  That depends on the spectrum: 8192 x 4096 with 256 strong directions takes 2.2 ms here at k = 64, 5.0 at
-// 128, 11.5 at 256, the reduction 35.8 whatever k; an isotropic matrix of n = 2048 12.8 ms at k = 64 against 11.3.
-// kKryMinN: at n = 384 the buffers just hold the eight steps of k <= 32.
+// two sides meet.  That depends on the spectrum: 8192 x 4096 with 256 strong directions takes 1.6 ms here at k = 64, 4.8 at
+// 128, 7.4 at 256, the reduction 35.5 whatever k; an isotropic matrix of n = 2048 7.6 ms at k = 64 against 11.3.
+// kKryMinN: at n = 384 the buffers just hold the eight steps of k <= 32.  256 strong directions take 0.94 ms there (the
+// reduction 1.6), isotropic matrices, which leave the steps unsettled, 2.5; from n = 768 on those are faster here as well (3.2
+// and 3.3 ms; n = 1024 4.4 and 4.6, 4096 5.7 and 35.6).
 bool krylov_applies(int n, int k, int ctas) {
     return n >= kKryMinN && k <= kKryMaxK && krylov_steps(n) >= (k <= 32 ? 8 : 10) && n / kB <= ctas;
 }
@@ -1057,10 +1059,10 @@ cudaError_t launch_krylov(const float *C, int n, int k, int max_iters, const Kry
                           cudaStream_t st) {
     cudaError_t e = cudaSuccess;
     const int most = krylov_steps(n);
-    // Steps at first, and twice as many whenever some eigenvalue has not settled.  Nine spectra (256 strong directions, power
-    // laws, exponential, 50 and 600 directions, isotropic; n = 1024 to 4096), k = 32, all nine together: from 6 steps 28.8 ms,
-    // from 8 26.6, 10 32.1, 12 27.0, 16 32.8.  k = 64, the six of them that end here: from 8 29.8 ms, 10 24.8, 12 22.9,
-    // 16 26.3; 10 is the best of the two with 256 strong directions (2.2 and 1.7 ms against 2.6 and 2.1 from 12).
+    // Steps at first, and twice as many whenever some eigenvalue has not settled.  Ten spectra (256 strong directions, power
+    // laws, exponential, 50 and 600 directions, isotropic; n = 1024 to 4096), all together: k = 32 from 6 steps 22.1 ms, from 8
+    // 19.7, 10 20.7, 12 20.7, 16 24.6; k = 64 from 6 41.0, 8 38.2, 10 32.3, 12 32.0, 16 35.8, without the two isotropic ones
+    // 10 19.3 and 12 20.1.
     int part_blocks = most + 3, q0 = 0, q = k <= 32 ? 8 : 10, launch = 0;
     while (true) {
         unsigned *bar = b.bar + launch;
