@@ -31,14 +31,14 @@ if ROOT not in sys.path:
 # recorded beside them: when the file has changed since the capture, the bench prints null instead.
 NCU_COUNTERS = {
     "source": "paper_2410_03090_b200/csrc/scores_tc.cu",
-    "sha256": "63ec9cc4ca159417c73a7a1b5d6a6475d335ea14ff2ec4b43a4276ee1c29d6a2",
+    "sha256": "8d63120913f70eb85182711785d3d40a80c0a9e1366e49830b849aa8c8dcc1f7",
     "capture": "ncu --set full, one launch per kernel, c3 scaled to N 16384 x 10 layers; summary in profiles/",
     "kernels": {
-        "gram_score_stats": {"dram_bytes_per_unit_token": (344.470528e6 + 31.993088e6) / (80 * 16384),
-                             "tensor_pipe_pct": 53.9, "xu_pipe_pct": 70.6},
-        "score_colsum": {"dram_bytes_per_unit_token": (346.816000e6 + 11.107584e6) / (80 * 16384),
-                         "tensor_pipe_pct": 37.8, "xu_pipe_pct": 76.1},
-        "gram_score_colsum": {"dram_bytes_per_unit_token": (345.092096e6 + 34.181632e6) / (80 * 16384),
+        "gram_score_stats": {"dram_bytes_per_unit_token": (344.410624e6 + 32.759552e6) / (80 * 16384),
+                             "tensor_pipe_pct": 54.0, "xu_pipe_pct": 70.7},
+        "score_colsum": {"dram_bytes_per_unit_token": (346.801664e6 + 8.760576e6) / (80 * 16384),
+                         "tensor_pipe_pct": 37.7, "xu_pipe_pct": 76.0},
+        "gram_score_colsum": {"dram_bytes_per_unit_token": (345.160192e6 + 34.720768e6) / (80 * 16384),
                               "tensor_pipe_pct": 54.6, "xu_pipe_pct": 70.3},
     },
 }
