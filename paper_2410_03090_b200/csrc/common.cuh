@@ -170,7 +170,10 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), const LaunchShape &s, cud
         attr[cfg.numAttrs].val.clusterDim.y = attr[cfg.numAttrs].val.clusterDim.z = 1;
         ++cfg.numAttrs;
     }
-    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+    // a refused launch is this call's error; the runtime also keeps it as its last one, where the caller's next check would find it
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 // Optional per-kernel timing with CUDA events on the launching stream (host objects only).
