@@ -99,7 +99,7 @@ void uncomp_destroy(uncomp_ctx *ctx);
  * largest eigenvalues (bracketed to 2e-8 of the spectral radius; the fp32 reduction is good to about
  * 1e-7).  fp32 input: Gram matrix and eigenvalues in fp64 throughout (Householder in registers,
  * brackets to 1e-13 of the spectral radius).  max_iters bounds the multi-section rounds (0 = the default
- * of the path, 10 or 14); a unit that has not reached its tolerance by then sets
+ * of the path, 10 or 14; more than 64 are as good as 64); a unit that has not reached its tolerance by then sets
  * UNCOMP_STATUS_NOT_CONVERGED and still writes its current estimate.
  *
  * Fusion with the scorer: the window scorer (uncomp_score_select) also sweeps over K and needs, before
